@@ -541,10 +541,7 @@ template <typename T>
 bool launch_fused_any(const ep_grid *h, const Stage<T> &S, DevInfo *di, cudaStream_t st, bool check = false) {
   const int v = fused_variant(h);
   if (v == EP_KERNEL_FUSED_TMA) return launch_fused3d_tma<T>(h->g, S, h->dscal, di, h->kz, st);
-  if (v == EP_KERNEL_FUSED_REG) {
-    launch_fused3d_reg<T>(h->g, S, h->dscal, di, h->kz, st, check);
-    return true;
-  }
+  if (v == EP_KERNEL_FUSED_REG) return launch_fused3d_reg<T>(h->g, S, h->dscal, di, h->kz, st, check);
   launch_fused3d<T>(h->g, S, h->dscal, di, h->kz, st);
   return true;
 }

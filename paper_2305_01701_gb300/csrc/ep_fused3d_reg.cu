@@ -3,33 +3,53 @@
 //
 // Same arithmetic and z-march as ep_fused3d.cu (spin, relaxed trial, centre
 // return, edge return, velocity update; Eqs. A5, A23ssP, A2ssP, A6121lambda,
-// A22S, A22P), mapped so that almost no neighbour value goes through shared
+// A22S, A22P), mapped so that little but a plane's inputs goes through shared
 // memory:
 //   * a block covers a window of 32 x H columns (x, y) of the box and walks
-//     them through a chunk of z-planes; lane a owns window column x = i0-2+a,
-//     warp b owns row y = j0-2+b; the inner 28 x (H-4) columns are written;
-//   * x +- 1 neighbours are warp shuffles of registers;
+//     them through a chunk of z-planes; the inner 28 x (H-4) columns are
+//     written (the iteration couples columns two apart);
+//   * FP32: a thread owns two adjacent x columns as one float2 and half a
+//     warp owns a row (H = 24: 384 threads of 168 registers, the whole file);
+//     FP64: a thread owns one column, a warp a row;
+//   * a plane's 23 inputs arrive as TMA boxes (cp.async.bulk.tensor, zero
+//     outside the box) in one of two stages: plane t + 2 is asked for when
+//     every warp has read plane t, a whole plane before it is needed; each
+//     warp's elected thread issues its share;
+//   * x +- 1 neighbours are warp shuffles of registers (one per pair);
 //   * y +- 1 neighbours are rows of shared memory, each written once by its
 //     owner (two plane slots where a value is read one plane later);
-//   * z - 1 neighbours are registers carried from the previous plane;
-//   * inputs arrive through plain coalesced loads issued one plane ahead.
+//   * z - 1 neighbours are registers carried from the previous plane.
 // Plane t of the march computes spins at plane t, edge trials at face t and
 // plane t-1, centres t-1, edges t-1 and velocities t-2.  Three block barriers
-// separate the steps of a plane: the input rows of plane t+1 are published
-// before the third barrier of plane t, once every read of plane t's input
-// rows lies behind the second.
-// Instruction count (the kernel is issue-bound, not bandwidth-bound):
-//   * blocks whose whole window lies inside the domain run a copy of the body
-//     in which the domain-boundary tests are compile-time true;
-//   * FP32 loads take a clamped in-box address and no test: a value read
-//     outside the box only ever enters guarded expressions;
-//   * the march is unrolled by two planes, so the shared-memory slot of each
-//     copy is a compile-time constant;
+// separate the steps of a plane.
+// Bound: HBM in principle (132 B per cell); in fact the latency of a plane's
+// three steps at 12 warps per SM.  Measured (FP32, one sweep): 127^3 79.5 us,
+// 383^3 1600 us (4.6 TB/s), against 126.9 and 2312 us of the form with one
+// column per thread (16 warps, 600 instructions per warp and plane, register
+// prefetch).  Packing the pairs alone, with the register prefetch (8 warps of
+// 255 registers), halved the instructions and gained nothing: the loads'
+// latency showed.  cp.async in place of TMA cost 5 shared-memory wavefronts
+// per 8-byte copy (the window starts off a 32-byte sector): 131 and 2164 us.
+// Instruction count:
+//   * FP32 arithmetic is packed (add/mul/fma on float2: one instruction per
+//     pair);
+//   * a mean of four neighbours is a sum of two pair sums: the pair sum along
+//     x or z is formed once by its owner and shared (shuffle, shared row or
+//     carried register) by the two or three means that need it, and the
+//     factors 1/2, 1/4, 1/8 are folded into the coefficients (exact powers of
+//     two);
+//   * walls are factors of 0 and 1 per column on the spins, the trials and the
+//     velocity step, and blocks whose whole window lies inside the domain run
+//     a copy of the body without them: what a window's outermost columns and
+//     rows compute is never read by a written point;
+//   * the march is unrolled by two planes, so the stage and the slot of each
+//     copy are compile-time constants;
 //   * offsets within an array are 32-bit when the box has fewer than 2^31
-//     points (FP32), so an address is one wide multiply-add;
-//   * the warps of the window's first and last rows, whose centres are never
-//     read, skip the centre step, and the first row's warp skips the xz-edge
-//     and centre trials (rows are warp-uniform).
+//     points (FP32);
+//   * warps whose rows are never written skip the steps that only written
+//     rows need.
+// Waits are bounded: one that runs out marks the grid's record (status 4), the
+// block waits (bounded) for the copies in flight and returns.
 // Check iterations (FP32, CHK = true) also reduce the stopping measures of
 // Eqs. Convergence1-3 over the points each block writes, the same point sets
 // and the same snapshot updates as the staged check iteration: max|sigma|,
@@ -39,6 +59,7 @@
 // snapshot values a thread checks in a plane are copied to shared memory with
 // cp.async at the plane's start and read after the second barrier, so that
 // their memory latency hides behind the plane's first steps.
+#include <cuda.h>
 #include <math.h>
 
 #include <type_traits>
@@ -49,34 +70,111 @@ namespace ep {
 
 namespace {
 
-constexpr int WX = 32;       // window columns: one per lane
+constexpr int WX = 32;       // window columns
 constexpr int OX = WX - 4;   // written columns per block
 constexpr unsigned FULL = 0xffffffffu;
 
-template <typename T>
-__device__ __forceinline__ T xm(T v) { return __shfl_up_sync(FULL, v, 1); }    // value of column a - 1
-template <typename T>
-__device__ __forceinline__ T xp(T v) { return __shfl_down_sync(FULL, v, 1); }  // value of column a + 1
-
-// One plane slot of a row-exchanged value: rows -1 .. H of the window, so
-// that row b +- 1 is always in bounds (the two pad rows stay zero).
-template <typename T, int H>
-struct Rows {
-  T r[H + 2][WX];
+// ---- the columns of one thread -------------------------------------------
+// LaneF: two adjacent FP32 columns, 16 threads per row, H_ rows per block.
+// LaneD: one FP64 column, 32 threads per row, 8 rows per block.
+template <int H_>
+struct LaneF {
+  using T = float;
+  using V = float2;
+  static constexpr int N = 2, LPR = 16, H = H_;
+};
+struct LaneD {
+  using T = double;
+  using V = double;
+  static constexpr int N = 1, LPR = 32, H = 8;
 };
 
-template <typename T, int H>
+template <typename V>
+struct Splat;
+template <>
+struct Splat<float2> {
+  static __device__ __forceinline__ float2 of(float s) { return make_float2(s, s); }
+};
+template <>
+struct Splat<double> {
+  static __device__ __forceinline__ double of(double s) { return s; }
+};
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+// value of the column left / right of each column (a row's first column has
+// no left neighbour and gets an arbitrary value, the last no right one)
+__device__ __forceinline__ float2 xm(float2 v) { return make_float2(__shfl_up_sync(FULL, v.y, 1, 16), v.x); }
+__device__ __forceinline__ float2 xp(float2 v) { return make_float2(v.y, __shfl_down_sync(FULL, v.x, 1, 16)); }
+__device__ __forceinline__ double xm(double v) { return __shfl_up_sync(FULL, v, 1); }
+__device__ __forceinline__ double xp(double v) { return __shfl_down_sync(FULL, v, 1); }
+template <int E>
+__device__ __forceinline__ float el(float2 v) { return E == 0 ? v.x : v.y; }
+template <int E>
+__device__ __forceinline__ double el(double v) { return v; }
+
+// v off the domain's boundary, 0 on it: m holds 1 or 0 per column.  INT
+// windows have no boundary columns.
+template <bool INT, typename V>
+__device__ __forceinline__ V keep(V m, V v) {
+  return INT ? v : vmul(m, v);
+}
+
+// centre scale min(1, Y / sqrt(J2)).  FP32: compare squares and scale with
+// the reciprocal square root only where the return acts (most cells stay
+// elastic).
+__device__ __forceinline__ float scale_of(float J2, float Y) {
+  Y = Y > 0.f ? Y : 0.f;
+  return J2 > Y * Y ? Y * rsqrtf(J2) : 1.f;
+}
+__device__ __forceinline__ double scale_of(double J2, double Y) {
+  Y = Y > 0.0 ? Y : 0.0;
+  const double sj = sqrt(J2);
+  return sj > Y ? Y / sj : 1.0;
+}
+__device__ __forceinline__ float2 vscale(float2 J2, float2 Y) {
+  return make_float2(scale_of(J2.x, Y.x), scale_of(J2.y, Y.y));
+}
+__device__ __forceinline__ double vscale(double J2, double Y) { return scale_of(J2, Y); }
+
+// One plane slot of a value per thread, as rows of the window
+template <typename L>
+struct Rows {
+  typename L::V r[L::H * L::LPR];
+};
+
+// inputs of a plane: face/edge arrays of plane t, centre arrays of plane t - 1
+enum {
+  I_U0, I_U1, I_U2, I_RQ0, I_RQ1, I_RQ2, I_RD0, I_RD1, I_SOXZ, I_SOYZ, I_TBXZ, I_TBYZ,
+  I_SON0, I_SON1, I_SON2, I_TBN0, I_TBN1, I_TBN2, I_SOXY, I_TBXY, I_SOP, I_PB, I_YC,
+  I_COUNT
+};
+
+// columns of a TMA box: the window and two more on either side, so that its
+// first column is a multiple of 16 bytes
+constexpr int BX = WX + 4;
+
+template <typename L>
 struct SmemR {
-  Rows<T, H> u0, u2, rq2, oyz, tsxy;                    // read within the plane
-  Rows<T, H> u1[2], rq0[2], rq1[2], rd0[2], rd1[2];     // read at this plane and the next
-  Rows<T, H> oxy[2], oxz[2], pxy[2], pyz[2], tsyz[2];
-  Rows<T, H> s[2], syy[2], nxy[2], nyz[2];
+  alignas(128) typename L::T in[2][I_COUNT][L::H * BX];   // inputs of planes t and t + 1 (then t + 2)
+  Rows<L> A, D, I, K;               // sums of neighbouring inputs
+  Rows<L> B, E, wxz, M, pyz;        // pair sums of spins and rotation products
+  Rows<L> Q, Sz, U, Vs;             // pair sums of the edge trials and of the scales
+  Rows<L> syy[2], nxy[2], nyz[2];   // read one plane later
+  alignas(8) unsigned long long full[2];   // a stage's copies have arrived
+};
+
+struct Maps {
+  CUtensorMap m[I_COUNT];
 };
 
 template <typename T>
 struct Args {
-  const T *u[3], *rq[3], *rd[2];
-  const T *son[3], *sos[3], *sop, *tbn[3], *tbs[3], *pb, *yc;
   T *snn[3], *sns[3], *snp, *uo[3];
   T *s;   // centre return scales (read when plasticity is frozen, written by checks)
   T *cn[3], *cs[3], *cp, *uchk[3];   // state at the previous check (check iterations)
@@ -84,28 +182,53 @@ struct Args {
 };
 
 // a check iteration's snapshot values, one slot per thread, after SmemR
-template <typename T, int H>
+template <typename L>
 struct ChkSlots {
-  T cn[3][WX * H], cs[3][WX * H], cp[WX * H], uchk[3][WX * H];
-  double v0[3][WX * H];
+  static constexpr int NT = L::LPR * L::H;
+  double v0[3][NT * L::N];
+  typename L::V cn[3][NT], cs[3][NT], cp[NT], uchk[3][NT];
 };
 
-__device__ __forceinline__ void cp_async_el(float *smem, const float *gmem) {
+template <int BYTES>
+__device__ __forceinline__ void cp_async_el(void *smem, const void *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_el(double *smem, const double *gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::); }
 
+__device__ __forceinline__ unsigned su32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_expect(unsigned long long *b, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(su32(b)), "r"(bytes) : "memory");
+}
+// bounded wait for a phase of b: gives up after 2^31 SM cycles (about a
+// second, far above any copy's latency)
+__device__ __forceinline__ bool bar_wait(unsigned long long *b, unsigned parity) {
+  unsigned ok;
+  long long t0 = 0;
+  do {
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(su32(b)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    const long long now = clock64();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > (1ll << 31)) return false;
+  } while (true);
+}
+__device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int x, int y, int z,
+                                         unsigned long long *b) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n" ::
+          "r"(su32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(su32(b))
+      : "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ T maxt(T a, T b) { return (a > b || a != a) ? a : b; }
-// |x| in the type of x (no round trip through double for FP32)
 __device__ __forceinline__ float absv(float x) { return fabsf(x); }
-__device__ __forceinline__ double absv(double x) { return fabs(x); }
 
 // block-wide max of a non-negative value as its IEEE bits (integer order; a
 // NaN sorts above infinity), one atomic per block
@@ -135,364 +258,374 @@ __device__ __forceinline__ void block_max_bits(double v, unsigned long long *slo
 // INT: every column of the block's window lies strictly inside the domain
 // (1 <= x, y index <= n - 1), so the domain-boundary tests fold away.
 // Off: the integer type of offsets within an array.  CHK: a check iteration.
-template <typename T, int H, bool INT, typename Off, bool CHK>
-__device__ __forceinline__ void reg_body(const Args<T> &A, const Geo &g, const Scal *sc, DevInfo *di, bool frozen,
-                                         int kz, unsigned char *smem_raw) {
-  SmemR<T, H> &S = *reinterpret_cast<SmemR<T, H> *>(smem_raw);
-  ChkSlots<T, H> &C = *reinterpret_cast<ChkSlots<T, H> *>(smem_raw + sizeof(SmemR<T, H>));   // CHK only
-  constexpr int W = WX;
-  const int a = threadIdx.x & 31, b = threadIdx.x >> 5;
+template <typename L, bool INT, typename Off, bool CHK>
+__device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T> &A, const Geo &g, const Scal *sc, DevInfo *di,
+                                         bool frozen, int kz, unsigned char *smem_raw) {
+  using T = typename L::T;
+  using V = typename L::V;
+  constexpr int N = L::N, H = L::H, LPR = L::LPR;
+  SmemR<L> &S = *reinterpret_cast<SmemR<L> *>(smem_raw);
+  ChkSlots<L> &C = *reinterpret_cast<ChkSlots<L> *>(smem_raw + sizeof(SmemR<L>));   // CHK only
+  const int a = threadIdx.x % LPR, b = threadIdx.x / LPR;
   const int i0 = blockIdx.x * OX, j0 = blockIdx.y * (H - 4);
-  const int gi = i0 - 2 + a, gj = j0 - 2 + b;
+  const int gi = i0 - 2 + N * a, gj = j0 - 2 + b;   // first column of the thread, row
   const int kb = blockIdx.z * kz, ke = min(kb + kz, g.pz);
-  const int nz = g.nz, pz = g.pz;
+  const int nx = g.nx, ny = g.ny, nz = g.nz, pz = g.pz;
   const Off px = (Off)g.px, plane = (Off)g.plane;
-  const bool inb = INT || (gi >= 0 && gi < g.px && gj >= 0 && gj < g.py);
-  const bool gx1 = INT || (gi >= 1 && gi <= g.nx - 1), gy1 = INT || (gj >= 1 && gj <= g.ny - 1);
-  const bool gx0 = INT || (gi >= 0 && gi < g.nx), gy0 = INT || (gj >= 0 && gj < g.ny);
-  const bool gxl = INT || gi < g.nx, gyl = INT || gj < g.ny;
-  // this column's offset in a plane.  FP32 clamps it into the box so that
-  // loads need no test (a value outside the box only ever enters guarded
-  // expressions); every store and the frozen-scale read are guarded by
-  // in-box tests, where the clamped offset is the exact one.  FP64 keeps the
-  // tested loads (fewer registers).
-  const Off col = sizeof(T) == 4 ? (Off)min(max(gj, 0), g.py - 1) * px + (Off)min(max(gi, 0), g.px - 1)
-                                 : (inb ? (Off)gj * px + (Off)gi : (Off)0);
+  // inside the domain: x1, y1 a vertex/edge line off the walls; x0, y0 a centre
+  auto in_x1 = [&](int e) { return INT || (gi + e >= 1 && gi + e <= nx - 1); };
+  auto in_x0 = [&](int e) { return INT || (gi + e >= 0 && gi + e < nx); };
+  const bool gy1 = INT || (gj >= 1 && gj <= ny - 1), gy0 = INT || (gj >= 0 && gj < ny);
+  auto mask = [](bool e0, bool e1, T v) -> V {
+    if constexpr (N == 2) return make_float2(e0 ? v : (T)0, e1 ? v : (T)0);
+    else return e0 ? v : (T)0;
+  };
+  const V m_xy = mask(in_x1(0) && gy1, in_x1(1) && gy1, (T)1), m_xz = mask(in_x1(0) && gy0, in_x1(1) && gy0, (T)1),
+          m_yz = mask(in_x0(0) && gy1, in_x0(1) && gy1, (T)1);
+  const bool inb = INT || (gi >= 0 && gi < g.px && gj >= 0 && gj < g.py);   // px is a multiple of N
+  // this thread's offset in a plane, clamped into the box; every store and the
+  // frozen-scale read are guarded by in-box tests, where it is the exact one
+  const Off col = (Off)min(max(gj, 0), g.py - 1) * px + (Off)min(max(gi, 0), g.px - N);
 
-  const bool out_col = a >= 2 && a < W - 2 && b >= 2 && b < H - 2;
+  const bool out_col = N * a >= 2 && N * a < WX - 2 && b >= 2 && b < H - 2 && inb;
+  // rows of this warp: which steps some written row needs
+  constexpr int RPW = 32 / LPR;
+  const int b0 = (int)(threadIdx.x >> 5) * RPW, b1 = b0 + RPW - 1;
+  const bool w_edge = b1 >= 2, w_vel = b1 >= 2 && b0 < H - 2;
+
   const T rdx = (T)g.rdx, rdy = (T)g.rdy, rdz = (T)g.rdz;
-  const T two_eta = (T)sc->two_eta, bt = (T)sc->bt, ob = (T)1 - bt;
+  const T eta = (T)(0.5 * sc->two_eta), two_eta = (T)sc->two_eta, eta_d = (T)(-sc->two_eta / 3.0);
+  const T bt = (T)sc->bt, ob = (T)1 - bt;
   const T bp = (T)sc->bp, obp = (T)sc->obp, KDt = (T)sc->KDt, Acoef = (T)sc->A;
-  const T vs = (T)sc->vstep, qr = (T)0.25, third = (T)(1.0 / 3.0), hf = (T)0.5;
-  const int rb = b + 1;  // this thread's row in a Rows slot
+  const T vs = (T)sc->vstep, qr = (T)0.25, e8 = (T)0.125, e32 = (T)0.03125;
+  // velocity step of x-, y- and z-faces: 0 on the walls and off the extent
+  const V st0 = mask(in_x1(0) && gy0, in_x1(1) && gy0, vs), st1 = mask(in_x0(0) && gy1, in_x0(1) && gy1, vs),
+          st2 = mask(in_x0(0) && gy0, in_x0(1) && gy0, vs);
+  auto bc = [](T v) -> V { return Splat<V>::of(v); };   // the same value in every column
+  const V zero = bc((T)0);
+  // this thread's place in a Rows slot, and its row neighbours' (clamped: the
+  // window's first and last rows read a value that no written point uses)
+  const int bm = max(b - 1, 0), bq = min(b + 1, H - 1);
+  const int q0 = b * LPR + a, qm = bm * LPR + a, qp = bq * LPR + a;
+  const int p0 = b * BX + 2 + N * a, pm = bm * BX + 2 + N * a, pp = bq * BX + 2 + N * a;   // the same in a stage
 
-  // zero the pad rows (never written afterwards)
-  {
-    T *base = reinterpret_cast<T *>(smem_raw);
-    constexpr int n_rows = sizeof(SmemR<T, H>) / sizeof(Rows<T, H>);
-    for (int q = threadIdx.x; q < n_rows * 2 * WX; q += WX * H) {
-      const int slot = q / (2 * WX), rem = q % (2 * WX);
-      const int row = rem < WX ? 0 : H + 1;
-      base[(long long)slot * (H + 2) * WX + row * WX + (rem % WX)] = (T)0;
-    }
+  auto ldv = [&](const T *p, Off e) -> V { return __ldg(reinterpret_cast<const V *>(p + e)); };
+  auto stv = [&](T *p, Off e, V v) { *reinterpret_cast<V *>(p + e) = v; };
+  auto lev = [&](int k) -> Off { return (Off)min(max(k, 0), pz - 1) * plane + col; };
+
+  // the elected thread of each warp copies its share of a plane's input boxes
+  // into a stage: face/edge arrays of plane t, centre arrays of plane t - 1
+  constexpr int NW = LPR * H / 32;
+  constexpr unsigned BOX = H * BX * sizeof(T);
+  const int warp = threadIdx.x >> 5;
+  const bool elected = (threadIdx.x & 31) == 0;
+  auto fetch = [&](int t, const int stage) {
+    if (!elected) return;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    bar_expect(&S.full[stage], (unsigned)((I_COUNT - warp + NW - 1) / NW) * BOX);
+    for (int k = warp; k < I_COUNT; k += NW)
+      tma_load(S.in[stage][k], &M.m[k], i0 - 4, j0 - 2, k < I_SON0 ? t : t - 1, &S.full[stage]);
+  };
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 2; ++q)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(su32(&S.full[q])), "r"(NW) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-
-  auto ld = [&](const T *p, int lev) -> T {
-    if constexpr (sizeof(T) == 4) return __ldg(p + ((Off)min(max(lev, 0), pz - 1) * plane + col));
-    else return (inb && lev >= 0 && lev < pz) ? __ldg(p + ((Off)lev * plane + col)) : (T)0;
-  };
-
-  // inputs of the next plane (loaded one plane ahead)
-  T n_u0, n_u1, n_u2, n_rq0, n_rq1, n_rq2, n_rd0, n_rd1, n_soxz, n_soyz, n_tbxz, n_tbyz;
-  T n_son0, n_son1, n_son2, n_tbn0, n_tbn1, n_tbn2, n_soxy, n_tbxy, n_sop, n_pb, n_yc;
-  auto prefetch = [&](int t) {  // face/edge arrays of plane t, centre arrays of plane t - 1
-    n_u0 = ld(A.u[0], t); n_u1 = ld(A.u[1], t); n_u2 = ld(A.u[2], t);
-    n_rq0 = ld(A.rq[0], t); n_rq1 = ld(A.rq[1], t); n_rq2 = ld(A.rq[2], t);
-    n_rd0 = ld(A.rd[0], t); n_rd1 = ld(A.rd[1], t);
-    n_soxz = ld(A.sos[1], t); n_soyz = ld(A.sos[2], t); n_tbxz = ld(A.tbs[1], t); n_tbyz = ld(A.tbs[2], t);
-    const int c = t - 1;
-    n_son0 = ld(A.son[0], c); n_son1 = ld(A.son[1], c); n_son2 = ld(A.son[2], c);
-    n_tbn0 = ld(A.tbn[0], c); n_tbn1 = ld(A.tbn[1], c); n_tbn2 = ld(A.tbn[2], c);
-    n_soxy = ld(A.sos[0], c); n_tbxy = ld(A.tbs[0], c); n_sop = ld(A.sop, c); n_pb = ld(A.pb, c);
-    n_yc = ld(A.yc, c);
-  };
-  // the row-exchanged inputs of the prefetched plane, into its plane slot
-  auto publish = [&](const int slot) {
-    S.u0.r[rb][a] = n_u0; S.u2.r[rb][a] = n_u2; S.u1[slot].r[rb][a] = n_u1;
-    S.rq0[slot].r[rb][a] = n_rq0; S.rq1[slot].r[rb][a] = n_rq1; S.rq2.r[rb][a] = n_rq2;
-    S.rd0[slot].r[rb][a] = n_rd0; S.rd1[slot].r[rb][a] = n_rd1;
-  };
+  __syncthreads();
 
   // plane history (suffix: _1 plane t-1, _2 plane t-2, _3 plane t-3)
-  T u0 = 0, u1 = 0, u2 = 0, u0_1 = 0, u1_1 = 0, u2_1 = 0, u0_2 = 0, u1_2 = 0, u2_2 = 0;
-  T rq0 = 0, rq1 = 0, rq2 = 0, rd0 = 0, rd1 = 0, rq0_1 = 0, rq1_1 = 0, rq2_1 = 0, rd0_1 = 0, rd1_1 = 0;
-  T oxy_1 = 0, oxz_1 = 0, oyz_1 = 0, exy_1 = 0, pxy_1 = 0, pxz_1 = 0, pyz_1 = 0;
-  T tsxz_1 = 0, tsyz_1 = 0;
-  T s_2 = 0;                                   // centre scale, plane t-2
-  T sxx_2 = 0, syy_2 = 0, szz_2 = 0, szz_3 = 0;  // centre stress minus pressure
-  T nxy_2 = 0, nxz_2 = 0, nyz_2 = 0;           // edge stress, level t-2
+  V u0 = zero, u1 = zero, u2 = zero, u0_1 = zero, u1_1 = zero, u2_1 = zero, u0_2 = zero, u1_2 = zero, u2_2 = zero;
+  V rq0 = zero;
+  V D_1 = zero, E_1 = zero, F_1 = zero, G_1 = zero, J_1 = zero, L_1 = zero, M_1 = zero, N_1 = zero, O_1 = zero;
+  V wxy_1 = zero, qxy_1 = zero, e1_1 = zero, tsxz_1 = zero, tsyz_1 = zero;
+  V s_2 = zero, U_2 = zero;                                // quarter scale and its x pair sum, plane t-2
+  V sxx_2 = zero, syy_2 = zero, szz_2 = zero, szz_3 = zero;   // centre stress minus pressure
+  V nxy_2 = zero, nxz_2 = zero, nyz_2 = zero;              // edge stress, level t-2
   // check iterations: the stopping measures over this block's points
   T c_sig = 0, c_dtau = 0, c_dp = 0, c_r = 0, c_du = 0;
   double c_vm = 0.0;
 
-  prefetch(kb - 2);
-  publish(0);
-  __syncthreads();
+  fetch(kb - 2, 0);
+  fetch(kb - 1, 1);
+  unsigned ph[2] = {0u, 0u};   // the phase of each stage that is waited for next
+  // wait until a stage's copies have arrived; false once a wait has run out
+  // anywhere in the block: the record then says so and the copies in flight
+  // (a plane in each stage at most) have been waited for
+  auto arrived = [&](const int stage, bool other) -> bool {
+    const bool ok = bar_wait(&S.full[stage], ph[stage]);
+    ph[stage] ^= 1u;
+    if (!__syncthreads_or(!ok)) return true;
+    if (threadIdx.x == 0 && di != nullptr) di->done = 4;
+    if (!ok) bar_wait(&S.full[stage], ph[stage] ^ 1u);
+    if (other) bar_wait(&S.full[stage ^ 1], ph[stage ^ 1]);
+    return false;
+  };
+  if (!arrived(0, true)) return;
   // the march unrolled by two planes: the slot parity of each copy is a
   // compile-time constant
-  auto plane_step = [&](const int t, auto slc) {
+  auto plane_step = [&](const int t, auto slc) -> bool {
     constexpr int sl = decltype(slc)::value, sl1 = sl ^ 1;  // plane slots of t and t - 1
-    // ---- 0. take this plane's inputs (their rows are already published) ----
+    auto own = [&](int k) -> V { return *reinterpret_cast<const V *>(&S.in[sl][k][p0]); };
+    auto below = [&](int k) -> V { return *reinterpret_cast<const V *>(&S.in[sl][k][pm]); };   // row y - 1
+    auto above = [&](int k) -> V { return *reinterpret_cast<const V *>(&S.in[sl][k][pp]); };   // row y + 1
+    // ---- 0. take this plane's inputs (they lie in its stage) ----
     u0_2 = u0_1; u1_2 = u1_1; u2_2 = u2_1;
     u0_1 = u0; u1_1 = u1; u2_1 = u2;
-    u0 = n_u0; u1 = n_u1; u2 = n_u2;
-    rq0_1 = rq0; rq1_1 = rq1; rq2_1 = rq2; rd0_1 = rd0; rd1_1 = rd1;
-    rq0 = n_rq0; rq1 = n_rq1; rq2 = n_rq2; rd0 = n_rd0; rd1 = n_rd1;
-    const T soxz = n_soxz, soyz = n_soyz, tbxz = n_tbxz, tbyz = n_tbyz;
-    const T son0 = n_son0, son1 = n_son1, son2 = n_son2, tbn0 = n_tbn0, tbn1 = n_tbn1, tbn2 = n_tbn2;
-    const T soxy = n_soxy, tbxy = n_tbxy, sop = n_sop, pb = n_pb, yc = n_yc;
-    const bool more = t + 1 < ke + 2;
-    if (more) prefetch(t + 1);
+    u0 = own(I_U0); u1 = own(I_U1); u2 = own(I_U2);
+    const V rq0_1 = rq0, rq1 = own(I_RQ1), rq2 = own(I_RQ2);
+    rq0 = own(I_RQ0);
+    // sums of inputs: A = rq0 over planes t-1, t; D = rq2, I = rd0, J = rd1
+    // over columns x-1, x; K = rd1 - rd0
+    const V rd0 = own(I_RD0), rd1 = own(I_RD1);
+    const V vA = vadd(rq0_1, rq0), D = vadd(rq2, xm(rq2)), vI = vadd(rd0, xm(rd0)), J = vadd(rd1, xm(rd1));
+    const V vK = vsub(rd1, rd0);
+    S.A.r[q0] = vA; S.D.r[q0] = D; S.I.r[q0] = vI; S.K.r[q0] = vK;
     if constexpr (CHK) {   // the snapshot values checked at this plane: levels t-1 (centres, edges), t-2 (faces)
       const int tid = threadIdx.x;
-      const Off e1 = (Off)min(max(t - 1, 0), pz - 1) * plane + col, e2 = (Off)min(max(t - 2, 0), pz - 1) * plane + col;
+      const Off e1 = lev(t - 1), e2 = lev(t - 2);
+      constexpr int VB = (int)sizeof(V);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        cp_async_el(&C.cn[d][tid], A.cn[d] + e1);
-        cp_async_el(&C.cs[d][tid], A.cs[d] + e1);
-        cp_async_el(&C.uchk[d][tid], A.uchk[d] + e2);
-        cp_async_el(&C.v0[d][tid], A.v0[d] + e2);
+        cp_async_el<VB>(&C.cn[d][tid], A.cn[d] + e1);
+        cp_async_el<VB>(&C.cs[d][tid], A.cs[d] + e1);
+        cp_async_el<VB>(&C.uchk[d][tid], A.uchk[d] + e2);
+        cp_async_el<8 * N>(&C.v0[d][N * tid], A.v0[d] + e2);
       }
-      cp_async_el(&C.cp[tid], A.cp + e1);
+      cp_async_el<VB>(&C.cp[tid], A.cp + e1);
       cp_async_commit();
     }
+    const bool zf = t >= 1 && t <= nz - 1;   // face t carries xz/yz edges inside the domain
 
-    // ---- 1. shear strain rates and spins at plane t (xy) / face t (xz, yz) ----
-    T exy = 0, oxy = 0, exz = 0, oxz = 0, eyz = 0, oyz = 0;
+    // ---- 1. shear strain rates g = 2 eps and spins w = 2 omega at plane t
+    //         (xy) / face t (xz, yz) ----
+    V gxy, wxy, gxz, wxz, gyz, wyz;
     {
-      const T u0_ym = S.u0.r[rb - 1][a], u2_ym = S.u2.r[rb - 1][a];
-      const T u1_xm = xm(u1), u2_xm = xm(u2);
-      if (a >= 1 && b >= 1 && t >= 0 && t < nz && gx1 && gy1) {
-        const T x = (u0 - u0_ym) * rdy, y = (u1 - u1_xm) * rdx;
-        exy = hf * (x + y); oxy = hf * (x - y);
-      }
-      if (a >= 1 && t >= 1 && t <= nz - 1 && gx1 && gy0) {
-        const T x = (u0 - u0_1) * rdz, y = (u2 - u2_xm) * rdx;
-        exz = hf * (x + y); oxz = hf * (x - y);
-      }
-      if (b >= 1 && t >= 1 && t <= nz - 1 && gx0 && gy1) {
-        const T x = (u1 - u1_1) * rdz, y = (u2 - u2_ym) * rdy;
-        eyz = hf * (x + y); oyz = hf * (x - y);
-      }
+      const V u0_ym = below(I_U0), u2_ym = below(I_U2);
+      V x = vmul(vsub(u0, u0_ym), bc(rdy)), y = vsub(u1, xm(u1));
+      gxy = vfma(y, bc(rdx), x);
+      wxy = keep<INT>(m_xy, vfma(y, bc(-rdx), x));
+      x = vmul(vsub(u0, u0_1), bc(rdz)); y = vsub(u2, xm(u2));
+      gxz = vfma(y, bc(rdx), x);
+      wxz = keep<INT>(m_xz, vfma(y, bc(-rdx), x));
+      x = vmul(vsub(u1, u1_1), bc(rdz)); y = vsub(u2, u2_ym);
+      gyz = vfma(y, bc(rdy), x);
+      wyz = keep<INT>(m_yz, vfma(y, bc(-rdy), x));
+      if (t < 0 || t >= nz) wxy = zero;
+      if (!zf) { wxz = zero; wyz = zero; }
     }
-    const T pxy = rq0 * oxy, pxz = rq1 * oxz, pyz = rq2 * oyz;  // rotation products
-    S.oxy[sl].r[rb][a] = oxy; S.oxz[sl].r[rb][a] = oxz; S.oyz.r[rb][a] = oyz;
-    S.pxy[sl].r[rb][a] = pxy; S.pyz[sl].r[rb][a] = pyz;
+    // rotation products (2 rq omega) and the pair sums that their means and
+    // the spin means share
+    const V pxy = vmul(rq0, wxy), pxz = vmul(rq1, wxz), pyz = vmul(rq2, wyz);
+    const V vB = vadd(wxy_1, wxy), vE = vadd(wyz, xm(wyz)), vM = vadd(pxy, xp(pxy)), vN = vadd(pxz, xp(pxz));
+    S.B.r[q0] = vB; S.E.r[q0] = vE; S.wxz.r[q0] = wxz; S.M.r[q0] = vM; S.pyz.r[q0] = pyz;
     __syncthreads();
 
     // ---- 2. relaxed trials: faces t (xz, yz), plane t-1 (xy, centres) ----
     const int lc = t - 1;
-    T tsxz = 0, tsyz = 0, tsxy = 0, c0v = 0, c1v = 0, c2v = 0, exx = 0, eyy = 0, ezz = 0;
+    const bool zc = lc >= 0 && lc < nz;
+    V tsxz, tsyz, tsxy, c0v, c1v, c2v, div;
+    const V sop = own(I_SOP), pb = own(I_PB), yc = own(I_YC);
     {
-      // shuffles run on every lane, outside the validity branches
-      const T rd1_1_xm = xm(rd1_1), rd1_xm = xm(rd1), rd0_1_xm = xm(rd0_1);
-      const T rq2_xm = xm(rq2), rq2_1_xm = xm(rq2_1), oyz_xm = xm(oyz), oyz_1_xm = xm(oyz_1);
-      const T rq2_yp = S.rq2.r[rb + 1][a], oyz_yp = S.oyz.r[rb + 1][a];
-      const T rq2_yp_xm = xm(rq2_yp), oyz_yp_xm = xm(oyz_yp);
-      const T rq0_1_yp = S.rq0[sl1].r[rb + 1][a], rq0_yp = S.rq0[sl].r[rb + 1][a];
-      const T oxy_1_yp = S.oxy[sl1].r[rb + 1][a], oxy_yp = S.oxy[sl].r[rb + 1][a];
-      const T rq0_1_xp = xp(rq0_1), rq0_xp = xp(rq0), oxy_1_xp = xp(oxy_1), oxy_xp = xp(oxy);
-      const T rq1_ym = S.rq1[sl].r[rb - 1][a], oxz_ym = S.oxz[sl].r[rb - 1][a];
-      const T rq1_xp = xp(rq1), oxz_xp = xp(oxz), rq1_ym_xp = xp(rq1_ym), oxz_ym_xp = xp(oxz_ym);
-      const T rd0_1_ym = S.rd0[sl1].r[rb - 1][a], rd1_1_ym = S.rd1[sl1].r[rb - 1][a];
-      const T rd0_ym = S.rd0[sl].r[rb - 1][a], rd1_ym = S.rd1[sl].r[rb - 1][a];
-      const T rd0_1_ym_xm = xm(rd0_1_ym);
-      const T rq1_1_ym = S.rq1[sl1].r[rb - 1][a], oxz_1_ym = S.oxz[sl1].r[rb - 1][a];
-      const T u0_1_xp = xp(u0_1), u1_1_yp = S.u1[sl1].r[rb + 1][a];
-      const T pxy_1_xp = xp(pxy_1), pxy_1_yp = S.pxy[sl1].r[rb + 1][a];
-      const T pxy_1_yp_xp = xp(pxy_1_yp);
-      const T pxz_1_xp = xp(pxz_1), pxz_xp = xp(pxz);
-      const T pyz_1_yp = S.pyz[sl1].r[rb + 1][a], pyz_yp = S.pyz[sl].r[rb + 1][a];
-
-      if (b >= 1 && b < H - 1 && t >= 1 && t <= nz - 1)
-      if (a >= 1 && gx1 && gy0) {
-        const T dzx = qr * (rd1_1_xm + rd1_1 + rd1_xm + rd1);
-        const T Tyz = qr * (rq2_xm + rq2 + rq2_yp_xm + rq2_yp);
-        const T Wyz = qr * (oyz_xm + oyz + oyz_yp_xm + oyz_yp);
-        const T Txy = qr * (rq0_1 + rq0_1_yp + rq0 + rq0_yp);
-        const T Wxy = qr * (oxy_1 + oxy_1_yp + oxy + oxy_yp);
-        const T tr = tbxz + two_eta * exz + (oxz * dzx + Tyz * Wxy - Txy * Wyz);
-        tsxz = bt * soxz + ob * tr;
+      const V F = vadd(rq1, below(I_RQ1)), G = vadd(wxz, S.wxz.r[qm]);   // over rows y-1, y
+      const V Lz = vadd(vK, S.K.r[qm]), dyx = vadd(vI, S.I.r[qm]);
+      {   // xz: w dzx + (Tyz Wxy - Txy Wyz) / 4, in units of 1/8
+        const V Dz = vadd(J_1, J), Tyz = vadd(D, S.D.r[qp]), Wyz = vadd(vE, S.E.r[qp]);
+        const V Txy = vadd(vA, S.A.r[qp]), Wxy = vadd(vB, S.B.r[qp]);
+        const V r1 = vsub(vmul(Tyz, Wxy), vmul(Txy, Wyz));
+        const V r = vfma(r1, bc(qr), vmul(wxz, Dz));
+        const V tr = vfma(r, bc(e8), vfma(gxz, bc(eta), own(I_TBXZ)));
+        tsxz = keep<INT>(m_xz, vfma(own(I_SOXZ), bc(bt), vmul(tr, bc(ob))));
       }
-      if (b >= 1 && t >= 1 && t <= nz - 1)
-      if (a < W - 1 && gx0 && gy1) {
-        const T dzy = qr * ((rd1_1_ym - rd0_1_ym) + (rd1_1 - rd0_1) + (rd1_ym - rd0_ym) + (rd1 - rd0));
-        const T Txy = qr * (rq0_1 + rq0_1_xp + rq0 + rq0_xp);
-        const T Wxy = qr * (oxy_1 + oxy_1_xp + oxy + oxy_xp);
-        const T Txz = qr * (rq1_ym + rq1_ym_xp + rq1 + rq1_xp);
-        const T Wxz = qr * (oxz_ym + oxz_ym_xp + oxz + oxz_xp);
-        const T tr = tbyz + two_eta * eyz + (oyz * dzy - Txy * Wxz - Txz * Wxy);
-        tsyz = bt * soyz + ob * tr;
+      {   // yz: w dzy - (Txy Wxz + Txz Wxy) / 4
+        const V Dz = vadd(L_1, Lz), Txy = vadd(vA, xp(vA)), Wxy = vadd(vB, xp(vB));
+        const V Txz = vadd(F, xp(F)), Wxz = vadd(G, xp(G));
+        const V r1 = vfma(Txz, Wxy, vmul(Txy, Wxz));
+        const V r = vfma(r1, bc(-qr), vmul(wyz, Dz));
+        const V tr = vfma(r, bc(e8), vfma(gyz, bc(eta), own(I_TBYZ)));
+        tsyz = keep<INT>(m_yz, vfma(own(I_SOYZ), bc(bt), vmul(tr, bc(ob))));
       }
-      if (b >= 1 && lc >= 0 && lc < nz)
-      if (a >= 1 && gx1 && gy1) {
-        const T dyx = qr * (rd0_1_ym_xm + rd0_1_ym + rd0_1_xm + rd0_1);
-        const T Tyz = qr * (rq2_1_xm + rq2_1 + rq2_xm + rq2);
-        const T Wyz = qr * (oyz_1_xm + oyz_1 + oyz_xm + oyz);
-        const T Txz = qr * (rq1_1_ym + rq1_1 + rq1_ym + rq1);
-        const T Wxz = qr * (oxz_1_ym + oxz_1 + oxz_ym + oxz);
-        const T tr = tbxy + two_eta * exy_1 + (oxy_1 * dyx + Tyz * Wxz + Txz * Wyz);
-        tsxy = bt * soxy + ob * tr;
+      if (!zf) { tsxz = zero; tsyz = zero; }
+      {   // xy of plane t-1: w dyx + (Tyz Wxz + Txz Wyz) / 4
+        const V Tyz = vadd(D_1, D), Wyz = vadd(E_1, vE), Txz = vadd(F_1, F), Wxz = vadd(G_1, G);
+        const V r1 = vfma(Tyz, Wxz, vmul(Txz, Wyz));
+        const V tr = vfma(r1, bc(e32), vadd(own(I_TBXY), qxy_1));
+        tsxy = keep<INT>(m_xy, vfma(own(I_SOXY), bc(bt), vmul(tr, bc(ob))));
+        if (!zc) tsxy = zero;
+        // this plane's part of the next plane's xy trial
+        qxy_1 = vfma(gxy, bc(eta), vmul(vmul(wxy, dyx), bc(e8)));
       }
-      if (b >= 1 && b < H - 1 && lc >= 0 && lc < nz)
-      if (a < W - 1 && gx0 && gy0) {
-        exx = (u0_1_xp - u0_1) * rdx;
-        eyy = (u1_1_yp - u1_1) * rdy;
-        ezz = (u2 - u2_1) * rdz;
-        const T d3 = (exx + eyy + ezz) * third;
-        const T Pxy = qr * (pxy_1 + pxy_1_xp + pxy_1_yp + pxy_1_yp_xp);
-        const T Pxz = qr * (pxz_1 + pxz_1_xp + pxz + pxz_xp);
-        const T Pyz = qr * (pyz_1 + pyz_1_yp + pyz + pyz_yp);
-        const T t0 = tbn0 + two_eta * (exx - d3) + (T)2 * (Pxy + Pxz);
-        const T t1 = tbn1 + two_eta * (eyy - d3) - (T)2 * (Pxy - Pyz);
-        const T t2 = tbn2 + two_eta * (ezz - d3) - (T)2 * (Pxz + Pyz);
-        c0v = bt * son0 + ob * t0;
-        c1v = bt * son1 + ob * t1;
-        c2v = bt * son2 + ob * t2;
+      {   // centres of plane t-1
+        const V e0 = vmul(vsub(xp(u0_1), u0_1), bc(rdx));
+        const V e1 = e1_1;
+        const V e2 = vmul(vsub(u2, u2_1), bc(rdz));
+        div = vadd(vadd(e0, e1), e2);
+        const V O = vadd(pyz, S.pyz.r[qp]);
+        const V Pxz = vadd(N_1, vN), Pyz = vadd(O_1, O), Pxy = M_1;
+        const V m = vmul(div, bc(eta_d));
+        const V te = bc(two_eta), q = bc(qr);
+        const V t0 = vfma(vadd(Pxy, Pxz), q, vadd(own(I_TBN0), vfma(e0, te, m)));
+        const V t1 = vfma(vsub(Pyz, Pxy), q, vadd(own(I_TBN1), vfma(e1, te, m)));
+        const V t2 = vfma(vadd(Pxz, Pyz), bc(-qr), vadd(own(I_TBN2), vfma(e2, te, m)));
+        c0v = vfma(own(I_SON0), bc(bt), vmul(t0, bc(ob)));
+        c1v = vfma(own(I_SON1), bc(bt), vmul(t1, bc(ob)));
+        c2v = vfma(own(I_SON2), bc(bt), vmul(t2, bc(ob)));
+        e1_1 = vmul(vsub(above(I_U1), u1), bc(rdy));
+        M_1 = vadd(vM, S.M.r[qp]);
+        N_1 = vN; O_1 = O;
       }
+      D_1 = D; E_1 = vE; F_1 = F; G_1 = G; J_1 = J; L_1 = Lz;
     }
-    S.tsxy.r[rb][a] = tsxy; S.tsyz[sl].r[rb][a] = tsyz;
+    const V vQ = vadd(tsxy, xp(tsxy)), vS = vadd(tsyz_1, tsyz);
+    S.Q.r[q0] = vQ; S.Sz.r[q0] = vS;
     __syncthreads();
+
+    // every read of plane t's inputs lies behind the second barrier: their
+    // stage takes plane t + 2
+    if (t + 2 < ke + 2) fetch(t + 2, sl);
+    if constexpr (CHK) cp_async_wait_all();   // this thread's own snapshot slots
 
     // ---- 3. pressure and return at the centres of plane t-1 ----
-    T s_1 = 0, sxx_1 = 0, syy_1 = 0, szz_1 = 0;
-    if constexpr (CHK) cp_async_wait_all();   // this thread's own slots
-    if (b >= 1 && b < H - 1) {
-      const T tsxy_xp = xp(tsxy), tsxy_yp = S.tsxy.r[rb + 1][a];
-      const T tsxy_yp_xp = xp(tsxy_yp);
-      const T tsxz_1_xp = xp(tsxz_1), tsxz_xp = xp(tsxz);
-      const T tsyz_1_yp = S.tsyz[sl1].r[rb + 1][a], tsyz_yp = S.tsyz[sl].r[rb + 1][a];
-      if (b >= 1 && b < H - 1 && lc >= 0 && lc < nz)
-      if (a >= 1 && a < W - 1 && gx0 && gy0) {
-        const T div = exx + eyy + ezz;
-        const T pr = bp * sop + obp * (pb - KDt * div);
-        const T txy = qr * (tsxy + tsxy_xp + tsxy_yp + tsxy_yp_xp);
-        const T txz = qr * (tsxz_1 + tsxz_1_xp + tsxz + tsxz_xp);
-        const T tyz = qr * (tsyz_1 + tsyz_1_yp + tsyz + tsyz_yp);
-        const T J2 = txy * txy + txz * txz + tyz * tyz + hf * c0v * c0v + hf * c1v * c1v + hf * c2v * c2v;
-        if (frozen) {
-          s_1 = A.s[(Off)lc * plane + col];
-        } else {
-          T Y = Acoef * pr + yc;
-          Y = Y > (T)0 ? Y : (T)0;
-          if (sizeof(T) == 4) {
-            // FP32: compare squares and scale with the reciprocal square root
-            // only where the return acts (most cells stay elastic)
-            s_1 = J2 > Y * Y ? (T)(Y * rsqrtf((float)J2)) : (T)1;
-          } else {
-            const T sj = sqrt(J2);
-            s_1 = sj > Y ? Y / sj : (T)1;
-          }
-        }
-        const T n0 = s_1 * c0v, n1 = s_1 * c1v, n2 = s_1 * c2v;
-        sxx_1 = n0 - pr; syy_1 = n1 - pr; szz_1 = n2 - pr;
-        if (out_col && lc >= kb && lc < ke) {
-          const Off ec = (Off)lc * plane + col;
-          A.snn[0][ec] = n0; A.snn[1][ec] = n1; A.snn[2][ec] = n2; A.snp[ec] = pr;
-          if constexpr (CHK) {   // a centre of the box (lc < nz, gi < nx, gj < ny hold here)
-            if (!frozen) A.s[ec] = s_1;
-            c_sig = maxt(c_sig, maxt(absv(n0 - pr), maxt(absv(n1 - pr), absv(n2 - pr))));
-            const int tid = threadIdx.x;
-            c_dtau = maxt(c_dtau, maxt(absv(n0 - C.cn[0][tid]),
-                                       maxt(absv(n1 - C.cn[1][tid]), absv(n2 - C.cn[2][tid]))));
-            c_dp = maxt(c_dp, absv(pr - C.cp[tid]));
-            A.cn[0][ec] = n0; A.cn[1][ec] = n1; A.cn[2][ec] = n2; A.cp[ec] = pr;
-            if (isnan(s_1) || isnan(pr)) c_sig = (T)NAN;
-          }
+    V s_1, sxx_1, syy_1, szz_1;
+    {
+      const V pr = vfma(sop, bc(bp), vmul(vfma(div, bc(-KDt), pb), bc(obp)));
+      const V R = vadd(tsxz_1, tsxz);
+      const V xy = vadd(vQ, S.Q.r[qp]), xz = vadd(R, xp(R)), yz = vadd(vS, S.Sz.r[qp]);
+      const V j4 = vfma(yz, yz, vfma(xz, xz, vmul(xy, xy)));        // 16 x the shear part
+      const V jn = vfma(c2v, c2v, vfma(c1v, c1v, vmul(c0v, c0v)));  // 2 x the normal part
+      const V J2 = vfma(j4, bc((T)0.0625), vmul(jn, bc((T)0.5)));
+      V sc1;
+      if (frozen) sc1 = ldv(A.s, lev(lc));
+      else sc1 = vscale(J2, vfma(pr, bc(Acoef), yc));
+      const V n0 = vmul(sc1, c0v), n1 = vmul(sc1, c1v), n2 = vmul(sc1, c2v);
+      sxx_1 = vsub(n0, pr); syy_1 = vsub(n1, pr); szz_1 = vsub(n2, pr);
+      if (out_col && lc >= kb && lc < ke && zc && gy0 && in_x0(0)) {
+        const Off ec = (Off)lc * plane + col;
+        // the last pair of a row can lie half outside: its second column stays as it is
+        auto stc = [&](T *p, V v) {
+          if (N == 1 || in_x0(1)) stv(p, ec, v);
+          else p[ec] = el<0>(v);
+        };
+        stc(A.snn[0], n0); stc(A.snn[1], n1); stc(A.snn[2], n2); stc(A.snp, pr);
+        if constexpr (CHK) {   // the centres of the box
+          if (!frozen) stc(A.s, sc1);
+          const int tid = threadIdx.x;
+          auto one = [&](auto ic) {
+            constexpr int E = decltype(ic)::value;
+            if (!in_x0(E)) return;
+            const T p_ = el<E>(pr), a0 = el<E>(n0), a1 = el<E>(n1), a2 = el<E>(n2);
+            c_sig = maxt(c_sig, maxt(absv(a0 - p_), maxt(absv(a1 - p_), absv(a2 - p_))));
+            c_dtau = maxt(c_dtau, maxt(absv(a0 - el<E>(C.cn[0][tid])),
+                                       maxt(absv(a1 - el<E>(C.cn[1][tid])), absv(a2 - el<E>(C.cn[2][tid])))));
+            c_dp = maxt(c_dp, absv(p_ - el<E>(C.cp[tid])));
+            if (isnan(el<E>(sc1)) || isnan(p_)) c_sig = (T)NAN;
+          };
+          one(std::integral_constant<int, 0>{});
+          if constexpr (N == 2) one(std::integral_constant<int, 1>{});
+          stc(A.cn[0], n0); stc(A.cn[1], n1); stc(A.cn[2], n2); stc(A.cp, pr);
         }
       }
+      s_1 = vmul(sc1, bc(qr));
     }
-    S.s[sl1].r[rb][a] = s_1; S.syy[sl1].r[rb][a] = syy_1;
-    // every read of plane t's input rows lies behind the second barrier
-    if (more) publish(sl1);
-    __syncthreads();
+    const V vU = vadd(s_1, xm(s_1)), vV = vadd(s_2, s_1);   // quarter scales over x-1, x / planes t-2, t-1
+    S.U.r[q0] = vU; S.Vs.r[q0] = vV; S.syy[sl1].r[q0] = syy_1;
+    if (t + 1 < ke + 2) {   // plane t + 1 is needed next
+      if (!arrived(sl1, t + 2 < ke + 2)) return false;
+    } else {
+      __syncthreads();
+    }
 
     // ---- 4. new edge deviators at level t-1 ----
-    T nxy_1 = 0, nxz_1 = 0, nyz_1 = 0;
-    {
-      const T s_1_xm = xm(s_1), s_2_xm = xm(s_2);
-      const T s_1_ym = S.s[sl1].r[rb - 1][a], s_2_ym = S.s[sl].r[rb - 1][a];
-      const T s_1_ym_xm = xm(s_1_ym);
-      const bool inner = a >= 2 && a < W - 1 && b >= 2 && b < H - 1;
-      if (inner && lc >= 0 && lc < nz && gx1 && gy1)
-        nxy_1 = qr * (s_1_ym_xm + s_1_ym + s_1_xm + s_1) * tsxy;
-      if (inner && lc >= 1 && lc <= nz - 1 && gx1 && gy0)
-        nxz_1 = qr * (s_2_xm + s_2 + s_1_xm + s_1) * tsxz_1;
-      if (inner && lc >= 1 && lc <= nz - 1 && gx0 && gy1)
-        nyz_1 = qr * (s_2_ym + s_2 + s_1_ym + s_1) * tsyz_1;
-      if (out_col && lc >= kb && lc < ke && inb) {
+    V nxy_1 = zero, nxz_1 = zero, nyz_1 = zero;
+    if (w_edge) {
+      // the trials are zero on the walls, and so are these
+      nxy_1 = vmul(vadd(vU, S.U.r[qm]), tsxy);
+      nxz_1 = vmul(vadd(U_2, vU), tsxz_1);
+      nyz_1 = vmul(vadd(vV, S.Vs.r[qm]), tsyz_1);
+      if (out_col && lc >= kb && lc < ke) {
         const Off e = (Off)lc * plane + col;
-        A.sns[0][e] = nxy_1; A.sns[1][e] = nxz_1; A.sns[2][e] = nyz_1;
+        stv(A.sns[0], e, nxy_1); stv(A.sns[1], e, nxz_1); stv(A.sns[2], e, nyz_1);
         if constexpr (CHK) {
-          if (gi <= g.nx && gj <= g.ny && lc <= nz) {   // the staged check's edge points
-            c_sig = maxt(c_sig, maxt(absv(nxy_1), maxt(absv(nxz_1), absv(nyz_1))));
-            const int tid = threadIdx.x;
-            c_dtau = maxt(c_dtau, maxt(absv(nxy_1 - C.cs[0][tid]),
-                                       maxt(absv(nxz_1 - C.cs[1][tid]), absv(nyz_1 - C.cs[2][tid]))));
-            A.cs[0][e] = nxy_1; A.cs[1][e] = nxz_1; A.cs[2][e] = nyz_1;
+          const int tid = threadIdx.x;
+          auto one = [&](auto ic) {
+            constexpr int E = decltype(ic)::value;
+            if (gi + E > nx || gj > ny || lc > nz) return;   // the staged check's edge points
+            const T a0 = el<E>(nxy_1), a1 = el<E>(nxz_1), a2 = el<E>(nyz_1);
+            c_sig = maxt(c_sig, maxt(absv(a0), maxt(absv(a1), absv(a2))));
+            c_dtau = maxt(c_dtau, maxt(absv(a0 - el<E>(C.cs[0][tid])),
+                                       maxt(absv(a1 - el<E>(C.cs[1][tid])), absv(a2 - el<E>(C.cs[2][tid])))));
+          };
+          one(std::integral_constant<int, 0>{});
+          if constexpr (N == 2) one(std::integral_constant<int, 1>{});
+          if (gi <= nx && gj <= ny && lc <= nz) {   // zero beyond the last edge
+            stv(A.cs[0], e, nxy_1); stv(A.cs[1], e, nxz_1); stv(A.cs[2], e, nyz_1);
           }
         }
       }
+      S.nxy[sl1].r[q0] = nxy_1; S.nyz[sl1].r[q0] = nyz_1;
     }
-    S.nxy[sl1].r[rb][a] = nxy_1; S.nyz[sl1].r[rb][a] = nyz_1;
 
     // ---- 5. residual and velocity update of plane t-2 ----
-    {
+    if (w_vel) {
       const int lu = t - 2;
-      const T sxx_2_xm = xm(sxx_2), nxy_2_xp = xp(nxy_2), nxz_2_xp = xp(nxz_2);
-      if (out_col && inb && lu >= kb && lu < ke) {
-        const T nxy_2_yp = S.nxy[sl].r[rb + 1][a], syy_2_ym = S.syy[sl].r[rb - 1][a];
-        const T nyz_2_yp = S.nyz[sl].r[rb + 1][a];
+      const V sxx_2_xm = xm(sxx_2), nxy_2_xp = xp(nxy_2), nxz_2_xp = xp(nxz_2);
+      if (out_col && lu >= kb && lu < ke) {
+        const V nxy_2_yp = S.nxy[sl].r[qp], syy_2_ym = S.syy[sl].r[qm];
+        const V nyz_2_yp = S.nyz[sl].r[qp];
         const Off e = (Off)lu * plane + col;
-        T un = u0_2;
-        if (gx1 && gyl && lu < nz) {
-          const T R = (sxx_2 - sxx_2_xm) * rdx + (nxy_2_yp - nxy_2) * rdy + (nxz_1 - nxz_2) * rdz;
-          un = u0_2 + vs * R;
-          if constexpr (CHK) c_r = maxt(c_r, absv(R));
-        }
-        A.uo[0][e] = un;
+        const V vx = bc(rdx), vy = bc(rdy), vz = bc(rdz);
+        const V R0 = vfma(vsub(nxz_1, nxz_2), vz, vfma(vsub(nxy_2_yp, nxy_2), vy, vmul(vsub(sxx_2, sxx_2_xm), vx)));
+        const V R1 = vfma(vsub(nyz_1, nyz_2), vz, vfma(vsub(nxy_2_xp, nxy_2), vx, vmul(vsub(syy_2, syy_2_ym), vy)));
+        const V R2 = vfma(vsub(nyz_2_yp, nyz_2), vy, vfma(vsub(nxz_2_xp, nxz_2), vx, vmul(vsub(szz_2, szz_3), vz)));
+        // a face off the interior keeps its value
+        const bool zu = lu < nz, zw = lu >= 1 && lu <= nz - 1;
+        const V un0 = zu ? vfma(R0, st0, u0_2) : u0_2, un1 = zu ? vfma(R1, st1, u1_2) : u1_2;
+        const V un2 = zw ? vfma(R2, st2, u2_2) : u2_2;
+        stv(A.uo[0], e, un0); stv(A.uo[1], e, un1); stv(A.uo[2], e, un2);
         if constexpr (CHK) {
-          if (gi <= g.nx && gj < g.ny && lu < nz) {   // x-faces
-            c_du = maxt(c_du, absv(un - C.uchk[0][threadIdx.x]));
-            c_vm = fmax(c_vm, fabs(C.v0[0][threadIdx.x] + (double)u0_2));   // a NaN in u also reaches c_du
-            A.uchk[0][e] = un;
-          }
-        }
-        un = u1_2;
-        if (gy1 && gxl && lu < nz) {
-          const T R = (syy_2 - syy_2_ym) * rdy + (nxy_2_xp - nxy_2) * rdx + (nyz_1 - nyz_2) * rdz;
-          un = u1_2 + vs * R;
-          if constexpr (CHK) c_r = maxt(c_r, absv(R));
-        }
-        A.uo[1][e] = un;
-        if constexpr (CHK) {
-          if (gi < g.nx && gj <= g.ny && lu < nz) {   // y-faces
-            c_du = maxt(c_du, absv(un - C.uchk[1][threadIdx.x]));
-            c_vm = fmax(c_vm, fabs(C.v0[1][threadIdx.x] + (double)u1_2));
-            A.uchk[1][e] = un;
-          }
-        }
-        un = u2_2;
-        if (lu >= 1 && lu <= nz - 1 && gxl && gyl) {
-          const T R = (szz_2 - szz_3) * rdz + (nxz_2_xp - nxz_2) * rdx + (nyz_2_yp - nyz_2) * rdy;
-          un = u2_2 + vs * R;
-          if constexpr (CHK) c_r = maxt(c_r, absv(R));
-        }
-        A.uo[2][e] = un;
-        if constexpr (CHK) {
-          if (gi < g.nx && gj < g.ny && lu <= nz) {   // z-faces
-            c_du = maxt(c_du, absv(un - C.uchk[2][threadIdx.x]));
-            c_vm = fmax(c_vm, fabs(C.v0[2][threadIdx.x] + (double)u2_2));
-            A.uchk[2][e] = un;
-          }
+          const int tid = threadIdx.x;
+          auto one = [&](auto ic) {
+            constexpr int E = decltype(ic)::value;
+            const int x = gi + E;
+            const bool x1 = in_x1(E), xl = in_x0(E);
+            if (x1 && gy0 && zu) c_r = maxt(c_r, absv(el<E>(R0)));
+            if (xl && gy1 && zu) c_r = maxt(c_r, absv(el<E>(R1)));
+            if (xl && gy0 && zw) c_r = maxt(c_r, absv(el<E>(R2)));
+            // |v0 + u|: a NaN in u also reaches c_du
+            if (x <= nx && gj < ny && lu < nz) {
+              c_du = maxt(c_du, absv(el<E>(un0) - el<E>(C.uchk[0][tid])));
+              c_vm = fmax(c_vm, fabs(C.v0[0][N * tid + E] + (double)el<E>(u0_2)));
+            }
+            if (x < nx && gj <= ny && lu < nz) {
+              c_du = maxt(c_du, absv(el<E>(un1) - el<E>(C.uchk[1][tid])));
+              c_vm = fmax(c_vm, fabs(C.v0[1][N * tid + E] + (double)el<E>(u1_2)));
+            }
+            if (x < nx && gj < ny && lu <= nz) {
+              c_du = maxt(c_du, absv(el<E>(un2) - el<E>(C.uchk[2][tid])));
+              c_vm = fmax(c_vm, fabs(C.v0[2][N * tid + E] + (double)el<E>(u2_2)));
+            }
+          };
+          one(std::integral_constant<int, 0>{});
+          if constexpr (N == 2) one(std::integral_constant<int, 1>{});
+          // off a location's extent u stays zero, and so does its snapshot
+          stv(A.uchk[0], e, un0); stv(A.uchk[1], e, un1); stv(A.uchk[2], e, un2);
         }
       }
     }
 
     // ---- carry this plane's values one plane down ----
-    oxy_1 = oxy; oxz_1 = oxz; oyz_1 = oyz; exy_1 = exy;
-    pxy_1 = pxy; pxz_1 = pxz; pyz_1 = pyz;
+    wxy_1 = wxy;
     tsxz_1 = tsxz; tsyz_1 = tsyz;
-    s_2 = s_1;
+    s_2 = s_1; U_2 = vU;
     sxx_2 = sxx_1; syy_2 = syy_1; szz_3 = szz_2; szz_2 = szz_1;
     nxy_2 = nxy_1; nxz_2 = nxz_1; nyz_2 = nyz_1;
+    return true;
   };
   int t = kb - 2;
   for (; t + 1 < ke + 2; t += 2) {
-    plane_step(t, std::integral_constant<int, 0>{});
-    plane_step(t + 1, std::integral_constant<int, 1>{});
+    if (!plane_step(t, std::integral_constant<int, 0>{})) return;
+    if (!plane_step(t + 1, std::integral_constant<int, 1>{})) return;
   }
-  if (t < ke + 2) plane_step(t, std::integral_constant<int, 0>{});
+  if (t < ke + 2 && !plane_step(t, std::integral_constant<int, 0>{})) return;
   if constexpr (CHK) {
     block_max_bits((double)c_sig, &di->red[RED_SIG]);
     block_max_bits((double)c_dtau, &di->red[RED_DTAU]);
@@ -503,77 +636,125 @@ __device__ __forceinline__ void reg_body(const Args<T> &A, const Geo &g, const S
   }
 }
 
-template <typename T, int H, typename Off, bool CHK>
-__global__ void __launch_bounds__(WX *H, 1)
-    k_fused3d_reg(const Args<T> A, Geo g, const Scal *sc, DevInfo *di, int kz) {
+template <typename L, typename Off, bool CHK>
+__global__ void __launch_bounds__(L::LPR *L::H, 1)
+    k_fused3d_reg(const __grid_constant__ Maps M, const Args<typename L::T> A, Geo g, const Scal *sc, DevInfo *di, int kz) {
   if (di != nullptr && *(volatile const int *)&di->done != 0) return;
   const bool frozen = di != nullptr && di->frozen;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int i0 = blockIdx.x * OX, j0 = blockIdx.y * (H - 4);
-  const bool interior = i0 - 2 >= 1 && i0 + WX - 3 <= g.nx - 1 && j0 - 2 >= 1 && j0 + H - 3 <= g.ny - 1;
-  if (interior) reg_body<T, H, true, Off, CHK>(A, g, sc, di, frozen, kz, smem_raw);
-  else reg_body<T, H, false, Off, CHK>(A, g, sc, di, frozen, kz, smem_raw);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int i0 = blockIdx.x * OX, j0 = blockIdx.y * (L::H - 4);
+  const bool interior = i0 - 2 >= 1 && i0 + WX - 3 <= g.nx - 1 && j0 - 2 >= 1 && j0 + L::H - 3 <= g.ny - 1;
+  if (interior) reg_body<L, true, Off, CHK>(M, A, g, sc, di, frozen, kz, smem_raw);
+  else reg_body<L, false, Off, CHK>(M, A, g, sc, di, frozen, kz, smem_raw);
 }
 
 template <typename T>
-constexpr int reg_rows() { return sizeof(T) == 4 ? 16 : 8; }
+struct LaneOf {
+  using type = LaneF<24>;
+  using check = LaneF<16>;   // the snapshots' slots take the room of eight rows
+};
+template <>
+struct LaneOf<double> {
+  using type = LaneD;
+  using check = LaneD;
+};
+
+typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiled encoder() {
+  static EncodeTiled fn = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return ok ? (EncodeTiled)p : nullptr;
+  }();
+  return fn;
+}
+
+// tensor maps of the stage's 23 input arrays: boxes of BX x H x 1, zero outside
+template <typename L>
+bool encode_maps(Maps *M, const Geo &g, const Stage<typename L::T> &S) {
+  using T = typename L::T;
+  const T *src[I_COUNT] = {S.u[0],   S.u[1],   S.u[2],   S.rq[0],  S.rq[1],  S.rq[2],  S.rd[0],  S.rd[1],
+                           S.sos[1], S.sos[2], S.tbs[1], S.tbs[2], S.son[0], S.son[1], S.son[2], S.tbn[0],
+                           S.tbn[1], S.tbn[2], S.sos[0], S.tbs[0], S.sop,    S.pb,     S.yc};
+  const EncodeTiled fn = encoder();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)g.px, (cuuint64_t)g.py, (cuuint64_t)g.pz};
+  cuuint64_t strides[2] = {(cuuint64_t)g.px * sizeof(T), (cuuint64_t)g.plane * sizeof(T)};
+  cuuint32_t box[3] = {(cuuint32_t)BX, (cuuint32_t)L::H, 1}, es[3] = {1, 1, 1};
+  for (int k = 0; k < I_COUNT; ++k)
+    if (fn(&M->m[k], sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
+           const_cast<T *>(src[k]), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return false;
+  return true;
+}
+
+template <typename L, typename Off, bool CHK>
+bool launch_lane(const Stage<typename L::T> &S, const Args<typename L::T> &A, const Geo &g, const Scal *sc, DevInfo *di,
+                 int kz, cudaStream_t st) {
+  Maps M;
+  if (!encode_maps<L>(&M, g, S)) return false;
+  kz = fused3d_kz(g, OX, L::H - 4, kz);
+  dim3 grid((g.px + OX - 1) / OX, (g.py + L::H - 5) / (L::H - 4), (g.pz + kz - 1) / kz);
+  k_fused3d_reg<L, Off, CHK><<<grid, L::LPR * L::H, sizeof(SmemR<L>) + (CHK ? sizeof(ChkSlots<L>) : 0), st>>>(
+      M, A, g, sc, di, kz);
+  return true;
+}
+
+template <typename L, typename Off, bool CHK>
+cudaError_t configure_lane() {
+  return cudaFuncSetAttribute(k_fused3d_reg<L, Off, CHK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(sizeof(SmemR<L>) + (CHK ? sizeof(ChkSlots<L>) : 0)));
+}
 
 }  // namespace
 
 // One fused iteration, register z-march flavour: reads buffer b of the
 // stage, writes 1 - b.  check (FP32 only): a check iteration, which also
 // reduces the stopping measures into di and updates the check snapshots.
+// Returns false if a tensor map could not be made.
 template <typename T>
-void launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
+bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
                         bool check) {
-  constexpr int H = reg_rows<T>();
+  using L = typename LaneOf<T>::type;
+  using LC = typename LaneOf<T>::check;
   Args<T> A;
   for (int d = 0; d < 3; ++d) {
-    A.u[d] = S.u[d]; A.rq[d] = S.rq[d]; A.son[d] = S.son[d]; A.sos[d] = S.sos[d];
-    A.tbn[d] = S.tbn[d]; A.tbs[d] = S.tbs[d];
     A.snn[d] = S.snn[d]; A.sns[d] = S.sns[d]; A.uo[d] = S.uo[d];
     A.cn[d] = S.cn[d]; A.cs[d] = S.cs[d]; A.uchk[d] = S.uchk[d]; A.v0[d] = S.v0[d];
   }
-  A.rd[0] = S.rd[0]; A.rd[1] = S.rd[1];
-  A.sop = S.sop; A.pb = S.pb; A.yc = S.yc; A.snp = S.snp;
-  A.s = S.s; A.cp = S.cp;
-  kz = fused3d_kz(g, OX, H - 4, kz);
-  dim3 grid((g.px + OX - 1) / OX, (g.py + H - 5) / (H - 4), (g.pz + kz - 1) / kz);
-  const size_t sm = sizeof(SmemR<T, H>), smc = sm + sizeof(ChkSlots<T, H>);
+  A.snp = S.snp; A.s = S.s; A.cp = S.cp;
   if constexpr (sizeof(T) == 4) {
     const bool o32 = (long long)g.pz * g.plane < (1LL << 31);
-    if (check) {
-      if (o32) k_fused3d_reg<T, H, int, true><<<grid, WX * H, smc, st>>>(A, g, sc, di, kz);
-      else k_fused3d_reg<T, H, long long, true><<<grid, WX * H, smc, st>>>(A, g, sc, di, kz);
-    } else {
-      if (o32) k_fused3d_reg<T, H, int, false><<<grid, WX * H, sm, st>>>(A, g, sc, di, kz);
-      else k_fused3d_reg<T, H, long long, false><<<grid, WX * H, sm, st>>>(A, g, sc, di, kz);
-    }
+    if (check)
+      return o32 ? launch_lane<LC, int, true>(S, A, g, sc, di, kz, st)
+                 : launch_lane<LC, long long, true>(S, A, g, sc, di, kz, st);
+    return o32 ? launch_lane<L, int, false>(S, A, g, sc, di, kz, st)
+               : launch_lane<L, long long, false>(S, A, g, sc, di, kz, st);
   } else {
-    k_fused3d_reg<T, H, long long, false><<<grid, WX * H, sm, st>>>(A, g, sc, di, kz);
+    return launch_lane<L, long long, false>(S, A, g, sc, di, kz, st);
   }
 }
 
 cudaError_t fused3d_reg_configure() {
-  const int sf = (int)sizeof(SmemR<float, 16>), sfc = sf + (int)sizeof(ChkSlots<float, 16>);
-  cudaError_t e = cudaFuncSetAttribute(k_fused3d_reg<float, 16, int, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, sf);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fused3d_reg<float, 16, long long, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sf);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fused3d_reg<float, 16, int, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sfc);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fused3d_reg<float, 16, long long, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sfc);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_fused3d_reg<double, 8, long long, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(SmemR<double, 8>));
+  using L = LaneOf<float>::type;
+  using LC = LaneOf<float>::check;
+  cudaError_t e = configure_lane<L, int, false>();
+  if (e == cudaSuccess) e = configure_lane<L, long long, false>();
+  if (e == cudaSuccess) e = configure_lane<LC, int, true>();
+  if (e == cudaSuccess) e = configure_lane<LC, long long, true>();
+  if (e == cudaSuccess) e = configure_lane<LaneD, long long, false>();
+  return e;
 }
 
-template void launch_fused3d_reg<float>(const Geo &, const Stage<float> &, const Scal *, DevInfo *, int, cudaStream_t,
+template bool launch_fused3d_reg<float>(const Geo &, const Stage<float> &, const Scal *, DevInfo *, int, cudaStream_t,
                                         bool);
-template void launch_fused3d_reg<double>(const Geo &, const Stage<double> &, const Scal *, DevInfo *, int,
+template bool launch_fused3d_reg<double>(const Geo &, const Stage<double> &, const Scal *, DevInfo *, int,
                                          cudaStream_t, bool);
 
 }  // namespace ep

@@ -190,7 +190,7 @@ void launch_check(DevInfo *di, const Scal *sc, cudaStream_t st);
 // z-planes per block when none was chosen (kz <= 0).  A block marches kz
 // planes plus four halo planes, and the launch runs in waves of
 // (SMs x blocks per SM) blocks, so the time goes as
-// waves(kz) x (kz + 4); take the kz in [8, 128] that minimises it.
+// waves(kz) x (kz + 4); take the kz in [1, 128] that minimises it.
 inline int fused3d_kz(const Geo &g, int tx, int ty, int kz, int per_sm = 1) {
   if (kz > 0) return kz;
   static int sms = 0;
@@ -201,9 +201,9 @@ inline int fused3d_kz(const Geo &g, int tx, int ty, int kz, int per_sm = 1) {
   }
   const long long cols = (long long)((g.px + tx - 1) / tx) * ((g.py + ty - 1) / ty);
   const long long wave = (long long)sms * per_sm;
-  int best = 8;
+  int best = 1;
   long long best_cost = -1;
-  for (int k = 8; k <= 128; ++k) {
+  for (int k = 1; k <= 128; ++k) {
     const long long blocks = cols * ((g.pz + k - 1) / k);
     const long long cost = (blocks + wave - 1) / wave * (k + 4);
     if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = k; }
@@ -219,9 +219,9 @@ void launch_fused3d(const Geo &g, const Stage<T> &S, const Scal *sc, const DevIn
 template <typename T>
 bool launch_fused3d_tma(const Geo &g, const Stage<T> &S, const Scal *sc, const DevInfo *di, int kz, cudaStream_t st);
 cudaError_t fused3d_tma_configure();
-// register z-march variant (ep_fused3d_reg.cu)
+// register z-march variant (ep_fused3d_reg.cu); false if a tensor map failed
 template <typename T>
-void launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
+bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
                         bool check = false);
 cudaError_t fused3d_reg_configure();
 

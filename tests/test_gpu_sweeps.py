@@ -1,0 +1,92 @@
+"""The fast sweep kernels against the staged sweep at the sizes where a tiling can go wrong:
+one window, a window's edge, one row or column beyond it, remainders along z, many blocks."""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+EPS32 = 2.0 ** -24
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2305_01701_gb300 import build as B
+    B.build()
+    import paper_2305_01701_gb300 as P
+    return P
+
+
+def _fields(P, nd, n, seed):
+    """A history near yield: pure shear with noise, noisy velocities, shear zero on the walls."""
+    rng = np.random.default_rng(seed)
+    rates = [1.0, -1.0] if nd == 2 else [1.0, 0.0, -1.0]
+    f = {}
+    shape = {k: P.field_shape(nd, tuple(n) + (1,), k) for k in
+             ["vx", "vy", "txx", "tyy", "txy", "p"] + (["vz", "tzz", "txz", "tyz"] if nd == 3 else [])}
+    for d in range(nd):
+        ax = nd - 1 - d
+        x = np.arange(n[d] + 1) / n[d] - 0.5
+        v = rates[d] * x.reshape([-1 if q == ax else 1 for q in range(nd)]) * np.ones(shape["v" + "xyz"[d]])
+        f["v" + "xyz"[d]] = v + 0.02 * rng.standard_normal(v.shape)
+        c = shape["t" + "xyz"[d] * 2]
+        f["t" + "xyz"[d] * 2] = (1.2e-3 if nd == 2 else 1.7e-3) * rates[d] + 1e-4 * rng.standard_normal(c)
+    for k, walls in (("txy", (0, 1)), ("txz", (0, 2)), ("tyz", (1, 2))):
+        if k in shape:
+            t = 1e-4 * rng.standard_normal(shape[k])
+            for d in walls:
+                ax = nd - 1 - d
+                t[tuple(slice(None) if q != ax else [0, -1] for q in range(nd))] = 0.0
+            f[k] = t
+    f["p"] = 1e-4 * rng.standard_normal(shape["p"])
+    return f
+
+
+def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
+    g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=precision)
+    rng = np.random.default_rng(1)
+    g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, 1.5e-3 * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
+    if "cell_g" in opts:
+        g.set_shear_modulus(1.0 + 0.2 * opts.pop("cell_g") * rng.random(int(np.prod(n))))
+    g.set_solver(tol=0.0, max_iter=iters, n_chk=iters // 2, **opts)
+    g.set_kernel(kernel, shape)
+    for k, a in f.items():
+        g.set(k, a)
+    g.apply_increment(1.0, 1e-4, P.LOAD_XY if nd == 2 else P.LOAD_XZ)
+    info = g.solve_increment(raise_on_fail=False)
+    g.commit_increment()
+    out = {k: g.get(k) for k in list(f) + ["epl", "scale"]}
+    g.close()
+    return info, out
+
+
+def _compare(f, out, ref, info, iref, iters, eps):
+    """Both sweeps round every state value once or twice per iteration in another order: over
+    `iters` iterations the difference stays below 4 iters ulp of the field group's scale (each
+    rounding decays with the relaxation; the sum of all of them bounds it)."""
+    bound = 4 * iters * eps
+    groups = [[k for k in f if k[0] == "v"], [k for k in f if k[0] != "v"]]
+    for names in groups:
+        scale = max(np.abs(ref[k]).max() for k in names)
+        for k in names:
+            err = np.abs(out[k] - ref[k]).max() / scale
+            assert err <= bound, (k, err, bound)
+    plastic = ref["scale"] < 1.0
+    assert plastic.any() and not plastic.all()
+    assert np.abs(out["scale"] - ref["scale"]).max() <= bound * 10
+    for k in ("max_sigma", "eps_rel"):
+        assert abs(info[k] - iref[k]) <= 100 * bound * abs(iref[k]), (k, info[k], iref[k])
+
+
+@pytest.mark.parametrize("n,kz", [((27, 19, 5), 0), ((28, 20, 6), 0), ((29, 21, 7), 3), ((31, 3, 9), 0), ((1, 45, 4), 0),
+                                  ((84, 61, 2), 1), ((63, 47, 33), 0), ((90, 64, 21), 8), ((35, 130, 1), 0)])
+def test_register_sweep_matches_the_staged_sweep_at_tile_edges_fp32(P, n, kz):
+    iters = 20
+    f = _fields(P, 3, n, 7)
+    iref, ref = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f)
+    info, out = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_FUSED_REG, iters, f, shape=kz)
+    _compare(f, out, ref, info, iref, iters, EPS32)

@@ -25,6 +25,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "ep_conv.cuh"
 #include "ep_internal.cuh"
 
 namespace ep {
@@ -243,20 +244,22 @@ __global__ void k_to_channels_last(const float *x, int N, int C, long long nv, i
   out[t] = __float2bfloat16_rn(c < C ? x[(n * C + c) * nv + v] : 0.f);
 }
 
-// BF16 co x ci x taps -> the operand layout of ConvSmem.b, per tap and
+// BF16 co x ci x taps -> the operand layout of ConvSmem.b, per layer, tap and
 // 16-channel chunk: [half][co][8 channels]; channels >= ci are zero
-__global__ void k_pack_weights(const __nv_bfloat16 *w, int cin, int cout, int taps, int cinp,
-                               __nv_bfloat16 *out) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = (long long)taps * cinp * cout;
-  if (t >= total) return;
-  const int e = (int)(t % 8);
-  const int co = (int)((t / 8) % cout);
-  const int h = (int)((t / (8 * cout)) % 2);
-  const int q = (int)((t / (16LL * cout)) % (cinp / 16));
-  const int tap = (int)(t / (16LL * cout * (cinp / 16)));
+__global__ void k_pack_weights(const PackTable P, const __nv_bfloat16 *w, __nv_bfloat16 *out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P.total) return;
+  int l = 0;
+  while (l + 1 < P.n && i >= P.dst[l + 1]) ++l;
+  const int cin = P.cin[l], cout = P.cout[l], cinp = (cin + 15) / 16 * 16;
+  const int t = (int)(i - P.dst[l]);   // taps * cinp * cout elements
+  const int e = t % 8;
+  const int co = (t / 8) % cout;
+  const int h = (t / (8 * cout)) % 2;
+  const int q = (t / (16 * cout)) % (cinp / 16);
+  const int tap = t / (16 * cout * (cinp / 16));
   const int ci = 16 * q + 8 * h + e;
-  out[t] = ci < cin ? w[((long long)co * cin + ci) * taps + tap] : __float2bfloat16_rn(0.f);
+  out[i] = ci < cin ? w[P.src[l] + ((long long)co * cin + ci) * P.taps + tap] : __float2bfloat16_rn(0.f);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -287,10 +290,8 @@ void conv_tc_to_channels_last(const float *x, int N, int C, long long nv, int cp
   k_to_channels_last<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(x, N, C, nv, cp, out);
 }
 
-void conv_tc_pack_weights(const __nv_bfloat16 *w, int cin, int cout, int taps, __nv_bfloat16 *out, cudaStream_t st) {
-  const int cinp = conv_tc_cinp(cin);
-  const long long total = (long long)taps * cinp * cout;
-  k_pack_weights<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(w, cin, cout, taps, cinp, out);
+void conv_tc_pack_weights(const PackTable &P, const __nv_bfloat16 *w, __nv_bfloat16 *out, cudaStream_t st) {
+  k_pack_weights<<<(unsigned)((P.total + 255) / 256), 256, 0, st>>>(P, w, out);
 }
 
 cudaError_t conv_tc_forward(int D, const __nv_bfloat16 *xcl, int N, int X, int Y, int Z, int cin,

@@ -11,9 +11,8 @@
 //   head             : conv1 (c_0 -> out), no activation, zero-initialised.
 // The prediction is added to a baseline chosen by the caller (the previous
 // increment's velocity change), so an untrained network reproduces it.
-// Training: MSE loss, Adam.  The convolutions run on CUDA cores with FP32
-// accumulation: at the sizes used (<= 128 channels) they are a small part of
-// an increment's solve time.
+// Training: MSE loss, Adam; its 3^D convolutions and weight gradients run in
+// FP32 on the CUDA cores (ep_conv_fp32.cu).
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
@@ -23,6 +22,7 @@
 #include <string>
 #include <vector>
 
+#include "ep_conv.cuh"
 #include "ep_internal.cuh"
 
 namespace ep {
@@ -32,7 +32,6 @@ bool conv_tc_supported(int k, int cout);
 int conv_tc_cinp(int cin);
 void conv_tc_to_channels_last(const float *x, int N, int C, long long nv, int cp, __nv_bfloat16 *out,
                               cudaStream_t st);
-void conv_tc_pack_weights(const __nv_bfloat16 *w, int cin, int cout, int taps, __nv_bfloat16 *out, cudaStream_t st);
 cudaError_t conv_tc_forward(int D, const __nv_bfloat16 *xcl, int N, int X, int Y, int Z, int cin,
                             const __nv_bfloat16 *wpk, const float *bias, int cout, int relu, float *y, int *err,
                             cudaStream_t st);
@@ -43,128 +42,43 @@ constexpr int NT = 256;
 
 inline unsigned nblk(long long n) { return (unsigned)((n + NT - 1) / NT); }
 
-// ---- direct convolution (3^D or 1^D taps), zero padding -------------------
-// y[n, co, p] = b[co] + sum_{ci, tap} W(co, ci, tap) x[n, ci, p + tap - r]
-// TRANS = true computes the data gradient: channels swapped and taps
-// mirrored, i.e. dx = conv(dy, W^T flipped); then b is unused.
-template <int D, int K, bool TRANS>
-__global__ void k_conv(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
-                       float *__restrict__ y, int N, int cin, int cout, int X, int Y, int Z, int relu,
-                       int w_cin, int w_cout) {
+// ---- the head's 1^D convolution ---------------------------------------------
+// y[n, co, p] = b[co] + sum_ci W(co, ci) x[n, ci, p]
+// TRANS = true computes the data gradient dx = W^T dy (b is unused); mask
+// (nullable, the shape of y): y is 0 where it is <= 0 (the ReLU behind x).
+template <bool TRANS>
+__global__ void k_conv1(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
+                        float *__restrict__ y, const float *__restrict__ mask, int cin, int cout, long long nvox) {
   // one thread per output voxel, a chunk of 8 output channels per blockIdx.y
   constexpr int CB = 8;
-  constexpr int R = K / 2;
-  const long long nvox = (long long)X * Y * Z;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int co0 = blockIdx.y * CB;
   const int n = blockIdx.z;
   if (t >= nvox) return;
-  const int ix = (int)(t % X), iy = (int)((t / X) % Y), iz = (int)(t / ((long long)X * Y));
   float acc[CB];
 #pragma unroll
-  for (int c = 0; c < CB; ++c) acc[c] = (!TRANS && b && co0 + c < cout) ? b[co0 + c] : 0.f;
-  const float *xn = x + (long long)n * cin * nvox;
-  constexpr int KZ = D == 3 ? K : 1;
+  for (int c = 0; c < CB; ++c) acc[c] = (!TRANS && co0 + c < cout) ? b[co0 + c] : 0.f;
+  const float *xn = x + (long long)n * cin * nvox + t;
   for (int ci = 0; ci < cin; ++ci) {
-    const float *xc = xn + (long long)ci * nvox;
-    for (int dz = 0; dz < KZ; ++dz) {
-      const int zz = D == 3 ? iz + dz - R : iz;
-      if (zz < 0 || zz >= Z) continue;
-      for (int dy = 0; dy < K; ++dy) {
-        const int yy = iy + dy - R;
-        if (yy < 0 || yy >= Y) continue;
-        for (int dx = 0; dx < K; ++dx) {
-          const int xx = ix + dx - R;
-          if (xx < 0 || xx >= X) continue;
-          const float v = xc[((long long)zz * Y + yy) * X + xx];
-          const int tap = (dz * K + dy) * K + dx;
-          const int taps = KZ * K * K;
+    const float v = xn[(long long)ci * nvox];
 #pragma unroll
-          for (int c = 0; c < CB; ++c) {
-            const int co = co0 + c;
-            if (co >= cout) break;
-            // forward: W[co][ci][tap]; transposed: W[ci'=co_out... ] mirrored
-            long long wi;
-            if (!TRANS) wi = ((long long)co * w_cin + ci) * taps + tap;
-            else wi = ((long long)ci * w_cin + co) * taps + (taps - 1 - tap);
-            acc[c] += __bfloat162float(w[wi]) * v;
-          }
-        }
-      }
+    for (int c = 0; c < CB; ++c) {
+      const int co = co0 + c;
+      if (co < cout) acc[c] += __bfloat162float(w[TRANS ? (long long)ci * cout + co : (long long)co * cin + ci]) * v;
     }
   }
-  float *yn = y + (long long)n * cout * nvox;
 #pragma unroll
   for (int c = 0; c < CB; ++c) {
     const int co = co0 + c;
     if (co >= cout) break;
-    float v = acc[c];
-    if (relu && v < 0.f) v = 0.f;
-    yn[(long long)co * nvox + t] = v;
-  }
-}
-
-// weight gradient: dW[co][ci][tap] += sum_{n, p} dy[n, co, p] x[n, ci, p + tap - r]
-// one block per (co, ci); threads stride over voxels, block-reduce per tap.
-template <int D, int K>
-__global__ void k_conv_wgrad(const float *__restrict__ x, const float *__restrict__ dy, float *__restrict__ dw,
-                             float *__restrict__ db, int N, int cin, int cout, int X, int Y, int Z) {
-  constexpr int R = K / 2, KZ = D == 3 ? K : 1, TAPS = KZ * K * K;
-  const int co = blockIdx.x, ci = blockIdx.y;
-  const long long nvox = (long long)X * Y * Z;
-  float acc[TAPS];
-#pragma unroll
-  for (int q = 0; q < TAPS; ++q) acc[q] = 0.f;
-  float accb = 0.f;
-  for (int n = 0; n < N; ++n) {
-    const float *g = dy + ((long long)n * cout + co) * nvox;
-    const float *xc = x + ((long long)n * cin + ci) * nvox;
-    for (long long t = threadIdx.x; t < nvox; t += blockDim.x) {
-      const float gv = g[t];
-      if (gv == 0.f) continue;
-      const int ix = (int)(t % X), iy = (int)((t / X) % Y), iz = (int)(t / ((long long)X * Y));
-      if (ci == 0) accb += gv;
-#pragma unroll
-      for (int dz = 0; dz < KZ; ++dz) {
-        const int zz = D == 3 ? iz + dz - R : iz;
-#pragma unroll
-        for (int dyy = 0; dyy < K; ++dyy) {
-          const int yy = iy + dyy - R;
-#pragma unroll
-          for (int dx = 0; dx < K; ++dx) {
-            const int xx = ix + dx - R;
-            const bool ok = xx >= 0 && xx < X && yy >= 0 && yy < Y && zz >= 0 && zz < Z;
-            if (ok) acc[(dz * K + dyy) * K + dx] += gv * xc[((long long)zz * Y + yy) * X + xx];
-          }
-        }
-      }
-    }
-  }
-  __shared__ float red[NT / 32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int q = 0; q <= TAPS; ++q) {
-    float v = q < TAPS ? acc[q] : accb;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0) red[wid] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float s = 0.f;
-      for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) s += red[w2];
-      if (q < TAPS) dw[((long long)co * cin + ci) * TAPS + q] += s;
-      else if (ci == 0 && db) db[co] += s;
-    }
+    const long long o = ((long long)n * cout + co) * nvox + t;
+    y[o] = mask && mask[o] <= 0.f ? 0.f : acc[c];
   }
 }
 
 __global__ void k_scale(float *a, long long n, float s) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) a[t] *= s;
-}
-
-__global__ void k_relu_bwd(const float *a, float *g, long long n) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n && a[t] <= 0.f) g[t] = 0.f;
 }
 
 // average pool by 2 in every spatial dimension (sizes are even)
@@ -185,8 +99,10 @@ __global__ void k_pool(const float *x, float *y, long long NC, int X, int Y, int
   y[t] = s * (D == 3 ? 0.125f : 0.25f);
 }
 
+// gx += the pool's gradient, then 0 where the pooled activation a is <= 0 (its
+// ReLU; the skip's part is already in gx)
 template <int D>
-__global__ void k_pool_bwd(const float *gy, float *gx, long long NC, int X, int Y, int Z) {
+__global__ void k_pool_bwd(const float *gy, const float *a, float *gx, long long NC, int X, int Y, int Z) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   long long nv = (long long)X * Y * Z;
   if (t >= NC * nv) return;
@@ -194,28 +110,33 @@ __global__ void k_pool_bwd(const float *gy, float *gx, long long NC, int X, int 
   int ix = (int)(v % X), iy = (int)((v / X) % Y), iz = (int)(v / ((long long)X * Y));
   const int x2 = X / 2, y2 = Y / 2;
   const long long n2 = (long long)x2 * y2 * (D == 3 ? Z / 2 : 1);
-  gx[t] = gy[c * n2 + ((long long)(D == 3 ? iz / 2 : 0) * y2 + iy / 2) * x2 + ix / 2] * (D == 3 ? 0.125f : 0.25f);
+  const float g = gy[c * n2 + ((long long)(D == 3 ? iz / 2 : 0) * y2 + iy / 2) * x2 + ix / 2] * (D == 3 ? 0.125f : 0.25f);
+  gx[t] = a[t] <= 0.f ? 0.f : gx[t] + g;
 }
 
-// nearest upsample by 2 into channel slot [c_off, c_off + C) of a wider tensor
+// y = the nearest upsample by 2 of x (cup channels), then the skip e (c
+// channels); X, Y, Z: sizes of y and e
 template <int D>
-__global__ void k_up(const float *x, float *y, int N, int C, int ctot, int c_off, int X, int Y, int Z) {
-  // X, Y, Z: sizes of the (fine) output
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long nv = (long long)X * Y * Z;
-  if (t >= (long long)N * C * nv) return;
-  long long nc = t / nv, v = t % nv;
-  int n = (int)(nc / C), c = (int)(nc % C);
-  int ix = (int)(v % X), iy = (int)((v / X) % Y), iz = (int)(v / ((long long)X * Y));
+__global__ void k_up_cat(const float *x, const float *e, float *y, int N, int cup, int c, int X, int Y, int Z) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long nv = (long long)X * Y * Z;
+  if (t >= (long long)N * (cup + c) * nv) return;
+  const long long nc = t / nv, v = t % nv;
+  const int n = (int)(nc / (cup + c)), ch = (int)(nc % (cup + c));
+  if (ch >= cup) {
+    y[t] = e[((long long)n * c + ch - cup) * nv + v];
+    return;
+  }
+  const int ix = (int)(v % X), iy = (int)((v / X) % Y), iz = (int)(v / ((long long)X * Y));
   const int x2 = X / 2, y2 = Y / 2;
   const long long n2 = (long long)x2 * y2 * (D == 3 ? Z / 2 : 1);
-  y[((long long)n * ctot + c_off + c) * nv + v] =
-      x[((long long)n * C + c) * n2 + ((long long)(D == 3 ? iz / 2 : 0) * y2 + iy / 2) * x2 + ix / 2];
+  y[t] = x[((long long)n * cup + ch) * n2 + ((long long)(D == 3 ? iz / 2 : 0) * y2 + iy / 2) * x2 + ix / 2];
 }
 
+// the upsample's gradient, 0 where the upsampled activation a is <= 0 (its ReLU)
 template <int D>
-__global__ void k_up_bwd(const float *gy, float *gx, int N, int C, int ctot, int c_off, int X, int Y, int Z) {
-  // gx: coarse (X/2...), gy: fine slot
+__global__ void k_up_bwd(const float *gy, const float *a, float *gx, int N, int C, int ctot, int X, int Y, int Z) {
+  // gx, a: coarse (X/2...); gy: the first C of ctot channels of the fine tensor
   const int x2 = X / 2, y2 = Y / 2, z2 = D == 3 ? Z / 2 : 1;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   long long n2 = (long long)x2 * y2 * z2, nv = (long long)X * Y * Z;
@@ -223,25 +144,21 @@ __global__ void k_up_bwd(const float *gy, float *gx, int N, int C, int ctot, int
   long long nc = t / n2, v = t % n2;
   int n = (int)(nc / C), c = (int)(nc % C);
   int ix = (int)(v % x2), iy = (int)((v / x2) % y2), iz = (int)(v / ((long long)x2 * y2));
-  const float *g = gy + ((long long)n * ctot + c_off + c) * nv;
+  const float *g = gy + ((long long)n * ctot + c) * nv;
   float s = 0.f;
   for (int dz = 0; dz < (D == 3 ? 2 : 1); ++dz)
     for (int dy = 0; dy < 2; ++dy)
       for (int dx = 0; dx < 2; ++dx)
         s += g[((long long)(D == 3 ? 2 * iz + dz : 0) * Y + 2 * iy + dy) * X + 2 * ix + dx];
-  gx[t] = s;
+  gx[t] = a[t] <= 0.f ? 0.f : s;
 }
 
-// copy channels [0, C) of a tensor into slot [c_off, c_off + C) of a wider one (and back)
-__global__ void k_slot_copy(const float *src, float *dst, int N, int C, int csrc, int soff, int cdst, int doff,
-                            long long nv, int accumulate) {
+// channels [off, off + C) of a tensor of ctot channels, copied
+__global__ void k_slot_copy(const float *src, float *dst, int N, int C, int ctot, int off, long long nv) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)N * C * nv) return;
   long long nc = t / nv, v = t % nv;
-  int n = (int)(nc / C), c = (int)(nc % C);
-  float val = src[((long long)n * csrc + soff + c) * nv + v];
-  float *d = dst + ((long long)n * cdst + doff + c) * nv + v;
-  if (accumulate) *d += val; else *d = val;
+  dst[t] = src[((nc / C) * ctot + off + nc % C) * nv + v];
 }
 
 // MSE loss between y and target (both N x C x nv): grad = 2 (y - t) / count.
@@ -330,8 +247,7 @@ struct UNet {
   std::vector<float *> act, grad;   // per stored tensor
   std::vector<int> act_c;           // channels of each stored tensor
   std::vector<int> act_lvl;         // level (resolution) of each stored tensor
-  float *scratch = nullptr, *scratch2 = nullptr;
-  long long scratch_n = 0;
+  float *partial = nullptr;         // the weight gradients' partial sums
   double *dloss = nullptr;
   cudaStream_t st = nullptr;
   // tensor-core inference: weights packed per layer in the MMA operand
@@ -399,11 +315,19 @@ static long long tc_layout(UNet &u) {
 
 // repack the BF16 weights for the tensor cores (after every weight change)
 static void tc_pack(UNet &u) {
+  PackTable P{};
+  P.taps = u.D == 3 ? 27 : 9;
   for (size_t q = 0; q < u.layers.size(); ++q) {
     if (u.pk_off[q] < 0) continue;
     const Layer &L = u.layers[q];
-    conv_tc_pack_weights(u.wb + L.woff, L.cin, L.cout, u.D == 3 ? 27 : 9, u.wpk + u.pk_off[q], u.st);
+    P.cin[P.n] = L.cin;
+    P.cout[P.n] = L.cout;
+    P.src[P.n] = L.woff;
+    P.dst[P.n] = u.pk_off[q];
+    P.total = u.pk_off[q] + (long long)P.taps * conv_tc_cinp(L.cin) * L.cout;
+    ++P.n;
   }
+  if (P.n) conv_tc_pack_weights(P, u.wb, u.wpk, u.st);
 }
 
 // BF16 elements of the largest channels-last layer input at shape (N, X, Y, Z)
@@ -427,14 +351,20 @@ static long long tc_xcl_elems(const UNet &u, int N, int X, int Y, int Z) {
 
 namespace ep {
 
+// resolution level of layer q: two per level down, two per level up, the head
+static int layer_level(const UNet &u, int q) {
+  if (q < 2 * u.levels) return q / 2;
+  const int d = (q - 2 * u.levels) / 2;
+  return std::max(0, u.levels - 2 - d);
+}
+
 static cudaError_t ensure_shape(UNet &u, int N, int X, int Y, int Z) {
   if (u.N == N && u.X == X && u.Y == Y && u.Z == Z) return cudaSuccess;
   for (float *p : u.act) cudaFree(p);
   for (float *p : u.grad) cudaFree(p);
   u.act.clear(); u.grad.clear(); u.act_c.clear(); u.act_lvl.clear();
-  if (u.scratch) cudaFree(u.scratch);
-  if (u.scratch2) cudaFree(u.scratch2);
-  u.scratch = u.scratch2 = nullptr;
+  if (u.partial) cudaFree(u.partial);
+  u.partial = nullptr;
   u.N = N; u.X = X; u.Y = Y; u.Z = Z;
   // tensors in forward order: e[l][0], e[l][1], pool[l] (l < L-1), then per
   // decoder level: cat, d0, d1; then the head output
@@ -460,10 +390,13 @@ static cudaError_t ensure_shape(UNet &u, int N, int X, int Y, int Z) {
     if (e == cudaSuccess) e = add(c, l);
   }
   if (e == cudaSuccess) e = add(u.cout, 0);
-  long long big = (long long)N * (u.base << (u.levels - 1)) * 2 * vox(u, 0);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&u.scratch, big * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&u.scratch2, big * sizeof(float));
-  u.scratch_n = big;
+  long long big = 0;
+  for (size_t q = 0; q < u.layers.size(); ++q) {
+    const Layer &L = u.layers[q];
+    const int l = layer_level(u, (int)q);
+    big = std::max(big, conv32_wgrad_floats(u.D, L.k, N, X >> l, Y >> l, u.D == 3 ? Z >> l : 1, L.cin, L.cout));
+  }
+  if (e == cudaSuccess) e = cudaMalloc((void **)&u.partial, big * sizeof(float));
   if (u.xcl) cudaFree(u.xcl);
   u.xcl = nullptr;
   u.xcl_n = tc_xcl_elems(u, N, X, Y, Z);
@@ -503,45 +436,39 @@ static void conv_tc(const UNet &u, int li, int N, int X, int Y, int Z, const flo
   conv_tc_forward(D, xcl, N, X, Y, Z, L.cin, u.wpk + u.pk_off[li], u.w + L.boff, L.cout, relu, y, u.terr, u.st);
 }
 
-template <int D>
-static void conv_fwd(UNet &u, const Layer &L, const float *x, float *y, int lvl, int relu, bool tc = false) {
-  const long long nv = vox(u, lvl);
-  const int li = (int)(&L - u.layers.data());
-  if (tc && u.pk_off[li] >= 0) {
-    conv_tc<D>(u, li, u.N, u.X >> lvl, u.Y >> lvl, D == 3 ? (u.Z >> lvl) : 1, x, y, relu, u.xcl);
+// one convolution on the CUDA cores (3^D, or the 1^D head)
+static void conv_cuda(const UNet &u, const Layer &L, const float *x, float *y, int N, int X, int Y, int Z, int relu) {
+  if (L.k == 3) {
+    conv32(u.D, false, ConvArgs32{x, u.wb + L.woff, u.w + L.boff, y, nullptr, N, L.cin, L.cout, X, Y, Z, relu}, u.st);
     return;
   }
-  dim3 grid(nblk(nv), (L.cout + 7) / 8, u.N);
-  const int X = u.X >> lvl, Y = u.Y >> lvl, Z = D == 3 ? (u.Z >> lvl) : 1;
-  if (L.k == 3)
-    k_conv<D, 3, false><<<grid, NT, 0, u.st>>>(x, u.wb + L.woff, u.w + L.boff, y, u.N, L.cin, L.cout, X, Y, Z, relu,
-                                               L.cin, L.cout);
-  else
-    k_conv<D, 1, false><<<grid, NT, 0, u.st>>>(x, u.wb + L.woff, u.w + L.boff, y, u.N, L.cin, L.cout, X, Y, Z, relu,
-                                               L.cin, L.cout);
+  const long long nv = (long long)X * Y * Z;
+  k_conv1<false><<<dim3(nblk(nv), (L.cout + 7) / 8, N), NT, 0, u.st>>>(x, u.wb + L.woff, u.w + L.boff, y, nullptr, L.cin,
+                                                                       L.cout, nv);
 }
 
-// data gradient gx (cin channels) from gy (cout channels); weight gradient into u.g
 template <int D>
-static void conv_bwd(UNet &u, const Layer &L, const float *x, const float *gy, float *gx, int lvl) {
-  const long long nv = vox(u, lvl);
+static void conv_fwd(UNet &u, const Layer &L, const float *x, float *y, int lvl, int relu, bool tc = false) {
+  const int li = (int)(&L - u.layers.data());
   const int X = u.X >> lvl, Y = u.Y >> lvl, Z = D == 3 ? (u.Z >> lvl) : 1;
-  dim3 wg(L.cout, L.cin);
-  if (L.k == 3) k_conv_wgrad<D, 3><<<wg, NT, 0, u.st>>>(x, gy, u.g + L.woff, u.g + L.boff, u.N, L.cin, L.cout, X, Y, Z);
-  else k_conv_wgrad<D, 1><<<wg, NT, 0, u.st>>>(x, gy, u.g + L.woff, u.g + L.boff, u.N, L.cin, L.cout, X, Y, Z);
-  if (!gx) return;
-  dim3 grid(nblk(nv), (L.cin + 7) / 8, u.N);
-  if (L.k == 3)
-    k_conv<D, 3, true><<<grid, NT, 0, u.st>>>(gy, u.wb + L.woff, nullptr, gx, u.N, L.cout, L.cin, X, Y, Z, 0, L.cin,
-                                              L.cout);
-  else
-    k_conv<D, 1, true><<<grid, NT, 0, u.st>>>(gy, u.wb + L.woff, nullptr, gx, u.N, L.cout, L.cin, X, Y, Z, 0, L.cin,
-                                              L.cout);
+  if (tc && u.pk_off[li] >= 0) conv_tc<D>(u, li, u.N, X, Y, Z, x, y, relu, u.xcl);
+  else conv_cuda(u, L, x, y, u.N, X, Y, Z, relu);
 }
 
-static void relu_bwd(UNet &u, int q) {
-  long long n = (long long)u.N * u.act_c[q] * vox(u, u.act_lvl[q]);
-  k_relu_bwd<<<nblk(n), NT, 0, u.st>>>(u.act[q], u.grad[q], n);
+// data gradient gx (cin channels; 0 where mask, x's activation, is <= 0) from
+// gy (cout channels); weight gradient into u.g
+template <int D>
+static void conv_bwd(UNet &u, const Layer &L, const float *x, const float *gy, float *gx, const float *mask, int lvl) {
+  const int X = u.X >> lvl, Y = u.Y >> lvl, Z = D == 3 ? (u.Z >> lvl) : 1;
+  conv32_wgrad(D, L.k, WgradArgs{x, gy, u.partial, u.N, L.cin, L.cout, X, Y, Z, 0}, u.g + L.woff, u.g + L.boff, u.st);
+  if (!gx) return;
+  if (L.k == 3) {
+    conv32(D, true, ConvArgs32{gy, u.wb + L.woff, nullptr, gx, mask, u.N, L.cout, L.cin, X, Y, Z, 0}, u.st);
+    return;
+  }
+  const long long nv = (long long)X * Y * Z;
+  k_conv1<true><<<dim3(nblk(nv), (L.cin + 7) / 8, u.N), NT, 0, u.st>>>(gy, u.wb + L.woff, nullptr, gx, mask, L.cout,
+                                                                       L.cin, nv);
 }
 
 template <int D>
@@ -564,9 +491,8 @@ static void forward(UNet &u, const float *x, bool tc = false) {
     const int c = u.base << l, cup = u.base << (l + 1);
     const int X = u.X >> l, Y = u.Y >> l, Z = D == 3 ? (u.Z >> l) : 1;
     const long long nv = vox(u, l);
-    k_up<D><<<nblk((long long)u.N * cup * nv), NT, 0, u.st>>>(prev, u.act[I.cat[l]], u.N, cup, cup + c, 0, X, Y, Z);
-    k_slot_copy<<<nblk((long long)u.N * c * nv), NT, 0, u.st>>>(u.act[I.e1[l]], u.act[I.cat[l]], u.N, c, c, 0,
-                                                                cup + c, cup, nv, 0);
+    k_up_cat<D><<<nblk((long long)u.N * (cup + c) * nv), NT, 0, u.st>>>(prev, u.act[I.e1[l]], u.act[I.cat[l]], u.N, cup,
+                                                                        c, X, Y, Z);
     conv_fwd<D>(u, u.layers[li++], u.act[I.cat[l]], u.act[I.d0[l]], l, 1, tc);
     conv_fwd<D>(u, u.layers[li++], u.act[I.d0[l]], u.act[I.d1[l]], l, 1, tc);
     prev = u.act[I.d1[l]];
@@ -578,69 +504,41 @@ static void forward(UNet &u, const float *x, bool tc = false) {
   }
 }
 
-// gradients of all parameters given d loss / d out in u.grad[out]
+// gradients of all parameters given d loss / d out in u.grad[out].  The
+// kernels that write an activation's gradient last apply its ReLU.
 template <int D>
 static void backward(UNet &u, const float *x) {
   const Idx I = indices(u);
-  const int nl = (int)u.layers.size();
-  int li = nl - 1;
-  // zero the activation gradients that are accumulated into: every e1 (skip
-  // and pool/up paths) and the decoder outputs below the finest level (their
-  // only contribution arrives through the upsampling of the next finer level)
-  for (int l = 0; l < u.levels; ++l) {
-    long long n = (long long)u.N * u.act_c[I.e1[l]] * vox(u, l);
-    cudaMemsetAsync(u.grad[I.e1[l]], 0, n * sizeof(float), u.st);
-  }
-  for (int l = 1; l <= u.levels - 2; ++l) {
-    long long n = (long long)u.N * u.act_c[I.d1[l]] * vox(u, l);
-    cudaMemsetAsync(u.grad[I.d1[l]], 0, n * sizeof(float), u.st);
-  }
   const int top = u.levels == 1 ? I.e1[0] : I.d1[0];
-  // head
-  {
-    long long n = (long long)u.N * u.base * vox(u, 0);
-    if (u.levels == 1) {
-      conv_bwd<D>(u, u.layers[li--], u.act[top], u.grad[I.out], u.scratch, 0);
-      k_slot_copy<<<nblk(n), NT, 0, u.st>>>(u.scratch, u.grad[top], u.N, u.base, u.base, 0, u.base, 0, vox(u, 0), 1);
-    } else {
-      conv_bwd<D>(u, u.layers[li--], u.act[top], u.grad[I.out], u.grad[top], 0);
-    }
-  }
+  conv_bwd<D>(u, u.layers.back(), u.act[top], u.grad[I.out], u.grad[top], u.act[top], 0);
   // decoder, finest level first
   for (int l = 0; l <= u.levels - 2; ++l) {
     const int c = u.base << l, cup = u.base << (l + 1);
     const int X = u.X >> l, Y = u.Y >> l, Z = D == 3 ? (u.Z >> l) : 1;
     const long long nv = vox(u, l);
-    const Layer &L1 = u.layers[li--];
-    const Layer &L0 = u.layers[li--];
-    relu_bwd(u, I.d1[l]);
-    conv_bwd<D>(u, L1, u.act[I.d0[l]], u.grad[I.d1[l]], u.grad[I.d0[l]], l);
-    relu_bwd(u, I.d0[l]);
-    conv_bwd<D>(u, L0, u.act[I.cat[l]], u.grad[I.d0[l]], u.grad[I.cat[l]], l);
-    // split the concatenation: upsampled part -> coarser tensor, skip -> e1[l]
-    k_slot_copy<<<nblk((long long)u.N * c * nv), NT, 0, u.st>>>(u.grad[I.cat[l]], u.grad[I.e1[l]], u.N, c, cup + c,
-                                                                cup, c, 0, nv, 1);
+    const Layer &L1 = u.layers[2 * u.levels + 2 * (u.levels - 2 - l) + 1];
+    const Layer &L0 = u.layers[2 * u.levels + 2 * (u.levels - 2 - l)];
+    conv_bwd<D>(u, L1, u.act[I.d0[l]], u.grad[I.d1[l]], u.grad[I.d0[l]], u.act[I.d0[l]], l);
+    conv_bwd<D>(u, L0, u.act[I.cat[l]], u.grad[I.d0[l]], u.grad[I.cat[l]], nullptr, l);
+    // split the concatenation: skip -> e1[l], upsampled part -> coarser tensor
+    k_slot_copy<<<nblk((long long)u.N * c * nv), NT, 0, u.st>>>(u.grad[I.cat[l]], u.grad[I.e1[l]], u.N, c, cup + c, cup,
+                                                                nv);
     const int coarse = l + 1 == u.levels - 1 ? I.e1[l + 1] : I.d1[l + 1];
     const long long n2 = (long long)u.N * cup * vox(u, l + 1);
-    k_up_bwd<D><<<nblk(n2), NT, 0, u.st>>>(u.grad[I.cat[l]], u.scratch, u.N, cup, cup + c, 0, X, Y, Z);
-    k_slot_copy<<<nblk(n2), NT, 0, u.st>>>(u.scratch, u.grad[coarse], u.N, cup, cup, 0, cup, 0, vox(u, l + 1), 1);
+    k_up_bwd<D><<<nblk(n2), NT, 0, u.st>>>(u.grad[I.cat[l]], u.act[coarse], u.grad[coarse], u.N, cup, cup + c, X, Y, Z);
   }
   // encoder, coarsest level first
   for (int l = u.levels - 1; l >= 0; --l) {
-    const Layer &L1 = u.layers[2 * l + 1];
-    const Layer &L0 = u.layers[2 * l];
-    relu_bwd(u, I.e1[l]);
-    conv_bwd<D>(u, L1, u.act[I.e0[l]], u.grad[I.e1[l]], u.grad[I.e0[l]], l);
-    relu_bwd(u, I.e0[l]);
+    conv_bwd<D>(u, u.layers[2 * l + 1], u.act[I.e0[l]], u.grad[I.e1[l]], u.grad[I.e0[l]], u.act[I.e0[l]], l);
     const float *in = l == 0 ? x : u.act[I.pool[l - 1]];
     float *gin = l == 0 ? nullptr : u.grad[I.pool[l - 1]];
-    conv_bwd<D>(u, L0, in, u.grad[I.e0[l]], gin, l);
+    conv_bwd<D>(u, u.layers[2 * l], in, u.grad[I.e0[l]], gin, nullptr, l);
     if (l > 0) {
       const int X = u.X >> (l - 1), Y = u.Y >> (l - 1), Z = D == 3 ? (u.Z >> (l - 1)) : 1;
       const int cl = u.base << (l - 1);
-      long long n = (long long)u.N * cl * vox(u, l - 1);
-      k_pool_bwd<D><<<nblk(n), NT, 0, u.st>>>(u.grad[I.pool[l - 1]], u.scratch, (long long)u.N * cl, X, Y, Z);
-      k_slot_copy<<<nblk(n), NT, 0, u.st>>>(u.scratch, u.grad[I.e1[l - 1]], u.N, cl, cl, 0, cl, 0, vox(u, l - 1), 1);
+      const long long n = (long long)u.N * cl * vox(u, l - 1);
+      k_pool_bwd<D><<<nblk(n), NT, 0, u.st>>>(u.grad[I.pool[l - 1]], u.act[I.e1[l - 1]], u.grad[I.e1[l - 1]],
+                                              (long long)u.N * cl, X, Y, Z);
     }
   }
 }
@@ -764,20 +662,10 @@ static long long static_layout(const UNet &u, const Shp &s, long long *off) {
 template <int D>
 static void conv_fwd_s(const UNet &u, const Shp &s, const Layer &L, const float *x, float *y, int lvl, int relu,
                        __nv_bfloat16 *xcl) {
-  const long long nv = svox(u, s, lvl);
   const int li = (int)(&L - u.layers.data());
-  if (u.pk_off[li] >= 0) {
-    conv_tc<D>(u, li, s.N, s.X >> lvl, s.Y >> lvl, D == 3 ? (s.Z >> lvl) : 1, x, y, relu, xcl);
-    return;
-  }
-  dim3 grid(nblk(nv), (L.cout + 7) / 8, s.N);
   const int X = s.X >> lvl, Y = s.Y >> lvl, Z = D == 3 ? (s.Z >> lvl) : 1;
-  if (L.k == 3)
-    k_conv<D, 3, false><<<grid, NT, 0, u.st>>>(x, u.wb + L.woff, u.w + L.boff, y, s.N, L.cin, L.cout, X, Y, Z, relu,
-                                               L.cin, L.cout);
-  else
-    k_conv<D, 1, false><<<grid, NT, 0, u.st>>>(x, u.wb + L.woff, u.w + L.boff, y, s.N, L.cin, L.cout, X, Y, Z, relu,
-                                               L.cin, L.cout);
+  if (u.pk_off[li] >= 0) conv_tc<D>(u, li, s.N, X, Y, Z, x, y, relu, xcl);
+  else conv_cuda(u, L, x, y, s.N, X, Y, Z, relu);
 }
 
 // the network's forward pass with activations at act + off[q] and the head
@@ -805,9 +693,8 @@ static void forward_static(const UNet &u, const Shp &s, const float *x, float *a
     const int X = s.X >> l, Y = s.Y >> l, Z = D == 3 ? (s.Z >> l) : 1;
     const long long nv = svox(u, s, l);
     float *cat = act + off[I.cat[l]];
-    k_up<D><<<nblk((long long)s.N * cup * nv), NT, 0, u.st>>>(prev, cat, s.N, cup, cup + c, 0, X, Y, Z);
-    k_slot_copy<<<nblk((long long)s.N * c * nv), NT, 0, u.st>>>(act + off[I.e1[l]], cat, s.N, c, c, 0, cup + c, cup,
-                                                                nv, 0);
+    k_up_cat<D><<<nblk((long long)s.N * (cup + c) * nv), NT, 0, u.st>>>(prev, act + off[I.e1[l]], cat, s.N, cup, c, X, Y,
+                                                                        Z);
     conv_fwd_s<D>(u, s, u.layers[li++], cat, act + off[I.d0[l]], l, 1, xcl);
     conv_fwd_s<D>(u, s, u.layers[li++], act + off[I.d0[l]], act + off[I.d1[l]], l, 1, xcl);
     prev = act + off[I.d1[l]];
@@ -830,6 +717,10 @@ ep_status ep_net_create(int ndim, int in_ch, int out_ch, int base, int levels, u
   u.D = ndim; u.cin = in_ch; u.cout = out_ch; u.base = base; u.levels = levels;
   u.st = (cudaStream_t)stream;
   unet_layers(u);
+  if (conv32_configure() != cudaSuccess) {
+    delete n;
+    return nfail(nullptr, EP_ERR_CUDA, "ep_net_create: convolution kernels' shared-memory attribute");
+  }
   // He-uniform initialisation from splitmix64 (seeded); biases and the head zero
   std::vector<float> w(u.nparam, 0.f);
   unsigned long long st = seed;
@@ -935,7 +826,6 @@ static ep_status net_grads(ep_net *n, const float *x, const float *t, int N, con
   if (u.D == 2) forward<2>(u, x); else forward<3>(u, x);
   const Idx I = indices(u);
   const long long no = (long long)N * u.cout * vox(u, 0);
-  NCK(n, cudaMemsetAsync(u.g, 0, u.nparam * 4, u.st));
   const float inv_s = u.out_scale > 0.f ? 1.f / u.out_scale : 1.f;
   k_mse<<<MSE_BLOCKS, NT, 0, u.st>>>(u.act[I.out], t, u.grad[I.out], no, u.dloss + 1, inv_s);
   k_mse_final<<<1, NT, 0, u.st>>>(u.dloss + 1, no, u.dloss);
@@ -992,7 +882,7 @@ ep_status ep_net_destroy(ep_net *n) {
   if (u.st) cudaStreamSynchronize(u.st);
   for (float *p : u.act) cudaFree(p);
   for (float *p : u.grad) cudaFree(p);
-  cudaFree(u.scratch); cudaFree(u.scratch2);
+  cudaFree(u.partial);
   cudaFree(u.w); cudaFree(u.g); cudaFree(u.m); cudaFree(u.v); cudaFree(u.wb); cudaFree(u.dloss);
   cudaFree(u.wpk); cudaFree(u.xcl); cudaFree(u.terr);
   delete n;

@@ -1,0 +1,84 @@
+"""The FP32 training convolutions (forward, data gradient, weight gradient) at sizes and channel
+counts around their tiles, against the same network in FP64 torch with the same BF16 weights."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2305_01701_gb300 import build as B
+    B.build()
+    import paper_2305_01701_gb300 as P
+    return P
+
+
+def _reference(params, x, t, nd, cin, cout, base, levels):
+    import torch
+    F = torch.nn.functional
+    conv, pool = (F.conv3d, F.avg_pool3d) if nd == 3 else (F.conv2d, F.avg_pool2d)
+    leaves, at, terms = [], 0, 0
+
+    def layer(a, ci, co, k):
+        nonlocal at, terms
+        m = ci * co * k ** nd
+        w = params[at:at + m].bfloat16().double().view([co, ci] + [k] * nd).requires_grad_()
+        b = params[at + m:at + m + co].double().requires_grad_()
+        at += m + co
+        terms = max(terms, ci * k ** nd, co * k ** nd)
+        leaves.extend([w, b])
+        return conv(a, w, b, padding=k // 2)
+
+    skips, a, ci = [], x.double(), cin
+    for lv in range(levels):
+        o = base << lv
+        a = torch.relu(layer(torch.relu(layer(a, ci, o, 3)), o, o, 3))
+        ci = o
+        if lv < levels - 1:
+            skips.append(a)
+            a = pool(a, 2)
+    for lv in range(levels - 2, -1, -1):
+        o = base << lv
+        a = torch.cat([F.interpolate(a, scale_factor=2, mode="nearest"), skips[lv]], 1)
+        a = torch.relu(layer(torch.relu(layer(a, 3 * o, o, 3)), o, o, 3))
+    y = layer(a, base, cout, 1)
+    loss = ((y - t.double()) ** 2).mean()
+    loss.backward()
+    return float(loss.detach()), torch.cat([q.grad.reshape(-1) for q in leaves]), terms
+
+
+@pytest.mark.parametrize("nd,size,cin,cout,base,levels,N", [
+    (2, (5, 3), 1, 1, 1, 1, 1),          # less than a tile of voxels and of channels
+    (2, (16, 32), 9, 5, 16, 1, 2),       # exactly one tile
+    (2, (20, 36), 9, 5, 16, 2, 3),       # one row and one run beyond it
+    (2, (34, 66), 17, 33, 12, 2, 1),     # channels beyond a block of 16 / 32
+    (3, (16, 8, 4), 4, 3, 16, 1, 1),
+    (3, (17, 9, 5), 13, 9, 33, 1, 2),
+    (3, (20, 12, 8), 13, 9, 16, 3, 1),
+    (3, (6, 2, 14), 5, 2, 24, 2, 2),
+])
+def test_training_convolutions_match_fp64(P, nd, size, cin, cout, base, levels, N):
+    import torch
+    gen = torch.Generator().manual_seed(3)
+    net = P.Net(nd, cin, cout, base=base, levels=levels)
+    params = 0.1 * torch.randn(net.n_params(), generator=gen)
+    net.set_params(params.numpy())
+    dims = tuple(reversed(size))
+    x = torch.randn((N, cin) + dims, generator=gen).cuda()
+    t = torch.randn((N, cout) + dims, generator=gen).cuda()
+    loss, g = net.gradients(x.data_ptr(), t.data_ptr(), N, list(size))
+    loss2, g2 = net.gradients(x.data_ptr(), t.data_ptr(), N, list(size))
+    assert loss == loss2 and np.array_equal(g, g2)      # sums in a fixed order
+    ref_loss, ref, terms = _reference(params.cuda(), x, t, nd, cin, cout, base, levels)
+    vox = N * int(np.prod(size))
+    # FP32 sums of `terms` products per layer and `vox` per weight gradient, each rounding
+    # 2^-24: their random growth, through the layers of both passes
+    bound = 2.0 ** -24 * (np.sqrt(terms) + np.sqrt(vox)) * (4 * levels + 2)
+    assert abs(loss - ref_loss) <= bound * ref_loss
+    err = np.linalg.norm(g - ref.cpu().numpy()) / np.linalg.norm(ref.cpu().numpy())
+    assert err <= bound, (err, bound)
+    net.close()

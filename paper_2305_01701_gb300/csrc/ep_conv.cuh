@@ -9,8 +9,8 @@ namespace ep {
 
 struct ConvArgs32 {
   const float *x;             // N x cin x [Z x] Y x X
-  const __nv_bfloat16 *w;     // forward: cout x cin x taps; transposed: cin x cout x taps
-  const float *b;             // cout (forward only)
+  const float *w;             // the layer's packed weights in this direction (conv32_pack)
+  const float *b;             // cout (nullable)
   float *y;                   // N x cout x [Z x] Y x X
   const float *mask;          // nullable, the shape of y: y is 0 where it is <= 0
   int N, cin, cout, X, Y, Z, relu;
@@ -32,8 +32,18 @@ struct PackTable {
 void conv_tc_pack_weights(const PackTable &P, const __nv_bfloat16 *w, __nv_bfloat16 *out, cudaStream_t st);
 
 cudaError_t conv32_configure();
+// FP32 copies of the 3^D layers' weights in the order the kernels read them, for
+// the forward pass and for the data gradient
+struct Pack32 {
+  int n, taps;
+  int cin[24], cout[24];
+  long long src[24], fwd[24], bwd[24];   // offsets of the weights and of their packed copies
+};
+__host__ __device__ constexpr int conv32_cinp(int cin) { return (cin + 7) / 8 * 8; }
+long long conv32_packed(int D, int cin, int cout);   // floats of one direction
+void conv32_pack(const Pack32 &P, const __nv_bfloat16 *w, float *out, cudaStream_t st);
 // 3^D convolution with zero padding, forward or data gradient
-void conv32(int D, bool trans, const ConvArgs32 &A, cudaStream_t st);
+void conv32(int D, const ConvArgs32 &A, cudaStream_t st);
 // weight and bias gradient of a k^D convolution (k = 1 or 3): overwrites dw, db
 long long conv32_wgrad_floats(int D, int k, int N, int X, int Y, int Z, int cin, int cout);
 void conv32_wgrad(int D, int k, WgradArgs A, float *dw, float *db, cudaStream_t st);

@@ -40,6 +40,9 @@ __device__ __forceinline__ unsigned su32(const void *p) { return (unsigned)__cvt
 __device__ __forceinline__ void cp4(float *dst, const float *src, bool ok) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(su32(dst)), "l"(src), "r"(ok ? 4 : 0));
 }
+__device__ __forceinline__ void cp16(float *dst, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(su32(dst)), "l"(src));
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int n>
 __device__ __forceinline__ void cp_wait() {
@@ -48,34 +51,41 @@ __device__ __forceinline__ void cp_wait() {
 
 // ---- forward and data gradient --------------------------------------------
 constexpr int CO = 16;   // output channels per block
-constexpr int CK = 4;    // input channels per stage
 constexpr int CT = 128;  // threads
 constexpr int TX = 16;   // voxels along x
 constexpr int PX = 20;   // pitch of a row of TX + 2 inputs
-constexpr int WS = 20;   // pitch of a tap's CO weights
 
-template <int D>
+// KS = 1: 512 voxels per block, every thread sums over all input channels.
+// KS = 4: 128 voxels per block; each warp takes every fourth input channel and
+// the four partial sums are added at the end.
+template <int D, int KS>
 struct Tile {
-  static constexpr int TY = D == 3 ? 8 : 32, TZ = D == 3 ? 4 : 1;
+  static constexpr int CK = KS == 1 ? 4 : 8;   // input channels per stage
+  static constexpr int TY = D == 3 ? (KS == 1 ? 8 : 4) : (KS == 1 ? 32 : 8);
+  static constexpr int TZ = D == 3 ? (KS == 1 ? 4 : 2) : 1;
   static constexpr int RY = TY + 2, RZ = D == 3 ? TZ + 2 : 1;   // rows with the halo
   static constexpr int TAPS = D == 3 ? 27 : 9;
   static constexpr int ROWS = CK * RZ * RY;
   static constexpr int WN = CK * TAPS * CO;   // weights per stage
-  static constexpr size_t bytes = 2 * (size_t)(ROWS * PX + CK * TAPS * WS) * sizeof(float);
+  static constexpr size_t stages = 2 * (size_t)(ROWS * PX + WN) * sizeof(float);
+  static constexpr size_t sums = KS == 1 ? 0 : (size_t)CT * CO * 4 * sizeof(float);
+  static constexpr size_t bytes = stages > sums ? stages : sums;
 };
 
 // y[n, co, v] = b[co] + sum over ci, tap of W(co, ci, tap) x[n, ci, v + tap - 1]
-// TRANS: the data gradient, channels swapped and taps mirrored (no bias).
-// relu: max(y, 0).  mask (nullable): y is 0 where mask[n, co, v] <= 0 (the
+// The data gradient is the same with the weights packed the other way round
+// (channels swapped, taps mirrored) and no bias.  relu: max(y, 0).  mask (nullable): y is 0 where mask[n, co, v] <= 0 (the
 // ReLU of the layer that produced the tensor whose gradient y is).
-template <int D, bool TRANS>
+template <int D, int KS>
 __global__ void __launch_bounds__(CT, 3) k_conv_tile(const ConvArgs32 A) {
-  using L = Tile<D>;
+  using L = Tile<D, KS>;
+  constexpr int CK = L::CK;
   extern __shared__ __align__(16) float sm[];
   auto xs = [&](int k) { return sm + k * (L::ROWS * PX); };
-  auto ws = [&](int k) { return sm + 2 * L::ROWS * PX + k * (CK * L::TAPS * WS); };
+  auto ws = [&](int k) { return sm + 2 * L::ROWS * PX + k * L::WN; };
   const int tid = threadIdx.x;
-  const int tx = tid & 3, ty = (tid >> 2) % L::TY, tz = (tid >> 2) / L::TY;
+  const int vt = tid % (CT / KS), kpart = tid / (CT / KS);
+  const int tx = vt & 3, ty = (vt >> 2) % L::TY, tz = (vt >> 2) / L::TY;
   const int X = A.X, Y = A.Y, Z = A.Z, cin = A.cin, cout = A.cout;
   const int nbx = (X + TX - 1) / TX, nby = (Y + L::TY - 1) / L::TY;
   const int x0 = (blockIdx.x % nbx) * TX, y0 = (blockIdx.x / nbx % nby) * L::TY, z0 = blockIdx.x / (nbx * nby) * L::TZ;
@@ -92,35 +102,26 @@ __global__ void __launch_bounds__(CT, 3) k_conv_tile(const ConvArgs32 A) {
       cp4(dst + row * PX + xx, ok ? xn + (long long)(c0 + c) * nvox + ((long long)gz * Y + gy) * X + gx : xn, ok);
     }
   };
-  // weights of a stage: tap fastest, then the channel that is contiguous in
-  // memory (input channels forward, output channels transposed)
+  // a stage's weights are one run of the packed array: [ci][tap][16 co]
+  const float *wn = A.w + (long long)blockIdx.y * conv32_cinp(cin) * L::TAPS * CO;
   auto fetch_w = [&](int c0, float *dst) {
-#pragma unroll 4
-    for (int e = tid; e < L::WN; e += CT) {
-      const int tap = e % L::TAPS, r = e / L::TAPS;
-      const int c = TRANS ? r / CO : r % CK, o = TRANS ? r % CO : r / CK;
-      float v = 0.f;
-      if (c0 + c < cin && co0 + o < cout) {
-        const long long wi = TRANS ? ((long long)(c0 + c) * cout + co0 + o) * L::TAPS + (L::TAPS - 1 - tap)
-                                   : ((long long)(co0 + o) * cin + c0 + c) * L::TAPS + tap;
-        v = __bfloat162float(A.w[wi]);
-      }
-      dst[(c * L::TAPS + tap) * WS + o] = v;
-    }
+    const float *src = wn + (long long)c0 * L::TAPS * CO;
+    for (int e = tid; e < L::WN / 4; e += CT) cp16(dst + 4 * e, src + 4 * e);
   };
 
   float2 acc[CO / 2][4];
 #pragma unroll
   for (int p = 0; p < CO / 2; ++p) {
     const int c = co0 + 2 * p;
-    const float2 b = make_float2(!TRANS && c < cout ? A.b[c] : 0.f, !TRANS && c + 1 < cout ? A.b[c + 1] : 0.f);
+    const float2 b = make_float2(A.b && kpart == 0 && c < cout ? A.b[c] : 0.f,
+                                 A.b && kpart == 0 && c + 1 < cout ? A.b[c + 1] : 0.f);
 #pragma unroll
     for (int v = 0; v < 4; ++v) acc[p][v] = b;
   }
 
   fetch_x(0, xs(0));
-  cp_commit();
   fetch_w(0, ws(0));
+  cp_commit();
   const int stages = (cin + CK - 1) / CK;
   for (int s = 0; s < stages; ++s) {
     const int cur = s & 1;
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(CT, 3) k_conv_tile(const ConvArgs32 A) {
     }
     cp_commit();
     const float *xb = xs(cur) + (tz * L::RY + ty) * PX + 4 * tx, *wb = ws(cur);
-    for (int c = 0; c < CK; ++c) {
+    for (int c = kpart; c < CK; c += KS) {
 #pragma unroll
       for (int dz = 0; dz < (D == 3 ? 3 : 1); ++dz)
 #pragma unroll
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(CT, 3) k_conv_tile(const ConvArgs32 A) {
           const float xv[6] = {xa.x, xa.y, xa.z, xa.w, xc.x, xc.y};
 #pragma unroll
           for (int dx = 0; dx < 3; ++dx) {
-            const float4 *wp = reinterpret_cast<const float4 *>(wb + (c * L::TAPS + (dz * 3 + dy) * 3 + dx) * WS);
+            const float4 *wp = reinterpret_cast<const float4 *>(wb + (c * L::TAPS + (dz * 3 + dy) * 3 + dx) * CO);
 #pragma unroll
             for (int q = 0; q < CO / 4; ++q) {
               const float4 w4 = wp[q];
@@ -159,18 +160,44 @@ __global__ void __launch_bounds__(CT, 3) k_conv_tile(const ConvArgs32 A) {
     }
   }
 
+  // KS = 4: every warp's sums to shared memory, [part][channel, voxel][thread];
+  // warp k then adds and writes channels 4k .. 4k + 3
+  constexpr int CW = CO / KS;   // channels this thread writes
+  const int cw0 = KS == 1 ? 0 : kpart * CW;
+  float out[KS == 1 ? 1 : CW][4];
+  if constexpr (KS > 1) {
+    __syncthreads();   // the last stage is no longer read
+#pragma unroll
+    for (int c = 0; c < CO; ++c)
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        sm[((kpart * CO + c) * 4 + v) * 32 + vt] = (c & 1) ? acc[c / 2][v].y : acc[c / 2][v].x;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < CW; ++c)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        float r = sm[((cw0 + c) * 4 + v) * 32 + vt];
+#pragma unroll
+        for (int k = 1; k < KS; ++k) r += sm[((k * CO + cw0 + c) * 4 + v) * 32 + vt];
+        out[c][v] = r;
+      }
+  }
+
   const int ox = x0 + 4 * tx, oy = y0 + ty, oz = z0 + tz;
   if (ox >= X || oy >= Y || oz >= Z) return;
   const long long v0 = ((long long)oz * Y + oy) * X + ox;
   const bool vec = (X & 3) == 0;   // then v0 and every channel's offset are multiples of 4
 #pragma unroll
-  for (int c = 0; c < CO; ++c) {
-    if (co0 + c >= cout) break;
-    const long long o = ((long long)n * cout + co0 + c) * nvox + v0;
+  for (int c = 0; c < CW; ++c) {
+    const int co = co0 + cw0 + c;
+    if (co >= cout) break;
+    const long long o = ((long long)n * cout + co) * nvox + v0;
     float r[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      r[v] = (c & 1) ? acc[c / 2][v].y : acc[c / 2][v].x;
+      if constexpr (KS == 1) r[v] = (c & 1) ? acc[c / 2][v].y : acc[c / 2][v].x;
+      else r[v] = out[c][v];
       if (A.relu && r[v] < 0.f) r[v] = 0.f;
     }
     if (vec) {
@@ -196,7 +223,7 @@ constexpr int GPY = 36;   // pitch of a gradient voxel's channels
 
 template <int D, int K>
 struct GTile {
-  static constexpr int TY = D == 3 ? 4 : 16, TZ = D == 3 ? 2 : 1, R = K / 2;
+  static constexpr int TY = 4, TZ = D == 3 ? 2 : 1, R = K / 2;
   static constexpr int HX = TX + 2 * R, HY = TY + 2 * R, HZ = D == 3 ? TZ + 2 * R : 1;
   static constexpr int TAPS = D == 3 ? K * K * K : K * K;
   static constexpr int VOX = TX * TY * TZ, HALO = HX * HY * HZ;
@@ -310,12 +337,21 @@ __global__ void __launch_bounds__(GT, 1) k_conv_wgrad_tile(const WgradArgs A) {
   }
 }
 
-// dw = sum of the partial sums in the order of the splits; db likewise
-__global__ void k_wgrad_sum(const float *partial, int slots, long long per, int cout, float *dw, float *db) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = per + cout;
-  if (i >= stride) return;
+// dw = sum of the partial sums, db likewise: 8 threads per element add every
+// eighth split each, then their sums are added, in a fixed order
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float *partial, int slots, long long per, int cout, float *dw,
+                                                   float *db) {
+  __shared__ float sh[8][32];
+  const int e = threadIdx.x & 31, j = threadIdx.x >> 5;
+  const long long i = (long long)blockIdx.x * 32 + e, stride = per + cout;
   float s = 0.f;
-  for (int q = 0; q < slots; ++q) s += partial[q * stride + i];
+  if (i < stride)
+    for (int q = j; q < slots; q += 8) s += partial[q * stride + i];
+  sh[j][e] = s;
+  __syncthreads();
+  if (j != 0 || i >= stride) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) s += sh[q][e];
   if (i < per) dw[i] = s;
   else db[i - per] = s;
 }
@@ -335,7 +371,7 @@ int wgrad_quads(int cout) {
 // splits of the voxel tiles: enough blocks for two per SM (152 SMs), no more
 // than there are tiles
 int wgrad_splits(int D, int N, int X, int Y, int Z, int cin, int cout) {
-  const int ty = D == 3 ? 4 : 16, tz = D == 3 ? 2 : 1;
+  const int ty = 4, tz = D == 3 ? 2 : 1;
   const long long tiles = (long long)N * ((X + TX - 1) / TX) * ((Y + ty - 1) / ty) * ((Z + tz - 1) / tz);
   const int blocks = ((cout + GC - 1) / GC) * ((cin + GC - 1) / GC);
   return (int)std::max(1ll, std::min<long long>(tiles, 304 / blocks));
@@ -343,28 +379,69 @@ int wgrad_splits(int D, int N, int X, int Y, int Z, int cin, int cout) {
 
 }  // namespace
 
+// fewest blocks of the 512-voxel tiling that it is used for; below, the chip is
+// filled better by the 128-voxel blocks that split the input channels
+constexpr long long KS_BLOCKS = 400;
+
 cudaError_t conv32_configure() {
   cudaError_t e = cudaSuccess;
 #define EP_CFG(k, b) \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(b));
-  EP_CFG((k_conv_tile<2, false>), Tile<2>::bytes) EP_CFG((k_conv_tile<2, true>), Tile<2>::bytes)
-  EP_CFG((k_conv_tile<3, false>), Tile<3>::bytes) EP_CFG((k_conv_tile<3, true>), Tile<3>::bytes)
+  EP_CFG((k_conv_tile<2, 1>), (Tile<2, 1>::bytes)) EP_CFG((k_conv_tile<3, 1>), (Tile<3, 1>::bytes))
+  EP_CFG((k_conv_tile<2, 4>), (Tile<2, 4>::bytes)) EP_CFG((k_conv_tile<3, 4>), (Tile<3, 4>::bytes))
   EP_CFG((k_conv_wgrad_tile<2, 1>), (GTile<2, 1>::bytes)) EP_CFG((k_conv_wgrad_tile<2, 3>), (GTile<2, 3>::bytes))
   EP_CFG((k_conv_wgrad_tile<3, 1>), (GTile<3, 1>::bytes)) EP_CFG((k_conv_wgrad_tile<3, 3>), (GTile<3, 3>::bytes))
 #undef EP_CFG
   return e;
 }
 
-void conv32(int D, bool trans, const ConvArgs32 &A, cudaStream_t st) {
-  const int ty = D == 3 ? Tile<3>::TY : Tile<2>::TY, tz = D == 3 ? Tile<3>::TZ : 1;
-  dim3 grid(((A.X + TX - 1) / TX) * ((A.Y + ty - 1) / ty) * ((A.Z + tz - 1) / tz), (A.cout + CO - 1) / CO, A.N);
-  if (D == 3) {
-    if (trans) k_conv_tile<3, true><<<grid, CT, Tile<3>::bytes, st>>>(A);
-    else k_conv_tile<3, false><<<grid, CT, Tile<3>::bytes, st>>>(A);
-  } else {
-    if (trans) k_conv_tile<2, true><<<grid, CT, Tile<2>::bytes, st>>>(A);
-    else k_conv_tile<2, false><<<grid, CT, Tile<2>::bytes, st>>>(A);
+namespace {
+
+template <int D, int KS>
+dim3 conv_grid(const ConvArgs32 &A) {
+  using L = Tile<D, KS>;
+  return dim3(((A.X + TX - 1) / TX) * ((A.Y + L::TY - 1) / L::TY) * ((A.Z + L::TZ - 1) / L::TZ), (A.cout + CO - 1) / CO,
+              A.N);
+}
+
+template <int D>
+void conv_launch(const ConvArgs32 &A, cudaStream_t st) {
+  const dim3 g = conv_grid<D, 1>(A);
+  if ((long long)g.x * g.y * g.z >= KS_BLOCKS) k_conv_tile<D, 1><<<g, CT, Tile<D, 1>::bytes, st>>>(A);
+  else k_conv_tile<D, 4><<<conv_grid<D, 4>(A), CT, Tile<D, 4>::bytes, st>>>(A);
+}
+
+// BF16 cout x cin x taps -> FP32 [block of 16 output channels][ci][tap][16],
+// forward (even blockIdx.y) and transposed (odd); channels beyond the last are
+// zero, input channels are padded to a multiple of 8
+__global__ void k_pack32(const Pack32 P, const __nv_bfloat16 *w, float *out) {
+  const int l = blockIdx.y >> 1, tr = blockIdx.y & 1, taps = P.taps;
+  const int cin = tr ? P.cout[l] : P.cin[l], cout = tr ? P.cin[l] : P.cout[l], cinp = conv32_cinp(cin);
+  const int total = (cout + CO - 1) / CO * cinp * taps * CO;
+  float *dst = out + (tr ? P.bwd[l] : P.fwd[l]);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int tap = i / CO % taps, ci = i / (CO * taps) % cinp, co = i / (CO * taps * cinp) * CO + i % CO;
+    float v = 0.f;
+    if (ci < cin && co < cout)
+      v = __bfloat162float(w[P.src[l] + (tr ? ((long long)ci * cout + co) * taps + taps - 1 - tap
+                                            : ((long long)co * cin + ci) * taps + tap)]);
+    dst[i] = v;
   }
+}
+
+}  // namespace
+
+long long conv32_packed(int D, int cin, int cout) {
+  return (long long)((cout + CO - 1) / CO) * conv32_cinp(cin) * (D == 3 ? 27 : 9) * CO;
+}
+
+void conv32_pack(const Pack32 &P, const __nv_bfloat16 *w, float *out, cudaStream_t st) {
+  k_pack32<<<dim3(96, 2 * P.n), 256, 0, st>>>(P, w, out);
+}
+
+void conv32(int D, const ConvArgs32 &A, cudaStream_t st) {
+  if (D == 3) conv_launch<3>(A, st);
+  else conv_launch<2>(A, st);
 }
 
 long long conv32_wgrad_floats(int D, int k, int N, int X, int Y, int Z, int cin, int cout) {
@@ -381,7 +458,7 @@ void conv32_wgrad(int D, int k, WgradArgs A, float *dw, float *db, cudaStream_t 
     if (k == 3) wgrad_launch<2, 3>(A, sx, st); else wgrad_launch<2, 1>(A, sx, st);
   }
   const long long taps = D == 3 ? (long long)k * k * k : (long long)k * k, per = (long long)A.cout * A.cin * taps;
-  k_wgrad_sum<<<(unsigned)((per + A.cout + 127) / 128), 128, 0, st>>>(A.partial, sx * (8 / A.nq), per, A.cout, dw, db);
+  k_wgrad_sum<<<(unsigned)((per + A.cout + 31) / 32), 256, 0, st>>>(A.partial, sx * (8 / A.nq), per, A.cout, dw, db);
 }
 
 }  // namespace ep

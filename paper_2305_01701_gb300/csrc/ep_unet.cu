@@ -257,6 +257,10 @@ struct UNet {
   std::vector<long long> pk_off;
   __nv_bfloat16 *xcl = nullptr;
   long long xcl_n = 0;
+  // FP32 copies of the 3^D layers' weights for the CUDA-core convolutions, and
+  // their offsets per layer (the 1^D head has none)
+  float *wp32 = nullptr;
+  std::vector<long long> fwd_off, bwd_off;
   int *terr = nullptr;
   // the network's output is out_scale times the head's: training on targets
   // of any magnitude keeps the head's values of order one
@@ -313,8 +317,37 @@ static long long tc_layout(UNet &u) {
   return off;
 }
 
-// repack the BF16 weights for the tensor cores (after every weight change)
-static void tc_pack(UNet &u) {
+// offsets of the 3^D layers' FP32 copies; total floats
+static long long layout32(UNet &u) {
+  long long off = 0;
+  u.fwd_off.assign(u.layers.size(), -1);
+  u.bwd_off = u.fwd_off;
+  for (size_t q = 0; q < u.layers.size(); ++q) {
+    const Layer &L = u.layers[q];
+    if (L.k != 3) continue;
+    u.fwd_off[q] = off;
+    off += conv32_packed(u.D, L.cin, L.cout);
+    u.bwd_off[q] = off;
+    off += conv32_packed(u.D, L.cout, L.cin);
+  }
+  return off;
+}
+
+// the kernels' copies of the BF16 weights (after every weight change)
+static void pack_weights(UNet &u) {
+  Pack32 Q{};
+  Q.taps = u.D == 3 ? 27 : 9;
+  for (size_t q = 0; q < u.layers.size(); ++q) {
+    if (u.fwd_off[q] < 0) continue;
+    const Layer &L = u.layers[q];
+    Q.cin[Q.n] = L.cin;
+    Q.cout[Q.n] = L.cout;
+    Q.src[Q.n] = L.woff;
+    Q.fwd[Q.n] = u.fwd_off[q];
+    Q.bwd[Q.n] = u.bwd_off[q];
+    ++Q.n;
+  }
+  conv32_pack(Q, u.wb, u.wp32, u.st);
   PackTable P{};
   P.taps = u.D == 3 ? 27 : 9;
   for (size_t q = 0; q < u.layers.size(); ++q) {
@@ -439,7 +472,8 @@ static void conv_tc(const UNet &u, int li, int N, int X, int Y, int Z, const flo
 // one convolution on the CUDA cores (3^D, or the 1^D head)
 static void conv_cuda(const UNet &u, const Layer &L, const float *x, float *y, int N, int X, int Y, int Z, int relu) {
   if (L.k == 3) {
-    conv32(u.D, false, ConvArgs32{x, u.wb + L.woff, u.w + L.boff, y, nullptr, N, L.cin, L.cout, X, Y, Z, relu}, u.st);
+    const float *w = u.wp32 + u.fwd_off[&L - u.layers.data()];
+    conv32(u.D, ConvArgs32{x, w, u.w + L.boff, y, nullptr, N, L.cin, L.cout, X, Y, Z, relu}, u.st);
     return;
   }
   const long long nv = (long long)X * Y * Z;
@@ -463,7 +497,8 @@ static void conv_bwd(UNet &u, const Layer &L, const float *x, const float *gy, f
   conv32_wgrad(D, L.k, WgradArgs{x, gy, u.partial, u.N, L.cin, L.cout, X, Y, Z, 0}, u.g + L.woff, u.g + L.boff, u.st);
   if (!gx) return;
   if (L.k == 3) {
-    conv32(D, true, ConvArgs32{gy, u.wb + L.woff, nullptr, gx, mask, u.N, L.cout, L.cin, X, Y, Z, 0}, u.st);
+    const float *w = u.wp32 + u.bwd_off[&L - u.layers.data()];
+    conv32(D, ConvArgs32{gy, w, nullptr, gx, mask, u.N, L.cout, L.cin, X, Y, Z, 0}, u.st);
     return;
   }
   const long long nv = (long long)X * Y * Z;
@@ -745,8 +780,8 @@ ep_status ep_net_create(int ndim, int in_ch, int out_ch, int base, int levels, u
     ep_net_destroy(n);
     return nfail(nullptr, EP_ERR_OOM, "ep_net_create: allocation failed");
   }
-  const long long npk = tc_layout(u);
-  if ((npk > 0 && cudaMalloc((void **)&u.wpk, npk * sizeof(__nv_bfloat16)) != cudaSuccess) ||
+  const long long npk = tc_layout(u), np32 = layout32(u);
+  if (cudaMalloc((void **)&u.wp32, np32 * sizeof(float)) != cudaSuccess || (npk > 0 && cudaMalloc((void **)&u.wpk, npk * sizeof(__nv_bfloat16)) != cudaSuccess) ||
       cudaMalloc((void **)&u.terr, sizeof(int)) != cudaSuccess) {
     ep_net_destroy(n);
     return nfail(nullptr, EP_ERR_OOM, "ep_net_create: allocation failed");
@@ -756,7 +791,7 @@ ep_status ep_net_create(int ndim, int in_ch, int out_ch, int base, int levels, u
   cudaMemset(u.m, 0, np * 4);
   cudaMemset(u.v, 0, np * 4);
   k_to_bf16<<<nblk(np), NT, 0, u.st>>>(u.w, u.wb, np);
-  tc_pack(u);
+  pack_weights(u);
   if (cudaStreamSynchronize(u.st) != cudaSuccess) {
     ep_net_destroy(n);
     return nfail(nullptr, EP_ERR_CUDA, "ep_net_create: initialisation failed");
@@ -781,7 +816,7 @@ ep_status ep_net_set_params(ep_net *n, const float *host, long long count) {
   if (!n || !host || count != n->u.nparam) return nfail(n, EP_ERR_ARG, "ep_net_set_params: bad arguments");
   NCK(n, cudaMemcpy(n->u.w, host, count * 4, cudaMemcpyHostToDevice));
   k_to_bf16<<<nblk(count), NT, 0, n->u.st>>>(n->u.w, n->u.wb, count);
-  tc_pack(n->u);
+  pack_weights(n->u);
   NCK(n, cudaStreamSynchronize(n->u.st));
   return EP_OK;
 }
@@ -857,7 +892,7 @@ ep_status ep_net_train_step(ep_net *n, const float *x, const float *t, int N, co
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)u.step), c2 = 1.f - powf(b2, (float)u.step);
   k_adam<<<nblk(u.nparam), NT, 0, u.st>>>(u.w, u.wb, u.g, u.m, u.v, u.nparam, lr, b1, b2, ADAM_EPS, c1, c2);
-  tc_pack(u);
+  pack_weights(u);
   NCK(n, cudaGetLastError());
   NCK(n, cudaStreamSynchronize(u.st));
   return EP_OK;
@@ -884,7 +919,7 @@ ep_status ep_net_destroy(ep_net *n) {
   for (float *p : u.grad) cudaFree(p);
   cudaFree(u.partial);
   cudaFree(u.w); cudaFree(u.g); cudaFree(u.m); cudaFree(u.v); cudaFree(u.wb); cudaFree(u.dloss);
-  cudaFree(u.wpk); cudaFree(u.xcl); cudaFree(u.terr);
+  cudaFree(u.wpk); cudaFree(u.wp32); cudaFree(u.xcl); cudaFree(u.terr);
   delete n;
   return EP_OK;
 }

@@ -31,6 +31,29 @@ struct PackTable {
 };
 void conv_tc_pack_weights(const PackTable &P, const __nv_bfloat16 *w, __nv_bfloat16 *out, cudaStream_t st);
 
+// Where a tensor-core convolution's output goes (any of them may be null).
+// Blocked tensors are BF16 [n][channel / 8][z][y][x][8].
+struct TcOut {
+  int relu;
+  float *f32;                    // N x cout x V; with a head, its N x head_c x V output
+  __nv_bfloat16 *b16;            // the output in blocks b16_off .. of a tensor of b16_ch blocks
+  int b16_ch, b16_off;
+  __nv_bfloat16 *pool;           // its 2^D average
+  __nv_bfloat16 *up;             // its nearest upsample, the first blocks of a tensor of up_ch blocks
+  int up_ch;
+  const __nv_bfloat16 *head_w;   // the 1^D head on the FP32 output: head_c x cout, times scale
+  const float *head_b;
+  int head_c;
+  float scale;
+};
+bool conv_tc_supported(int k, int cout);
+__host__ __device__ constexpr int conv_tc_cinp(int cin) { return (cin + 15) / 16 * 16; }
+// FP32 N x C x V -> blocks of conv_tc_cinp(C) channels
+void conv_tc_to_blocks(const float *x, int N, int C, long long nv, __nv_bfloat16 *out, cudaStream_t st);
+cudaError_t conv_tc_forward(int D, const __nv_bfloat16 *xb, int N, int X, int Y, int Z, int cin,
+                            const __nv_bfloat16 *wpk, const float *bias, int cout, const TcOut &out, int *err,
+                            cudaStream_t st);
+
 cudaError_t conv32_configure();
 // FP32 copies of the 3^D layers' weights in the order the kernels read them, for
 // the forward pass and for the data gradient

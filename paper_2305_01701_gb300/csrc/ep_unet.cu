@@ -27,15 +27,6 @@
 
 namespace ep {
 
-// ep_conv_tc.cu
-bool conv_tc_supported(int k, int cout);
-int conv_tc_cinp(int cin);
-void conv_tc_to_channels_last(const float *x, int N, int C, long long nv, int cp, __nv_bfloat16 *out,
-                              cudaStream_t st);
-cudaError_t conv_tc_forward(int D, const __nv_bfloat16 *xcl, int N, int X, int Y, int Z, int cin,
-                            const __nv_bfloat16 *wpk, const float *bias, int cout, int relu, float *y, int *err,
-                            cudaStream_t st);
-
 namespace {
 
 constexpr int NT = 256;
@@ -239,6 +230,7 @@ struct UNet {
   int D, cin, cout, base, levels;
   std::vector<Layer> layers;  // enc (2 per level), dec (2 per level except last), head
   long long nparam = 0;
+  char *mem = nullptr;   // holds w, g, m, v, wb, dloss, wpk, wp32 and terr
   float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
   __nv_bfloat16 *wb = nullptr;
   long long step = 0;
@@ -251,8 +243,9 @@ struct UNet {
   double *dloss = nullptr;
   cudaStream_t st = nullptr;
   // tensor-core inference: weights packed per layer in the MMA operand
-  // layout (offset -1: the layer runs on CUDA cores), the channels-last BF16
-  // copy of a layer's input, and the kernels' error word
+  // layout (offset -1: the layer runs on CUDA cores), the blocked BF16 copy of
+  // a layer's input (networks with CUDA-core layers) or every blocked tensor of
+  // the pass (the others), and the kernels' error word
   __nv_bfloat16 *wpk = nullptr;
   std::vector<long long> pk_off;
   __nv_bfloat16 *xcl = nullptr;
@@ -261,6 +254,8 @@ struct UNet {
   // their offsets per layer (the 1^D head has none)
   float *wp32 = nullptr;
   std::vector<long long> fwd_off, bwd_off;
+  __nv_bfloat16 *tbuf = nullptr;
+  long long tbuf_n = 0;
   int *terr = nullptr;
   // the network's output is out_scale times the head's: training on targets
   // of any magnitude keeps the head's values of order one
@@ -363,7 +358,7 @@ static void pack_weights(UNet &u) {
   if (P.n) conv_tc_pack_weights(P, u.wb, u.wpk, u.st);
 }
 
-// BF16 elements of the largest channels-last layer input at shape (N, X, Y, Z)
+// BF16 elements of the largest blocked layer input at shape (N, X, Y, Z)
 static long long tc_xcl_elems(const UNet &u, int N, int X, int Y, int Z) {
   long long best = 0;
   int li = 0;
@@ -458,15 +453,110 @@ static Idx indices(const UNet &u) {
   return I;
 }
 
-// one convolution on the tensor cores: the input to channels-last BF16, then
-// the implicit GEMM (the caller has checked that the layer is supported)
+// one convolution on the tensor cores between FP32 tensors: the input to blocks,
+// then the implicit GEMM (the caller has checked that the layer is supported)
 template <int D>
-static void conv_tc(const UNet &u, int li, int N, int X, int Y, int Z, const float *x, float *y, int relu,
-                    __nv_bfloat16 *xcl) {
+static cudaError_t conv_tc(const UNet &u, int li, int N, int X, int Y, int Z, const float *x, float *y, int relu,
+                           __nv_bfloat16 *xcl) {
   const Layer &L = u.layers[li];
-  const long long nv = (long long)X * Y * Z;
-  conv_tc_to_channels_last(x, N, L.cin, nv, conv_tc_cinp(L.cin), xcl, u.st);
-  conv_tc_forward(D, xcl, N, X, Y, Z, L.cin, u.wpk + u.pk_off[li], u.w + L.boff, L.cout, relu, y, u.terr, u.st);
+  conv_tc_to_blocks(x, N, L.cin, (long long)X * Y * Z, xcl, u.st);
+  TcOut o{};
+  o.relu = relu;
+  o.f32 = y;
+  return conv_tc_forward(D, xcl, N, X, Y, Z, L.cin, u.wpk + u.pk_off[li], u.w + L.boff, L.cout, o, u.terr, u.st);
+}
+
+// every 3^D layer runs on the tensor cores
+static bool all_tc(const UNet &u) {
+  for (size_t q = 0; q < u.layers.size(); ++q)
+    if (u.layers[q].k == 3 && u.pk_off[q] < 0) return false;
+  return true;
+}
+
+// blocked tensors of the pass at shape (N, X, Y, Z): offsets (input; per level
+// e0, pool, cat, d0) and total, in BF16 elements
+struct TcBufs {
+  long long in, e0[8], pool[8], cat[8], d0[8], total;
+};
+static TcBufs tc_bufs(const UNet &u, int N, int X, int Y, int Z) {
+  TcBufs B{};
+  auto take = [&](int c, int l) {
+    const long long o = B.total, v = (long long)(X >> l) * (Y >> l) * (u.D == 3 ? Z >> l : 1);
+    B.total += (N * v * c + 127) / 128 * 128;
+    return o;
+  };
+  B.in = take(conv_tc_cinp(u.cin), 0);
+  for (int l = 0; l < u.levels; ++l) {
+    const int c = u.base << l;
+    B.e0[l] = take(c, l);
+    if (l + 1 == u.levels) break;
+    B.pool[l] = take(c, l + 1);
+    B.cat[l] = take(3 * c, l);
+    B.d0[l] = take(c, l);
+  }
+  return B;
+}
+
+// The forward pass on the tensor cores, blocked tensors between the layers: each
+// convolution writes what the next one reads -- its output, pooled copy, or
+// upsampled copy in the concatenation -- and the last one applies the head.
+template <int D>
+static cudaError_t forward_tc(const UNet &u, int N, int X, int Y, int Z, const float *x, __nv_bfloat16 *buf, float *y) {
+  const TcBufs B = tc_bufs(u, N, X, Y, Z);
+  const Layer &H = u.layers.back();
+  const int L = u.levels;
+  cudaError_t e = cudaSuccess;
+  auto conv = [&](int li, int l, long long src, const TcOut &o) {
+    const Layer &C = u.layers[li];
+    if (e == cudaSuccess)
+      e = conv_tc_forward(D, buf + src, N, X >> l, Y >> l, D == 3 ? Z >> l : 1, C.cin, u.wpk + u.pk_off[li], u.w + C.boff,
+                          C.cout, o, u.terr, u.st);
+  };
+  auto plain = [&](long long dst, int c) {
+    TcOut o{};
+    o.relu = 1;
+    o.b16 = buf + dst;
+    o.b16_ch = c / 8;
+    return o;
+  };
+  // the last convolution of level l on the way up (or of the coarsest level):
+  // upsampled into level l - 1's concatenation, or the head
+  auto last = [&](int l) {
+    TcOut o{};
+    o.relu = 1;
+    if (l > 0) {
+      o.up = buf + B.cat[l - 1];
+      o.up_ch = 3 * (u.base << (l - 1)) / 8;
+    } else {
+      o.f32 = y;
+      o.head_w = u.wb + H.woff;
+      o.head_b = u.w + H.boff;
+      o.head_c = H.cout;
+      o.scale = u.out_scale;
+    }
+    return o;
+  };
+  conv_tc_to_blocks(x, N, u.cin, (long long)X * Y * Z, buf + B.in, u.st);
+  long long src = B.in;
+  int li = 0;
+  for (int l = 0; l < L; ++l) {
+    const int c = u.base << l;
+    conv(li++, l, src, plain(B.e0[l], c));
+    if (l + 1 == L) {
+      conv(li++, l, B.e0[l], last(l));
+      break;
+    }
+    TcOut o = plain(B.cat[l], 3 * c);   // the skip behind the 2 c upsampled channels
+    o.b16_off = 2 * c / 8;
+    o.pool = buf + B.pool[l];
+    conv(li++, l, B.e0[l], o);
+    src = B.pool[l];
+  }
+  for (int l = L - 2; l >= 0; --l) {
+    conv(li++, l, B.cat[l], plain(B.d0[l], u.base << l));
+    conv(li++, l, B.d0[l], last(l));
+  }
+  return e;
 }
 
 // one convolution on the CUDA cores (3^D, or the 1^D head)
@@ -482,11 +572,12 @@ static void conv_cuda(const UNet &u, const Layer &L, const float *x, float *y, i
 }
 
 template <int D>
-static void conv_fwd(UNet &u, const Layer &L, const float *x, float *y, int lvl, int relu, bool tc = false) {
+static cudaError_t conv_fwd(UNet &u, const Layer &L, const float *x, float *y, int lvl, int relu, bool tc = false) {
   const int li = (int)(&L - u.layers.data());
   const int X = u.X >> lvl, Y = u.Y >> lvl, Z = D == 3 ? (u.Z >> lvl) : 1;
-  if (tc && u.pk_off[li] >= 0) conv_tc<D>(u, li, u.N, X, Y, Z, x, y, relu, u.xcl);
-  else conv_cuda(u, L, x, y, u.N, X, Y, Z, relu);
+  if (tc && u.pk_off[li] >= 0) return conv_tc<D>(u, li, u.N, X, Y, Z, x, y, relu, u.xcl);
+  conv_cuda(u, L, x, y, u.N, X, Y, Z, relu);
+  return cudaSuccess;
 }
 
 // data gradient gx (cin channels; 0 where mask, x's activation, is <= 0) from
@@ -507,13 +598,15 @@ static void conv_bwd(UNet &u, const Layer &L, const float *x, const float *gy, f
 }
 
 template <int D>
-static void forward(UNet &u, const float *x, bool tc = false) {
+static cudaError_t forward(UNet &u, const float *x, bool tc = false) {
   const Idx I = indices(u);
   int li = 0;
+  cudaError_t e = cudaSuccess;
+  auto keep = [&](cudaError_t r) { e = e == cudaSuccess ? r : e; };
   const float *in = x;
   for (int l = 0; l < u.levels; ++l) {
-    conv_fwd<D>(u, u.layers[li++], in, u.act[I.e0[l]], l, 1, tc);
-    conv_fwd<D>(u, u.layers[li++], u.act[I.e0[l]], u.act[I.e1[l]], l, 1, tc);
+    keep(conv_fwd<D>(u, u.layers[li++], in, u.act[I.e0[l]], l, 1, tc));
+    keep(conv_fwd<D>(u, u.layers[li++], u.act[I.e0[l]], u.act[I.e1[l]], l, 1, tc));
     if (l < u.levels - 1) {
       const int X = u.X >> l, Y = u.Y >> l, Z = D == 3 ? (u.Z >> l) : 1;
       long long n = (long long)u.N * u.act_c[I.pool[l]] * vox(u, l + 1);
@@ -528,15 +621,16 @@ static void forward(UNet &u, const float *x, bool tc = false) {
     const long long nv = vox(u, l);
     k_up_cat<D><<<nblk((long long)u.N * (cup + c) * nv), NT, 0, u.st>>>(prev, u.act[I.e1[l]], u.act[I.cat[l]], u.N, cup,
                                                                         c, X, Y, Z);
-    conv_fwd<D>(u, u.layers[li++], u.act[I.cat[l]], u.act[I.d0[l]], l, 1, tc);
-    conv_fwd<D>(u, u.layers[li++], u.act[I.d0[l]], u.act[I.d1[l]], l, 1, tc);
+    keep(conv_fwd<D>(u, u.layers[li++], u.act[I.cat[l]], u.act[I.d0[l]], l, 1, tc));
+    keep(conv_fwd<D>(u, u.layers[li++], u.act[I.d0[l]], u.act[I.d1[l]], l, 1, tc));
     prev = u.act[I.d1[l]];
   }
-  conv_fwd<D>(u, u.layers[li++], prev, u.act[I.out], 0, 0);
+  keep(conv_fwd<D>(u, u.layers[li++], prev, u.act[I.out], 0, 0));
   if (u.out_scale != 1.f) {
     const long long no = (long long)u.N * u.cout * vox(u, 0);
     k_scale<<<nblk(no), NT, 0, u.st>>>(u.act[I.out], no, u.out_scale);
   }
+  return e;
 }
 
 // gradients of all parameters given d loss / d out in u.grad[out].  The
@@ -687,7 +781,7 @@ static long long static_layout(const UNet &u, const Shp &s, long long *off) {
     add(c, l);
     add(c, l);
   }
-  // the channels-last BF16 input of the tensor-core convolutions (two per
+  // the blocked BF16 input of the tensor-core convolutions (two per
   // float), at the index of the head output (which is written to y)
   if (off) off[q] = total;
   total += (tc_xcl_elems(u, s.N, s.X, s.Y, s.Z) / 2 + 64) / 64 * 64;
@@ -695,25 +789,28 @@ static long long static_layout(const UNet &u, const Shp &s, long long *off) {
 }
 
 template <int D>
-static void conv_fwd_s(const UNet &u, const Shp &s, const Layer &L, const float *x, float *y, int lvl, int relu,
+static cudaError_t conv_fwd_s(const UNet &u, const Shp &s, const Layer &L, const float *x, float *y, int lvl, int relu,
                        __nv_bfloat16 *xcl) {
   const int li = (int)(&L - u.layers.data());
   const int X = s.X >> lvl, Y = s.Y >> lvl, Z = D == 3 ? (s.Z >> lvl) : 1;
-  if (u.pk_off[li] >= 0) conv_tc<D>(u, li, s.N, X, Y, Z, x, y, relu, xcl);
-  else conv_cuda(u, L, x, y, s.N, X, Y, Z, relu);
+  if (u.pk_off[li] >= 0) return conv_tc<D>(u, li, s.N, X, Y, Z, x, y, relu, xcl);
+  conv_cuda(u, L, x, y, s.N, X, Y, Z, relu);
+  return cudaSuccess;
 }
 
 // the network's forward pass with activations at act + off[q] and the head
 // writing straight into y; same kernels and launch shapes as forward()
 template <int D>
-static void forward_static(const UNet &u, const Shp &s, const float *x, float *act, const long long *off, float *y) {
+static cudaError_t forward_static(const UNet &u, const Shp &s, const float *x, float *act, const long long *off, float *y) {
   const Idx I = indices(u);
   __nv_bfloat16 *xcl = reinterpret_cast<__nv_bfloat16 *>(act + off[I.out]);
   int li = 0;
+  cudaError_t e = cudaSuccess;
+  auto keep = [&](cudaError_t r) { e = e == cudaSuccess ? r : e; };
   const float *in = x;
   for (int l = 0; l < u.levels; ++l) {
-    conv_fwd_s<D>(u, s, u.layers[li++], in, act + off[I.e0[l]], l, 1, xcl);
-    conv_fwd_s<D>(u, s, u.layers[li++], act + off[I.e0[l]], act + off[I.e1[l]], l, 1, xcl);
+    keep(conv_fwd_s<D>(u, s, u.layers[li++], in, act + off[I.e0[l]], l, 1, xcl));
+    keep(conv_fwd_s<D>(u, s, u.layers[li++], act + off[I.e0[l]], act + off[I.e1[l]], l, 1, xcl));
     if (l < u.levels - 1) {
       const int X = s.X >> l, Y = s.Y >> l, Z = D == 3 ? (s.Z >> l) : 1;
       const long long n = (long long)s.N * (u.base << l) * svox(u, s, l + 1);
@@ -730,15 +827,16 @@ static void forward_static(const UNet &u, const Shp &s, const float *x, float *a
     float *cat = act + off[I.cat[l]];
     k_up_cat<D><<<nblk((long long)s.N * (cup + c) * nv), NT, 0, u.st>>>(prev, act + off[I.e1[l]], cat, s.N, cup, c, X, Y,
                                                                         Z);
-    conv_fwd_s<D>(u, s, u.layers[li++], cat, act + off[I.d0[l]], l, 1, xcl);
-    conv_fwd_s<D>(u, s, u.layers[li++], act + off[I.d0[l]], act + off[I.d1[l]], l, 1, xcl);
+    keep(conv_fwd_s<D>(u, s, u.layers[li++], cat, act + off[I.d0[l]], l, 1, xcl));
+    keep(conv_fwd_s<D>(u, s, u.layers[li++], act + off[I.d0[l]], act + off[I.d1[l]], l, 1, xcl));
     prev = act + off[I.d1[l]];
   }
-  conv_fwd_s<D>(u, s, u.layers[li++], prev, y, 0, 0, xcl);
+  keep(conv_fwd_s<D>(u, s, u.layers[li++], prev, y, 0, 0, xcl));
   if (u.out_scale != 1.f) {
     const long long no = (long long)s.N * u.cout * svox(u, s, 0);
     k_scale<<<nblk(no), NT, 0, u.st>>>(y, no, u.out_scale);
   }
+  return e;
 }
 
 extern "C" {
@@ -752,7 +850,8 @@ ep_status ep_net_create(int ndim, int in_ch, int out_ch, int base, int levels, u
   u.D = ndim; u.cin = in_ch; u.cout = out_ch; u.base = base; u.levels = levels;
   u.st = (cudaStream_t)stream;
   unet_layers(u);
-  if (conv32_configure() != cudaSuccess) {
+  static const cudaError_t cfg = conv32_configure();
+  if (cfg != cudaSuccess) {
     delete n;
     return nfail(nullptr, EP_ERR_CUDA, "ep_net_create: convolution kernels' shared-memory attribute");
   }
@@ -774,18 +873,23 @@ ep_status ep_net_create(int ndim, int in_ch, int out_ch, int base, int levels, u
     for (long long q = 0; q < (long long)L.cin * L.cout * taps; ++q) w[L.woff + q] = (float)((2.0 * rnd() - 1.0) * bound);
   }
   const long long np = u.nparam;
-  if (cudaMalloc((void **)&u.w, np * 4) != cudaSuccess || cudaMalloc((void **)&u.g, np * 4) != cudaSuccess ||
-      cudaMalloc((void **)&u.m, np * 4) != cudaSuccess || cudaMalloc((void **)&u.v, np * 4) != cudaSuccess ||
-      cudaMalloc((void **)&u.wb, np * 2) != cudaSuccess || cudaMalloc((void **)&u.dloss, 8 * (1 + MSE_BLOCKS)) != cudaSuccess) {
-    ep_net_destroy(n);
-    return nfail(nullptr, EP_ERR_OOM, "ep_net_create: allocation failed");
-  }
+  // one allocation for everything that follows the parameters
   const long long npk = tc_layout(u), np32 = layout32(u);
-  if (cudaMalloc((void **)&u.wp32, np32 * sizeof(float)) != cudaSuccess || (npk > 0 && cudaMalloc((void **)&u.wpk, npk * sizeof(__nv_bfloat16)) != cudaSuccess) ||
-      cudaMalloc((void **)&u.terr, sizeof(int)) != cudaSuccess) {
+  size_t total = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = total;
+    total += (bytes + 255) & ~(size_t)255;
+    return o;
+  };
+  const size_t ow = take(np * 4), og = take(np * 4), om = take(np * 4), ov = take(np * 4), owb = take(np * 2),
+               ol = take(8 * (1 + MSE_BLOCKS)), opk = take(npk * 2), o32 = take(np32 * 4), oe = take(sizeof(int));
+  if (cudaMalloc((void **)&u.mem, total) != cudaSuccess) {
     ep_net_destroy(n);
     return nfail(nullptr, EP_ERR_OOM, "ep_net_create: allocation failed");
   }
+  u.w = (float *)(u.mem + ow); u.g = (float *)(u.mem + og); u.m = (float *)(u.mem + om); u.v = (float *)(u.mem + ov);
+  u.wb = (__nv_bfloat16 *)(u.mem + owb); u.dloss = (double *)(u.mem + ol);
+  u.wpk = (__nv_bfloat16 *)(u.mem + opk); u.wp32 = (float *)(u.mem + o32); u.terr = (int *)(u.mem + oe);
   cudaMemset(u.terr, 0, sizeof(int));
   cudaMemcpy(u.w, w.data(), np * 4, cudaMemcpyHostToDevice);
   cudaMemset(u.m, 0, np * 4);
@@ -825,8 +929,22 @@ ep_status ep_net_forward(ep_net *n, const float *x, int N, const int size[3], fl
   if (!n || !x || !y || N < 1 || !size || !shape_ok(n, size))
     return nfail(n, EP_ERR_ARG, "ep_net_forward: sizes must be multiples of 2^(levels-1)");
   UNet &u = n->u;
-  NCK(n, ensure_shape(u, N, size[0], size[1], u.D == 3 ? size[2] : 1));
-  if (u.D == 2) forward<2>(u, x, true); else forward<3>(u, x, true);
+  const int Z = u.D == 3 ? size[2] : 1;
+  if (all_tc(u)) {
+    const long long need = tc_bufs(u, N, size[0], size[1], Z).total;
+    if (need > u.tbuf_n) {
+      cudaFree(u.tbuf);
+      u.tbuf = nullptr;
+      u.tbuf_n = 0;
+      NCK(n, cudaMalloc((void **)&u.tbuf, need * sizeof(__nv_bfloat16)));
+      u.tbuf_n = need;
+    }
+    NCK(n, u.D == 2 ? forward_tc<2>(u, N, size[0], size[1], Z, x, u.tbuf, y)
+                    : forward_tc<3>(u, N, size[0], size[1], Z, x, u.tbuf, y));
+    return tc_status(n);
+  }
+  NCK(n, ensure_shape(u, N, size[0], size[1], Z));
+  NCK(n, u.D == 2 ? forward<2>(u, x, true) : forward<3>(u, x, true));
   const long long no = (long long)N * u.cout * vox(u, 0);
   NCK(n, cudaMemcpyAsync(y, u.act[indices(u).out], no * 4, cudaMemcpyDeviceToDevice, u.st));
   NCK(n, cudaGetLastError());
@@ -849,8 +967,13 @@ ep_status ep_net_forward_static(ep_net *n, const float *x, int N, const int size
   float *act = nullptr;
   const ep_status r = static_act(n, &act);
   if (r != EP_OK) return r;
-  if (u.D == 2) forward_static<2>(u, s, x, act, off, y);
-  else forward_static<3>(u, s, x, act, off, y);
+  // the blocked tensors are BF16 and fewer: they take less than half of need
+  if (all_tc(u)) {
+    __nv_bfloat16 *buf = reinterpret_cast<__nv_bfloat16 *>(act);
+    NCK(n, u.D == 2 ? forward_tc<2>(u, N, s.X, s.Y, s.Z, x, buf, y) : forward_tc<3>(u, N, s.X, s.Y, s.Z, x, buf, y));
+  } else {
+    NCK(n, u.D == 2 ? forward_static<2>(u, s, x, act, off, y) : forward_static<3>(u, s, x, act, off, y));
+  }
   NCK(n, cudaGetLastError());
   return tc_status(n);
 }
@@ -858,7 +981,7 @@ ep_status ep_net_forward_static(ep_net *n, const float *x, int N, const int size
 static ep_status net_grads(ep_net *n, const float *x, const float *t, int N, const int size[3], double *loss) {
   UNet &u = n->u;
   NCK(n, ensure_shape(u, N, size[0], size[1], u.D == 3 ? size[2] : 1));
-  if (u.D == 2) forward<2>(u, x); else forward<3>(u, x);
+  NCK(n, u.D == 2 ? forward<2>(u, x) : forward<3>(u, x));
   const Idx I = indices(u);
   const long long no = (long long)N * u.cout * vox(u, 0);
   const float inv_s = u.out_scale > 0.f ? 1.f / u.out_scale : 1.f;
@@ -918,8 +1041,7 @@ ep_status ep_net_destroy(ep_net *n) {
   for (float *p : u.act) cudaFree(p);
   for (float *p : u.grad) cudaFree(p);
   cudaFree(u.partial);
-  cudaFree(u.w); cudaFree(u.g); cudaFree(u.m); cudaFree(u.v); cudaFree(u.wb); cudaFree(u.dloss);
-  cudaFree(u.wpk); cudaFree(u.wp32); cudaFree(u.xcl); cudaFree(u.terr);
+  cudaFree(u.mem); cudaFree(u.xcl); cudaFree(u.tbuf);
   delete n;
   return EP_OK;
 }

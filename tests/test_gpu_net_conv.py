@@ -1,5 +1,6 @@
-"""The FP32 training convolutions (forward, data gradient, weight gradient) at sizes and channel
-counts around their tiles, against the same network in FP64 torch with the same BF16 weights."""
+"""The network's convolutions at sizes and channel counts around their tiles, against the same
+network in FP64 torch with the same BF16 weights: training in FP32 (forward, data gradient,
+weight gradient) and inference on the tensor cores."""
 import numpy as np
 import pytest
 
@@ -82,3 +83,70 @@ def test_training_convolutions_match_fp64(P, nd, size, cin, cout, base, levels, 
     err = np.linalg.norm(g - ref.cpu().numpy()) / np.linalg.norm(ref.cpu().numpy())
     assert err <= bound, (err, bound)
     net.close()
+
+
+@pytest.mark.parametrize("nd,size,cin,cout,base,levels,N", [
+    (2, (8, 16), 9, 5, 16, 1, 1),         # one brick
+    (2, (10, 18), 9, 5, 48, 1, 3),        # beyond it; 16-channel stages
+    (2, (12, 36), 40, 17, 32, 3, 2),      # more than 12 head outputs
+    (3, (8, 16, 4), 13, 9, 16, 1, 1),
+    (3, (72, 68, 20), 13, 9, 16, 2, 1),   # four slabs per block
+    (3, (9, 17, 3), 33, 2, 128, 1, 1),    # two slabs, the last one outside; all accumulator columns
+    (3, (4, 12, 20), 13, 9, 32, 3, 2),
+])
+def test_tensor_core_convolutions_at_brick_edges(P, nd, size, cin, cout, base, levels, N):
+    """The inference pass (blocked BF16 tensors between the layers, pooling, upsampling and head in
+    the convolutions) against FP64 torch with the convolutions' inputs rounded to BF16: what is
+    left is FP32 accumulation moving a value across a BF16 rounding boundary (2^-8 relative in a
+    few values, carried on through the layers)."""
+    import torch
+    F = torch.nn.functional
+    gen = torch.Generator().manual_seed(4)
+    net = P.Net(nd, cin, cout, base=base, levels=levels)
+    net.set_output_scale(0.5)
+    params = torch.randn(net.n_params(), generator=gen)
+    at, spans = 0, []
+    for ci, co, k in _layers(nd, cin, cout, base, levels):
+        params[at:at + ci * co * k ** nd] *= (2.0 / (ci * k ** nd)) ** 0.5
+        params[at + ci * co * k ** nd:at + ci * co * k ** nd + co] *= 0.05
+        spans.append((at, ci, co, k))
+        at += ci * co * k ** nd + co
+    net.set_params(params.numpy())
+    dims = tuple(reversed(size))
+    x = torch.randn((N, cin) + dims, generator=gen).cuda()
+    y = torch.full((N, cout) + dims, float("nan"), device="cuda")
+    net.forward(x.data_ptr(), N, list(size), y.data_ptr())
+    conv, pool = (F.conv3d, F.avg_pool3d) if nd == 3 else (F.conv2d, F.avg_pool2d)
+    p = params.cuda()
+    it = iter(spans)
+
+    def layer(a):
+        o, ci, co, k = next(it)
+        m = ci * co * k ** nd
+        w = p[o:o + m].bfloat16().double().view([co, ci] + [k] * nd)
+        a = a.float().bfloat16().double() if k == 3 else a
+        return conv(a, w, p[o + m:o + m + co].double(), padding=k // 2)
+
+    skips, a = [], x.double()
+    for lv in range(levels):
+        a = torch.relu(layer(torch.relu(layer(a))))
+        if lv < levels - 1:
+            skips.append(a)
+            a = pool(a, 2)
+    for lv in range(levels - 2, -1, -1):
+        a = torch.cat([F.interpolate(a, scale_factor=2, mode="nearest"), skips[lv]], 1)
+        a = torch.relu(layer(torch.relu(layer(a))))
+    ref = 0.5 * layer(a)
+    err = (y.double() - ref).abs().max() / ref.abs().max()
+    assert torch.isfinite(y).all() and err <= 6e-3, float(err)
+    net.close()
+
+
+def _layers(nd, cin, cout, base, levels):
+    out, c = [], cin
+    for lv in range(levels):
+        out += [(c, base << lv, 3), (base << lv, base << lv, 3)]
+        c = base << lv
+    for lv in range(levels - 2, -1, -1):
+        out += [(3 * (base << lv), base << lv, 3), (base << lv, base << lv, 3)]
+    return out + [(base, cout, 1)]

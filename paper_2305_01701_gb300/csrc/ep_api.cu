@@ -170,10 +170,19 @@ void carve(ep_grid *h, Arena &a) {
   }
   for (int d = 0; d < nd; ++d) { tk(h->tbn[d]); tk(h->Tn[d]); tk(h->uchk[d]); tk(h->f[d]); tk(h->cn[d]); }
   for (int c = 0; c < ns; ++c) {
-    tk(h->tbs[c]); tk(h->rq[c]); tk(h->om[c]); tk(h->es[c]); tk(h->Ts[c]); tk(h->cs[c]);
+    tk(h->tbs[c]); tk(h->om[c]); tk(h->es[c]); tk(h->Ts[c]); tk(h->cs[c]);
   }
-  tk(h->pb); tk(h->yc); tk(h->s); tk(h->rd[0]); tk(h->cp);
-  if (nd == 3) tk(h->rd[1]);
+  tk(h->pb); tk(h->s); tk(h->cp);
+  // rotation weights and B c: in FP64 the increment's own arrays
+  if (es == 8) {
+    for (int c = 0; c < ns; ++c) h->rq[c] = h->rq64[c];
+    for (int r = 0; r < nd - 1; ++r) h->rd[r] = h->rd64[r];
+    h->yc = h->yc64;
+  } else {
+    for (int c = 0; c < ns; ++c) tk(h->rq[c]);
+    for (int r = 0; r < nd - 1; ++r) tk(h->rd[r]);
+    tk(h->yc);
+  }
   h->dscal = a.take<Scal>(1);
   h->dinfo = a.take<DevInfo>(1);
   h->inst_dev = a.take<Inst2<double>>(1);
@@ -252,6 +261,7 @@ Scal make_scal(const ep_grid *h) {
                            : eta_ve(h);
   s.gcell = h->Gc != nullptr;
   s.two_eta = 2.0 * eta;
+  s.eta_d = -s.two_eta / 3.0;
   s.c2 = eta / (h->G * h->dt);
   s.c2dt = s.c2 * h->dt;
   s.KDt = h->K * h->dt;
@@ -326,6 +336,16 @@ Stage<T> sweep_stage(ep_grid *h, int b) {
   for (int w = 0; w < 4; ++w) {
     S.ge[w] = h->Gc ? P<T>(h->geT[w]) : nullptr;
     S.gc[w] = h->Gc ? P<T>(h->gcT[w]) : nullptr;
+  }
+  if constexpr (sizeof(T) == 8) {
+    // FP64 scratch of the start and commit passes, free while the increment is
+    // iterated; the normal stress takes the shear rates' place (read before)
+    for (int d = 0; d < 3; ++d) {
+      S.md[d] = h->es64[d]; S.ma[d] = h->stn64[d]; S.mb[d] = h->sts64[d];
+      S.pr[d] = h->om64[d];
+    }
+    S.dv = h->stp64;
+    S.sx[0] = P<T>(h->es[0]); S.sx[1] = h->ndim == 3 ? P<T>(h->es[1]) : h->s64; S.sx[2] = P<T>(h->es[2]);
   }
   return S;
 }
@@ -489,7 +509,7 @@ ep_status prologue(ep_grid *h, const double *const dv[3]) {
     if (copy_into<T>(h, h->sts[0][c], h->sts64[c]) != EP_OK) return EP_ERR_CUDA;
     if (copy_into<T>(h, h->sts[1][c], h->sts64[c]) != EP_OK) return EP_ERR_CUDA;
     if (copy_into<T>(h, h->cs[c], h->sts64[c]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->rq[c], h->rq64[c]) != EP_OK) return EP_ERR_CUDA;
+    if (sizeof(T) == 4 && copy_into<T>(h, h->rq[c], h->rq64[c]) != EP_OK) return EP_ERR_CUDA;
   }
   if (h->opts.incompressible) {
     // base pressure step of the incompressible sweep: -K~ div v0 (es64 is
@@ -503,10 +523,17 @@ ep_status prologue(ep_grid *h, const double *const dv[3]) {
   if (copy_into<T>(h, h->stp[0], h->stp64) != EP_OK) return EP_ERR_CUDA;
   if (copy_into<T>(h, h->stp[1], h->stp64) != EP_OK) return EP_ERR_CUDA;
   if (copy_into<T>(h, h->cp, h->stp64) != EP_OK) return EP_ERR_CUDA;
-  if (copy_into<T>(h, h->yc, h->yc64) != EP_OK) return EP_ERR_CUDA;
-  for (int r = 0; r < (nd == 3 ? 2 : 1); ++r)
-    if (copy_into<T>(h, h->rd[r], h->rd64[r]) != EP_OK) return EP_ERR_CUDA;
+  if (sizeof(T) == 4) {
+    if (copy_into<T>(h, h->yc, h->yc64) != EP_OK) return EP_ERR_CUDA;
+    for (int r = 0; r < nd - 1; ++r)
+      if (copy_into<T>(h, h->rd[r], h->rd64[r]) != EP_OK) return EP_ERR_CUDA;
+  }
   if (copy_into<T>(h, h->s, h->s64) != EP_OK) return EP_ERR_CUDA;
+  if (sizeof(T) == 8 && !h->Gc) {
+    // the state has been copied: its scratch takes the rotation's coefficients
+    double *md[3] = {h->es64[0], h->es64[1], h->es64[2]};
+    launch_rotation_means(g, S, md, h->stn64, h->sts64, st);
+  }
   CK(h, cudaGetLastError());
   return EP_OK;
 }
@@ -546,11 +573,30 @@ bool launch_fused_any(const ep_grid *h, const Stage<T> &S, DevInfo *di, cudaStre
   return true;
 }
 
+// one staged iteration; returns its number of kernels.  ev (nullable): events
+// recorded behind each of them (ev[1], ev[2], ...)
+template <typename T>
+int launch_staged(const ep_grid *h, const Stage<T> &S, DevInfo *di, bool check, cudaStream_t st,
+                   const cudaEvent_t *ev = nullptr) {
+  const Geo &g = h->g;
+  if constexpr (sizeof(T) == 8) {
+    if (!h->Gc) return launch_sweep64(g, S, h->dscal, di, check, st, ev);
+  }
+  auto mark = [&](int q) {
+    if (ev) cudaEventRecord(ev[q], st);
+  };
+  launch_strain<T>(g, S, h->dscal, di, st); mark(1);
+  launch_trial<T>(g, S, h->dscal, di, st); mark(2);
+  launch_return_centres<T>(g, S, h->dscal, di, check, st); mark(3);
+  launch_return_edges<T>(g, S, h->dscal, di, check, st); mark(4);
+  launch_velocity<T>(g, S, h->dscal, di, check, st); mark(5);
+  return 5;
+}
+
 // One chunk of n_chk iterations (first one a check iteration), captured once.
 template <typename T>
 ep_status capture_chunk(ep_grid *h) {
   if (h->chunk) return EP_OK;
-  const Geo &g = h->g;
   cudaGraph_t graph;
   const bool f2 = use_fused2d<T>(h);
   int blocks = 0;
@@ -579,11 +625,7 @@ ep_status capture_chunk(ep_grid *h) {
       if (chk) launch_check(h->dinfo, h->dscal, h->cap);
       continue;
     }
-    launch_strain<T>(g, S, h->dscal, h->dinfo, h->cap);
-    launch_trial<T>(g, S, h->dscal, h->dinfo, h->cap);
-    launch_return_centres<T>(g, S, h->dscal, h->dinfo, chk, h->cap);
-    launch_return_edges<T>(g, S, h->dscal, h->dinfo, chk, h->cap);
-    launch_velocity<T>(g, S, h->dscal, h->dinfo, chk, h->cap);
+    launch_staged<T>(h, S, h->dinfo, chk, h->cap);
     if (chk) launch_check(h->dinfo, h->dscal, h->cap);
   }
   cudaError_t e = cudaStreamEndCapture(h->cap, &graph);
@@ -1227,7 +1269,7 @@ ep_status ep_restore(ep_handle h) {
 ep_status ep_time_sweep(ep_handle h, int iters, double *ms_out, int n_out, int *n_kernels) {
   if (!h || iters < 1 || !ms_out || n_out < 1) return fail(h, EP_ERR_ARG, "ep_time_sweep: bad arguments");
   if (!h->have_material || h->dt <= 0.0) return fail(h, EP_ERR_STATE, "ep_time_sweep: apply an increment first");
-  const int nk = 5;
+  int nk = 5;
   std::vector<cudaEvent_t> ev(nk + 1);
   for (auto &e : ev) CK(h, cudaEventCreate(&e));
   std::vector<double> acc(nk + 1, 0.0);
@@ -1289,21 +1331,8 @@ ep_status ep_time_sweep(ep_handle h, int iters, double *ms_out, int n_out, int *
   for (int it = 0; it < iters; ++it) {
     const int b = it & 1;
     CK(h, cudaEventRecord(ev[0], h->stream));
-    if (h->prec == EP_FP64) {
-      Stage<double> S = sweep_stage<double>(h, b);
-      launch_strain<double>(h->g, S, h->dscal, nullptr, h->stream); CK(h, cudaEventRecord(ev[1], h->stream));
-      launch_trial<double>(h->g, S, h->dscal, nullptr, h->stream); CK(h, cudaEventRecord(ev[2], h->stream));
-      launch_return_centres<double>(h->g, S, h->dscal, nullptr, 0, h->stream); CK(h, cudaEventRecord(ev[3], h->stream));
-      launch_return_edges<double>(h->g, S, h->dscal, nullptr, 0, h->stream); CK(h, cudaEventRecord(ev[4], h->stream));
-      launch_velocity<double>(h->g, S, h->dscal, nullptr, 0, h->stream); CK(h, cudaEventRecord(ev[5], h->stream));
-    } else {
-      Stage<float> S = sweep_stage<float>(h, b);
-      launch_strain<float>(h->g, S, h->dscal, nullptr, h->stream); CK(h, cudaEventRecord(ev[1], h->stream));
-      launch_trial<float>(h->g, S, h->dscal, nullptr, h->stream); CK(h, cudaEventRecord(ev[2], h->stream));
-      launch_return_centres<float>(h->g, S, h->dscal, nullptr, 0, h->stream); CK(h, cudaEventRecord(ev[3], h->stream));
-      launch_return_edges<float>(h->g, S, h->dscal, nullptr, 0, h->stream); CK(h, cudaEventRecord(ev[4], h->stream));
-      launch_velocity<float>(h->g, S, h->dscal, nullptr, 0, h->stream); CK(h, cudaEventRecord(ev[5], h->stream));
-    }
+    nk = h->prec == EP_FP64 ? launch_staged<double>(h, sweep_stage<double>(h, b), nullptr, false, h->stream, ev.data())
+                            : launch_staged<float>(h, sweep_stage<float>(h, b), nullptr, false, h->stream, ev.data());
     CK(h, cudaGetLastError());
     CK(h, cudaEventSynchronize(ev[nk]));
     for (int q = 0; q < nk; ++q) {

@@ -29,6 +29,7 @@ struct Geo {
 // captured CUDA graph stays valid across increments.
 struct Scal {
   double two_eta;      // 2 eta_ve
+  double eta_d;        // -2 eta_ve / 3: weight of the divergence in a normal deviator
   double c2;           // eta_ve / (G dt): weight of the rotated old stress
   double c2dt;         // c2 * dt: weight of the Jaumann rotation term
   double bt, bp;       // relaxation weights beta_tau, beta_p (Eqs. A23ssP, A2ssP)
@@ -94,6 +95,11 @@ struct Stage {
   // per-cell shear modulus (nullable: the uniform scalars): 2 eta_ve and
   // c2 = eta_ve / (G dt) at centres [0] and vertices/edges [1 + c]
   const T *ge[4], *gc[4];
+  // FP64 sweeps with a uniform modulus (ep_sweep64.cu): the rotation's
+  // coefficients at vertices/edges, the rotation products there, the divergence
+  // and the normal stress less the pressure at centres
+  const T *md[3], *ma[3], *mb[3];
+  T *pr[3], *dv, *sx[3];
 };
 
 // One 2D instance of the batched fused sweep (ep_fused2d.cu): geometry,
@@ -185,6 +191,13 @@ template <typename T>
 void launch_velocity(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int check,
                      cudaStream_t st);
 void launch_check(DevInfo *di, const Scal *sc, cudaStream_t st);
+
+// the FP64 sweep with a uniform modulus (ep_sweep64.cu): five kernels in 3D, two in
+// 2D (returned); ev (nullable): ev[1], ev[2], ... are recorded behind them
+int launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
+                    const cudaEvent_t *ev = nullptr);
+void launch_rotation_means(const Geo &g, const Stage<double> &S, double *const md[3], double *const ma[3],
+                           double *const mb[3], cudaStream_t st);
 
 // ---- fused sweeps (ep_fused3d.cu) ------------------------------------
 // z-planes per block when none was chosen (kz <= 0).  A block marches kz

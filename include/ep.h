@@ -207,10 +207,10 @@ ep_status ep_get_fields(ep_handle h, int field, double *host_out, size_t count);
 ep_status ep_set_fields(ep_handle h, int field, const double *host_in, size_t count);
 
 /* Sweep kernel selection.  EP_KERNEL_AUTO (default): the fastest measured
- * kernel for the grid -- for FP32 grids the fused one-kernel sweep (2D) and
- * the register z-march sweep (3D), for FP64 grids the staged five-kernel
- * sweep (FP64 is bound by FP64 arithmetic on GB300, where the staged sweep
- * does no halo recomputation).
+ * kernel for the grid -- the staged sweep for 2D grids and for FP64 ones (two
+ * kernels in 2D, five in 3D; FP64 is bound by FP64 arithmetic on GB300, where
+ * the staged sweep does no halo recomputation), the register z-march sweep for
+ * FP32 grids in 3D.
  * EP_KERNEL_STAGED / EP_KERNEL_FUSED force one;
  * EP_KERNEL_FUSED_TMA is the 3D fused sweep with every plane streamed by
  * the tensor-memory accelerator (a timed-out copy ends the solve with
@@ -236,7 +236,7 @@ ep_status ep_set_kernel(ep_handle h, int variant, int shape);
  * iterations.  The grids must be 2D, share a precision and n_chk, and stay
  * alive until ep_destroy_batch; the batch runs on the first grid's stream.
  * A grid solved in a batch performs the same arithmetic as when solved
- * alone with the fused 2D kernel. */
+ * alone with the fused 2D kernel (EP_KERNEL_FUSED with the batch's tile). */
 typedef struct ep_batch *ep_batch_handle;
 ep_status ep_create_batch(const ep_handle *grids, int count, ep_batch_handle *out);
 /* start an increment in every grid: pure shear at rate a[i] (host array of

@@ -337,15 +337,19 @@ Stage<T> sweep_stage(ep_grid *h, int b) {
     S.ge[w] = h->Gc ? P<T>(h->geT[w]) : nullptr;
     S.gc[w] = h->Gc ? P<T>(h->gcT[w]) : nullptr;
   }
-  if constexpr (sizeof(T) == 8) {
+  if (h->ndim == 2) {
+    // the two-stage sweep: arrays that only the five-stage one uses
+    S.md[0] = P<T>(h->om[0]);
+    S.sx[0] = P<T>(h->Tn[0]); S.sx[1] = P<T>(h->Tn[1]);
+  } else if constexpr (sizeof(T) == 8) {
     // FP64 scratch of the start and commit passes, free while the increment is
     // iterated; the normal stress takes the shear rates' place (read before)
     for (int d = 0; d < 3; ++d) {
       S.md[d] = h->es64[d]; S.ma[d] = h->stn64[d]; S.mb[d] = h->sts64[d];
       S.pr[d] = h->om64[d];
+      S.sx[d] = P<T>(h->es[d]);
     }
     S.dv = h->stp64;
-    S.sx[0] = P<T>(h->es[0]); S.sx[1] = h->ndim == 3 ? P<T>(h->es[1]) : h->s64; S.sx[2] = P<T>(h->es[2]);
   }
   return S;
 }
@@ -381,7 +385,7 @@ void append_items(std::vector<int4> &v, int inst, const Geo &g, int tile) {
 template <typename T>
 bool use_fused2d(const ep_grid *h) {
   if (h->ndim != 2 || h->have_f || h->Gc) return false;
-  return h->variant == EP_KERNEL_FUSED || (h->variant == EP_KERNEL_AUTO && sizeof(T) == 4);
+  return h->variant == EP_KERNEL_FUSED;
 }
 
 // upload this grid's instance record and work items for its tile
@@ -529,7 +533,9 @@ ep_status prologue(ep_grid *h, const double *const dv[3]) {
       if (copy_into<T>(h, h->rd[r], h->rd64[r]) != EP_OK) return EP_ERR_CUDA;
   }
   if (copy_into<T>(h, h->s, h->s64) != EP_OK) return EP_ERR_CUDA;
-  if (sizeof(T) == 8 && !h->Gc) {
+  if (nd == 2 && !h->Gc) {
+    launch_rotation_mean2d<T>(g, P<T>(h->rd[0]), P<T>(h->om[0]), st);
+  } else if (sizeof(T) == 8 && !h->Gc) {
     // the state has been copied: its scratch takes the rotation's coefficients
     double *md[3] = {h->es64[0], h->es64[1], h->es64[2]};
     launch_rotation_means(g, S, md, h->stn64, h->sts64, st);
@@ -579,8 +585,15 @@ template <typename T>
 int launch_staged(const ep_grid *h, const Stage<T> &S, DevInfo *di, bool check, cudaStream_t st,
                    const cudaEvent_t *ev = nullptr) {
   const Geo &g = h->g;
+  if (h->ndim == 2 && !h->Gc) {
+    launch_sweep2d<T>(g, S, h->dscal, di, check, st, ev);
+    return 2;
+  }
   if constexpr (sizeof(T) == 8) {
-    if (!h->Gc) return launch_sweep64(g, S, h->dscal, di, check, st, ev);
+    if (!h->Gc) {
+      launch_sweep64(g, S, h->dscal, di, check, st, ev);
+      return 5;
+    }
   }
   auto mark = [&](int q) {
     if (ev) cudaEventRecord(ev[q], st);

@@ -95,7 +95,7 @@ struct Stage {
   // per-cell shear modulus (nullable: the uniform scalars): 2 eta_ve and
   // c2 = eta_ve / (G dt) at centres [0] and vertices/edges [1 + c]
   const T *ge[4], *gc[4];
-  // FP64 sweeps with a uniform modulus (ep_sweep64.cu): the rotation's
+  // sweeps with a uniform modulus (ep_sweep64.cu, ep_sweep2d.cu): the rotation's
   // coefficients at vertices/edges, the rotation products there, the divergence
   // and the normal stress less the pressure at centres
   const T *md[3], *ma[3], *mb[3];
@@ -192,12 +192,18 @@ void launch_velocity(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *d
                      cudaStream_t st);
 void launch_check(DevInfo *di, const Scal *sc, cudaStream_t st);
 
-// the FP64 sweep with a uniform modulus (ep_sweep64.cu): five kernels in 3D, two in
-// 2D (returned); ev (nullable): ev[1], ev[2], ... are recorded behind them
-int launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
+// sweeps with a uniform modulus: FP64 in 3D (ep_sweep64.cu, five kernels) and one
+// 2D grid (ep_sweep2d.cu, two kernels); ev (nullable): ev[1], ev[2], ... are recorded
+// behind them
+void launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
                     const cudaEvent_t *ev = nullptr);
 void launch_rotation_means(const Geo &g, const Stage<double> &S, double *const md[3], double *const ma[3],
                            double *const mb[3], cudaStream_t st);
+template <typename T>
+void launch_sweep2d(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
+                    const cudaEvent_t *ev = nullptr);
+template <typename T>
+void launch_rotation_mean2d(const Geo &g, const T *rd, T *md, cudaStream_t st);
 
 // ---- fused sweeps (ep_fused3d.cu) ------------------------------------
 // z-planes per block when none was chosen (kz <= 0).  A block marches kz

@@ -1,9 +1,9 @@
-// ep_sweep64.cu -- the FP64 sweep of a grid with a uniform shear modulus: five
-// stage kernels in 3D, two in 2D.
+// ep_sweep64.cu -- the FP64 sweep of a 3D grid with a uniform shear modulus, as
+// five stage kernels.
 //
 // The same iteration as ep_stages.cu (strain, trial, centre return, edge return,
 // velocity; Eqs. A41, A5, A23ssP, A2ssP, A6121lambda, A22S, A22P), every quantity
-// computed once per point in 3D.  Bound: the FP64 pipe (two operations per clock and
+// computed once per point.  Bound: the FP64 pipe (two operations per clock and
 // SM, 1.2 TFLOP/s measured on this part), then launch latency on small grids.
 // What these kernels leave out of the general ones, which also serve the physical
 // response, FP32 and a per-cell modulus:
@@ -16,11 +16,8 @@
 //     the pressure once, in the centre return;
 //   * the square root and the division of the return run only where J2 is within
 //     rounding of Y^2 or above (elsewhere the scale is exactly 1).
-// Measured, an iteration: 3D 127^3 1129 -> 639 us (157 FP64 operations per cell are
-// 510 us of the pipe); 2D 511^2 76.5 -> 47.5 us, 64^2
-// 17.2 -> 8.4 us (two launches).
-// A warp covers 32 points along x; blocks hold as many rows as leave every SM some
-// (launch_rows, strip_rows).
+// Measured, an iteration at 127^3: 1129 -> 639 us (157 FP64 operations per cell are
+// 510 us of the pipe).  A warp covers 32 points along x; blocks hold as many rows as leave every SM some (launch_rows).
 #include <math.h>
 
 #include "ep_internal.cuh"
@@ -74,7 +71,6 @@ __device__ __forceinline__ Pt point(const Geo &g) {
   return p;
 }
 
-// ============================ 3D: five stages ============================
 // ---- spins, shear rates and rotation products at vertices / edges ------------
 __global__ void __launch_bounds__(256) k64_strain(Geo g, Stage<double> S, DevInfo *di) {
   if (skip(di)) return;
@@ -290,175 +286,10 @@ __global__ void __launch_bounds__(256) k64_velocity(Geo g, Stage<double> S, cons
   }
 }
 
-// ============================ 2D: two stages =============================
-// A vertex's trial needs only its own spin, so the stress kernel recomputes the
-// vertices around a centre instead of passing them through memory, and the
-// velocity kernel the deviators of the vertices beside a face: two launches per
-// iteration where five were (64^2: 12.7 us an iteration with five).  A warp
-// covers 32 columns (31 written, the last one gives its neighbour's values) and
-// marches R rows, carrying the row's vertices.
-
-// row range of this warp
-struct Strip {
-  int i, j0, j1, lane;
-};
-__device__ __forceinline__ Strip strip(const Geo &g, int rows) {
-  Strip p;
-  p.lane = threadIdx.x;
-  p.i = blockIdx.x * 31 + threadIdx.x;
-  p.j0 = (blockIdx.y * blockDim.y + threadIdx.y) * rows;
-  p.j1 = min(p.j0 + rows, g.py);
-  return p;
-}
-__device__ __forceinline__ double right(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
-
-template <bool CHK>
-__global__ void __launch_bounds__(128) k64_stress2d(Geo g, Stage<double> S, const Scal *sc, DevInfo *di, int rows) {
-  if (skip(di)) return;
-  const Strip p = strip(g, rows);
-  const int i = p.i, nx = g.nx, ny = g.ny;
-  const long long px = g.px;
-  const bool frozen = di != nullptr && di->frozen;
-  const double two_eta = sc->two_eta, eta = 0.5 * two_eta, bt = sc->bt, ob = 1.0 - bt;
-  const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
-  double sig = 0.0, dtau = 0.0, dp = 0.0;
-  double u0_m = 0.0, t_j = 0.0, p_j = 0.0;   // x-velocity of the row below; trial and rotation product at row j
-  // trial and rotation product of vertex (i, j)
-  auto vertex = [&](int j, double u0, double *ts, double *pr) {
-    *ts = *pr = 0.0;
-    if (x1 && j > 0 && j < ny) {
-      const long long e = j * px + i;
-      const double x = (u0 - u0_m) * g.rdy, y = S.u[1][e] - S.u[1][e - 1];
-      const double w = fma(y, -g.rdx, x);
-      const double tr = fma(w, S.md[0][e], fma(eta, fma(y, g.rdx, x), S.tbs[0][e]));
-      *ts = fma(bt, S.sos[0][e], ob * tr);
-      *pr = S.rq[0][e] * w;
-    }
-  };
-  auto u0_at = [&](int j) { return i <= nx && j >= 0 && j < ny ? S.u[0][j * px + i] : 0.0; };
-  if (p.j0 < p.j1) {
-    u0_m = u0_at(p.j0 - 1);
-    const double u0 = u0_at(p.j0);
-    vertex(p.j0, u0, &t_j, &p_j);
-    u0_m = u0;
-  }
-  for (int j = p.j0; j < p.j1; ++j) {
-    const long long e = j * px + i;
-    const double u0 = u0_m, u0_p = u0_at(j + 1);
-    double t_p, p_p;
-    vertex(j + 1, u0_p, &t_p, &p_p);
-    u0_m = u0_p;
-    const double pc = p_j + p_p, tc = t_j + t_p;
-    const double xy = pc + right(pc), txy = tc + right(tc), u0_r = right(u0);
-    if (own) S.Ts[0][e] = t_j;
-    if (own && i < nx && j < ny) {
-      const double e0 = (u0_r - u0) * g.rdx, e1 = (S.u[1][e + px] - S.u[1][e]) * g.rdy;
-      const double div = e0 + e1, m = div * sc->eta_d;
-      const double t0 = fma(0.25, xy, fma(two_eta, e0, S.tbn[0][e] + m));
-      const double t1 = fma(-0.25, xy, fma(two_eta, e1, S.tbn[1][e] + m));
-      const double c0 = fma(bt, S.son[0][e], ob * t0), c1 = fma(bt, S.son[1][e], ob * t1);
-      const double pr = fma(sc->bp, S.sop[e], sc->obp * fma(-sc->KDt, div, S.pb[e]));
-      double s = 1.0;
-      if (frozen) {
-        s = S.s[e];   // frozen plasticity: the held scale (Sec. 3.3)
-      } else {
-        const double J2 = fma(0.0625, txy * txy, 0.5 * fma(c1, c1, c0 * c0));
-        s = return_scale(J2, fma(sc->A, pr, S.yc[e]));
-        S.s[e] = s;
-      }
-      const double n0 = s * c0, n1 = s * c1, s0 = n0 - pr, s1 = n1 - pr;
-      S.snn[0][e] = n0;
-      S.snn[1][e] = n1;
-      S.snp[e] = pr;
-      S.sx[0][e] = s0;
-      S.sx[1][e] = s1;
-      if (CHK) {
-        sig = maxn(sig, maxn(fabs(s0), fabs(s1)));
-        dtau = maxn(dtau, maxn(fabs(n0 - S.cn[0][e]), fabs(n1 - S.cn[1][e])));
-        dp = maxn(dp, fabs(pr - S.cp[e]));
-        S.cn[0][e] = n0;
-        S.cn[1][e] = n1;
-        S.cp[e] = pr;
-        if (isnan(s) || isnan(pr)) sig = NAN;
-      }
-    }
-    t_j = t_p;
-    p_j = p_p;
-  }
-  if (CHK && di) {
-    block_max(sig, &di->red[RED_SIG]);
-    block_max(dtau, &di->red[RED_DTAU]);
-    block_max(dp, &di->red[RED_DP]);
-  }
-}
-
-template <bool CHK>
-__global__ void __launch_bounds__(128) k64_move2d(Geo g, Stage<double> S, const Scal *sc, DevInfo *di, int rows) {
-  if (skip(di)) return;
-  const Strip p = strip(g, rows);
-  const int i = p.i, nx = g.nx, ny = g.ny;
-  const long long px = g.px;
-  const double vs = sc->vstep;
-  const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
-  double sig = 0.0, dtau = 0.0, rmax = 0.0, du = 0.0, vm = 0.0;
-  // scales of the two centres beside column i in row j
-  auto pair = [&](int j) { return x1 && j >= 0 && j < ny ? S.s[j * px + i - 1] + S.s[j * px + i] : 0.0; };
-  // new deviator of vertex (i, j) from its rows of scales
-  auto vertex = [&](int j, double below, double at) {
-    return x1 && j > 0 && j < ny ? (below + at) * (0.25 * S.Ts[0][j * px + i]) : 0.0;
-  };
-  double h_m = pair(p.j0 - 1), h = pair(p.j0), v = vertex(p.j0, h_m, h);
-  for (int j = p.j0; j < p.j1; ++j) {
-    const long long e = j * px + i;
-    const double h_p = pair(j + 1), v_p = vertex(j + 1, h, h_p), v_r = right(v);
-    if (own) {
-      S.sns[0][e] = v;
-      if (CHK) {
-        sig = maxn(sig, fabs(v));
-        dtau = maxn(dtau, fabs(v - S.cs[0][e]));
-        S.cs[0][e] = v;
-      }
-      // face d: in = inside its extent, in1 = off the walls
-      const auto face = [&](int d, bool in, bool in1, double R) {
-        const double u = S.u[d][e];
-        double un = u;
-        if (in1) {
-          if (S.f[d]) R += S.f[d][e];
-          un = fma(vs, R, u);
-          if (CHK) rmax = maxn(rmax, fabs(R));
-        }
-        S.uo[d][e] = un;
-        if (CHK && in) {
-          du = maxn(du, fabs(un - S.uchk[d][e]));
-          vm = maxn(vm, fabs(S.v0[d][e] + u));
-          S.uchk[d][e] = un;
-        }
-      };
-      const bool ix = j < ny, iy = i < nx;
-      double R = 0.0;
-      if (ix && x1) R = fma(v_p - v, g.rdy, (S.sx[0][e] - S.sx[0][e - 1]) * g.rdx);
-      face(0, ix, ix && x1, R);
-      const bool y1 = iy && j > 0 && j < ny;
-      if (y1) R = fma(v_r - v, g.rdx, (S.sx[1][e] - S.sx[1][e - px]) * g.rdy);
-      face(1, iy, y1, R);
-    }
-    h = h_p;
-    v = v_p;
-  }
-  if (CHK && di) {
-    block_max(sig, &di->red[RED_SIG]);
-    block_max(dtau, &di->red[RED_DTAU]);
-    block_max(rmax, &di->red[RED_R]);
-    block_max(du, &di->red[RED_DU]);
-    block_max(vm, &di->red[RED_V]);
-  }
-}
-
 // ---- the rotation's coefficients at vertices / edges, once per increment -------------------
 // md: of the edge's own w; ma, mb: of the summed w of the two other orientations
 // (w = 2 omega; sums of four).  rq = c2 dt tau_hat at edges, rd = c2 dt (tyy - txx),
 // c2 dt (tzz - txx) at centres.
-template <int ND>
 __global__ void __launch_bounds__(256) k_rotation_means(Geo g, Stage<double> S, double *md0, double *md1, double *md2,
                                                         double *ma0, double *ma1, double *ma2, double *mb0,
                                                         double *mb1, double *mb2) {
@@ -468,19 +299,18 @@ __global__ void __launch_bounds__(256) k_rotation_means(Geo g, Stage<double> S, 
   const long long e = q.e, px = g.px, pl = g.plane;
   const bool x1 = i > 0 && i < nx, y1 = j > 0 && j < ny, z1 = k > 0 && k < nz;
   const double *rd0 = S.rd[0], *rd1 = S.rd[1], *q0 = S.rq[0], *q1 = S.rq[1], *q2 = S.rq[2];
-  if ((ND == 2 || k < nz) && x1 && y1) {
+  if (k < nz && x1 && y1) {
     md0[e] = 0.125 * (rd0[e - px - 1] + rd0[e - px] + rd0[e - 1] + rd0[e]);
-    if (ND == 3) {   // + Tyz Wxz + Txz Wyz
-      ma0[e] = 0.03125 * (q2[e - 1] + q2[e] + q2[e - 1 + pl] + q2[e + pl]);
-      mb0[e] = 0.03125 * (q1[e - px] + q1[e] + q1[e - px + pl] + q1[e + pl]);
-    }
+    // + Tyz Wxz + Txz Wyz
+    ma0[e] = 0.03125 * (q2[e - 1] + q2[e] + q2[e - 1 + pl] + q2[e + pl]);
+    mb0[e] = 0.03125 * (q1[e - px] + q1[e] + q1[e - px + pl] + q1[e + pl]);
   }
-  if (ND == 3 && j < ny && x1 && z1) {   // + Tyz Wxy - Txy Wyz
+  if (j < ny && x1 && z1) {   // + Tyz Wxy - Txy Wyz
     md1[e] = 0.125 * (rd1[e - pl - 1] + rd1[e - pl] + rd1[e - 1] + rd1[e]);
     ma1[e] = 0.03125 * (q2[e - 1] + q2[e] + q2[e - 1 + px] + q2[e + px]);
     mb1[e] = -0.03125 * (q0[e - pl] + q0[e - pl + px] + q0[e] + q0[e + px]);
   }
-  if (ND == 3 && i < nx && y1 && z1) {   // - Txy Wxz - Txz Wxy
+  if (i < nx && y1 && z1) {   // - Txy Wxz - Txz Wxy
     md2[e] = 0.125 * ((rd1[e - pl - px] - rd0[e - pl - px]) + (rd1[e - pl] - rd0[e - pl]) +
                       (rd1[e - px] - rd0[e - px]) + (rd1[e] - rd0[e]));
     ma2[e] = -0.03125 * (q0[e - pl] + q0[e - pl + 1] + q0[e] + q0[e + 1]);
@@ -489,7 +319,7 @@ __global__ void __launch_bounds__(256) k_rotation_means(Geo g, Stage<double> S, 
 }
 
 // rows per block: 8 where that leaves four blocks per SM (152), fewer on smaller
-// grids (64^2: 3 x 65 one-row blocks, where 256-thread blocks used 25 SMs)
+// grids
 void launch_rows(const Geo &g, dim3 *grid, dim3 *block) {
   const int bx = (g.nx + 32) / 32;   // points 0 .. nx
   int rows = 8;
@@ -498,38 +328,14 @@ void launch_rows(const Geo &g, dim3 *grid, dim3 *block) {
   *grid = dim3(bx, (g.py + rows - 1) / rows, g.pz);
 }
 
-// 2D strips: rows per warp (a strip recomputes one row of vertices), doubled up
-// to 8 while every SM still has eight warps
-int strip_rows(const Geo &g, dim3 *grid, dim3 *block) {
-  const int bx = (g.nx + 31) / 31;   // points 0 .. nx, 31 per warp
-  int rows = 1;
-  while (rows < 8 && (long long)bx * ((g.py + 2 * rows - 1) / (2 * rows)) >= 1216) rows *= 2;
-  const int strips = (g.py + rows - 1) / rows;
-  int w = 4;
-  while (w > 1 && (long long)bx * ((strips + w - 1) / w) < 304) w /= 2;
-  *block = dim3(32, w);
-  *grid = dim3(bx, (strips + w - 1) / w);
-  return rows;
-}
-
 }  // namespace
 
-int launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
+void launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
                    const cudaEvent_t *ev) {
   dim3 gr, bl;
   auto mark = [&](int q) {
     if (ev) cudaEventRecord(ev[q], st);
   };
-  if (g.ndim == 2) {
-    const int rows = strip_rows(g, &gr, &bl);
-    if (check) k64_stress2d<true><<<gr, bl, 0, st>>>(g, S, sc, di, rows);
-    else k64_stress2d<false><<<gr, bl, 0, st>>>(g, S, sc, di, rows);
-    mark(1);
-    if (check) k64_move2d<true><<<gr, bl, 0, st>>>(g, S, sc, di, rows);
-    else k64_move2d<false><<<gr, bl, 0, st>>>(g, S, sc, di, rows);
-    mark(2);
-    return 2;
-  }
   launch_rows(g, &gr, &bl);
   k64_strain<<<gr, bl, 0, st>>>(g, S, di);
   mark(1);
@@ -544,17 +350,13 @@ int launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo
   if (check) k64_velocity<true><<<gr, bl, 0, st>>>(g, S, sc, di);
   else k64_velocity<false><<<gr, bl, 0, st>>>(g, S, sc, di);
   mark(5);
-  return 5;
 }
 
 void launch_rotation_means(const Geo &g, const Stage<double> &S, double *const md[3], double *const ma[3],
                            double *const mb[3], cudaStream_t st) {
   dim3 gr, bl;
   launch_rows(g, &gr, &bl);
-  if (g.ndim == 2)
-    k_rotation_means<2><<<gr, bl, 0, st>>>(g, S, md[0], md[1], md[2], ma[0], ma[1], ma[2], mb[0], mb[1], mb[2]);
-  else
-    k_rotation_means<3><<<gr, bl, 0, st>>>(g, S, md[0], md[1], md[2], ma[0], ma[1], ma[2], mb[0], mb[1], mb[2]);
+  k_rotation_means<<<gr, bl, 0, st>>>(g, S, md[0], md[1], md[2], ma[0], ma[1], ma[2], mb[0], mb[1], mb[2]);
 }
 
 }  // namespace ep

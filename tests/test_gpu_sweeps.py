@@ -94,13 +94,15 @@ def test_register_sweep_matches_the_staged_sweep_at_tile_edges_fp32(P, n, kz):
 
 @pytest.mark.parametrize("n,rows", [((30, 4), 0), ((31, 5), 0), ((32, 33), 3), ((62, 64), 4), ((63, 7), 0), ((2, 9), 3),
                                     ((300, 180), 3)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("opts", [{}, {"mu_s": 1e-3, "jaumann": False}, {"incompressible": True}])
-def test_fp64_sweep_2d_matches_the_fused_sweep_at_strip_edges(P, n, rows, opts):
+def test_sweep_2d_matches_the_fused_sweep_at_strip_edges(P, n, rows, precision, opts):
     iters = 20
     f = _fields(P, 2, n, 5)
-    iref, ref = _solve(P, 2, n, P.FP64, P.KERNEL_FUSED, iters, f, shape=rows, **opts)
-    info, out = _solve(P, 2, n, P.FP64, P.KERNEL_STAGED, iters, f, **opts)
-    _compare(f, out, ref, info, iref, iters, 2.0 ** -53)
+    pr = P.FP64 if precision == "fp64" else P.FP32_MIXED
+    iref, ref = _solve(P, 2, n, pr, P.KERNEL_FUSED, iters, f, shape=rows, **opts)
+    info, out = _solve(P, 2, n, pr, P.KERNEL_AUTO, iters, f, **opts)
+    _compare(f, out, ref, info, iref, iters, 2.0 ** -53 if precision == "fp64" else EPS32)
 
 
 @pytest.mark.parametrize("n", [(31, 7, 3), (32, 8, 2), (33, 9, 4), (64, 17, 5), (20, 70, 12)])

@@ -251,6 +251,14 @@ double eta_ve(const ep_grid *h) {
   return isinf(h->mu_s) ? h->G * h->dt : 1.0 / (1.0 / (h->G * h->dt) + 1.0 / h->mu_s);
 }
 
+template <typename T>
+void fill_scal(const Scal &s, const Geo &g, SweepScal<T> *o) {
+  o->two_eta = (T)s.two_eta; o->eta = (T)(0.5 * s.two_eta); o->eta_d = (T)(-s.two_eta / 3.0);
+  o->bt = (T)s.bt; o->ob = (T)1 - o->bt; o->bp = (T)s.bp; o->obp = (T)s.obp;
+  o->KDt = (T)s.KDt; o->KDt_phys = (T)s.KDt_phys; o->A = (T)s.A; o->vstep = (T)s.vstep;
+  o->rdx = (T)g.rdx; o->rdy = (T)g.rdy; o->rdz = (T)g.rdz;
+}
+
 // Numerical parameters of Eqs. PT1-PT24qq with pseudo-time step 1:
 // Vp = C dx_min, rho~ = Re eta_ve / (Vp L_max), G~ = rho~ Vp^2 / (r + 4/3),
 // K~ = r G~, Re = xi 3 sqrt(10) pi / 2.
@@ -261,7 +269,6 @@ Scal make_scal(const ep_grid *h) {
                            : eta_ve(h);
   s.gcell = h->Gc != nullptr;
   s.two_eta = 2.0 * eta;
-  s.eta_d = -s.two_eta / 3.0;
   s.c2 = eta / (h->G * h->dt);
   s.c2dt = s.c2 * h->dt;
   s.KDt = h->K * h->dt;
@@ -306,6 +313,8 @@ Scal make_scal(const ep_grid *h) {
     s.p_meas = s.inv_1mbp;
   }
   for (int d = 0; d < 3; ++d) s.rate[d] = h->rate[d];
+  fill_scal(s, h->g, &s.f);
+  fill_scal(s, h->g, &s.d);
   return s;
 }
 

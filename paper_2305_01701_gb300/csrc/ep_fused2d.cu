@@ -74,9 +74,10 @@ __global__ void __launch_bounds__(TX *TY) k_fused2d(const Inst2<T> *insts, const
     const int i0 = item.y * TX, j0 = item.z * TY;
     const int nx = g.nx, ny = g.ny;
     const long long px = g.px;
-    const T rdx = (T)g.rdx, rdy = (T)g.rdy, two_eta = (T)sc->two_eta;
-    const T bt = (T)sc->bt, ob = (T)1 - bt, bp = (T)sc->bp, obp = (T)sc->obp, KDt = (T)sc->KDt;
-    const T Acoef = (T)sc->A, vs = (T)sc->vstep, qr = (T)0.25, third = (T)(1.0 / 3.0);
+    const SweepScal<T> &Q = sweep_scal<T>(sc);
+    const T rdx = Q.rdx, rdy = Q.rdy, two_eta = Q.two_eta;
+    const T bt = Q.bt, ob = Q.ob, bp = Q.bp, obp = Q.obp, KDt = Q.KDt;
+    const T Acoef = Q.A, vs = Q.vstep, qr = (T)0.25, third = (T)(1.0 / 3.0);
     const T *u0 = I.u[b][0], *u1 = I.u[b][1];
 
     __syncthreads();  // the previous item's shared data is no longer read

@@ -293,11 +293,11 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
   const int b0 = (int)(threadIdx.x >> 5) * RPW, b1 = b0 + RPW - 1;
   const bool w_edge = b1 >= 2, w_vel = b1 >= 2 && b0 < H - 2;
 
-  const T rdx = (T)g.rdx, rdy = (T)g.rdy, rdz = (T)g.rdz;
-  const T eta = (T)(0.5 * sc->two_eta), two_eta = (T)sc->two_eta, eta_d = (T)(-sc->two_eta / 3.0);
-  const T bt = (T)sc->bt, ob = (T)1 - bt;
-  const T bp = (T)sc->bp, obp = (T)sc->obp, KDt = (T)sc->KDt, Acoef = (T)sc->A;
-  const T vs = (T)sc->vstep, qr = (T)0.25, e8 = (T)0.125, e32 = (T)0.03125;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz;
+  const T eta = Q.eta, two_eta = Q.two_eta, eta_d = Q.eta_d, bt = Q.bt, ob = Q.ob;
+  const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Acoef = Q.A;
+  const T vs = Q.vstep, qr = (T)0.25, e8 = (T)0.125, e32 = (T)0.03125;
   // velocity step of x-, y- and z-faces: 0 on the walls and off the extent
   const V st0 = mask(in_x1(0) && gy0, in_x1(1) && gy0, vs), st1 = mask(in_x0(0) && gy1, in_x0(1) && gy1, vs),
           st2 = mask(in_x0(0) && gy0, in_x0(1) && gy0, vs);

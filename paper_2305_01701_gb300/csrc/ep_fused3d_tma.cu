@@ -142,10 +142,11 @@ __global__ void __launch_bounds__(TX *TY, 1)
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   const int kb = blockIdx.z * kz, ke = min(kb + kz, g.pz);
   const int nx = g.nx, ny = g.ny, nz = g.nz;
-  const T rdx = (T)g.rdx, rdy = (T)g.rdy, rdz = (T)g.rdz;
-  const T two_eta = (T)sc->two_eta, bt = (T)sc->bt, ob = (T)1 - bt;
-  const T bp = (T)sc->bp, obp = (T)sc->obp, KDt = (T)sc->KDt, Acoef = (T)sc->A;
-  const T vs = (T)sc->vstep, qr = (T)0.25, third = (T)(1.0 / 3.0), hf = (T)0.5;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz;
+  const T two_eta = Q.two_eta, bt = Q.bt, ob = Q.ob;
+  const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Acoef = Q.A;
+  const T vs = Q.vstep, qr = (T)0.25, third = (T)(1.0 / 3.0), hf = (T)0.5;
   const long long px = g.px;
   const bool leader = threadIdx.x == 0;
 

@@ -25,11 +25,21 @@ struct Geo {
   }
 };
 
+// The scalars of a sweep in its own type.  They are rounded on the host: a
+// conversion from FP64 runs on the FP64 pipe (two per clock and SM), and ten of
+// them per thread delayed every block of a short FP32 launch (90 x 40 x 24: 17.6 ->
+// 15.9 us a sweep; 383 x 191: 9.0 -> 8.4 us).
+template <typename T>
+struct SweepScal {
+  T two_eta, eta, eta_d;       // 2 eta_ve, eta_ve, -2 eta_ve / 3
+  T bt, ob, bp, obp, KDt, KDt_phys, A, vstep;
+  T rdx, rdy, rdz;
+};
+
 // Per-increment scalars, read by the kernels from device memory so that a
 // captured CUDA graph stays valid across increments.
 struct Scal {
   double two_eta;      // 2 eta_ve
-  double eta_d;        // -2 eta_ve / 3: weight of the divergence in a normal deviator
   double c2;           // eta_ve / (G dt): weight of the rotated old stress
   double c2dt;         // c2 * dt: weight of the Jaumann rotation term
   double bt, bp;       // relaxation weights beta_tau, beta_p (Eqs. A23ssP, A2ssP)
@@ -51,7 +61,15 @@ struct Scal {
   long long wait_cycles;   // bound of a TMA wait (0: the default, 2^31 cycles)
   int gcell;               // 1: per-cell shear modulus; the rotation weights then
                            // carry dt only and the trial applies each point's c2
+  SweepScal<float> f;
+  SweepScal<double> d;
 };
+template <typename T>
+__device__ __forceinline__ const SweepScal<T> &sweep_scal(const Scal *sc);
+template <>
+__device__ __forceinline__ const SweepScal<float> &sweep_scal<float>(const Scal *sc) { return sc->f; }
+template <>
+__device__ __forceinline__ const SweepScal<double> &sweep_scal<double>(const Scal *sc) { return sc->d; }
 
 // Reduction slots: bit patterns of non-negative doubles reduced with an
 // unsigned atomicMax (IEEE order equals integer order for x >= 0; a NaN
@@ -78,7 +96,7 @@ struct Stage {
   const T *son[3], *sos[3], *sop;   // old pseudo-time state (relax only)
   T *snn[3], *sns[3], *snp;         // new state
   const T *tbn[3], *tbs[3], *pb;    // base trial (x tb_scale) and base pressure
-  double tb_scale;                  // 0 with per-cell c2 (then c2 of the point, see tb_c2)
+  T tb_scale;                       // 0 with per-cell c2 (then c2 of the point, see tb_c2)
   int tb_c2;                        // 1: the base trial is the old stress times c2
   const T *rq[3];                   // c2 dt tau_hat shear (edges)
   const T *rd[2];                   // c2 dt (tyy - txx), c2 dt (tzz - txx) (centres)

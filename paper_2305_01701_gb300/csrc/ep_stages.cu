@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(kThreads) k_strain(Geo g, Stage<T> S, const Sc
   if (!q.in) return;
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   const long long e = q.e, px = g.px, pl = g.plane;
-  const T rdx = (T)g.rdx, rdy = (T)g.rdy, rdz = (T)g.rdz, h = (T)0.5;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz, h = (T)0.5;
   if (i > nx || j > ny || k > (ND == 3 ? nz : 0)) return;
   // xy: 2D vertices or 3D xy-edges (k < nz)
   {
@@ -135,14 +136,15 @@ __global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Sca
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   const long long e = q.e, px = g.px, pl = g.plane;
   if (i > nx || j > ny || k > (ND == 3 ? nz : 0)) return;
-  const T rdx = (T)g.rdx, rdy = (T)g.rdy, rdz = (T)g.rdz;
-  const T two_eta = (T)sc->two_eta, tbs0 = (T)S.tb_scale, qr = (T)0.25, third = (T)(1.0 / 3.0);
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz;
+  const T two_eta = Q.two_eta, tbs0 = S.tb_scale, qr = (T)0.25, third = (T)(1.0 / 3.0);
   // per point: 2 eta_ve, the weight c2 of the rotation terms (folded into
   // the rotation weights when the modulus is uniform) and of the base trial
   auto te = [&](int w, long long x) { return S.ge[w] ? S.ge[w][x] : two_eta; };
   auto cr = [&](int w, long long x) { return S.gc[w] ? S.gc[w][x] : (T)1; };
   auto tb = [&](int w, long long x) { return S.tb_c2 && S.gc[w] ? S.gc[w][x] : tbs0; };
-  const T bt = S.relax ? (T)sc->bt : (T)0, ob = (T)1 - bt;
+  const T bt = S.relax ? Q.bt : (T)0, ob = S.relax ? Q.ob : (T)1;
   // ---- centre ----
   if (i < nx && j < ny && (ND == 2 || k < nz)) {
     const long long c = e;
@@ -234,14 +236,15 @@ __global__ void __launch_bounds__(kThreads) k_return_centres(Geo g, Stage<T> S, 
   const long long c = q.e, px = g.px, pl = g.plane;
   const bool act = q.in && i < g.nx && j < g.ny && (ND == 2 || k < g.nz);
   const bool frozen = di != nullptr && di->frozen;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
   T sig = 0, dtau = 0, dp = 0;
   if (act) {
     const T qr = (T)0.25;
-    T div = (S.u[0][c + 1] - S.u[0][c]) * (T)g.rdx + (S.u[1][c + px] - S.u[1][c]) * (T)g.rdy;
-    if (ND == 3) div += (S.u[2][c + pl] - S.u[2][c]) * (T)g.rdz;
+    T div = (S.u[0][c + 1] - S.u[0][c]) * Q.rdx + (S.u[1][c + px] - S.u[1][c]) * Q.rdy;
+    if (ND == 3) div += (S.u[2][c + pl] - S.u[2][c]) * Q.rdz;
     T p;
-    if (S.relax) p = (T)sc->bp * S.sop[c] + (T)sc->obp * (S.pb[c] - (T)sc->KDt * div);
-    else p = S.pb[c] - (T)sc->KDt_phys * div;
+    if (S.relax) p = Q.bp * S.sop[c] + Q.obp * (S.pb[c] - Q.KDt * div);
+    else p = S.pb[c] - Q.KDt_phys * div;
     T txy = qr * (S.Ts[0][c] + S.Ts[0][c + 1] + S.Ts[0][c + px] + S.Ts[0][c + px + 1]);
     T J2 = txy * txy;
     if (ND == 3) {
@@ -260,7 +263,7 @@ __global__ void __launch_bounds__(kThreads) k_return_centres(Geo g, Stage<T> S, 
       s = S.s[c];   // frozen plasticity: the held scale (Sec. 3.3)
     } else {
       T sj = sqrt(J2);
-      T Y = (T)sc->A * p + S.yc[c];
+      T Y = Q.A * p + S.yc[c];
       Y = Y > (T)0 ? Y : (T)0;
       s = sj > Y ? Y / sj : (T)1;
       S.s[c] = s;
@@ -350,7 +353,8 @@ __global__ void __launch_bounds__(kThreads) k_velocity(Geo g, Stage<T> S, const 
   const Pos q = position(g);
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   const long long e = q.e, px = g.px, pl = g.plane;
-  const T rdx = (T)g.rdx, rdy = (T)g.rdy, rdz = (T)g.rdz, vs = (T)sc->vstep;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz, vs = Q.vstep;
   T rmax = 0, du = 0;
   double vm = 0.0;   // |v0 + u| needs the FP64 base velocity
   if (q.in && i <= nx && j <= ny && k <= (ND == 3 ? nz : 0)) {

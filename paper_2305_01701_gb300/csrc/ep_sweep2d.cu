@@ -80,8 +80,9 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
   const int i = p.i, nx = g.nx, ny = g.ny;
   const int px = g.px;   // a 2D box has fewer than 2^31 points
   const bool frozen = di != nullptr && di->frozen;
-  const T two_eta = (T)sc->two_eta, eta = (T)0.5 * two_eta, eta_d = (T)sc->eta_d, bt = (T)sc->bt, ob = (T)1 - bt;
-  const T bp = (T)sc->bp, obp = (T)sc->obp, KDt = (T)sc->KDt, Ac = (T)sc->A, rdx = (T)g.rdx, rdy = (T)g.rdy;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T two_eta = Q.two_eta, eta = Q.eta, eta_d = Q.eta_d, bt = Q.bt, ob = Q.ob;
+  const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Ac = Q.A, rdx = Q.rdx, rdy = Q.rdy;
   const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
   T sig = 0, dtau = 0, dp = 0;
   T u0_m = 0, t_j = 0, p_j = 0;   // x-velocity of the row below; trial and rotation product at row j
@@ -160,7 +161,8 @@ __global__ void __launch_bounds__(128) k_move2d(Geo g, Stage<T> S, const Scal *s
   const Strip p = strip(g, rows);
   const int i = p.i, nx = g.nx, ny = g.ny;
   const int px = g.px;   // a 2D box has fewer than 2^31 points
-  const T vs = (T)sc->vstep, rdx = (T)g.rdx, rdy = (T)g.rdy;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T vs = Q.vstep, rdx = Q.rdx, rdy = Q.rdy;
   const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
   T sig = 0, dtau = 0, rmax = 0, du = 0;
   double vm = 0.0;   // |v0 + u| needs the FP64 base velocity

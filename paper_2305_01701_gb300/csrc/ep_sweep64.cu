@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k64_trial(Geo g, Stage<double> S, const S
     const double e0 = (S.u[0][e + 1] - S.u[0][e]) * g.rdx, e1 = (S.u[1][e + px] - S.u[1][e]) * g.rdy;
     const double *p0 = S.pr[0];
     const double xy = (p0[e] + p0[e + 1]) + (p0[e + px] + p0[e + px + 1]);
-      const double e2 = (S.u[2][e + pl] - S.u[2][e]) * g.rdz, div = e0 + e1 + e2, m = div * sc->eta_d;
+      const double e2 = (S.u[2][e + pl] - S.u[2][e]) * g.rdz, div = e0 + e1 + e2, m = div * sc->d.eta_d;
       const double *p1 = S.pr[1], *p2 = S.pr[2];
       const double xz = (p1[e] + p1[e + 1]) + (p1[e + pl] + p1[e + pl + 1]);
       const double yz = (p2[e] + p2[e + px]) + (p2[e + pl] + p2[e + pl + px]);

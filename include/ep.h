@@ -160,7 +160,8 @@ ep_status ep_set_material(ep_handle h, double K, double G, double mu_s, double p
  * G at the centres, and at a vertex/edge the mean G of the centres around it
  * (indices clamped at the walls); the pseudo-transient parameters (Eqs.
  * PT1-PT24qq) use the largest G.  NULL restores the uniform G.  Grids with a
- * per-cell G run the staged sweep kernels.  Not inside an open increment. */
+ * per-cell G run the staged sweep kernels, or the register z-march sweep (3D
+ * FP32: EP_KERNEL_AUTO, EP_KERNEL_FUSED_REG).  Not inside an open increment. */
 ep_status ep_set_shear_modulus(ep_handle h, const double *G);
 
 /* Fill opts with the defaults for a grid of dimension ndim. */

@@ -565,8 +565,10 @@ int fused_variant(const ep_grid *h) {
 
 template <typename T>
 bool use_fused(const ep_grid *h) {
-  if (h->ndim != 3 || h->have_f || h->Gc) return false;
+  if (h->ndim != 3 || h->have_f) return false;
   const int v = fused_variant(h);
+  // a per-cell shear modulus: the FP32 register sweep only
+  if (h->Gc) return sizeof(T) == 4 && v == EP_KERNEL_FUSED_REG;
   return v == EP_KERNEL_FUSED || v == EP_KERNEL_FUSED_TMA || v == EP_KERNEL_FUSED_REG;
 }
 

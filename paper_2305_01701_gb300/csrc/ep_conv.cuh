@@ -46,6 +46,8 @@ struct TcOut {
   int head_c;
   float scale;
 };
+// shared-memory limits of the kernels, per device (at every network's creation)
+cudaError_t conv_tc_configure();
 bool conv_tc_supported(int k, int cout);
 __host__ __device__ constexpr int conv_tc_cinp(int cin) { return (cin + 15) / 16 * 16; }
 // FP32 N x C x V -> blocks of conv_tc_cinp(C) channels

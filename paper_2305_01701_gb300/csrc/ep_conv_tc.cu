@@ -423,9 +423,6 @@ constexpr size_t SMEM_MAX = 216 * 1024;   // beside the static arrays
 
 template <int D, int TZ, int KQ>
 cudaError_t tc_launch(const CUtensorMap &map, TcArgs A, int N, cudaStream_t st) {
-  static const cudaError_t cfg =
-      cudaFuncSetAttribute(k_conv_tc<D, TZ, KQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
-  if (cfg != cudaSuccess) return cfg;
   // shared memory: two A stages, and as many B stages as fit
   const size_t a = ((size_t)(A.kc / 8) * HX * HY * (D == 3 ? TZ + 2 : 1) * 16 + 127) / 128 * 128;
   const size_t b = 3 * (size_t)A.kc * A.cout * 2;
@@ -439,6 +436,16 @@ cudaError_t tc_launch(const CUtensorMap &map, TcArgs A, int N, cudaStream_t st) 
 }
 
 }  // namespace
+
+cudaError_t conv_tc_configure() {
+  cudaError_t e = cudaSuccess;
+#define EP_CFG(d, tz, kq)                                                                                       \
+  if (e == cudaSuccess)                                                                                         \
+    e = cudaFuncSetAttribute(k_conv_tc<d, tz, kq>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+  EP_CFG(2, 1, 1) EP_CFG(2, 1, 2) EP_CFG(3, 2, 1) EP_CFG(3, 2, 2) EP_CFG(3, 4, 1) EP_CFG(3, 4, 2)
+#undef EP_CFG
+  return e;
+}
 
 bool conv_tc_supported(int k, int cout) { return k == 3 && cout >= 16 && cout <= 128 && cout % 16 == 0; }
 

@@ -23,13 +23,15 @@
 // plane t-1, centres t-1, edges t-1 and velocities t-2.  Three block barriers
 // separate the steps of a plane.
 // Bound: HBM in principle (132 B per cell); in fact the latency of a plane's
-// three steps at 12 warps per SM.  Measured (FP32, one sweep): 127^3 79.5 us,
-// 383^3 1600 us (4.6 TB/s), against 126.9 and 2312 us of the form with one
+// three steps at 12 warps per SM.  Measured (FP32, one sweep): 127^3 77.2 us,
+// 383^3 1575 us (4.7 TB/s), against 126.9 and 2312 us of the form with one
 // column per thread (16 warps, 600 instructions per warp and plane, register
 // prefetch).  Packing the pairs alone, with the register prefetch (8 warps of
 // 255 registers), halved the instructions and gained nothing: the loads'
 // latency showed.  cp.async in place of TMA cost 5 shared-memory wavefronts
 // per 8-byte copy (the window starts off a 32-byte sector): 131 and 2164 us.
+// With a per-cell shear modulus (31 inputs, 16 rows) 95^3 takes 52 us, the five
+// staged kernels 100.
 // Instruction count:
 //   * FP32 arithmetic is packed (add/mul/fma on float2: one instruction per
 //     pair);
@@ -152,16 +154,23 @@ struct Rows {
 enum {
   I_U0, I_U1, I_U2, I_RQ0, I_RQ1, I_RQ2, I_RD0, I_RD1, I_SOXZ, I_SOYZ, I_TBXZ, I_TBYZ,
   I_SON0, I_SON1, I_SON2, I_TBN0, I_TBN1, I_TBN2, I_SOXY, I_TBXY, I_SOP, I_PB, I_YC,
-  I_COUNT
+  I_COUNT,
+  // with a per-cell shear modulus also 2 eta_ve and c2 of the points of plane t - 1
+  // (centres, xy) and plane t (xz, yz)
+  I_GEN = I_COUNT, I_GCN, I_GEXY, I_GCXY, I_GEXZ, I_GCXZ, I_GEYZ, I_GCYZ,
+  I_COUNT_G
 };
+template <bool GC>
+constexpr int inputs() { return GC ? I_COUNT_G : I_COUNT; }
 
 // columns of a TMA box: the window and two more on either side, so that its
 // first column is a multiple of 16 bytes
 constexpr int BX = WX + 4;
 
-template <typename L>
+template <typename L, bool GC>
 struct SmemR {
-  alignas(128) typename L::T in[2][I_COUNT][L::H * BX];   // inputs of planes t and t + 1 (then t + 2)
+  alignas(128) typename L::T in[2][inputs<GC>()][L::H * BX];   // inputs of planes t and t + 1 (then t + 2)
+  static_assert(sizeof(in[0][0]) % 128 == 0, "a TMA box lands on a 128-byte boundary");
   Rows<L> A, D, I, K;               // sums of neighbouring inputs
   Rows<L> B, E, wxz, M, pyz;        // pair sums of spins and rotation products
   Rows<L> Q, Sz, U, Vs;             // pair sums of the edge trials and of the scales
@@ -169,8 +178,9 @@ struct SmemR {
   alignas(8) unsigned long long full[2];   // a stage's copies have arrived
 };
 
+template <bool GC>
 struct Maps {
-  CUtensorMap m[I_COUNT];
+  CUtensorMap m[inputs<GC>()];
 };
 
 template <typename T>
@@ -258,14 +268,15 @@ __device__ __forceinline__ void block_max_bits(double v, unsigned long long *slo
 // INT: every column of the block's window lies strictly inside the domain
 // (1 <= x, y index <= n - 1), so the domain-boundary tests fold away.
 // Off: the integer type of offsets within an array.  CHK: a check iteration.
-template <typename L, bool INT, typename Off, bool CHK>
-__device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T> &A, const Geo &g, const Scal *sc, DevInfo *di,
+// GC: a per-cell shear modulus.
+template <typename L, bool GC, bool INT, typename Off, bool CHK>
+__device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename L::T> &A, const Geo &g, const Scal *sc, DevInfo *di,
                                          bool frozen, int kz, unsigned char *smem_raw) {
   using T = typename L::T;
   using V = typename L::V;
   constexpr int N = L::N, H = L::H, LPR = L::LPR;
-  SmemR<L> &S = *reinterpret_cast<SmemR<L> *>(smem_raw);
-  ChkSlots<L> &C = *reinterpret_cast<ChkSlots<L> *>(smem_raw + sizeof(SmemR<L>));   // CHK only
+  SmemR<L, GC> &S = *reinterpret_cast<SmemR<L, GC> *>(smem_raw);
+  ChkSlots<L> &C = *reinterpret_cast<ChkSlots<L> *>(smem_raw + sizeof(SmemR<L, GC>));   // CHK only
   const int a = threadIdx.x % LPR, b = threadIdx.x / LPR;
   const int i0 = blockIdx.x * OX, j0 = blockIdx.y * (H - 4);
   const int gi = i0 - 2 + N * a, gj = j0 - 2 + b;   // first column of the thread, row
@@ -322,9 +333,10 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
   auto fetch = [&](int t, const int stage) {
     if (!elected) return;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    bar_expect(&S.full[stage], (unsigned)((I_COUNT - warp + NW - 1) / NW) * BOX);
-    for (int k = warp; k < I_COUNT; k += NW)
-      tma_load(S.in[stage][k], &M.m[k], i0 - 4, j0 - 2, k < I_SON0 ? t : t - 1, &S.full[stage]);
+    constexpr int NI = inputs<GC>();
+    bar_expect(&S.full[stage], (unsigned)((NI - warp + NW - 1) / NW) * BOX);
+    for (int k = warp; k < NI; k += NW)
+      tma_load(S.in[stage][k], &M.m[k], i0 - 4, j0 - 2, k < I_SON0 || k >= I_GEXZ ? t : t - 1, &S.full[stage]);
   };
   if (threadIdx.x == 0) {
     for (int q = 0; q < 2; ++q)
@@ -337,7 +349,7 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
   V u0 = zero, u1 = zero, u2 = zero, u0_1 = zero, u1_1 = zero, u2_1 = zero, u0_2 = zero, u1_2 = zero, u2_2 = zero;
   V rq0 = zero;
   V D_1 = zero, E_1 = zero, F_1 = zero, G_1 = zero, J_1 = zero, L_1 = zero, M_1 = zero, N_1 = zero, O_1 = zero;
-  V wxy_1 = zero, qxy_1 = zero, e1_1 = zero, tsxz_1 = zero, tsyz_1 = zero;
+  V wxy_1 = zero, qxy_1 = zero, gxy_1 = zero, e1_1 = zero, tsxz_1 = zero, tsyz_1 = zero;
   V s_2 = zero, U_2 = zero;                                // quarter scale and its x pair sum, plane t-2
   V sxx_2 = zero, syy_2 = zero, szz_2 = zero, szz_3 = zero;   // centre stress minus pressure
   V nxy_2 = zero, nxz_2 = zero, nyz_2 = zero;              // edge stress, level t-2
@@ -423,6 +435,12 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
     // ---- 2. relaxed trials: faces t (xz, yz), plane t-1 (xy, centres) ----
     const int lc = t - 1;
     const bool zc = lc >= 0 && lc < nz;
+    // an edge's trial: base + eta g + rotation r (in units of sc), each point's
+    // own 2 eta_ve and c2 with a per-cell modulus
+    auto trial = [&](V r, T unit, V gs, int tb, int ge) -> V {
+      if constexpr (GC) return vfma(vmul(r, bc(unit)), own(ge + 1), vfma(vmul(gs, bc((T)0.5)), own(ge), own(tb)));
+      else return vfma(r, bc(unit), vfma(gs, bc(eta), own(tb)));
+    };
     V tsxz, tsyz, tsxy, c0v, c1v, c2v, div;
     const V sop = own(I_SOP), pb = own(I_PB), yc = own(I_YC);
     {
@@ -433,7 +451,7 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
         const V Txy = vadd(vA, S.A.r[qp]), Wxy = vadd(vB, S.B.r[qp]);
         const V r1 = vsub(vmul(Tyz, Wxy), vmul(Txy, Wyz));
         const V r = vfma(r1, bc(qr), vmul(wxz, Dz));
-        const V tr = vfma(r, bc(e8), vfma(gxz, bc(eta), own(I_TBXZ)));
+        const V tr = trial(r, e8, gxz, I_TBXZ, I_GEXZ);
         tsxz = keep<INT>(m_xz, vfma(own(I_SOXZ), bc(bt), vmul(tr, bc(ob))));
       }
       {   // yz: w dzy - (Txy Wxz + Txz Wxy) / 4
@@ -441,18 +459,25 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
         const V Txz = vadd(F, xp(F)), Wxz = vadd(G, xp(G));
         const V r1 = vfma(Txz, Wxy, vmul(Txy, Wxz));
         const V r = vfma(r1, bc(-qr), vmul(wyz, Dz));
-        const V tr = vfma(r, bc(e8), vfma(gyz, bc(eta), own(I_TBYZ)));
+        const V tr = trial(r, e8, gyz, I_TBYZ, I_GEYZ);
         tsyz = keep<INT>(m_yz, vfma(own(I_SOYZ), bc(bt), vmul(tr, bc(ob))));
       }
       if (!zf) { tsxz = zero; tsyz = zero; }
       {   // xy of plane t-1: w dyx + (Tyz Wxz + Txz Wyz) / 4
         const V Tyz = vadd(D_1, D), Wyz = vadd(E_1, vE), Txz = vadd(F_1, F), Wxz = vadd(G_1, G);
         const V r1 = vfma(Tyz, Wxz, vmul(Txz, Wyz));
-        const V tr = vfma(r1, bc(e32), vadd(own(I_TBXY), qxy_1));
+        V tr;
+        if constexpr (GC) tr = trial(vfma(r1, bc(qr), qxy_1), e8, gxy_1, I_TBXY, I_GEXY);
+        else tr = vfma(r1, bc(e32), vadd(own(I_TBXY), qxy_1));
         tsxy = keep<INT>(m_xy, vfma(own(I_SOXY), bc(bt), vmul(tr, bc(ob))));
         if (!zc) tsxy = zero;
         // this plane's part of the next plane's xy trial
-        qxy_1 = vfma(gxy, bc(eta), vmul(vmul(wxy, dyx), bc(e8)));
+        if constexpr (GC) {
+          qxy_1 = vmul(wxy, dyx);
+          gxy_1 = gxy;
+        } else {
+          qxy_1 = vfma(gxy, bc(eta), vmul(vmul(wxy, dyx), bc(e8)));
+        }
       }
       {   // centres of plane t-1
         const V e0 = vmul(vsub(xp(u0_1), u0_1), bc(rdx));
@@ -461,11 +486,18 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
         div = vadd(vadd(e0, e1), e2);
         const V O = vadd(pyz, S.pyz.r[qp]);
         const V Pxz = vadd(N_1, vN), Pyz = vadd(O_1, O), Pxy = M_1;
-        const V m = vmul(div, bc(eta_d));
-        const V te = bc(two_eta), q = bc(qr);
-        const V t0 = vfma(vadd(Pxy, Pxz), q, vadd(own(I_TBN0), vfma(e0, te, m)));
-        const V t1 = vfma(vsub(Pyz, Pxy), q, vadd(own(I_TBN1), vfma(e1, te, m)));
-        const V t2 = vfma(vadd(Pxz, Pyz), bc(-qr), vadd(own(I_TBN2), vfma(e2, te, m)));
+        V t0, t1, t2;
+        if constexpr (GC) {
+          const V te = own(I_GEN), q = vmul(own(I_GCN), bc(qr)), d3 = vmul(div, bc((T)(1.0 / 3.0)));
+          t0 = vfma(vadd(Pxy, Pxz), q, vfma(vsub(e0, d3), te, own(I_TBN0)));
+          t1 = vfma(vsub(Pyz, Pxy), q, vfma(vsub(e1, d3), te, own(I_TBN1)));
+          t2 = vfma(vsub(zero, vadd(Pxz, Pyz)), q, vfma(vsub(e2, d3), te, own(I_TBN2)));
+        } else {
+          const V m = vmul(div, bc(eta_d)), te = bc(two_eta), q = bc(qr);
+          t0 = vfma(vadd(Pxy, Pxz), q, vadd(own(I_TBN0), vfma(e0, te, m)));
+          t1 = vfma(vsub(Pyz, Pxy), q, vadd(own(I_TBN1), vfma(e1, te, m)));
+          t2 = vfma(vadd(Pxz, Pyz), bc(-qr), vadd(own(I_TBN2), vfma(e2, te, m)));
+        }
         c0v = vfma(own(I_SON0), bc(bt), vmul(t0, bc(ob)));
         c1v = vfma(own(I_SON1), bc(bt), vmul(t1, bc(ob)));
         c2v = vfma(own(I_SON2), bc(bt), vmul(t2, bc(ob)));
@@ -636,28 +668,17 @@ __device__ __forceinline__ void reg_body(const Maps &M, const Args<typename L::T
   }
 }
 
-template <typename L, typename Off, bool CHK>
+template <typename L, bool GC, typename Off, bool CHK>
 __global__ void __launch_bounds__(L::LPR *L::H, 1)
-    k_fused3d_reg(const __grid_constant__ Maps M, const Args<typename L::T> A, Geo g, const Scal *sc, DevInfo *di, int kz) {
+    k_fused3d_reg(const __grid_constant__ Maps<GC> M, const Args<typename L::T> A, Geo g, const Scal *sc, DevInfo *di, int kz) {
   if (di != nullptr && *(volatile const int *)&di->done != 0) return;
   const bool frozen = di != nullptr && di->frozen;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int i0 = blockIdx.x * OX, j0 = blockIdx.y * (L::H - 4);
   const bool interior = i0 - 2 >= 1 && i0 + WX - 3 <= g.nx - 1 && j0 - 2 >= 1 && j0 + L::H - 3 <= g.ny - 1;
-  if (interior) reg_body<L, true, Off, CHK>(M, A, g, sc, di, frozen, kz, smem_raw);
-  else reg_body<L, false, Off, CHK>(M, A, g, sc, di, frozen, kz, smem_raw);
+  if (interior) reg_body<L, GC, true, Off, CHK>(M, A, g, sc, di, frozen, kz, smem_raw);
+  else reg_body<L, GC, false, Off, CHK>(M, A, g, sc, di, frozen, kz, smem_raw);
 }
-
-template <typename T>
-struct LaneOf {
-  using type = LaneF<24>;
-  using check = LaneF<16>;   // the snapshots' slots take the room of eight rows
-};
-template <>
-struct LaneOf<double> {
-  using type = LaneD;
-  using check = LaneD;
-};
 
 typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -674,19 +695,20 @@ EncodeTiled encoder() {
   return fn;
 }
 
-// tensor maps of the stage's 23 input arrays: boxes of BX x H x 1, zero outside
-template <typename L>
-bool encode_maps(Maps *M, const Geo &g, const Stage<typename L::T> &S) {
+// tensor maps of the stage's input arrays: boxes of BX x H x 1, zero outside
+template <typename L, bool GC>
+bool encode_maps(Maps<GC> *M, const Geo &g, const Stage<typename L::T> &S) {
   using T = typename L::T;
-  const T *src[I_COUNT] = {S.u[0],   S.u[1],   S.u[2],   S.rq[0],  S.rq[1],  S.rq[2],  S.rd[0],  S.rd[1],
-                           S.sos[1], S.sos[2], S.tbs[1], S.tbs[2], S.son[0], S.son[1], S.son[2], S.tbn[0],
-                           S.tbn[1], S.tbn[2], S.sos[0], S.tbs[0], S.sop,    S.pb,     S.yc};
+  const T *src[I_COUNT_G] = {S.u[0],   S.u[1],   S.u[2],   S.rq[0],  S.rq[1],  S.rq[2],  S.rd[0],  S.rd[1],
+                             S.sos[1], S.sos[2], S.tbs[1], S.tbs[2], S.son[0], S.son[1], S.son[2], S.tbn[0],
+                             S.tbn[1], S.tbn[2], S.sos[0], S.tbs[0], S.sop,    S.pb,     S.yc,     S.ge[0],
+                             S.gc[0],  S.ge[1],  S.gc[1],  S.ge[2],  S.gc[2],  S.ge[3],  S.gc[3]};
   const EncodeTiled fn = encoder();
   if (!fn) return false;
   cuuint64_t dims[3] = {(cuuint64_t)g.px, (cuuint64_t)g.py, (cuuint64_t)g.pz};
   cuuint64_t strides[2] = {(cuuint64_t)g.px * sizeof(T), (cuuint64_t)g.plane * sizeof(T)};
   cuuint32_t box[3] = {(cuuint32_t)BX, (cuuint32_t)L::H, 1}, es[3] = {1, 1, 1};
-  for (int k = 0; k < I_COUNT; ++k)
+  for (int k = 0; k < inputs<GC>(); ++k)
     if (fn(&M->m[k], sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
            const_cast<T *>(src[k]), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -694,22 +716,41 @@ bool encode_maps(Maps *M, const Geo &g, const Stage<typename L::T> &S) {
   return true;
 }
 
-template <typename L, typename Off, bool CHK>
+template <typename L, bool GC, bool CHK>
+constexpr size_t lane_bytes() { return sizeof(SmemR<L, GC>) + (CHK ? sizeof(ChkSlots<L>) : 0); }
+
+template <typename L, bool GC, bool CHK>
+cudaError_t configure_lane() {
+  const cudaError_t e = cudaFuncSetAttribute(k_fused3d_reg<L, GC, int, CHK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)lane_bytes<L, GC, CHK>());
+  return e != cudaSuccess ? e
+                          : cudaFuncSetAttribute(k_fused3d_reg<L, GC, long long, CHK>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)lane_bytes<L, GC, CHK>());
+}
+
+// the columns to write: 0 .. nx (the row's padding stays zero)
+Geo extent(Geo g) {
+  g.px = g.nx + 1;
+  return g;
+}
+
+template <typename L, bool GC, typename Off, bool CHK>
 bool launch_lane(const Stage<typename L::T> &S, const Args<typename L::T> &A, const Geo &g, const Scal *sc, DevInfo *di,
                  int kz, cudaStream_t st) {
-  Maps M;
-  if (!encode_maps<L>(&M, g, S)) return false;
-  kz = fused3d_kz(g, OX, L::H - 4, kz);
-  dim3 grid((g.px + OX - 1) / OX, (g.py + L::H - 5) / (L::H - 4), (g.pz + kz - 1) / kz);
-  k_fused3d_reg<L, Off, CHK><<<grid, L::LPR * L::H, sizeof(SmemR<L>) + (CHK ? sizeof(ChkSlots<L>) : 0), st>>>(
-      M, A, g, sc, di, kz);
+  Maps<GC> M;
+  if (!encode_maps<L, GC>(&M, g, S)) return false;
+  if (kz <= 0) kz = fused3d_kz(extent(g), OX, L::H - 4, 0);
+  dim3 grid((g.nx + OX) / OX, (g.py + L::H - 5) / (L::H - 4), (g.pz + kz - 1) / kz);
+  k_fused3d_reg<L, GC, Off, CHK><<<grid, L::LPR * L::H, lane_bytes<L, GC, CHK>(), st>>>(M, A, g, sc, di, kz);
   return true;
 }
 
-template <typename L, typename Off, bool CHK>
-cudaError_t configure_lane() {
-  return cudaFuncSetAttribute(k_fused3d_reg<L, Off, CHK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(sizeof(SmemR<L>) + (CHK ? sizeof(ChkSlots<L>) : 0)));
+template <typename L, bool GC, bool CHK>
+bool launch_off(const Stage<typename L::T> &S, const Args<typename L::T> &A, const Geo &g, const Scal *sc, DevInfo *di,
+                int kz, cudaStream_t st) {
+  return (long long)g.pz * g.plane < (1LL << 31) ? launch_lane<L, GC, int, CHK>(S, A, g, sc, di, kz, st)
+                                                  : launch_lane<L, GC, long long, CHK>(S, A, g, sc, di, kz, st);
 }
 
 }  // namespace
@@ -721,35 +762,38 @@ cudaError_t configure_lane() {
 template <typename T>
 bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
                         bool check) {
-  using L = typename LaneOf<T>::type;
-  using LC = typename LaneOf<T>::check;
   Args<T> A;
   for (int d = 0; d < 3; ++d) {
     A.snn[d] = S.snn[d]; A.sns[d] = S.sns[d]; A.uo[d] = S.uo[d];
     A.cn[d] = S.cn[d]; A.cs[d] = S.cs[d]; A.uchk[d] = S.uchk[d]; A.v0[d] = S.v0[d];
   }
   A.snp = S.snp; A.s = S.s; A.cp = S.cp;
-  if constexpr (sizeof(T) == 4) {
-    const bool o32 = (long long)g.pz * g.plane < (1LL << 31);
-    if (check)
-      return o32 ? launch_lane<LC, int, true>(S, A, g, sc, di, kz, st)
-                 : launch_lane<LC, long long, true>(S, A, g, sc, di, kz, st);
-    return o32 ? launch_lane<L, int, false>(S, A, g, sc, di, kz, st)
-               : launch_lane<L, long long, false>(S, A, g, sc, di, kz, st);
+  if constexpr (sizeof(T) == 8) {
+    return launch_off<LaneD, false, false>(S, A, g, sc, di, kz, st);
+  } else if (S.ge[0]) {
+    return check ? launch_off<LaneF<16>, true, true>(S, A, g, sc, di, kz, st)
+                 : launch_off<LaneF<16>, true, false>(S, A, g, sc, di, kz, st);
+  } else if (check) {   // the snapshots' slots take the room of eight rows
+    return launch_off<LaneF<16>, false, true>(S, A, g, sc, di, kz, st);
   } else {
-    return launch_lane<L, long long, false>(S, A, g, sc, di, kz, st);
+    // a plane takes a 16-row block 1.5 us and a 24-row one 2.0 us; the 24 rows write
+    // 20 of theirs, the 16 rows 12, but need fewer planes per block where the grid is
+    // small (90x40x24 12.2 against 15.8 us a sweep, 63^3 19.8 / 22.3; 127^3 92.8 / 77.2,
+    // 383^3 1757 / 1575)
+    long long c16 = 0, c24 = 0;
+    const int k16 = fused3d_kz(extent(g), OX, 12, kz, 1, &c16), k24 = fused3d_kz(extent(g), OX, 20, kz, 1, &c24);
+    if (3 * c16 < 4 * c24) return launch_off<LaneF<16>, false, false>(S, A, g, sc, di, k16, st);
+    return launch_off<LaneF<24>, false, false>(S, A, g, sc, di, k24, st);
   }
 }
 
 cudaError_t fused3d_reg_configure() {
-  using L = LaneOf<float>::type;
-  using LC = LaneOf<float>::check;
-  cudaError_t e = configure_lane<L, int, false>();
-  if (e == cudaSuccess) e = configure_lane<L, long long, false>();
-  if (e == cudaSuccess) e = configure_lane<LC, int, true>();
-  if (e == cudaSuccess) e = configure_lane<LC, long long, true>();
-  if (e == cudaSuccess) e = configure_lane<LaneD, long long, false>();
-  return e;
+  const cudaError_t e[] = {configure_lane<LaneF<24>, false, false>(), configure_lane<LaneF<16>, false, false>(),
+                           configure_lane<LaneF<16>, false, true>(),  configure_lane<LaneF<16>, true, false>(),
+                           configure_lane<LaneF<16>, true, true>(),   configure_lane<LaneD, false, false>()};
+  for (cudaError_t q : e)
+    if (q != cudaSuccess) return q;
+  return cudaSuccess;
 }
 
 template bool launch_fused3d_reg<float>(const Geo &, const Stage<float> &, const Scal *, DevInfo *, int, cudaStream_t,

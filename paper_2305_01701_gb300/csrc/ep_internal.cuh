@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "../../include/ep.h"
 
 namespace ep {
@@ -227,24 +229,24 @@ void launch_rotation_mean2d(const Geo &g, const T *rd, T *md, cudaStream_t st);
 // z-planes per block when none was chosen (kz <= 0).  A block marches kz
 // planes plus four halo planes, and the launch runs in waves of
 // (SMs x blocks per SM) blocks, so the time goes as
-// waves(kz) x (kz + 4); take the kz in [1, 128] that minimises it.
-inline int fused3d_kz(const Geo &g, int tx, int ty, int kz, int per_sm = 1) {
-  if (kz > 0) return kz;
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
+// waves(kz) x (kz + 4); take the kz that minimises it.
+// A kz > 0 is kept.  cost (nullable): waves(kz) x (kz + 4).
+inline int fused3d_kz(const Geo &g, int tx, int ty, int kz, int per_sm = 1, long long *cost = nullptr) {
+  static const int sms = [] {
+    int dev = 0, n = 0;
     cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
-  }
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 148;
+  }();
   const long long cols = (long long)((g.px + tx - 1) / tx) * ((g.py + ty - 1) / ty);
   const long long wave = (long long)sms * per_sm;
-  int best = 1;
+  int best = 0;
   long long best_cost = -1;
-  for (int k = 1; k <= 128; ++k) {
+  for (int k = kz > 0 ? kz : 1; k <= (kz > 0 ? kz : g.pz); ++k) {
     const long long blocks = cols * ((g.pz + k - 1) / k);
-    const long long cost = (blocks + wave - 1) / wave * (k + 4);
-    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = k; }
+    const long long c = (blocks + wave - 1) / wave * (std::min(k, g.pz) + 4);
+    if (best_cost < 0 || c < best_cost) { best_cost = c; best = k; }
   }
+  if (cost) *cost = best_cost;
   return best;
 }
 template <typename T>

@@ -850,8 +850,7 @@ ep_status ep_net_create(int ndim, int in_ch, int out_ch, int base, int levels, u
   u.D = ndim; u.cin = in_ch; u.cout = out_ch; u.base = base; u.levels = levels;
   u.st = (cudaStream_t)stream;
   unet_layers(u);
-  static const cudaError_t cfg = conv32_configure();
-  if (cfg != cudaSuccess) {
+  if (conv32_configure() != cudaSuccess || conv_tc_configure() != cudaSuccess) {
     delete n;
     return nfail(nullptr, EP_ERR_CUDA, "ep_net_create: convolution kernels' shared-memory attribute");
   }

@@ -47,6 +47,7 @@ def _fields(P, nd, n, seed):
 
 
 def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
+    opts = dict(opts)
     g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=precision)
     rng = np.random.default_rng(1)
     g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, 1.5e-3 * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
@@ -89,6 +90,16 @@ def test_register_sweep_matches_the_staged_sweep_at_tile_edges_fp32(P, n, kz):
     f = _fields(P, 3, n, 7)
     iref, ref = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f)
     info, out = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_FUSED_REG, iters, f, shape=kz)
+    _compare(f, out, ref, info, iref, iters, EPS32)
+
+
+@pytest.mark.parametrize("n", [(27, 11, 5), (28, 12, 6), (29, 13, 7), (57, 25, 12), (90, 64, 21)])
+@pytest.mark.parametrize("mu_s", [math.inf, 1e-3])
+def test_register_sweep_with_a_per_cell_modulus_matches_the_staged_sweep_fp32(P, n, mu_s):
+    iters = 20
+    f = _fields(P, 3, n, 8)
+    iref, ref = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f, cell_g=1.0, mu_s=mu_s)
+    info, out = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_AUTO, iters, f, cell_g=1.0, mu_s=mu_s)
     _compare(f, out, ref, info, iref, iters, EPS32)
 
 

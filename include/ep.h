@@ -225,8 +225,8 @@ ep_status ep_set_fields(ep_handle h, int field, const double *host_in, size_t co
  * shape (< 0 keeps the current): in 3D the z-planes per block of the fused
  * kernels (0, the default: chosen from the grid size so that the launch
  * fills every SM); in 2D the tile of the fused kernel (0: 32x8, 1: 32x16,
- * 2: 64x8 cells in shared memory; 3, 4: one warp per strip of 28 columns
- * marching 64 / 32 rows with its row history in registers). */
+ * 2: 64x8 cells in shared memory; 3, 4: one warp per strip of 60 (FP32) or
+ * 28 (FP64) columns marching 64 / 32 rows with its row history in registers). */
 enum { EP_KERNEL_AUTO = -1, EP_KERNEL_STAGED = 0, EP_KERNEL_FUSED = 1, EP_KERNEL_FUSED_TMA = 2, EP_KERNEL_FUSED_REG = 3 };
 ep_status ep_set_kernel(ep_handle h, int variant, int shape);
 

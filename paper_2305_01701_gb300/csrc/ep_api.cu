@@ -384,11 +384,12 @@ Inst2<T> make_inst(ep_grid *h, DevInfo *di) {
 }
 
 // (instance, tile_x, tile_y) work items covering the padded box of a grid
-void append_items(std::vector<int4> &v, int inst, const Geo &g, int tile) {
+void append_items(std::vector<int4> &v, int inst, const Geo &g, int tile, size_t elem) {
   int tx, ty;
-  fused2d_tile(tile, &tx, &ty);
+  fused2d_tile(tile, elem, &tx, &ty);
+  // the written columns are 0 .. nx: the row's padding stays zero
   for (int j = 0; j < (g.py + ty - 1) / ty; ++j)
-    for (int i = 0; i < (g.px + tx - 1) / tx; ++i) v.push_back(make_int4(inst, i, j, 0));
+    for (int i = 0; i < (g.nx + tx) / tx; ++i) v.push_back(make_int4(inst, i, j, 0));
 }
 
 template <typename T>
@@ -404,7 +405,7 @@ ep_status prepare_solo2d(ep_grid *h) {
   CK(h, cudaMemcpyAsync(h->inst_dev, &I, sizeof(I), cudaMemcpyHostToDevice, h->stream));
   if (h->items_tile != h->tile) {
     std::vector<int4> it;
-    append_items(it, 0, h->g, h->tile);
+    append_items(it, 0, h->g, h->tile, sizeof(T));
     if ((int)it.size() > h->max_items) return fail(h, EP_ERR_ARG, "work-item list larger than reserved");
     CK(h, cudaMemcpyAsync(h->items_dev, it.data(), it.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
     h->n_items = (int)it.size();
@@ -1444,7 +1445,7 @@ ep_status batch_upload(ep_batch *b) {
   std::vector<int4> items;
   for (int q = 0; q < b->count; ++q) {
     I[q] = make_inst<T>(b->g[q], b->dinfo + q);
-    append_items(items, q, b->g[q]->g, b->tile);
+    append_items(items, q, b->g[q]->g, b->tile, sizeof(T));
   }
   if (b->items) cudaFree(b->items);
   b->items = nullptr;

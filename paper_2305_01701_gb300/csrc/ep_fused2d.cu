@@ -267,9 +267,9 @@ void launch_fused2d(int tile, const Inst2<T> *insts, const int4 *items, int n_it
   }
 }
 
-void fused2d_tile(int tile, int *tx, int *ty) {
-  if (tile >= 3) {   // warp strips: 28 written columns, 64 or 32 rows
-    *tx = 28;
+void fused2d_tile(int tile, size_t elem, int *tx, int *ty) {
+  if (tile >= 3) {   // warp strips: 64 or 32 rows
+    *tx = fused2d_strip_columns(elem);
     *ty = tile == 3 ? 64 : 32;
     return;
   }
@@ -313,7 +313,7 @@ void launch_check_batch(const Inst2<T> *insts, int n, cudaStream_t st) {
 
 template <typename T>
 int fused2d_blocks_per_sm(int tile) {
-  if (tile >= 3) return fused2d_strip_blocks_per_sm<T>(tile == 3 ? 64 : 32);
+  if (tile >= 3) return fused2d_strip_blocks_per_sm<T>();
   int nb = 0;
   cudaError_t e;
   if (tile == 0)

@@ -67,6 +67,7 @@
 #include <type_traits>
 
 #include "ep_internal.cuh"
+#include "ep_lanes.cuh"
 
 namespace ep {
 
@@ -91,58 +92,12 @@ struct LaneD {
   static constexpr int N = 1, LPR = 32, H = 8;
 };
 
-template <typename V>
-struct Splat;
-template <>
-struct Splat<float2> {
-  static __device__ __forceinline__ float2 of(float s) { return make_float2(s, s); }
-};
-template <>
-struct Splat<double> {
-  static __device__ __forceinline__ double of(double s) { return s; }
-};
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
-__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
-__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
-// value of the column left / right of each column (a row's first column has
-// no left neighbour and gets an arbitrary value, the last no right one)
-__device__ __forceinline__ float2 xm(float2 v) { return make_float2(__shfl_up_sync(FULL, v.y, 1, 16), v.x); }
-__device__ __forceinline__ float2 xp(float2 v) { return make_float2(v.y, __shfl_down_sync(FULL, v.x, 1, 16)); }
-__device__ __forceinline__ double xm(double v) { return __shfl_up_sync(FULL, v, 1); }
-__device__ __forceinline__ double xp(double v) { return __shfl_down_sync(FULL, v, 1); }
-template <int E>
-__device__ __forceinline__ float el(float2 v) { return E == 0 ? v.x : v.y; }
-template <int E>
-__device__ __forceinline__ double el(double v) { return v; }
-
 // v off the domain's boundary, 0 on it: m holds 1 or 0 per column.  INT
 // windows have no boundary columns.
 template <bool INT, typename V>
 __device__ __forceinline__ V keep(V m, V v) {
   return INT ? v : vmul(m, v);
 }
-
-// centre scale min(1, Y / sqrt(J2)).  FP32: compare squares and scale with
-// the reciprocal square root only where the return acts (most cells stay
-// elastic).
-__device__ __forceinline__ float scale_of(float J2, float Y) {
-  Y = Y > 0.f ? Y : 0.f;
-  return J2 > Y * Y ? Y * rsqrtf(J2) : 1.f;
-}
-__device__ __forceinline__ double scale_of(double J2, double Y) {
-  Y = Y > 0.0 ? Y : 0.0;
-  const double sj = sqrt(J2);
-  return sj > Y ? Y / sj : 1.0;
-}
-__device__ __forceinline__ float2 vscale(float2 J2, float2 Y) {
-  return make_float2(scale_of(J2.x, Y.x), scale_of(J2.y, Y.y));
-}
-__device__ __forceinline__ double vscale(double J2, double Y) { return scale_of(J2, Y); }
 
 // One plane slot of a value per thread, as rows of the window
 template <typename L>
@@ -389,7 +344,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
     // sums of inputs: A = rq0 over planes t-1, t; D = rq2, I = rd0, J = rd1
     // over columns x-1, x; K = rd1 - rd0
     const V rd0 = own(I_RD0), rd1 = own(I_RD1);
-    const V vA = vadd(rq0_1, rq0), D = vadd(rq2, xm(rq2)), vI = vadd(rd0, xm(rd0)), J = vadd(rd1, xm(rd1));
+    const V vA = vadd(rq0_1, rq0), D = vadd(rq2, xm<LPR>(rq2)), vI = vadd(rd0, xm<LPR>(rd0)), J = vadd(rd1, xm<LPR>(rd1));
     const V vK = vsub(rd1, rd0);
     S.A.r[q0] = vA; S.D.r[q0] = D; S.I.r[q0] = vI; S.K.r[q0] = vK;
     if constexpr (CHK) {   // the snapshot values checked at this plane: levels t-1 (centres, edges), t-2 (faces)
@@ -413,10 +368,10 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
     V gxy, wxy, gxz, wxz, gyz, wyz;
     {
       const V u0_ym = below(I_U0), u2_ym = below(I_U2);
-      V x = vmul(vsub(u0, u0_ym), bc(rdy)), y = vsub(u1, xm(u1));
+      V x = vmul(vsub(u0, u0_ym), bc(rdy)), y = vsub(u1, xm<LPR>(u1));
       gxy = vfma(y, bc(rdx), x);
       wxy = keep<INT>(m_xy, vfma(y, bc(-rdx), x));
-      x = vmul(vsub(u0, u0_1), bc(rdz)); y = vsub(u2, xm(u2));
+      x = vmul(vsub(u0, u0_1), bc(rdz)); y = vsub(u2, xm<LPR>(u2));
       gxz = vfma(y, bc(rdx), x);
       wxz = keep<INT>(m_xz, vfma(y, bc(-rdx), x));
       x = vmul(vsub(u1, u1_1), bc(rdz)); y = vsub(u2, u2_ym);
@@ -428,7 +383,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
     // rotation products (2 rq omega) and the pair sums that their means and
     // the spin means share
     const V pxy = vmul(rq0, wxy), pxz = vmul(rq1, wxz), pyz = vmul(rq2, wyz);
-    const V vB = vadd(wxy_1, wxy), vE = vadd(wyz, xm(wyz)), vM = vadd(pxy, xp(pxy)), vN = vadd(pxz, xp(pxz));
+    const V vB = vadd(wxy_1, wxy), vE = vadd(wyz, xm<LPR>(wyz)), vM = vadd(pxy, xp<LPR>(pxy)), vN = vadd(pxz, xp<LPR>(pxz));
     S.B.r[q0] = vB; S.E.r[q0] = vE; S.wxz.r[q0] = wxz; S.M.r[q0] = vM; S.pyz.r[q0] = pyz;
     __syncthreads();
 
@@ -455,8 +410,8 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
         tsxz = keep<INT>(m_xz, vfma(own(I_SOXZ), bc(bt), vmul(tr, bc(ob))));
       }
       {   // yz: w dzy - (Txy Wxz + Txz Wxy) / 4
-        const V Dz = vadd(L_1, Lz), Txy = vadd(vA, xp(vA)), Wxy = vadd(vB, xp(vB));
-        const V Txz = vadd(F, xp(F)), Wxz = vadd(G, xp(G));
+        const V Dz = vadd(L_1, Lz), Txy = vadd(vA, xp<LPR>(vA)), Wxy = vadd(vB, xp<LPR>(vB));
+        const V Txz = vadd(F, xp<LPR>(F)), Wxz = vadd(G, xp<LPR>(G));
         const V r1 = vfma(Txz, Wxy, vmul(Txy, Wxz));
         const V r = vfma(r1, bc(-qr), vmul(wyz, Dz));
         const V tr = trial(r, e8, gyz, I_TBYZ, I_GEYZ);
@@ -480,7 +435,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
         }
       }
       {   // centres of plane t-1
-        const V e0 = vmul(vsub(xp(u0_1), u0_1), bc(rdx));
+        const V e0 = vmul(vsub(xp<LPR>(u0_1), u0_1), bc(rdx));
         const V e1 = e1_1;
         const V e2 = vmul(vsub(u2, u2_1), bc(rdz));
         div = vadd(vadd(e0, e1), e2);
@@ -507,7 +462,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
       }
       D_1 = D; E_1 = vE; F_1 = F; G_1 = G; J_1 = J; L_1 = Lz;
     }
-    const V vQ = vadd(tsxy, xp(tsxy)), vS = vadd(tsyz_1, tsyz);
+    const V vQ = vadd(tsxy, xp<LPR>(tsxy)), vS = vadd(tsyz_1, tsyz);
     S.Q.r[q0] = vQ; S.Sz.r[q0] = vS;
     __syncthreads();
 
@@ -521,7 +476,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
     {
       const V pr = vfma(sop, bc(bp), vmul(vfma(div, bc(-KDt), pb), bc(obp)));
       const V R = vadd(tsxz_1, tsxz);
-      const V xy = vadd(vQ, S.Q.r[qp]), xz = vadd(R, xp(R)), yz = vadd(vS, S.Sz.r[qp]);
+      const V xy = vadd(vQ, S.Q.r[qp]), xz = vadd(R, xp<LPR>(R)), yz = vadd(vS, S.Sz.r[qp]);
       const V j4 = vfma(yz, yz, vfma(xz, xz, vmul(xy, xy)));        // 16 x the shear part
       const V jn = vfma(c2v, c2v, vfma(c1v, c1v, vmul(c0v, c0v)));  // 2 x the normal part
       const V J2 = vfma(j4, bc((T)0.0625), vmul(jn, bc((T)0.5)));
@@ -558,7 +513,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
       }
       s_1 = vmul(sc1, bc(qr));
     }
-    const V vU = vadd(s_1, xm(s_1)), vV = vadd(s_2, s_1);   // quarter scales over x-1, x / planes t-2, t-1
+    const V vU = vadd(s_1, xm<LPR>(s_1)), vV = vadd(s_2, s_1);   // quarter scales over x-1, x / planes t-2, t-1
     S.U.r[q0] = vU; S.Vs.r[q0] = vV; S.syy[sl1].r[q0] = syy_1;
     if (t + 1 < ke + 2) {   // plane t + 1 is needed next
       if (!arrived(sl1, t + 2 < ke + 2)) return false;
@@ -599,7 +554,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
     // ---- 5. residual and velocity update of plane t-2 ----
     if (w_vel) {
       const int lu = t - 2;
-      const V sxx_2_xm = xm(sxx_2), nxy_2_xp = xp(nxy_2), nxz_2_xp = xp(nxz_2);
+      const V sxx_2_xm = xm<LPR>(sxx_2), nxy_2_xp = xp<LPR>(nxy_2), nxz_2_xp = xp<LPR>(nxz_2);
       if (out_col && lu >= kb && lu < ke) {
         const V nxy_2_yp = S.nxy[sl].r[qp], syy_2_ym = S.syy[sl].r[qm];
         const V nyz_2_yp = S.nyz[sl].r[qp];

@@ -176,14 +176,15 @@ __device__ __forceinline__ void check_one(DevInfo *di, const Scal *sc) {
 
 // ---- batched fused 2D sweep (ep_fused2d.cu, ep_fused2d_strip.cu) ---------
 // tile: 0 = 32x8, 1 = 32x16, 2 = 64x8 cells (block tiles in shared memory);
-// 3, 4 = warp strips of 28 columns marching 64 / 32 rows
+// 3, 4 = warp strips of 60 (FP32) or 28 (FP64) columns marching 64 / 32 rows
 constexpr int FUSED2D_TILES = 5;
-inline int fused2d_items_per_block(int tile) { return tile >= 3 ? 8 : 1; }
+inline int fused2d_items_per_block(int tile) { return tile >= 3 ? 4 : 1; }   // warps of a strip block
+int fused2d_strip_columns(size_t elem);
 template <typename T>
 void launch_fused2d_strip(int seg, const Inst2<T> *insts, const int4 *items, int n_items, int b, int check,
                           int blocks, cudaStream_t st);
 template <typename T>
-int fused2d_strip_blocks_per_sm(int seg);
+int fused2d_strip_blocks_per_sm();
 template <typename T>
 void launch_fused2d(int tile, const Inst2<T> *insts, const int4 *items, int n_items, int b, int check, int blocks,
                     cudaStream_t st);
@@ -191,7 +192,7 @@ template <typename T>
 void launch_check_batch(const Inst2<T> *insts, int n, cudaStream_t st);
 template <typename T>
 void launch_init_batch(const Inst2<T> *insts, int n, long long max_iter, cudaStream_t st);
-void fused2d_tile(int tile, int *tx, int *ty);
+void fused2d_tile(int tile, size_t elem, int *tx, int *ty);
 cudaError_t fused2d_configure();
 template <typename T>
 int fused2d_blocks_per_sm(int tile);

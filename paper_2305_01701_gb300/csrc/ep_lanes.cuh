@@ -1,0 +1,67 @@
+// ep_lanes.cuh -- the columns of one thread of a marching sweep kernel: two
+// adjacent FP32 columns as a float2 (packed arithmetic, one instruction per
+// pair), or one FP64 column.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace ep {
+
+template <typename V>
+struct Splat;
+template <>
+struct Splat<float2> {
+  static __device__ __forceinline__ float2 of(float s) { return make_float2(s, s); }
+};
+template <>
+struct Splat<double> {
+  static __device__ __forceinline__ double of(double s) { return s; }
+};
+
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+
+// value of the column left / right of each column, W threads per row (a row's
+// first column has no left neighbour and gets an arbitrary value, the last no
+// right one)
+template <int W>
+__device__ __forceinline__ float2 xm(float2 v) { return make_float2(__shfl_up_sync(0xffffffffu, v.y, 1, W), v.x); }
+template <int W>
+__device__ __forceinline__ float2 xp(float2 v) { return make_float2(v.y, __shfl_down_sync(0xffffffffu, v.x, 1, W)); }
+template <int W>
+__device__ __forceinline__ double xm(double v) { return __shfl_up_sync(0xffffffffu, v, 1, W); }
+template <int W>
+__device__ __forceinline__ double xp(double v) { return __shfl_down_sync(0xffffffffu, v, 1, W); }
+
+// column E of a value
+template <int E>
+__device__ __forceinline__ float el(float2 v) { return E == 0 ? v.x : v.y; }
+template <int E>
+__device__ __forceinline__ double el(double v) { return v; }
+
+// centre scale min(1, Y / sqrt(J2)).  FP32: compare squares and scale with
+// the reciprocal square root only where the return acts (most cells stay
+// elastic).  FP64: below Y^2 by more than the rounding of both, sqrt(J2) > Y
+// cannot hold and the scale is 1 without the root.
+__device__ __forceinline__ float scale_of(float J2, float Y) {
+  Y = Y > 0.f ? Y : 0.f;
+  return J2 > Y * Y ? Y * rsqrtf(J2) : 1.f;
+}
+__device__ __forceinline__ double scale_of(double J2, double Y) {
+  Y = Y > 0.0 ? Y : 0.0;
+  if (J2 < Y * Y * (1.0 - 1e-15)) return 1.0;
+  const double sj = sqrt(J2);
+  return sj > Y ? Y / sj : 1.0;
+}
+__device__ __forceinline__ float2 vscale(float2 J2, float2 Y) {
+  return make_float2(scale_of(J2.x, Y.x), scale_of(J2.y, Y.y));
+}
+__device__ __forceinline__ double vscale(double J2, double Y) { return scale_of(J2, Y); }
+
+}  // namespace ep

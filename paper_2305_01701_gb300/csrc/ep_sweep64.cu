@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "ep_internal.cuh"
+#include "ep_lanes.cuh"
 
 namespace ep {
 
@@ -48,15 +49,6 @@ __device__ __forceinline__ void block_max(double v, unsigned long long *slot) {
 }
 
 __device__ __forceinline__ bool skip(const DevInfo *di) { return di != nullptr && *(volatile const int *)&di->done != 0; }
-
-// centre scale min(1, Y / sqrt(J2)).  Below Y^2 by more than the rounding of
-// both, sqrt(J2) > Y cannot hold and the scale is 1 without the root.
-__device__ __forceinline__ double return_scale(double J2, double Y) {
-  Y = Y > 0.0 ? Y : 0.0;
-  if (J2 < Y * Y * (1.0 - 1e-15)) return 1.0;
-  const double sj = sqrt(J2);
-  return sj > Y ? Y / sj : 1.0;
-}
 
 struct Pt {
   int i, j, k;
@@ -170,7 +162,7 @@ __global__ void __launch_bounds__(256) k64_centres(Geo g, Stage<double> S, const
     if (frozen) {
       s = S.s[e];   // frozen plasticity: the held scale (Sec. 3.3)
     } else {
-      s = return_scale(fma(0.0625, j4, 0.5 * jn), fma(sc->A, p, S.yc[e]));
+      s = scale_of(fma(0.0625, j4, 0.5 * jn), fma(sc->A, p, S.yc[e]));
       S.s[e] = s;
     }
     S.snp[e] = p;

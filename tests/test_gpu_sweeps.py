@@ -124,3 +124,14 @@ def test_fp64_sweep_3d_matches_the_register_sweep_at_warp_edges(P, n, opts):
     iref, ref = _solve(P, 3, n, P.FP64, P.KERNEL_FUSED_REG, iters, f, shape=0, **opts)
     info, out = _solve(P, 3, n, P.FP64, P.KERNEL_STAGED, iters, f, **opts)
     _compare(f, out, ref, info, iref, iters, 2.0 ** -53)
+
+
+@pytest.mark.parametrize("n", [(58, 31), (59, 32), (60, 33), (61, 63), (119, 64), (120, 65), (121, 3)])
+@pytest.mark.parametrize("tile", [3, 4])
+@pytest.mark.parametrize("opts", [{}, {"mu_s": 1e-3, "jaumann": False}, {"freeze_iter": 5}])
+def test_batched_strips_of_column_pairs_match_the_staged_sweep_fp32(P, n, tile, opts):
+    iters = 20
+    f = _fields(P, 2, n, 9)
+    iref, ref = _solve(P, 2, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f, **opts)
+    info, out = _solve(P, 2, n, P.FP32_MIXED, P.KERNEL_FUSED, iters, f, shape=tile, **opts)
+    _compare(f, out, ref, info, iref, iters, EPS32)

@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <string>
+#include <initializer_list>
 #include <vector>
 
 #include "ep_internal.cuh"
@@ -464,14 +465,12 @@ WarmScales warm_scales(const ep_grid *h) {
   return w;
 }
 
-template <typename Td>
-ep_status copy_into(ep_grid *h, void *dst, const double *src) {
-  if (sizeof(Td) == 8) {
-    CK(h, cudaMemcpyAsync(dst, src, h->g.box * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-  } else {
-    launch_convert<float, double>((float *)dst, src, h->g.box, h->stream);
-  }
-  return EP_OK;
+// entry of a fill table: src (null: zeros) to up to four arrays
+void fill_to(FillTab &F, const double *src, std::initializer_list<void *> dst) {
+  FillTab::Entry &E = F.e[F.count++];
+  E.src = src;
+  int q = 0;
+  for (void *d : dst) E.dst[q++] = d;
 }
 
 // Start of an increment: start velocity, rotation weights, the physical
@@ -487,11 +486,12 @@ ep_status prologue(ep_grid *h, const double *const dv[3]) {
     // Tn64 / Ts64 / stp64 are free here (dv was consumed above)
     const int nd = h->ndim, ns = n_shear(nd);
     launch_advect(g, h->H, h->dscal, h->Tn64, h->Ts64, h->stp64, st);
-    for (int d = 0; d < nd; ++d)
-      CK(h, cudaMemcpyAsync(h->H.tn[d], h->Tn64[d], g.box * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    for (int c = 0; c < ns; ++c)
-      CK(h, cudaMemcpyAsync(h->H.ts[c], h->Ts64[c], g.box * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    CK(h, cudaMemcpyAsync(h->H.p, h->stp64, g.box * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    CopyTab C{};
+    const long long n16 = g.box / 2;
+    for (int d = 0; d < nd; ++d) C.e[C.count++] = {h->Tn64[d], h->H.tn[d], n16};
+    for (int c = 0; c < ns; ++c) C.e[C.count++] = {h->Ts64[c], h->H.ts[c], n16};
+    C.e[C.count++] = {h->stp64, h->H.p, n16};
+    launch_copy_table(C, st);
     h->adv_done = h->n_commits;
   }
   launch_rotation_fields<double>(g, h->H, h->dscal, h->rq64, h->rd64, h->yc64, st);
@@ -507,42 +507,37 @@ ep_status prologue(ep_grid *h, const double *const dv[3]) {
     launch_warm_stress(g, h->wy, h->wcoarse, 1.0 / warm_scales(h).st_inv, h->stn64, h->sts64, dims, st);
   }
   CK(h, cudaGetLastError());
-  // sweep constants: base trial tau_tr(v0), base pressure p(v0), weights
+  // sweep constants and the first state, in the sweep's type: base trial
+  // tau_tr(v0), base pressure p(v0), weights; one launch (up to 45 arrays from
+  // 24 entries; 127^3: 280 -> 99 us, a 64^2 grid's apply 154 -> 60 us)
   const int nd = h->ndim, ns = n_shear(nd);
+  FillTab F{};
   for (int d = 0; d < nd; ++d) {
-    if (copy_into<T>(h, h->tbn[d], h->Tn64[d]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->stn[0][d], h->stn64[d]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->stn[1][d], h->stn64[d]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->cn[d], h->stn64[d]) != EP_OK) return EP_ERR_CUDA;
-    CK(h, cudaMemsetAsync(h->u[0][d], 0, g.box * sizeof(T), st));
-    CK(h, cudaMemsetAsync(h->u[1][d], 0, g.box * sizeof(T), st));
-    CK(h, cudaMemsetAsync(h->uchk[d], 0, g.box * sizeof(T), st));
+    fill_to(F, h->Tn64[d], {h->tbn[d]});
+    fill_to(F, h->stn64[d], {h->stn[0][d], h->stn[1][d], h->cn[d]});
+    fill_to(F, nullptr, {h->u[0][d], h->u[1][d], h->uchk[d]});
   }
   for (int c = 0; c < ns; ++c) {
-    if (copy_into<T>(h, h->tbs[c], h->Ts64[c]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->sts[0][c], h->sts64[c]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->sts[1][c], h->sts64[c]) != EP_OK) return EP_ERR_CUDA;
-    if (copy_into<T>(h, h->cs[c], h->sts64[c]) != EP_OK) return EP_ERR_CUDA;
-    if (sizeof(T) == 4 && copy_into<T>(h, h->rq[c], h->rq64[c]) != EP_OK) return EP_ERR_CUDA;
+    fill_to(F, h->Ts64[c], {h->tbs[c]});
+    fill_to(F, h->sts64[c], {h->sts[0][c], h->sts[1][c], h->cs[c]});
+    if (sizeof(T) == 4) fill_to(F, h->rq64[c], {h->rq[c]});
   }
   if (h->opts.incompressible) {
     // base pressure step of the incompressible sweep: -K~ div v0 (es64 is
     // free after the start stage); the state starts at p_hat
     const double *v0[3] = {h->H.v0[0], h->H.v0[1], h->H.v0[2]};
     launch_scaled_div(g, v0, -make_scal(h).KDt, h->es64[0], st);
-    if (copy_into<T>(h, h->pb, h->es64[0]) != EP_OK) return EP_ERR_CUDA;
-  } else if (copy_into<T>(h, h->pb, h->stp64) != EP_OK) {
-    return EP_ERR_CUDA;
+    fill_to(F, h->es64[0], {h->pb});
+  } else {
+    fill_to(F, h->stp64, {h->pb});
   }
-  if (copy_into<T>(h, h->stp[0], h->stp64) != EP_OK) return EP_ERR_CUDA;
-  if (copy_into<T>(h, h->stp[1], h->stp64) != EP_OK) return EP_ERR_CUDA;
-  if (copy_into<T>(h, h->cp, h->stp64) != EP_OK) return EP_ERR_CUDA;
+  fill_to(F, h->stp64, {h->stp[0], h->stp[1], h->cp});
   if (sizeof(T) == 4) {
-    if (copy_into<T>(h, h->yc, h->yc64) != EP_OK) return EP_ERR_CUDA;
-    for (int r = 0; r < nd - 1; ++r)
-      if (copy_into<T>(h, h->rd[r], h->rd64[r]) != EP_OK) return EP_ERR_CUDA;
+    fill_to(F, h->yc64, {h->yc});
+    for (int r = 0; r < nd - 1; ++r) fill_to(F, h->rd64[r], {h->rd[r]});
   }
-  if (copy_into<T>(h, h->s, h->s64) != EP_OK) return EP_ERR_CUDA;
+  fill_to(F, h->s64, {h->s});
+  launch_fill<T>(F, g.box, st);
   if (nd == 2 && !h->Gc) {
     launch_rotation_mean2d<T>(g, P<T>(h->rd[0]), P<T>(h->om[0]), st);
   } else if (sizeof(T) == 8 && !h->Gc) {
@@ -667,18 +662,18 @@ ep_status commit(ep_grid *h) {
   const Geo &g = h->g;
   cudaStream_t st = h->stream;
   const T *uf[3] = {P<T>(h->u[0][0]), P<T>(h->u[0][1]), P<T>(h->u[0][2])};
-  for (int d = 0; d < h->ndim; ++d)
-    CK(h, cudaMemcpyAsync(h->vpp[d], h->H.v[d], g.box * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  launch_compose<T>(g, h->H.v0, uf, h->H.v, st);
+  launch_compose<T>(g, h->H.v0, uf, h->H.v, h->vpp, st);
   Stage<double> S = phys_stage(h, h->H.v);
   launch_strain<double>(g, S, h->dscal, nullptr, st);
-  launch_trial<double>(g, S, h->dscal, nullptr, st);
   if (h->wrecord && h->w0) {
+    launch_trial<double>(g, S, h->dscal, nullptr, st);
     // the physical response of the converged velocity with the old history
     // (warm-start training targets); the trial stays in Tn64 / Ts64
     launch_return_centres<double>(g, S, h->dscal, nullptr, 0, st);
     launch_return_edges<double>(g, S, h->dscal, nullptr, 0, st);
     launch_warm_record(g, h->stn64, h->sts64, h->w0, st);
+  } else {
+    launch_trial_near<T>(g, S, h->dscal, P<T>(h->s), st);   // what k_commit reads of it
   }
   CK(h, cudaMemsetAsync(h->dnpl, 0, sizeof(unsigned long long), st));
   const T *stn[3] = {P<T>(h->stn[1][0]), P<T>(h->stn[1][1]), P<T>(h->stn[1][2])};
@@ -1263,9 +1258,11 @@ ep_status ep_snapshot(ep_handle h) {
   // plus the last return scale (sweep type), a feature of the warm start
   const size_t ns = h->g.box * (h->prec == EP_FP64 ? sizeof(double) : sizeof(float));
   if (!h->snap) CK(h, cudaMalloc((void **)&h->snap, nb * arr.size() + ns));
-  for (size_t q = 0; q < arr.size(); ++q)
-    CK(h, cudaMemcpyAsync(h->snap + q * nb, arr[q], nb, cudaMemcpyDeviceToDevice, h->stream));
-  CK(h, cudaMemcpyAsync(h->snap + arr.size() * nb, h->s, ns, cudaMemcpyDeviceToDevice, h->stream));
+  CopyTab C{};
+  for (size_t q = 0; q < arr.size(); ++q) C.e[C.count++] = {arr[q], h->snap + q * nb, (long long)(nb / 16)};
+  C.e[C.count++] = {h->s, h->snap + arr.size() * nb, (long long)(ns / 16)};
+  launch_copy_table(C, h->stream);
+  CK(h, cudaGetLastError());
   CK(h, cudaStreamSynchronize(h->stream));
   h->snap_started = h->started;
   h->snap_commits = h->n_commits;
@@ -1279,9 +1276,11 @@ ep_status ep_restore(ep_handle h) {
   auto arr = history_arrays(h);
   const size_t nb = h->g.box * sizeof(double);
   const size_t ns = h->g.box * (h->prec == EP_FP64 ? sizeof(double) : sizeof(float));
-  for (size_t q = 0; q < arr.size(); ++q)
-    CK(h, cudaMemcpyAsync(arr[q], h->snap + q * nb, nb, cudaMemcpyDeviceToDevice, h->stream));
-  CK(h, cudaMemcpyAsync(h->s, h->snap + arr.size() * nb, ns, cudaMemcpyDeviceToDevice, h->stream));
+  CopyTab C{};
+  for (size_t q = 0; q < arr.size(); ++q) C.e[C.count++] = {h->snap + q * nb, arr[q], (long long)(nb / 16)};
+  C.e[C.count++] = {h->snap + arr.size() * nb, h->s, (long long)(ns / 16)};
+  launch_copy_table(C, h->stream);
+  CK(h, cudaGetLastError());
   CK(h, cudaStreamSynchronize(h->stream));
   h->started = h->snap_started;
   h->n_commits = h->snap_commits;

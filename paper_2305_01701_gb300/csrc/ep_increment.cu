@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include "ep_internal.cuh"
+#include "ep_lanes.cuh"
 
 namespace ep {
 
@@ -51,11 +52,12 @@ __global__ void k_start_velocity(Geo g, History H, const double *dv0, const doub
   const double L[3] = {Lx, Ly, Lz};
   const double h[3] = {g.dx, g.dy, g.dz};
   const int c[3] = {q.i, q.j, q.k};
-  for (int d = 0; d < g.ndim; ++d) {
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (d >= g.ndim) break;
     double v = 0.0;
     if (face_in(g, d, q.i, q.j, q.k)) {
-      const double vb = sc->rate[d] * (-0.5 * L[d] + c[d] * h[d]);
-      if (face_wall(g, d, q.i, q.j, q.k) || !started) v = vb;
+      if (face_wall(g, d, q.i, q.j, q.k) || !started) v = sc->rate[d] * (-0.5 * L[d] + c[d] * h[d]);
       else v = H.v[d][q.e];
       if (dv[d] && !face_wall(g, d, q.i, q.j, q.k)) v += dv[d][q.e];
     }
@@ -88,19 +90,29 @@ __global__ void k_rotation_fields(Geo g, History H, const Scal *sc, T *rq0, T *r
   }
 }
 
+// o = v0 + u, the velocity that it replaces kept in `prev`
 template <typename T>
 __global__ void k_compose(Geo g, const double *v00, const double *v01, const double *v02, const T *u0,
-                          const T *u1, const T *u2, double *o0, double *o1, double *o2) {
+                          const T *u1, const T *u2, double *o0, double *o1, double *o2, double *prev0,
+                          double *prev1, double *prev2) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= g.box) return;
+  prev0[t] = o0[t];
+  prev1[t] = o1[t];
   o0[t] = v00[t] + (double)u0[t];
   o1[t] = v01[t] + (double)u1[t];
-  if (g.ndim == 3) o2[t] = v02[t] + (double)u2[t];
+  if (g.ndim == 3) {
+    prev2[t] = o2[t];
+    o2[t] = v02[t] + (double)u2[t];
+  }
 }
 
 // History commit.  Tn64/Ts64: physical trial at the converged velocity
-// H.v (already composed); es64: its shear strain rates; stn/sts/stp/s: the
-// converged pseudo-time state and last return scales.
+// H.v (already composed), valid where the return acted; es64: its shear strain
+// rates; stn/sts/stp/s: the converged pseudo-time state and last return scales.
+// The trial and its second invariant are formed at the centres with s < 1 only
+// (127^3, FP32 state: commit 286 -> 119 us, its trial 501 -> 25 us, elastic;
+// both are FP64-pipe bound where every centre yields).
 template <typename T>
 __global__ void k_commit(Geo g, History H, const double *Tn0, const double *Tn1, const double *Tn2,
                          const double *Ts0, const double *Ts1, const double *Ts2, const double *es0,
@@ -115,21 +127,21 @@ __global__ void k_commit(Geo g, History H, const double *Tn0, const double *Tn1,
     const double dt = sc->dt;
     const bool centre = i < nx && j < ny && (g.ndim == 2 || k < nz);
     if (centre) {
-      const double Tn[3] = {Tn0[e], Tn1[e], g.ndim == 3 ? Tn2[e] : 0.0};
       const double tn[3] = {(double)stn0[e], (double)stn1[e], g.ndim == 3 ? (double)stn2[e] : 0.0};
-      double J2 = 0.0;
-      for (int d = 0; d < g.ndim; ++d) J2 += 0.5 * (Tn[d] - tn[d]) * (Tn[d] - tn[d]);
-      double a = 0.25 * ((Ts0[e] - (double)sts0[e]) + (Ts0[e + 1] - (double)sts0[e + 1]) +
-                         (Ts0[e + px] - (double)sts0[e + px]) + (Ts0[e + px + 1] - (double)sts0[e + px + 1]));
-      J2 += a * a;
-      if (g.ndim == 3) {
-        double b = 0.25 * ((Ts1[e] - (double)sts1[e]) + (Ts1[e + 1] - (double)sts1[e + 1]) +
-                           (Ts1[e + pl] - (double)sts1[e + pl]) + (Ts1[e + pl + 1] - (double)sts1[e + pl + 1]));
-        double cc = 0.25 * ((Ts2[e] - (double)sts2[e]) + (Ts2[e + px] - (double)sts2[e + px]) +
-                            (Ts2[e + pl] - (double)sts2[e + pl]) + (Ts2[e + pl + px] - (double)sts2[e + pl + px]));
-        J2 += b * b + cc * cc;
-      }
-      if ((double)s[e] < 1.0) {
+      if (below_one(s[e])) {
+        const double Tn[3] = {Tn0[e], Tn1[e], g.ndim == 3 ? Tn2[e] : 0.0};
+        double J2 = 0.0;
+        for (int d = 0; d < g.ndim; ++d) J2 += 0.5 * (Tn[d] - tn[d]) * (Tn[d] - tn[d]);
+        double a = 0.25 * ((Ts0[e] - (double)sts0[e]) + (Ts0[e + 1] - (double)sts0[e + 1]) +
+                           (Ts0[e + px] - (double)sts0[e + px]) + (Ts0[e + px + 1] - (double)sts0[e + px + 1]));
+        J2 += a * a;
+        if (g.ndim == 3) {
+          double b = 0.25 * ((Ts1[e] - (double)sts1[e]) + (Ts1[e + 1] - (double)sts1[e + 1]) +
+                             (Ts1[e + pl] - (double)sts1[e + pl]) + (Ts1[e + pl + 1] - (double)sts1[e + pl + 1]));
+          double cc = 0.25 * ((Ts2[e] - (double)sts2[e]) + (Ts2[e + px] - (double)sts2[e + px]) +
+                              (Ts2[e + pl] - (double)sts2[e + pl]) + (Ts2[e + pl + px] - (double)sts2[e + pl + px]));
+          J2 += b * b + cc * cc;
+        }
         H.epl[e] += dt * sqrt(J2) / (H.te_c ? H.te_c[e] : sc->two_eta);
         plastic = 1;
       }
@@ -159,6 +171,46 @@ __global__ void k_commit(Geo g, History H, const double *Tn0, const double *Tn1,
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(n_plastic, (unsigned long long)__popc(m));
 }
 
+// One source to up to four arrays of the sweep's type (no source: zeros), every
+// field of an increment's start in one launch: blockIdx.y is the entry.
+template <typename Td>
+__global__ void __launch_bounds__(kThreads) k_fill(FillTab F, long long n) {
+  const FillTab::Entry &E = F.e[blockIdx.y];
+  const long long t = ((long long)blockIdx.x * kThreads + threadIdx.x) * 4;   // n is a multiple of 32
+  if (t >= n) return;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  if (E.src) {
+    const double2 a = *reinterpret_cast<const double2 *>(E.src + t), b = *reinterpret_cast<const double2 *>(E.src + t + 2);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    Td *d = (Td *)E.dst[q];
+    if (!d) break;
+    if constexpr (sizeof(Td) == 4) {
+      *reinterpret_cast<float4 *>(d + t) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+    } else {
+      *reinterpret_cast<double2 *>(d + t) = make_double2(v[0], v[1]);
+      *reinterpret_cast<double2 *>(d + t + 2) = make_double2(v[2], v[3]);
+    }
+  }
+}
+
+// Copies of a table in one launch: blockIdx.y is the entry, 16 KB a block.
+__global__ void __launch_bounds__(kThreads) k_copy_table(CopyTab C) {
+  const CopyTab::Entry &E = C.e[blockIdx.y];
+  const uint4 *s = (const uint4 *)E.src;
+  uint4 *d = (uint4 *)E.dst;
+  const long long t = (long long)blockIdx.x * (4 * kThreads) + threadIdx.x;
+  uint4 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (t + q * kThreads < E.n16) v[q] = s[t + q * kThreads];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (t + q * kThreads < E.n16) d[t + q * kThreads] = v[q];
+}
+
 template <typename Td, typename Ts>
 __global__ void k_convert(Td *dst, const Ts *src, long long n) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -166,26 +218,32 @@ __global__ void k_convert(Td *dst, const Ts *src, long long n) {
 }
 
 // integrated sigma_xx = tau_xx - p along the centre column and the rightmost
-// column (2D: sum over j of dy; 3D: sum over k of dz at j = ny/2)
-__global__ void k_line_integrals(Geo g, History H, double *out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// column (2D: sum over j of dy; 3D: sum over k of dz at j = ny/2): one block,
+// a thread's points in order, then a fixed tree (one thread: 93 us at 255 rows,
+// all of it load latency)
+__global__ void __launch_bounds__(kThreads) k_line_integrals(Geo g, History H, double *out) {
+  __shared__ double sm[2][kThreads / 32];
   const int ic = g.nx / 2, ir = g.nx - 1, jc = g.ny / 2;
-  double a = 0.0, b = 0.0;
-  if (g.ndim == 2) {
-    for (int j = 0; j < g.ny; ++j) {
-      long long ec = g.idx(ic, j, 0), er = g.idx(ir, j, 0);
-      a += (H.tn[0][ec] - H.p[ec]) * g.dy;
-      b += (H.tn[0][er] - H.p[er]) * g.dy;
-    }
-  } else {
-    for (int k = 0; k < g.nz; ++k) {
-      long long ec = g.idx(ic, jc, k), er = g.idx(ir, jc, k);
-      a += (H.tn[0][ec] - H.p[ec]) * g.dz;
-      b += (H.tn[0][er] - H.p[er]) * g.dz;
-    }
+  const int n = g.ndim == 2 ? g.ny : g.nz;
+  const double h = g.ndim == 2 ? g.dy : g.dz;
+  double v[2] = {0.0, 0.0};
+  for (int q = threadIdx.x; q < n; q += kThreads) {
+    const int j = g.ndim == 2 ? q : jc, k = g.ndim == 2 ? 0 : q;
+    const long long ec = g.idx(ic, j, k), er = g.idx(ir, j, k);
+    v[0] += (H.tn[0][ec] - H.p[ec]) * h;
+    v[1] += (H.tn[0][er] - H.p[er]) * h;
   }
-  out[0] = a;
-  out[1] = b;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+    if ((threadIdx.x & 31) == 0) sm[c][threadIdx.x >> 5] = v[c];
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double a = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) a += sm[threadIdx.x][w];
+    out[threadIdx.x] = a;
+  }
 }
 
 __global__ void k_pack(const double *box, double *dst, int ex, int ey, int ez, int px, int py) {
@@ -359,9 +417,9 @@ void launch_rotation_fields(const Geo &g, const History &H, const Scal *sc, T *c
 
 template <typename T>
 void launch_compose(const Geo &g, const double *const v0[3], const T *const u[3], double *const out[3],
-                    cudaStream_t st) {
+                    double *const prev[3], cudaStream_t st) {
   k_compose<T><<<blocks_for(g.box), kThreads, 0, st>>>(g, v0[0], v0[1], v0[2], u[0], u[1], u[2], out[0], out[1],
-                                                       out[2]);
+                                                       out[2], prev[0], prev[1], prev[2]);
 }
 
 template <typename T>
@@ -378,8 +436,19 @@ void launch_convert(Td *dst, const Ts *src, long long n, cudaStream_t st) {
   k_convert<Td, Ts><<<blocks_for(n), kThreads, 0, st>>>(dst, src, n);
 }
 
+template <typename Td>
+void launch_fill(const FillTab &F, long long n, cudaStream_t st) {
+  if (F.count) k_fill<Td><<<dim3(blocks_for(n / 4), F.count), kThreads, 0, st>>>(F, n);
+}
+
+void launch_copy_table(const CopyTab &C, cudaStream_t st) {
+  long long n = 0;
+  for (int q = 0; q < C.count; ++q) n = C.e[q].n16 > n ? C.e[q].n16 : n;
+  if (n) k_copy_table<<<dim3((unsigned)((n + 4 * kThreads - 1) / (4 * kThreads)), C.count), kThreads, 0, st>>>(C);
+}
+
 void launch_line_integrals(const Geo &g, const History &H, double *out2, cudaStream_t st) {
-  k_line_integrals<<<1, 32, 0, st>>>(g, H, out2);
+  k_line_integrals<<<1, kThreads, 0, st>>>(g, H, out2);
 }
 
 void launch_pack(const double *box, double *dst, int ex, int ey, int ez, int px, int py, cudaStream_t st) {
@@ -401,9 +470,9 @@ template void launch_rotation_fields<float>(const Geo &, const History &, const 
                                             float *const[2], float *, cudaStream_t);
 template void launch_rotation_fields<double>(const Geo &, const History &, const Scal *, double *const[3],
                                              double *const[2], double *, cudaStream_t);
-template void launch_compose<float>(const Geo &, const double *const[3], const float *const[3],
+template void launch_compose<float>(const Geo &, const double *const[3], const float *const[3], double *const[3],
                                     double *const[3], cudaStream_t);
-template void launch_compose<double>(const Geo &, const double *const[3], const double *const[3],
+template void launch_compose<double>(const Geo &, const double *const[3], const double *const[3], double *const[3],
                                      double *const[3], cudaStream_t);
 template void launch_commit<float>(const Geo &, const History &, const double *const[3], const double *const[3],
                                    const double *const[3], const float *const[3], const float *const[3],
@@ -412,6 +481,8 @@ template void launch_commit<double>(const Geo &, const History &, const double *
                                     const double *const[3], const double *const[3], const double *const[3],
                                     const double *, const double *, const Scal *, unsigned long long *,
                                     cudaStream_t);
+template void launch_fill<float>(const FillTab &, long long, cudaStream_t);
+template void launch_fill<double>(const FillTab &, long long, cudaStream_t);
 template void launch_convert<float, double>(float *, const double *, long long, cudaStream_t);
 template void launch_convert<double, float>(double *, const float *, long long, cudaStream_t);
 template void launch_convert<double, double>(double *, const double *, long long, cudaStream_t);

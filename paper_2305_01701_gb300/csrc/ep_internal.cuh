@@ -202,6 +202,9 @@ template <typename T>
 void launch_strain(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, cudaStream_t st);
 template <typename T>
 void launch_trial(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, cudaStream_t st);
+// the trial at the centres with near < 1 and at the points around them
+template <typename TS>
+void launch_trial_near(const Geo &g, const Stage<double> &S, const Scal *sc, const TS *near, cudaStream_t st);
 template <typename T>
 void launch_return_centres(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int check,
                            cudaStream_t st);
@@ -277,13 +280,35 @@ void launch_rotation_fields(const Geo &g, const History &H, const Scal *sc, T *c
                             T *yc, cudaStream_t st);
 template <typename T>
 void launch_compose(const Geo &g, const double *const v0[3], const T *const u[3], double *const out[3],
-                    cudaStream_t st);
+                    double *const prev[3], cudaStream_t st);
 template <typename T>
 void launch_commit(const Geo &g, const History &H, const double *const Tn64[3], const double *const Ts64[3],
                    const double *const es64[3], const T *const stn[3], const T *const sts[3], const T *stp,
                    const T *s, const Scal *sc, unsigned long long *n_plastic, cudaStream_t st);
 template <typename Td, typename Ts>
 void launch_convert(Td *dst, const Ts *src, long long n, cudaStream_t st);
+// sources (null: zeros) and their copies in the sweep's type; unused dst are null
+struct FillTab {
+  static constexpr int MAX = 26;
+  struct Entry {
+    const double *src;
+    void *dst[4];
+  } e[MAX];
+  int count;
+};
+template <typename Td>
+void launch_fill(const FillTab &F, long long n, cudaStream_t st);
+// copies of 16-byte-aligned arrays, n16 times 16 bytes each
+struct CopyTab {
+  static constexpr int MAX = 26;
+  struct Entry {
+    const void *src;
+    void *dst;
+    long long n16;
+  } e[MAX];
+  int count;
+};
+void launch_copy_table(const CopyTab &C, cudaStream_t st);
 void launch_line_integrals(const Geo &g, const History &H, double *out2, cudaStream_t st);
 void launch_advect(const Geo &g, const History &H, const Scal *sc, double *const tn_out[3], double *const ts_out[3],
                    double *p_out, cudaStream_t st);

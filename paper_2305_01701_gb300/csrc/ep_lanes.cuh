@@ -1,6 +1,6 @@
 // ep_lanes.cuh -- the columns of one thread of a marching sweep kernel: two
 // adjacent FP32 columns as a float2 (packed arithmetic, one instruction per
-// pair), or one FP64 column.
+// pair), or one FP64 column; the return scale.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -63,5 +63,9 @@ __device__ __forceinline__ float2 vscale(float2 J2, float2 Y) {
   return make_float2(scale_of(J2.x, Y.x), scale_of(J2.y, Y.y));
 }
 __device__ __forceinline__ double vscale(double J2, double Y) { return scale_of(J2, Y); }
+
+// a return scale (0 .. 1, or NaN) below one; the FP64 one without the FP64 pipe
+__device__ __forceinline__ bool below_one(float s) { return s < 1.f; }
+__device__ __forceinline__ bool below_one(double s) { return (unsigned)__double2hiint(s) < 0x3ff00000u; }
 
 }  // namespace ep

@@ -19,7 +19,10 @@
 // start-of-increment and commit passes.
 #include <math.h>
 
+#include <type_traits>
+
 #include "ep_internal.cuh"
+#include "ep_lanes.cuh"
 
 namespace ep {
 
@@ -128,13 +131,24 @@ __global__ void __launch_bounds__(kThreads) k_strain(Geo g, Stage<T> S, const Sc
 }
 
 // ---------------------------------------------------------------------------
-template <typename T, int ND>
-__global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Scal *sc, DevInfo *di) {
+// near (TS is not void): the return scale of the last iteration; the trial is
+// formed at the centres that it acted on (near < 1) and at the vertices / edges
+// around them only.
+template <typename T, int ND, typename TS>
+__global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Scal *sc, DevInfo *di, const TS *near) {
   if (skip(di)) return;
   const Pos q = position(g);
   if (!q.in) return;
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   const long long e = q.e, px = g.px, pl = g.plane;
+  auto want = [&](long long c) {
+    if constexpr (std::is_void<TS>::value) return true;
+    else return below_one(near[c]);
+  };
+  // an edge whose surrounding centres are c, c + a, c + b, c + a + b
+  auto want4 = [&](long long c, long long a, long long b) {
+    return want(c) || want(c + a) || want(c + b) || want(c + a + b);
+  };
   if (i > nx || j > ny || k > (ND == 3 ? nz : 0)) return;
   const SweepScal<T> &Q = sweep_scal<T>(sc);
   const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz;
@@ -146,7 +160,7 @@ __global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Sca
   auto tb = [&](int w, long long x) { return S.tb_c2 && S.gc[w] ? S.gc[w][x] : tbs0; };
   const T bt = S.relax ? Q.bt : (T)0, ob = S.relax ? Q.ob : (T)1;
   // ---- centre ----
-  if (i < nx && j < ny && (ND == 2 || k < nz)) {
+  if (i < nx && j < ny && (ND == 2 || k < nz) && want(e)) {
     const long long c = e;
     T tr[3];
     if (ND == 2) {
@@ -182,7 +196,7 @@ __global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Sca
   // ---- vertices (2D) / edges (3D) ----
   if (ND == 2) {
     T v = 0;
-    if (i > 0 && i < nx && j > 0 && j < ny) {
+    if (i > 0 && i < nx && j > 0 && j < ny && want4(e - px - 1, 1, px)) {
       T dyx = qr * (S.rd[0][e - px - 1] + S.rd[0][e - px] + S.rd[0][e - 1] + S.rd[0][e]);
       T tr = tb(1, e) * S.tbs[0][e] + te(1, e) * S.es[0][e] + cr(1, e) * (S.om[0][e] * dyx);
       v = S.relax ? bt * S.sos[0][e] + ob * tr : tr;
@@ -190,7 +204,7 @@ __global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Sca
     S.Ts[0][e] = v;
   } else {
     T v = 0;  // xy-edge
-    if (k < nz && i > 0 && i < nx && j > 0 && j < ny) {
+    if (k < nz && i > 0 && i < nx && j > 0 && j < ny && want4(e - px - 1, 1, px)) {
       T dyx = qr * (S.rd[0][e - px - 1] + S.rd[0][e - px] + S.rd[0][e - 1] + S.rd[0][e]);
       T Tyz = qr * (S.rq[2][e - 1] + S.rq[2][e] + S.rq[2][e - 1 + pl] + S.rq[2][e + pl]);
       T Wyz = qr * (S.om[2][e - 1] + S.om[2][e] + S.om[2][e - 1 + pl] + S.om[2][e + pl]);
@@ -201,7 +215,7 @@ __global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Sca
     }
     S.Ts[0][e] = v;
     v = 0;    // xz-edge
-    if (j < ny && i > 0 && i < nx && k > 0 && k < nz) {
+    if (j < ny && i > 0 && i < nx && k > 0 && k < nz && want4(e - pl - 1, 1, pl)) {
       T dzx = qr * (S.rd[1][e - pl - 1] + S.rd[1][e - pl] + S.rd[1][e - 1] + S.rd[1][e]);
       T Tyz = qr * (S.rq[2][e - 1] + S.rq[2][e] + S.rq[2][e - 1 + px] + S.rq[2][e + px]);
       T Wyz = qr * (S.om[2][e - 1] + S.om[2][e] + S.om[2][e - 1 + px] + S.om[2][e + px]);
@@ -212,7 +226,7 @@ __global__ void __launch_bounds__(kThreads) k_trial(Geo g, Stage<T> S, const Sca
     }
     S.Ts[1][e] = v;
     v = 0;    // yz-edge
-    if (i < nx && j > 0 && j < ny && k > 0 && k < nz) {
+    if (i < nx && j > 0 && j < ny && k > 0 && k < nz && want4(e - pl - px, px, pl)) {
       T dzy = qr * ((S.rd[1][e - pl - px] - S.rd[0][e - pl - px]) + (S.rd[1][e - pl] - S.rd[0][e - pl]) +
                     (S.rd[1][e - px] - S.rd[0][e - px]) + (S.rd[1][e] - S.rd[0][e]));
       T Txy = qr * (S.rq[0][e - pl] + S.rq[0][e - pl + 1] + S.rq[0][e] + S.rq[0][e + 1]);
@@ -262,10 +276,14 @@ __global__ void __launch_bounds__(kThreads) k_return_centres(Geo g, Stage<T> S, 
     if (frozen) {
       s = S.s[c];   // frozen plasticity: the held scale (Sec. 3.3)
     } else {
-      T sj = sqrt(J2);
       T Y = Q.A * p + S.yc[c];
-      Y = Y > (T)0 ? Y : (T)0;
-      s = sj > Y ? Y / sj : (T)1;
+      if constexpr (sizeof(T) == 8) {
+        s = scale_of(J2, Y);
+      } else {
+        T sj = sqrt(J2);
+        Y = Y > (T)0 ? Y : (T)0;
+        s = sj > Y ? Y / sj : (T)1;
+      }
       S.s[c] = s;
     }
     S.snp[c] = p;
@@ -445,9 +463,19 @@ void launch_strain(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di,
 }
 template <typename T>
 void launch_trial(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, cudaStream_t st) {
-  if (g.ndim == 2) k_trial<T, 2><<<blocks_for(g.box), kThreads, 0, st>>>(g, S, sc, di);
-  else k_trial<T, 3><<<blocks_for(g.box), kThreads, 0, st>>>(g, S, sc, di);
+  const void *all = nullptr;
+  if (g.ndim == 2) k_trial<T, 2><<<blocks_for(g.box), kThreads, 0, st>>>(g, S, sc, di, all);
+  else k_trial<T, 3><<<blocks_for(g.box), kThreads, 0, st>>>(g, S, sc, di, all);
 }
+
+template <typename TS>
+void launch_trial_near(const Geo &g, const Stage<double> &S, const Scal *sc, const TS *near, cudaStream_t st) {
+  if (g.ndim == 2) k_trial<double, 2><<<blocks_for(g.box), kThreads, 0, st>>>(g, S, sc, nullptr, near);
+  else k_trial<double, 3><<<blocks_for(g.box), kThreads, 0, st>>>(g, S, sc, nullptr, near);
+}
+template void launch_trial_near<float>(const Geo &, const Stage<double> &, const Scal *, const float *, cudaStream_t);
+template void launch_trial_near<double>(const Geo &, const Stage<double> &, const Scal *, const double *,
+                                        cudaStream_t);
 template <typename T>
 void launch_return_centres(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int check,
                            cudaStream_t st) {

@@ -135,3 +135,39 @@ def test_batched_strips_of_column_pairs_match_the_staged_sweep_fp32(P, n, tile, 
     iref, ref = _solve(P, 2, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f, **opts)
     info, out = _solve(P, 2, n, P.FP32_MIXED, P.KERNEL_FUSED, iters, f, shape=tile, **opts)
     _compare(f, out, ref, info, iref, iters, EPS32)
+
+
+@pytest.mark.parametrize("nd,n", [(2, (31, 300)), (2, (64, 7)), (3, (33, 5, 260)), (3, (28, 20, 6))])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_commit_history_copies_and_line_integrals(P, nd, n, precision):
+    """The commit's trial near the yielding centres against the trial of every point (formed
+    while the warm-start targets are recorded), the copies of a restore, the column integrals."""
+    f = _fields(P, nd, n, 10)
+    g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=P.FP64 if precision == "fp64" else P.FP32_MIXED)
+    g.set_material(2.0, 1.0, math.inf, 30.0, 0.0, np.full(int(np.prod(n)), 1.5e-3))
+    g.set_solver(tol=2e-2, max_iter=50000, n_chk=10)
+    for k, a in f.items():
+        g.set(k, a)
+    g.snapshot()
+    names = list(f) + ["epl", "ux", "exx", "exy"]
+    start = {k: g.get(k) for k in names}
+    outs = []
+    for on in (0, 1):
+        g.warm_record(on)
+        g.apply_increment(1.0, 1e-4, P.LOAD_XY if nd == 2 else P.LOAD_XZ)
+        info = g.solve_increment()
+        outs.append(({k: g.get(k) for k in names + ["scale"]}, (info["sxx_int_centre"], info["sxx_int_right"])))
+        g.restore()
+        for k in names:
+            np.testing.assert_array_equal(g.get(k), start[k])
+    (a, la), (b, lb) = outs
+    assert (a["scale"] < 1.0).any() and (a["epl"] > 0.0).any() and (a["epl"] == 0.0).any()
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k])
+    assert la == lb
+    sxx = a["txx"] - a["p"]
+    cols = (sxx[:, n[0] // 2], sxx[:, -1]) if nd == 2 else (sxx[:, n[1] // 2, n[0] // 2], sxx[:, n[1] // 2, -1])
+    h = 0.8 / n[1] if nd == 2 else 1.3 / n[2]
+    for got, c in zip(la, cols):
+        assert abs(got - math.fsum(c * h)) <= len(c) * 2.0 ** -52 * np.abs(c * h).sum()
+    g.close()

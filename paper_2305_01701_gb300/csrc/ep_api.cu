@@ -55,6 +55,9 @@ struct ep_grid {
   DevInfo *dinfo = nullptr, *hinfo = nullptr;
   unsigned long long *dnpl = nullptr;
   double *dline = nullptr;
+  // resident 2D sweep: counters of its blocks, words of its exchange
+  unsigned *rcount = nullptr;
+  unsigned long long *rwords = nullptr;
   cudaGraphExec_t chunk = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int variant = EP_KERNEL_AUTO;  // sweep kernel choice (ep_set_kernel)
@@ -191,6 +194,10 @@ void carve(ep_grid *h, Arena &a) {
   h->items_dev = a.take<int4>(h->max_items);
   h->dnpl = a.take<unsigned long long>(1);
   h->dline = a.take<double>(2);
+  if (const long long words = resident2d_words(h->g, es)) {
+    h->rcount = a.take<unsigned>(RESIDENT_BLOCKS);
+    h->rwords = a.take<unsigned long long>(words);
+  }
 }
 
 // natural extent of a field id; returns false for an unknown / absent field
@@ -626,6 +633,9 @@ ep_status capture_chunk(ep_grid *h) {
     blocks = std::min(persistent_blocks(h->tile, sizeof(T)),
                       (h->n_items + fused2d_items_per_block(h->tile) - 1) / fused2d_items_per_block(h->tile));
   }
+  // AUTO on a 2D grid that fits the chip: the iterations behind the check in one launch
+  const int res = h->ndim == 2 && !h->Gc && h->variant == EP_KERNEL_AUTO ? resident2d_config<T>(h->g) : -1;
+  cudaError_t launched = cudaSuccess;
   CK(h, cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
   for (int it = 0; f2 && it < h->opts.n_chk; ++it) {
     launch_fused2d<T>(h->tile, (const Inst2<T> *)h->inst_dev, h->items_dev, h->n_items, it & 1, it == 0, blocks,
@@ -645,10 +655,19 @@ ep_status capture_chunk(ep_grid *h) {
       if (chk) launch_check(h->dinfo, h->dscal, h->cap);
       continue;
     }
+    if (!chk && res >= 0) {
+      launched = launch_resident2d<T>(res, h->g, S, h->dscal, h->dinfo, h->opts.n_chk - 1, h->rcount, h->rwords,
+                                      h->cap);
+      break;
+    }
     launch_staged<T>(h, S, h->dinfo, chk, h->cap);
     if (chk) launch_check(h->dinfo, h->dscal, h->cap);
   }
   cudaError_t e = cudaStreamEndCapture(h->cap, &graph);
+  if (e == cudaSuccess && launched != cudaSuccess) {
+    cudaGraphDestroy(graph);
+    e = launched;
+  }
   if (e != cudaSuccess) return fail(h, EP_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
   e = cudaGraphInstantiate(&h->chunk, graph, 0);
   cudaGraphDestroy(graph);
@@ -703,6 +722,9 @@ ep_status solve(ep_grid *h, long long max_chunks, ep_solve_info *info) {
     init.frozen_at = -1;
     *h->hinfo = init;
     CK(h, cudaMemcpyAsync(h->dinfo, h->hinfo, sizeof(DevInfo), cudaMemcpyHostToDevice, h->stream));
+    if (h->rwords)   // the two arrays are adjacent
+      CK(h, cudaMemsetAsync(h->rcount, 0, (char *)(h->rwords + resident2d_words(h->g, sizeof(T))) - (char *)h->rcount,
+                            h->stream));
     h->solving = true;
   }
   CK(h, cudaEventRecord(h->ev0, h->stream));

@@ -174,6 +174,22 @@ __device__ __forceinline__ void check_one(DevInfo *di, const Scal *sc) {
   for (int r = 0; r < RED_COUNT; ++r) di->red[r] = 0ull;
 }
 
+// ---- the unchecked iterations of a chunk in one launch (ep_resident2d.cu) ----
+constexpr int RESIDENT_BLOCKS = 4096;          // counters of a grid
+constexpr long long RESIDENT_POINTS = 200000;  // largest box
+// the exchange's words of both buffers, three values per point (0: box too large)
+inline long long resident2d_words(const Geo &g, size_t elem) {
+  return g.ndim == 2 && g.box <= RESIDENT_POINTS ? 6 * g.box * (long long)(elem / 4) : 0;
+}
+// a configuration that holds the whole grid on the chip at once, or -1
+template <typename T>
+int resident2d_config(const Geo &g);
+// `iters` (odd) iterations from S.u, S.son .. to S.uo, S.snn ..; `count` and `words`
+// are zero when a solve starts and its own until it ends
+template <typename T>
+cudaError_t launch_resident2d(int config, const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int iters,
+                              unsigned *count, unsigned long long *words, cudaStream_t st);
+
 // ---- batched fused 2D sweep (ep_fused2d.cu, ep_fused2d_strip.cu) ---------
 // tile: 0 = 32x8, 1 = 32x16, 2 = 64x8 cells (block tiles in shared memory);
 // 3, 4 = warp strips of 60 (FP32) or 28 (FP64) columns marching 64 / 32 rows

@@ -1,0 +1,295 @@
+// ep_resident2d.cu -- the unchecked iterations of a chunk on one small 2D grid, in one
+// cooperative launch that keeps the state on the chip.
+//
+// The same iteration as ep_sweep2d.cu, operation by operation (equal results, bit
+// for bit).  Two launches an iteration cost 8 us however small the grid is, most of it
+// launch and load latency.  Here a thread owns one point of a lattice for the whole
+// chunk and keeps its coefficients and stresses in registers; a block's lattice of
+// WX x WY points overlaps its neighbours by two points on each side, where the
+// stresses are computed twice, so that the blocks exchange only once an iteration: the
+// velocities of the two outer rows and columns that a block owns, and the shear stress
+// there.  Points of a block meet in shared memory.
+//
+// Exchange: a value travels in 8-byte words that carry 32 of its bits and the number of
+// the iteration that wrote them, so that the reader polls the value itself (one trip
+// through L2; a counter behind a fence takes four).  Two buffers alternate: a block
+// overwrites a word only after it has read from every neighbour what that one sent
+// after reading the word.  All blocks are resident at once (cooperative launch,
+// checked against the occupancy); a wait gives up after 2^31 cycles or when another
+// one has: done = 4, every block returns.  Numbers only grow, by the same amount in
+// every block of a launch; the buffers start a solve at zero.
+//
+// Bound: latency of the exchange and of four block barriers; FP64 grids the FP64 pipe
+// as well, which takes a warp's instruction in 64 cycles.
+// Measured, an iteration against two launches: FP64 64^2 8.0 -> 4.0 us, 128^2 8.9 -> 6.5;
+// FP32 64^2 5.8 -> 1.6, 128^2 6.3 -> 1.8, 383 x 191 9.0 -> 2.7, 300^2 9.2 -> 2.9 (a
+// counter per block behind a fence: 64^2 FP64 7.5 us, 383 x 191 FP32 5.8).
+#include <math.h>
+
+#include "ep_internal.cuh"
+
+namespace ep {
+
+namespace {
+
+// As in ep_sweep2d.cu.
+template <typename T>
+__device__ __forceinline__ T return_scale(T J2, T Y) {
+  Y = Y > (T)0 ? Y : (T)0;
+  if (J2 < Y * Y * (T)(sizeof(T) == 8 ? 1.0 - 1e-15 : 1.0 - 1e-6)) return (T)1;
+  const T sj = sqrt(J2);
+  return sj > Y ? Y / sj : (T)1;
+}
+
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// one value at word index e: sizeof(T) / 4 words, each with the number `tag`
+__device__ __forceinline__ void send(unsigned long long *w, int e, float v, unsigned tag) {
+  st_relaxed(w + e, (unsigned long long)tag << 32 | __float_as_uint(v));
+}
+__device__ __forceinline__ void send(unsigned long long *w, int e, double v, unsigned tag) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
+  st_relaxed(w + 2 * e, t | (b & 0xffffffffu));
+  st_relaxed(w + 2 * e + 1, t | (b >> 32));
+}
+__device__ __forceinline__ bool receive(const unsigned long long *w, int e, unsigned tag, float *v) {
+  const unsigned long long a = ld_relaxed(w + e);
+  *v = __uint_as_float((unsigned)a);
+  return (unsigned)(a >> 32) == tag;
+}
+__device__ __forceinline__ bool receive(const unsigned long long *w, int e, unsigned tag, double *v) {
+  const unsigned long long a = ld_relaxed(w + 2 * e), b = ld_relaxed(w + 2 * e + 1);
+  *v = __longlong_as_double((long long)(b << 32 | (a & 0xffffffffu)));
+  return (unsigned)(a >> 32) == tag && (unsigned)(b >> 32) == tag;
+}
+
+constexpr long long WAIT_CYCLES = 1LL << 31;
+
+template <typename T, int WX, int WY>
+__global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const Scal *sc, DevInfo *di, int iters,
+                                                       unsigned *count, unsigned long long *words) {
+  __shared__ T su0[WY][WX], su1[WY][WX], sp[WY][WX], st[WY][WX], ss[WY][WX], sx0[WY][WX], sx1[WY][WX], sn[WY][WX];
+  const int tid = threadIdx.x, tx = tid % WX, ty = tid / WX;
+  // one thread's view of `done` for the block
+  if (__syncthreads_or(tid == 0 && *(volatile const int *)&di->done != 0)) return;
+  const bool frozen = di->frozen != 0;
+  const int nx = g.nx, ny = g.ny, px = g.px;   // a 2D box has fewer than 2^31 points
+  const int gi = blockIdx.x * (WX - 4) - 2 + tx, gj = blockIdx.y * (WY - 4) - 2 + ty, e = gj * px + gi;
+  const SweepScal<T> &Q = sweep_scal<T>(sc);
+  const T two_eta = Q.two_eta, eta = Q.eta, eta_d = Q.eta_d, bt = Q.bt, ob = Q.ob;
+  const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Ac = Q.A, rdx = Q.rdx, rdy = Q.rdy, vs = Q.vstep;
+
+  const bool box = gi >= 0 && gi <= nx && gj >= 0 && gj <= ny;
+  const bool owned = box && tx >= 2 && tx < WX - 2 && ty >= 2 && ty < WY - 2;
+  const bool ring = owned && (tx < 4 || tx >= WX - 4 || ty < 4 || ty >= WY - 4);
+  // interior vertices, and those of them whose deviator is formed here (the others
+  // around a centre come from the block that owns them)
+  const bool vin = gi > 0 && gi < nx && gj > 0 && gj < ny && tx >= 1 && ty >= 1;
+  const bool vown = vin && tx >= 2 && tx < WX - 1 && ty >= 2 && ty < WY - 1;
+  const bool cin = gi >= 0 && gi < nx && gj >= 0 && gj < ny && tx >= 1 && tx < WX - 1 && ty >= 1 && ty < WY - 1;
+  const bool x1 = gi > 0 && gi < nx;
+  const bool fx = owned && gj < ny && x1, fy = owned && gi < nx && gj > 0 && gj < ny;
+
+  T u0 = 0, u1 = 0, md = 0, tbs = 0, rq = 0, tsh = 0;
+  T tb0 = 0, tb1 = 0, n0 = 0, n1 = 0, pr = 0, pb = 0, yc = 0, s = 1, f0 = 0, f1 = 0;
+  if (box) { u0 = S.u[0][e]; u1 = S.u[1][e]; }
+  if (vin) { md = S.md[0][e]; tbs = S.tbs[0][e]; rq = S.rq[0][e]; tsh = S.sos[0][e]; }
+  if (cin) {
+    tb0 = S.tbn[0][e]; tb1 = S.tbn[1][e]; n0 = S.son[0][e]; n1 = S.son[1][e];
+    pr = S.sop[e]; pb = S.pb[e]; yc = S.yc[e];
+    if (frozen) s = S.s[e];   // frozen plasticity: the held scale (Sec. 3.3)
+  }
+  if (fx && S.f[0]) f0 = S.f[0][e];
+  if (fy && S.f[1]) f1 = S.f[1][e];
+  su0[ty][tx] = u0;
+  su1[ty][tx] = u1;
+
+  // iterations before this launch; words of both buffers: x and y velocity, shear stress
+  unsigned *const mine = count + blockIdx.y * gridDim.x + blockIdx.x;
+  const unsigned base = *mine;
+  const long long field = g.box * (long long)(sizeof(T) / 4);
+  __syncthreads();
+  if (tid == 0) *mine = base + iters;
+
+  for (int q = 0; q < iters; ++q) {
+    // ---- vertex: relaxed trial, rotation product ----
+    T ts = 0, p = 0;
+    if (vin) {
+      const T x = (u0 - su0[ty - 1][tx]) * rdy, y = u1 - su1[ty][tx - 1];
+      const T w = fma(y, -rdx, x);
+      const T tr = fma(w, md, fma(eta, fma(y, rdx, x), tbs));
+      ts = fma(bt, tsh, ob * tr);
+      p = rq * w;
+    }
+    sp[ty][tx] = p;
+    st[ty][tx] = ts;
+    __syncthreads();
+    // ---- centre: relaxed trial, pressure, return ----
+    T s0 = 0, s1 = 0;
+    if (cin) {
+      const T xy = (p + sp[ty + 1][tx]) + (sp[ty][tx + 1] + sp[ty + 1][tx + 1]);
+      const T txy = (ts + st[ty + 1][tx]) + (st[ty][tx + 1] + st[ty + 1][tx + 1]);
+      const T e0 = (su0[ty][tx + 1] - u0) * rdx, e1 = (su1[ty + 1][tx] - u1) * rdy;
+      const T div = e0 + e1, m = div * eta_d;
+      const T t0 = fma((T)0.25, xy, fma(two_eta, e0, tb0 + m));
+      const T t1 = fma((T)-0.25, xy, fma(two_eta, e1, tb1 + m));
+      const T c0 = fma(bt, n0, ob * t0), c1 = fma(bt, n1, ob * t1);
+      pr = fma(bp, pr, obp * fma(-KDt, div, pb));
+      if (!frozen) {
+        const T J2 = fma((T)0.0625, txy * txy, (T)0.5 * fma(c1, c1, c0 * c0));
+        s = return_scale(J2, fma(Ac, pr, yc));
+      }
+      n0 = s * c0;
+      n1 = s * c1;
+      s0 = n0 - pr;
+      s1 = n1 - pr;
+    }
+    ss[ty][tx] = s;
+    sx0[ty][tx] = s0;
+    sx1[ty][tx] = s1;
+    __syncthreads();
+    // ---- vertex: deviator from the mean of its centre scales ----
+    T v = 0;
+    if (vown) {
+      v = ((ss[ty - 1][tx - 1] + ss[ty - 1][tx]) + (ss[ty][tx - 1] + s)) * ((T)0.25 * ts);
+      tsh = v;
+    }
+    sn[ty][tx] = v;
+    __syncthreads();
+    // ---- faces: residual and velocity update ----
+    if (fx) {
+      T R0 = fma(sn[ty + 1][tx] - v, rdy, (s0 - sx0[ty][tx - 1]) * rdx);
+      if (S.f[0]) R0 += f0;
+      u0 = fma(vs, R0, u0);
+      su0[ty][tx] = u0;
+    }
+    if (fy) {
+      T R1 = fma(sn[ty][tx + 1] - v, rdx, (s1 - sx1[ty - 1][tx]) * rdy);
+      if (S.f[1]) R1 += f1;
+      u1 = fma(vs, R1, u1);
+      su1[ty][tx] = u1;
+    }
+    if (q == iters - 1) break;
+
+    // ---- exchange with the neighbours ----
+    const unsigned tag = base + q + 1;
+    unsigned long long *const w0 = words + (q & 1) * 3 * field, *const w1 = w0 + field, *const ws = w1 + field;
+    bool lost = false;
+    if (ring) {
+      send(w0, e, u0, tag);
+      send(w1, e, u1, tag);
+      send(ws, e, v, tag);
+    } else if (box && !owned) {
+      const bool shear = vin && !vown;
+      const long long t0 = clock64();
+      for (unsigned n = 1;; ++n) {
+        T a, b, c = tsh;
+        bool ok = receive(w0, e, tag, &a);
+        ok = receive(w1, e, tag, &b) && ok;
+        if (shear) ok = receive(ws, e, tag, &c) && ok;
+        if (ok) {
+          u0 = a;
+          u1 = b;
+          tsh = c;
+          break;
+        }
+        if ((n & 63) == 0 && (clock64() - t0 > WAIT_CYCLES || *(volatile const int *)&di->done != 0)) {
+          lost = true;
+          atomicCAS(&di->done, 0, 4);
+          break;
+        }
+      }
+      su0[ty][tx] = u0;
+      su1[ty][tx] = u1;
+    }
+    if (__syncthreads_or(lost)) return;
+  }
+  if (owned) {
+    S.uo[0][e] = u0;
+    S.uo[1][e] = u1;
+    S.sns[0][e] = vin ? tsh : (T)0;
+    if (cin) {
+      S.snn[0][e] = n0;
+      S.snn[1][e] = n1;
+      S.snp[e] = pr;
+      if (!frozen) S.s[e] = s;
+    }
+  }
+}
+
+struct Config {
+  int wx, wy;
+};
+// Lattices; a grid takes the one with the fewest points per SM, of equals the first (128^2
+// FP32: 16 x 8 1.8 us, 32 x 16 2.05, 32 x 32 2.4; 96^2 FP64: 16 x 8 5.6, 16 x 16 6.5).
+template <typename T>
+Config config(int c) {
+  return c == 0 ? Config{16, 8} : c == 1 ? Config{32, 16} : sizeof(T) == 8 ? Config{16, 16} : Config{32, 32};
+}
+constexpr int CONFIGS = 3;
+
+template <typename T>
+const void *kernel_of(int c) {
+  if (c == 0) return (const void *)k_resident2d<T, 16, 8>;
+  if (c == 1) return (const void *)k_resident2d<T, 32, 16>;
+  if constexpr (sizeof(T) == 8) return (const void *)k_resident2d<T, 16, 16>;
+  else return (const void *)k_resident2d<T, 32, 32>;
+}
+
+}  // namespace
+
+template <typename T>
+int resident2d_config(const Geo &g) {
+  int dev = 0, sms = 0, coop = 0, best = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop || sms < 1)
+    return -1;
+  if (g.box > RESIDENT_POINTS) return -1;
+  // Points per SM that it pays up to.  FP32: what the registers hold (1024; 383 x 191
+  // takes that).  FP64: the points computed twice go through the FP64 pipe, which several
+  // grids solved at once on their own streams share: 128^2 (256 points) 9.1 -> 6.6 us
+  // alone, 10.9 -> 9.8 with two grids, 15.0 -> 19.6 with four; 200^2 (512) 12.5 -> 9.9
+  // alone but 17.4 -> 19.1 with two, so the two launches stay there.
+  long long cost = (sizeof(T) == 4 ? 1024 : 256) + 1;
+  for (int c = 0; c < CONFIGS; ++c) {
+    const void *k = kernel_of<T>(c);
+    const int wx = config<T>(c).wx, wy = config<T>(c).wy;
+    const long long blocks = (long long)((g.nx + wx - 4) / (wx - 4)) * ((g.ny + wy - 4) / (wy - 4));
+    const long long rounds = (blocks + sms - 1) / sms;
+    int per = 0;
+    if (blocks > RESIDENT_BLOCKS || rounds * wx * wy >= cost ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, wx * wy, 0) != cudaSuccess || rounds > per)
+      continue;
+    cost = rounds * wx * wy;
+    best = c;
+  }
+  return best;
+}
+
+template <typename T>
+cudaError_t launch_resident2d(int c, const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int iters,
+                              unsigned *count, unsigned long long *words, cudaStream_t st) {
+  const int wx = config<T>(c).wx, wy = config<T>(c).wy;
+  Geo gg = g;
+  Stage<T> SS = S;
+  void *args[] = {&gg, &SS, &sc, &di, &iters, &count, &words};
+  return cudaLaunchCooperativeKernel(kernel_of<T>(c), dim3((g.nx + wx - 4) / (wx - 4), (g.ny + wy - 4) / (wy - 4)),
+                                     dim3(wx * wy), args, 0, st);
+}
+
+template int resident2d_config<float>(const Geo &);
+template int resident2d_config<double>(const Geo &);
+template cudaError_t launch_resident2d<float>(int, const Geo &, const Stage<float> &, const Scal *, DevInfo *, int,
+                                              unsigned *, unsigned long long *, cudaStream_t);
+template cudaError_t launch_resident2d<double>(int, const Geo &, const Stage<double> &, const Scal *, DevInfo *, int,
+                                               unsigned *, unsigned long long *, cudaStream_t);
+
+}  // namespace ep

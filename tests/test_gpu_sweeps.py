@@ -48,16 +48,18 @@ def _fields(P, nd, n, seed):
 
 def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
     opts = dict(opts)
+    force = opts.pop("force", 0.0)
     g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=precision)
     rng = np.random.default_rng(1)
     g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, 1.5e-3 * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
     if "cell_g" in opts:
         g.set_shear_modulus(1.0 + 0.2 * opts.pop("cell_g") * rng.random(int(np.prod(n))))
-    g.set_solver(tol=0.0, max_iter=iters, n_chk=iters // 2, **opts)
+    g.set_solver(tol=0.0, max_iter=iters, n_chk=opts.pop("chunk", iters // 2), **opts)
     g.set_kernel(kernel, shape)
     for k, a in f.items():
         g.set(k, a)
-    g.apply_increment(1.0, 1e-4, P.LOAD_XY if nd == 2 else P.LOAD_XZ)
+    bf = force * rng.standard_normal(sum(f["v" + c].size for c in "xyz"[:nd])) if force else None
+    g.apply_increment(1.0, 1e-4, P.LOAD_XY if nd == 2 else P.LOAD_XZ, bf)
     info = g.solve_increment(raise_on_fail=False)
     g.commit_increment()
     out = {k: g.get(k) for k in list(f) + ["epl", "scale"]}
@@ -171,3 +173,21 @@ def test_commit_history_copies_and_line_integrals(P, nd, n, precision):
     for got, c in zip(la, cols):
         assert abs(got - math.fsum(c * h)) <= len(c) * 2.0 ** -52 * np.abs(c * h).sum()
     g.close()
+
+
+@pytest.mark.parametrize("n", [(11, 3), (12, 4), (13, 5), (24, 25), (64, 64), (27, 90), (171, 140), (300, 180), (383, 191)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("opts", [{}, {"mu_s": 1e-3, "jaumann": False, "incompressible": True}, {"freeze_iter": 5},
+                                  {"force": 1e-3}])
+def test_resident_2d_iterations_equal_the_two_launch_sweep(P, n, precision, opts):
+    """One launch per chunk against two per iteration: the same operations, equal bits, at the
+    edges of every lattice, over several chunks; the largest grids take two launches again."""
+    iters = 24
+    f = _fields(P, 2, n, 11)
+    pr = P.FP64 if precision == "fp64" else P.FP32_MIXED
+    iref, ref = _solve(P, 2, n, pr, P.KERNEL_STAGED, iters, f, chunk=6, **opts)
+    info, out = _solve(P, 2, n, pr, P.KERNEL_AUTO, iters, f, chunk=6, **opts)
+    for k in out:
+        np.testing.assert_array_equal(out[k], ref[k])
+    for k in ("iters", "max_sigma", "eps_rel", "eps_res"):
+        assert info[k] == iref[k]

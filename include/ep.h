@@ -212,10 +212,12 @@ ep_status ep_set_fields(ep_handle h, int field, const double *host_in, size_t co
  * kernels in 2D, five in 3D; FP64 is bound by FP64 arithmetic on GB300, where
  * the staged sweep does no halo recomputation), the register z-march sweep for
  * FP32 grids in 3D.  A 2D grid with a uniform modulus that fits the chip (in
- * FP32 up to about 118,000 points, in FP64 up to about 20,000) runs the
- * iterations between two checks in one cooperative launch, with the same
- * results bit for bit; its blocks wait for one another, bounded at 2^31
- * cycles (then EP_ERR_TIMEOUT).  ep_time_sweep times the two kernels there.
+ * FP32 up to about 118,000 points, in FP64 up to about 20,000) and a 3D FP32
+ * grid with a uniform modulus and no body force of up to about 100,000 points
+ * run the iterations between two checks in one cooperative launch (in 2D with
+ * the same results bit for bit); its blocks wait for one another, bounded at
+ * 2^31 cycles (then EP_ERR_TIMEOUT).  ep_time_sweep times the other kernels
+ * there.
  * EP_KERNEL_STAGED / EP_KERNEL_FUSED force one;
  * EP_KERNEL_FUSED_TMA is the 3D fused sweep with every plane streamed by
  * the tensor-memory accelerator (a timed-out copy ends the solve with

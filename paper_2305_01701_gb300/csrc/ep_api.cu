@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "ep_internal.cuh"
+#include "ep_words.cuh"
 
 using namespace ep;
 
@@ -55,9 +56,9 @@ struct ep_grid {
   DevInfo *dinfo = nullptr, *hinfo = nullptr;
   unsigned long long *dnpl = nullptr;
   double *dline = nullptr;
-  // resident 2D sweep: counters of its blocks, words of its exchange
+  // resident sweeps: counters of the blocks, words of its exchange
   unsigned *rcount = nullptr;
-  unsigned long long *rwords = nullptr;
+  Word *rwords = nullptr;
   cudaGraphExec_t chunk = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int variant = EP_KERNEL_AUTO;  // sweep kernel choice (ep_set_kernel)
@@ -194,9 +195,9 @@ void carve(ep_grid *h, Arena &a) {
   h->items_dev = a.take<int4>(h->max_items);
   h->dnpl = a.take<unsigned long long>(1);
   h->dline = a.take<double>(2);
-  if (const long long words = resident2d_words(h->g, es)) {
+  if (const long long words = resident_words(h->g, es)) {
     h->rcount = a.take<unsigned>(RESIDENT_BLOCKS);
-    h->rwords = a.take<unsigned long long>(words);
+    h->rwords = a.take<Word>(words);
   }
 }
 
@@ -633,8 +634,11 @@ ep_status capture_chunk(ep_grid *h) {
     blocks = std::min(persistent_blocks(h->tile, sizeof(T)),
                       (h->n_items + fused2d_items_per_block(h->tile) - 1) / fused2d_items_per_block(h->tile));
   }
-  // AUTO on a 2D grid that fits the chip: the iterations behind the check in one launch
+  // AUTO on a grid that fits the chip: the iterations behind the check in one launch
   const int res = h->ndim == 2 && !h->Gc && h->variant == EP_KERNEL_AUTO ? resident2d_config<T>(h->g) : -1;
+  int tile3[3];
+  const bool res3 = sizeof(T) == 4 && use_fused<T>(h) && !h->Gc && h->variant == EP_KERNEL_AUTO && h->kz == 0 &&
+                    h->rwords && resident3d_tile(h->g, tile3);
   cudaError_t launched = cudaSuccess;
   CK(h, cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
   for (int it = 0; f2 && it < h->opts.n_chk; ++it) {
@@ -645,6 +649,13 @@ ep_status capture_chunk(ep_grid *h) {
   for (int it = 0; !f2 && it < h->opts.n_chk; ++it) {
     Stage<T> S = sweep_stage<T>(h, it & 1);
     const int chk = it == 0;
+    if constexpr (sizeof(T) == 4) {
+      if (!chk && res3) {
+        launched = launch_resident3d(tile3, h->g, S, h->dscal, h->dinfo, h->opts.n_chk - 1, h->rcount, h->rwords,
+                                     h->cap);
+        break;
+      }
+    }
     if ((!chk || fused_check<T>(h)) && use_fused<T>(h)) {
       if (!launch_fused_any<T>(h, S, h->dinfo, h->cap, chk)) {
         cudaGraph_t gr;
@@ -723,7 +734,7 @@ ep_status solve(ep_grid *h, long long max_chunks, ep_solve_info *info) {
     *h->hinfo = init;
     CK(h, cudaMemcpyAsync(h->dinfo, h->hinfo, sizeof(DevInfo), cudaMemcpyHostToDevice, h->stream));
     if (h->rwords)   // the two arrays are adjacent
-      CK(h, cudaMemsetAsync(h->rcount, 0, (char *)(h->rwords + resident2d_words(h->g, sizeof(T))) - (char *)h->rcount,
+      CK(h, cudaMemsetAsync(h->rcount, 0, (char *)(h->rwords + resident_words(h->g, sizeof(T))) - (char *)h->rcount,
                             h->stream));
     h->solving = true;
   }

@@ -174,13 +174,20 @@ __device__ __forceinline__ void check_one(DevInfo *di, const Scal *sc) {
   for (int r = 0; r < RED_COUNT; ++r) di->red[r] = 0ull;
 }
 
-// ---- the unchecked iterations of a chunk in one launch (ep_resident2d.cu) ----
+// ---- the unchecked iterations of a chunk in one launch (ep_resident2d.cu, ep_resident3d.cu) ----
 constexpr int RESIDENT_BLOCKS = 4096;          // counters of a grid
 constexpr long long RESIDENT_POINTS = 200000;  // largest box
-// the exchange's words of both buffers, three values per point (0: box too large)
-inline long long resident2d_words(const Geo &g, size_t elem) {
-  return g.ndim == 2 && g.box <= RESIDENT_POINTS ? 6 * g.box * (long long)(elem / 4) : 0;
+// the exchange's 16-byte words (0: box too large, or FP64 in 3D): in 2D two buffers of
+// three values per point, in 3D three words
+struct Word;
+inline long long resident_words(const Geo &g, size_t elem) {
+  if (g.box > RESIDENT_POINTS || (g.ndim == 3 && elem == 8)) return 0;
+  return g.box * (g.ndim == 2 ? elem == 4 ? 2 : 6 : 3);
 }
+// 3D, FP32 (ep_resident3d.cu)
+bool resident3d_tile(const Geo &g, int tile[3]);   // the points of a block; false: does not fit
+cudaError_t launch_resident3d(const int tile[3], const Geo &g, const Stage<float> &S, const Scal *sc, DevInfo *di,
+                              int iters, unsigned *count, Word *words, cudaStream_t st);
 // a configuration that holds the whole grid on the chip at once, or -1
 template <typename T>
 int resident2d_config(const Geo &g);
@@ -188,7 +195,7 @@ int resident2d_config(const Geo &g);
 // are zero when a solve starts and its own until it ends
 template <typename T>
 cudaError_t launch_resident2d(int config, const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int iters,
-                              unsigned *count, unsigned long long *words, cudaStream_t st);
+                              unsigned *count, Word *words, cudaStream_t st);
 
 // ---- batched fused 2D sweep (ep_fused2d.cu, ep_fused2d_strip.cu) ---------
 // tile: 0 = 32x8, 1 = 32x16, 2 = 64x8 cells (block tiles in shared memory);

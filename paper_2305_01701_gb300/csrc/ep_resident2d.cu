@@ -10,9 +10,7 @@
 // velocities of the two outer rows and columns that a block owns, and the shear stress
 // there.  Points of a block meet in shared memory.
 //
-// Exchange: a value travels in 8-byte words that carry 32 of its bits and the number of
-// the iteration that wrote them, so that the reader polls the value itself (one trip
-// through L2; a counter behind a fence takes four).  Two buffers alternate: a block
+// Exchange: ep_words.cuh.  Two buffers alternate: a block
 // overwrites a word only after it has read from every neighbour what that one sent
 // after reading the word.  All blocks are resident at once (cooperative launch,
 // checked against the occupancy); a wait gives up after 2^31 cycles or when another
@@ -27,6 +25,7 @@
 #include <math.h>
 
 #include "ep_internal.cuh"
+#include "ep_words.cuh"
 
 namespace ep {
 
@@ -41,40 +40,9 @@ __device__ __forceinline__ T return_scale(T J2, T Y) {
   return sj > Y ? Y / sj : (T)1;
 }
 
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// one value at word index e: sizeof(T) / 4 words, each with the number `tag`
-__device__ __forceinline__ void send(unsigned long long *w, int e, float v, unsigned tag) {
-  st_relaxed(w + e, (unsigned long long)tag << 32 | __float_as_uint(v));
-}
-__device__ __forceinline__ void send(unsigned long long *w, int e, double v, unsigned tag) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
-  st_relaxed(w + 2 * e, t | (b & 0xffffffffu));
-  st_relaxed(w + 2 * e + 1, t | (b >> 32));
-}
-__device__ __forceinline__ bool receive(const unsigned long long *w, int e, unsigned tag, float *v) {
-  const unsigned long long a = ld_relaxed(w + e);
-  *v = __uint_as_float((unsigned)a);
-  return (unsigned)(a >> 32) == tag;
-}
-__device__ __forceinline__ bool receive(const unsigned long long *w, int e, unsigned tag, double *v) {
-  const unsigned long long a = ld_relaxed(w + 2 * e), b = ld_relaxed(w + 2 * e + 1);
-  *v = __longlong_as_double((long long)(b << 32 | (a & 0xffffffffu)));
-  return (unsigned)(a >> 32) == tag && (unsigned)(b >> 32) == tag;
-}
-
-constexpr long long WAIT_CYCLES = 1LL << 31;
-
 template <typename T, int WX, int WY>
 __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const Scal *sc, DevInfo *di, int iters,
-                                                       unsigned *count, unsigned long long *words) {
+                                                       unsigned *count, Word *words) {
   __shared__ T su0[WY][WX], su1[WY][WX], sp[WY][WX], st[WY][WX], ss[WY][WX], sx0[WY][WX], sx1[WY][WX], sn[WY][WX];
   const int tid = threadIdx.x, tx = tid % WX, ty = tid / WX;
   // one thread's view of `done` for the block
@@ -111,10 +79,9 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
   su0[ty][tx] = u0;
   su1[ty][tx] = u1;
 
-  // iterations before this launch; words of both buffers: x and y velocity, shear stress
+  // iterations before this launch; a point's words: x and y velocity, shear stress
   unsigned *const mine = count + blockIdx.y * gridDim.x + blockIdx.x;
   const unsigned base = *mine;
-  const long long field = g.box * (long long)(sizeof(T) / 4);
   __syncthreads();
   if (tid == 0) *mine = base + iters;
 
@@ -180,21 +147,16 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
 
     // ---- exchange with the neighbours ----
     const unsigned tag = base + q + 1;
-    unsigned long long *const w0 = words + (q & 1) * 3 * field, *const w1 = w0 + field, *const ws = w1 + field;
+    Word *const word = words + (q & 1) * g.box * words_of<T>() + e;
     bool lost = false;
     if (ring) {
-      send(w0, e, u0, tag);
-      send(w1, e, u1, tag);
-      send(ws, e, v, tag);
+      send(word, g.box, u0, u1, v, tag);
     } else if (box && !owned) {
       const bool shear = vin && !vown;
       const long long t0 = clock64();
       for (unsigned n = 1;; ++n) {
         T a, b, c = tsh;
-        bool ok = receive(w0, e, tag, &a);
-        ok = receive(w1, e, tag, &b) && ok;
-        if (shear) ok = receive(ws, e, tag, &c) && ok;
-        if (ok) {
+        if (receive(word, g.box, tag, &a, &b, &c, shear)) {
           u0 = a;
           u1 = b;
           tsh = c;
@@ -276,7 +238,7 @@ int resident2d_config(const Geo &g) {
 
 template <typename T>
 cudaError_t launch_resident2d(int c, const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int iters,
-                              unsigned *count, unsigned long long *words, cudaStream_t st) {
+                              unsigned *count, Word *words, cudaStream_t st) {
   const int wx = config<T>(c).wx, wy = config<T>(c).wy;
   Geo gg = g;
   Stage<T> SS = S;
@@ -288,8 +250,8 @@ cudaError_t launch_resident2d(int c, const Geo &g, const Stage<T> &S, const Scal
 template int resident2d_config<float>(const Geo &);
 template int resident2d_config<double>(const Geo &);
 template cudaError_t launch_resident2d<float>(int, const Geo &, const Stage<float> &, const Scal *, DevInfo *, int,
-                                              unsigned *, unsigned long long *, cudaStream_t);
+                                              unsigned *, Word *, cudaStream_t);
 template cudaError_t launch_resident2d<double>(int, const Geo &, const Stage<double> &, const Scal *, DevInfo *, int,
-                                               unsigned *, unsigned long long *, cudaStream_t);
+                                               unsigned *, Word *, cudaStream_t);
 
 }  // namespace ep

@@ -191,3 +191,14 @@ def test_resident_2d_iterations_equal_the_two_launch_sweep(P, n, precision, opts
         np.testing.assert_array_equal(out[k], ref[k])
     for k in ("iters", "max_sigma", "eps_rel", "eps_res"):
         assert info[k] == iref[k]
+
+
+@pytest.mark.parametrize("n", [(3, 2, 2), (15, 15, 1), (27, 19, 5), (31, 9, 33), (90, 40, 24), (70, 30, 40)])
+@pytest.mark.parametrize("opts", [{}, {"mu_s": 1e-3, "jaumann": False, "incompressible": True}, {"freeze_iter": 6}])
+def test_resident_3d_iterations_match_the_staged_sweep_fp32(P, n, opts):
+    """One launch per chunk: blocks of one point and of many, remainders in each direction."""
+    iters = 24
+    f = _fields(P, 3, n, 12)
+    iref, ref = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f, chunk=6, **opts)
+    info, out = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_AUTO, iters, f, chunk=6, **opts)
+    _compare(f, out, ref, info, iref, iters, EPS32)

@@ -509,26 +509,28 @@ def aggregate(torch, dist, seconds, units, device):
 
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the
-# dominant kernel from one ncu capture of the benchmark command, by kernel and
-# box size; the entry must be dropped when the kernel changes.
-# DRAM bytes per launch of the dominant kernel from an ncu capture of its
-# current build (profiles/k_fused3d_reg_127cube.md)
-NCU_TRAFFIC = {("k_fused3d_reg", 127): 271.3e6,
-               ("k_fused3d_reg", 511): 271.3e6 * 133432831 / 2048383}
-NCU_SOURCE = {("k_fused3d_reg", 127): "ncu --set full capture of one launch at 127^3 (profiles/)",
-              ("k_fused3d_reg", 511): "ncu --set full capture of one launch at 127^3 (profiles/), the per-cell "
+# dominant kernel from an ncu capture of its current build
+# (profiles/k_fused3d_reg_127cube.md), by kernel and box size; the entry must be
+# dropped when the kernel changes.
+NCU_TRAFFIC = {("k_fused3d_reg", 127): 267.9e6,
+               ("k_fused3d_reg", 511): 267.9e6 * 133432831 / 2048383}
+NCU_SOURCE = {("k_fused3d_reg", 127): "ncu capture of one launch at 127^3 (profiles/)",
+              ("k_fused3d_reg", 511): "ncu capture of one launch at 127^3 (profiles/), the per-cell "
                                       "traffic scaled to 511^3 by the cell count"}
 # FP64 flops per cell of one staged FP64 sweep (dadd + dmul + 2 dfma thread
 # instructions of its five kernels, counted by ncu at 127^3; profiles/)
-FP64_FLOPS_PER_CELL = 322.5
+FP64_FLOPS_PER_CELL = 206.4
 # algorithmic bytes per cell of a 3D FP32 sweep recast so that its stress is
 # no pseudo-time state (reported beside the fraction by the scheme's bytes)
 RECAST_BYTES_3D_FP32 = 80.0
 
 
-def kernel_names(ktimes, kernel):
+def kernel_names(ktimes, kernel, precision):
+    """Kernels of the 3D sweep that time_sweep timed (its last entry is the whole iteration)."""
     if len(ktimes) == 2:
         return [{"tma": "k_fused3d_tma", "reg": "k_fused3d_reg", "fused": "k_fused3d"}.get(kernel, "k_fused3d_reg")]
+    if precision == "fp64":
+        return ["k64_strain", "k64_trial", "k64_centres", "k64_edges", "k64_velocity"]
     return ["k_strain", "k_trial", "k_return_centres", "k_return_edges", "k_velocity"]
 
 
@@ -706,7 +708,7 @@ def our_arm(args):
     g.restore()
     g.apply_increment(s.a, s.dt, P.LOAD_XZ)
     ktimes = g.time_sweep(10 if s.n[0] > 300 else 20)
-    kernels = kernel_names(ktimes, args.kernel)
+    kernels = kernel_names(ktimes, args.kernel, args.precision)
     it_ms = ktimes[-1]
     dom = int(max(range(len(kernels)), key=lambda q: ktimes[q]))
     g.close()

@@ -47,11 +47,16 @@ __device__ __forceinline__ double el(double v) { return v; }
 
 // centre scale min(1, Y / sqrt(J2)).  FP32: compare squares and scale with
 // the reciprocal square root only where the return acts (most cells stay
-// elastic).  FP64: below Y^2 by more than the rounding of both, sqrt(J2) > Y
+// elastic), refined by a Newton step: its 2 ulp act on the same cells in every
+// iteration (95^3 with a per-cell modulus, error against 64 bits after 200 of them:
+// 11 % above that of sqrt and division, with the step 3 %; 52 -> 54 us an iteration,
+// 67 with sqrt and division).  FP64: below Y^2 by more than the rounding of both, sqrt(J2) > Y
 // cannot hold and the scale is 1 without the root.
 __device__ __forceinline__ float scale_of(float J2, float Y) {
   Y = Y > 0.f ? Y : 0.f;
-  return J2 > Y * Y ? Y * rsqrtf(J2) : 1.f;
+  if (!(J2 > Y * Y)) return 1.f;
+  const float r = rsqrtf(J2), q = Y * r, s = fmaf(0.5f * q, fmaf(-J2 * r, r, 1.f), q);
+  return s > 1.f ? 1.f : s;
 }
 __device__ __forceinline__ double scale_of(double J2, double Y) {
   Y = Y > 0.0 ? Y : 0.0;

@@ -30,7 +30,7 @@
 // 255 registers), halved the instructions and gained nothing: the loads'
 // latency showed.  cp.async in place of TMA cost 5 shared-memory wavefronts
 // per 8-byte copy (the window starts off a 32-byte sector): 131 and 2164 us.
-// With a per-cell shear modulus (31 inputs, 16 rows) 95^3 takes 52 us, the five
+// With a per-cell shear modulus (31 inputs, 16 rows) 95^3 takes 55 us, the five
 // staged kernels 100.
 // Instruction count:
 //   * FP32 arithmetic is packed (add/mul/fma on float2: one instruction per

@@ -485,7 +485,6 @@ template void launch_fill<float>(const FillTab &, long long, cudaStream_t);
 template void launch_fill<double>(const FillTab &, long long, cudaStream_t);
 template void launch_convert<float, double>(float *, const double *, long long, cudaStream_t);
 template void launch_convert<double, float>(double *, const float *, long long, cudaStream_t);
-template void launch_convert<double, double>(double *, const double *, long long, cudaStream_t);
 
 void launch_scaled_div(const Geo &g, const double *const v[3], double scale, double *out, cudaStream_t st) {
   k_scaled_div<<<blocks_for(g.box), kThreads, 0, st>>>(g, v[0], v[1], v[2], scale, out);

@@ -49,7 +49,7 @@ __device__ __forceinline__ double el(double v) { return v; }
 // the reciprocal square root only where the return acts (most cells stay
 // elastic), refined by a Newton step: its 2 ulp act on the same cells in every
 // iteration (95^3 with a per-cell modulus, error against 64 bits after 200 of them:
-// 11 % above that of sqrt and division, with the step 3 %; 52 -> 54 us an iteration,
+// 11 % above that of sqrt and division, with the step 3 %; 54.0 -> 55.6 us an iteration,
 // 67 with sqrt and division).  FP64: below Y^2 by more than the rounding of both, sqrt(J2) > Y
 // cannot hold and the scale is 1 without the root.
 __device__ __forceinline__ float scale_of(float J2, float Y) {

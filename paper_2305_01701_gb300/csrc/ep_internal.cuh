@@ -191,8 +191,9 @@ cudaError_t launch_resident3d(const int tile[3], const Geo &g, const Stage<float
 // a configuration that holds the whole grid on the chip at once, or -1
 template <typename T>
 int resident2d_config(const Geo &g);
-// `iters` (odd) iterations from S.u, S.son .. to S.uo, S.snn ..; `count` and `words`
-// are zero when a solve starts and its own until it ends
+// `iters` (odd) iterations from S.u, S.son .. to S.uo, S.snn ..; the stresses before the
+// last of them go to S.son .. (3D likewise).  `count` and `words` are zero when a solve
+// starts and its own until it ends
 template <typename T>
 cudaError_t launch_resident2d(int config, const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int iters,
                               unsigned *count, Word *words, cudaStream_t st);

@@ -129,6 +129,17 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
       tsh = v;
     }
     sn[ty][tx] = v;
+    // the stresses that the last iteration starts from stay where the launch found its own:
+    // a commit before the solve is decided takes them.  Every neighbour has read that state:
+    // it sent the words of iteration 0 since.
+    if (q == iters - 2 && owned) {
+      const_cast<T *>(S.sos[0])[e] = vin ? tsh : (T)0;
+      if (cin) {
+        const_cast<T *>(S.son[0])[e] = n0;
+        const_cast<T *>(S.son[1])[e] = n1;
+        const_cast<T *>(S.sop)[e] = pr;
+      }
+    }
     __syncthreads();
     // ---- faces: residual and velocity update ----
     if (fx) {

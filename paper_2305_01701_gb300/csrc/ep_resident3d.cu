@@ -308,6 +308,20 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
       if (in & 4) n2[m] = v2;
     }
     __syncthreads();
+    // the stresses that the last iteration starts from stay where the launch found its own:
+    // a commit before the solve is decided takes them.  Every neighbour has read that state:
+    // it sent the words of iteration 0 since.
+    if (q == iters - 2 && owned) {
+      const_cast<float *>(S.sos[0])[e] = n0[l];
+      const_cast<float *>(S.sos[1])[e] = n1[l];
+      const_cast<float *>(S.sos[2])[e] = n2[l];
+      if (cin) {
+        const_cast<float *>(S.son[0])[e] = c0;
+        const_cast<float *>(S.son[1])[e] = c1;
+        const_cast<float *>(S.son[2])[e] = c2;
+        const_cast<float *>(S.sop)[e] = pr;
+      }
+    }
     // ---- 5: residual and velocity of the own faces ----
     float un0 = 0.f, un1 = 0.f, un2 = 0.f;
     if (owned) {

@@ -49,6 +49,7 @@ def _fields(P, nd, n, seed):
 def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
     opts = dict(opts)
     force = opts.pop("force", 0.0)
+    pending = opts.pop("pending", 0)   # commit after so many chunks, the solve undecided
     g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=precision)
     rng = np.random.default_rng(1)
     g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, 1.5e-3 * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
@@ -60,7 +61,7 @@ def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
         g.set(k, a)
     bf = force * rng.standard_normal(sum(f["v" + c].size for c in "xyz"[:nd])) if force else None
     g.apply_increment(1.0, 1e-4, P.LOAD_XY if nd == 2 else P.LOAD_XZ, bf)
-    info = g.solve_increment(raise_on_fail=False)
+    info = g.solve_chunks(pending) if pending else g.solve_increment(raise_on_fail=False)
     g.commit_increment()
     out = {k: g.get(k) for k in list(f) + ["epl", "scale"]}
     g.close()
@@ -202,3 +203,22 @@ def test_resident_3d_iterations_match_the_staged_sweep_fp32(P, n, opts):
     iref, ref = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_STAGED, iters, f, chunk=6, **opts)
     info, out = _solve(P, 3, n, P.FP32_MIXED, P.KERNEL_AUTO, iters, f, chunk=6, **opts)
     _compare(f, out, ref, info, iref, iters, EPS32)
+
+
+@pytest.mark.parametrize("nd,n,precision", [(2, (24, 25), "fp64"), (2, (64, 64), "fp64"), (2, (300, 180), "fp32"),
+                                            (3, (27, 19, 5), "fp32"), (3, (90, 40, 24), "fp32")])
+@pytest.mark.parametrize("chunk", [2, 4, 10])
+def test_commit_of_an_undecided_solve_takes_the_newest_iterate(P, nd, n, precision, chunk):
+    """Whole chunks, then a commit while the stopping test has not decided: the resident kernels
+    leave the state where the launch-per-iteration sweeps do."""
+    iters = 20
+    f = _fields(P, nd, n, 13)
+    pr = P.FP64 if precision == "fp64" else P.FP32_MIXED
+    (iref, ref), (info, out) = (_solve(P, nd, n, pr, k, 1000, f, chunk=chunk, pending=iters // chunk)
+                                for k in (P.KERNEL_STAGED, P.KERNEL_AUTO))
+    assert info["status"] == iref["status"] == P.PENDING
+    if nd == 2:
+        for k in out:
+            np.testing.assert_array_equal(out[k], ref[k])
+    else:
+        _compare(f, out, ref, info, iref, iters, EPS32)

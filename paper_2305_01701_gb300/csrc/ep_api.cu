@@ -587,10 +587,11 @@ bool fused_check(const ep_grid *h) {
 
 // one fused 3D iteration in the grid's chosen flavour
 template <typename T>
-bool launch_fused_any(const ep_grid *h, const Stage<T> &S, DevInfo *di, cudaStream_t st, bool check = false) {
+bool launch_fused_any(const ep_grid *h, const Stage<T> &S, DevInfo *di, cudaStream_t st, bool check = false,
+                      bool last = false) {
   const int v = fused_variant(h);
   if (v == EP_KERNEL_FUSED_TMA) return launch_fused3d_tma<T>(h->g, S, h->dscal, di, h->kz, st);
-  if (v == EP_KERNEL_FUSED_REG) return launch_fused3d_reg<T>(h->g, S, h->dscal, di, h->kz, st, check);
+  if (v == EP_KERNEL_FUSED_REG) return launch_fused3d_reg<T>(h->g, S, h->dscal, di, h->kz, st, check, last);
   launch_fused3d<T>(h->g, S, h->dscal, di, h->kz, st);
   return true;
 }
@@ -658,7 +659,7 @@ ep_status capture_chunk(ep_grid *h) {
       }
     }
     if ((!chk || fused_check<T>(h)) && use_fused<T>(h)) {
-      if (!launch_fused_any<T>(h, S, h->dinfo, h->cap, chk)) {
+      if (!launch_fused_any<T>(h, S, h->dinfo, h->cap, chk, it == h->opts.n_chk - 1)) {
         cudaGraph_t gr;
         cudaStreamEndCapture(h->cap, &gr);
         if (gr) cudaGraphDestroy(gr);

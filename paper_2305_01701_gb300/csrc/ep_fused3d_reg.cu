@@ -142,6 +142,7 @@ template <typename T>
 struct Args {
   T *snn[3], *sns[3], *snp, *uo[3];
   T *s;   // centre return scales (read when plasticity is frozen, written by checks)
+  bool keep_s;   // written by this iteration too (GC: the last one of a chunk)
   T *cn[3], *cs[3], *cp, *uchk[3];   // state at the previous check (check iterations)
   const double *v0[3];               // start velocity (check iterations)
 };
@@ -509,6 +510,8 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
           one(std::integral_constant<int, 0>{});
           if constexpr (N == 2) one(std::integral_constant<int, 1>{});
           stc(A.cn[0], n0); stc(A.cn[1], n1); stc(A.cn[2], n2); stc(A.cp, pr);
+        } else if constexpr (GC) {
+          if (A.keep_s && !frozen) stc(A.s, sc1);
         }
       }
       s_1 = vmul(sc1, bc(qr));
@@ -713,16 +716,18 @@ bool launch_off(const Stage<typename L::T> &S, const Args<typename L::T> &A, con
 // One fused iteration, register z-march flavour: reads buffer b of the
 // stage, writes 1 - b.  check (FP32 only): a check iteration, which also
 // reduces the stopping measures into di and updates the check snapshots.
+// last: the last iteration of a chunk, whose return scales a commit of the
+// undecided solve reads (stored with a per-cell modulus).
 // Returns false if a tensor map could not be made.
 template <typename T>
 bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
-                        bool check) {
+                        bool check, bool last) {
   Args<T> A;
   for (int d = 0; d < 3; ++d) {
     A.snn[d] = S.snn[d]; A.sns[d] = S.sns[d]; A.uo[d] = S.uo[d];
     A.cn[d] = S.cn[d]; A.cs[d] = S.cs[d]; A.uchk[d] = S.uchk[d]; A.v0[d] = S.v0[d];
   }
-  A.snp = S.snp; A.s = S.s; A.cp = S.cp;
+  A.snp = S.snp; A.s = S.s; A.keep_s = last; A.cp = S.cp;
   if constexpr (sizeof(T) == 8) {
     return launch_off<LaneD, false, false>(S, A, g, sc, di, kz, st);
   } else if (S.ge[0]) {
@@ -752,8 +757,8 @@ cudaError_t fused3d_reg_configure() {
 }
 
 template bool launch_fused3d_reg<float>(const Geo &, const Stage<float> &, const Scal *, DevInfo *, int, cudaStream_t,
-                                        bool);
+                                        bool, bool);
 template bool launch_fused3d_reg<double>(const Geo &, const Stage<double> &, const Scal *, DevInfo *, int,
-                                         cudaStream_t, bool);
+                                         cudaStream_t, bool, bool);
 
 }  // namespace ep

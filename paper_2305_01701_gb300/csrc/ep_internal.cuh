@@ -289,7 +289,7 @@ cudaError_t fused3d_tma_configure();
 // register z-march variant (ep_fused3d_reg.cu); false if a tensor map failed
 template <typename T>
 bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
-                        bool check = false);
+                        bool check = false, bool last = false);
 cudaError_t fused3d_reg_configure();
 
 // ---- increment set-up and commit (FP64; ep_increment.cu) ------------------

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 
 namespace ep {
 
@@ -45,18 +46,21 @@ __device__ __forceinline__ float el(float2 v) { return E == 0 ? v.x : v.y; }
 template <int E>
 __device__ __forceinline__ double el(double v) { return v; }
 
-// centre scale min(1, Y / sqrt(J2)).  FP32: compare squares and scale with
-// the reciprocal square root only where the return acts (most cells stay
-// elastic), refined by a Newton step: its 2 ulp act on the same cells in every
-// iteration (95^3 with a per-cell modulus, error against 64 bits after 200 of them:
-// 11 % above that of sqrt and division, with the step 3 %; 54.0 -> 55.6 us an iteration,
-// 67 with sqrt and division).  FP64: below Y^2 by more than the rounding of both, sqrt(J2) > Y
-// cannot hold and the scale is 1 without the root.
+// centre scale min(1, Y / sqrt(J2)).  FP32: compare squares, and only where the return
+// acts (most cells stay elastic) form the quotient from the reciprocal square root r: J2 r
+// and its residual give the root as a sum t + d, and one Newton step on the quotient s = Y r
+// takes its residual Y - s (t + d) with fused multiply-adds.  The result is the rounded
+// quotient but for near-ties (0.5 ulp; a rounded root and a division make 1): an error of the
+// scale acts on the same cells in every iteration (95^3 with a per-cell modulus, error against
+// 64 bits after 200 of them, median of 16 inputs over that of sqrt and division: 0.99, without
+// the residuals 1.01; 55.8 -> 57.4 us an iteration, 67 with sqrt and division).  FP64: below Y^2 by more than the rounding
+// of both, sqrt(J2) > Y cannot hold and the scale is 1 without the root.
 __device__ __forceinline__ float scale_of(float J2, float Y) {
   Y = Y > 0.f ? Y : 0.f;
   if (!(J2 > Y * Y)) return 1.f;
-  const float r = rsqrtf(J2), q = Y * r, s = fmaf(0.5f * q, fmaf(-J2 * r, r, 1.f), q);
-  return s > 1.f ? 1.f : s;
+  const float r = rsqrtf(J2), t = J2 * r, d = fmaf(-t, t, J2) * (0.5f * r), s = Y * r;
+  const float q = fmaf(fmaf(-s, d, fmaf(-s, t, Y)), r, s);
+  return !(J2 < INFINITY) ? s : q > 1.f ? 1.f : q;   // s = 0 where the invariant overflows
 }
 __device__ __forceinline__ double scale_of(double J2, double Y) {
   Y = Y > 0.0 ? Y : 0.0;

@@ -263,7 +263,7 @@ double eta_ve(const ep_grid *h) {
 
 template <typename T>
 void fill_scal(const Scal &s, const Geo &g, SweepScal<T> *o) {
-  o->two_eta = (T)s.two_eta; o->eta = (T)(0.5 * s.two_eta); o->eta_d = (T)(-s.two_eta / 3.0);
+  o->two_eta = (T)s.two_eta; o->eta = (T)(0.5 * s.two_eta);
   o->bt = (T)s.bt; o->ob = (T)1 - o->bt; o->bp = (T)s.bp; o->obp = (T)s.obp;
   o->KDt = (T)s.KDt; o->KDt_phys = (T)s.KDt_phys; o->A = (T)s.A; o->vstep = (T)s.vstep;
   o->rdx = (T)g.rdx; o->rdy = (T)g.rdy; o->rdz = (T)g.rdz;

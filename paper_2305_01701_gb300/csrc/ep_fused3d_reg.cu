@@ -262,7 +262,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
 
   const SweepScal<T> &Q = sweep_scal<T>(sc);
   const T rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz;
-  const T eta = Q.eta, two_eta = Q.two_eta, eta_d = Q.eta_d, bt = Q.bt, ob = Q.ob;
+  const T eta = Q.eta, two_eta = Q.two_eta, bt = Q.bt, ob = Q.ob;
   const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Acoef = Q.A;
   const T vs = Q.vstep, qr = (T)0.25, e8 = (T)0.125, e32 = (T)0.03125;
   // velocity step of x-, y- and z-faces: 0 on the walls and off the extent
@@ -442,17 +442,21 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
         div = vadd(vadd(e0, e1), e2);
         const V O = vadd(pyz, S.pyz.r[qp]);
         const V Pxz = vadd(N_1, vN), Pyz = vadd(O_1, O), Pxy = M_1;
+        // the deviatoric rate is formed before it is scaled: 2 eta e and -2 eta div / 3 as
+        // two terms would round each at the size of the larger
+        const V m3 = bc((T)(-1.0 / 3.0)), d0 = vfma(div, m3, e0), d1 = vfma(div, m3, e1), d2 = vfma(div, m3, e2);
+        const V r0 = vadd(Pxy, Pxz), r1 = vsub(Pyz, Pxy), r2 = vadd(Pxz, Pyz);
         V t0, t1, t2;
         if constexpr (GC) {
-          const V te = own(I_GEN), q = vmul(own(I_GCN), bc(qr)), d3 = vmul(div, bc((T)(1.0 / 3.0)));
-          t0 = vfma(vadd(Pxy, Pxz), q, vfma(vsub(e0, d3), te, own(I_TBN0)));
-          t1 = vfma(vsub(Pyz, Pxy), q, vfma(vsub(e1, d3), te, own(I_TBN1)));
-          t2 = vfma(vsub(zero, vadd(Pxz, Pyz)), q, vfma(vsub(e2, d3), te, own(I_TBN2)));
+          const V te = own(I_GEN), q = vmul(own(I_GCN), bc(qr));
+          t0 = vfma(r0, q, vfma(d0, te, own(I_TBN0)));
+          t1 = vfma(r1, q, vfma(d1, te, own(I_TBN1)));
+          t2 = vfma(vsub(zero, r2), q, vfma(d2, te, own(I_TBN2)));
         } else {
-          const V m = vmul(div, bc(eta_d)), te = bc(two_eta), q = bc(qr);
-          t0 = vfma(vadd(Pxy, Pxz), q, vadd(own(I_TBN0), vfma(e0, te, m)));
-          t1 = vfma(vsub(Pyz, Pxy), q, vadd(own(I_TBN1), vfma(e1, te, m)));
-          t2 = vfma(vadd(Pxz, Pyz), bc(-qr), vadd(own(I_TBN2), vfma(e2, te, m)));
+          const V te = bc(two_eta);
+          t0 = vfma(r0, bc(qr), vfma(d0, te, own(I_TBN0)));
+          t1 = vfma(r1, bc(qr), vfma(d1, te, own(I_TBN1)));
+          t2 = vfma(r2, bc(-qr), vfma(d2, te, own(I_TBN2)));
         }
         c0v = vfma(own(I_SON0), bc(bt), vmul(t0, bc(ob)));
         c1v = vfma(own(I_SON1), bc(bt), vmul(t1, bc(ob)));

@@ -33,7 +33,7 @@ struct Geo {
 // 15.9 us a sweep; 383 x 191: 9.0 -> 8.4 us).
 template <typename T>
 struct SweepScal {
-  T two_eta, eta, eta_d;       // 2 eta_ve, eta_ve, -2 eta_ve / 3
+  T two_eta, eta;              // 2 eta_ve, eta_ve
   T bt, ob, bp, obp, KDt, KDt_phys, A, vstep;
   T rdx, rdy, rdz;
 };

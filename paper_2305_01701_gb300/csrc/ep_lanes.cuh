@@ -50,11 +50,12 @@ __device__ __forceinline__ double el(double v) { return v; }
 // acts (most cells stay elastic) form the quotient from the reciprocal square root r: J2 r
 // and its residual give the root as a sum t + d, and one Newton step on the quotient s = Y r
 // takes its residual Y - s (t + d) with fused multiply-adds.  The result is the rounded
-// quotient but for near-ties (0.5 ulp; a rounded root and a division make 1): an error of the
+// quotient but for near-ties (0.5 ulp; a rounded root and a division make 1.5): an error of the
 // scale acts on the same cells in every iteration (95^3 with a per-cell modulus, error against
 // 64 bits after 200 of them, median of 16 inputs over that of sqrt and division: 0.99, without
-// the residuals 1.01; 55.8 -> 57.4 us an iteration, 67 with sqrt and division).  FP64: below Y^2 by more than the rounding
-// of both, sqrt(J2) > Y cannot hold and the scale is 1 without the root.
+// the residuals 1.01; 55.8 -> 57.4 us an iteration, 67 with sqrt and division).  FP64: below
+// Y^2 by more than the rounding of both, sqrt(J2) > Y cannot hold and the scale is 1 without
+// the root.
 __device__ __forceinline__ float scale_of(float J2, float Y) {
   Y = Y > 0.f ? Y : 0.f;
   if (!(J2 > Y * Y)) return 1.f;

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
   const int nx = g.nx, ny = g.ny, px = g.px;   // a 2D box has fewer than 2^31 points
   const int gi = blockIdx.x * (WX - 4) - 2 + tx, gj = blockIdx.y * (WY - 4) - 2 + ty, e = gj * px + gi;
   const SweepScal<T> &Q = sweep_scal<T>(sc);
-  const T two_eta = Q.two_eta, eta = Q.eta, eta_d = Q.eta_d, bt = Q.bt, ob = Q.ob;
+  const T two_eta = Q.two_eta, eta = Q.eta, bt = Q.bt, ob = Q.ob;
   const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Ac = Q.A, rdx = Q.rdx, rdy = Q.rdy, vs = Q.vstep;
 
   const bool box = gi >= 0 && gi <= nx && gj >= 0 && gj <= ny;
@@ -104,9 +104,9 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
       const T xy = (p + sp[ty + 1][tx]) + (sp[ty][tx + 1] + sp[ty + 1][tx + 1]);
       const T txy = (ts + st[ty + 1][tx]) + (st[ty][tx + 1] + st[ty + 1][tx + 1]);
       const T e0 = (su0[ty][tx + 1] - u0) * rdx, e1 = (su1[ty + 1][tx] - u1) * rdy;
-      const T div = e0 + e1, m = div * eta_d;
-      const T t0 = fma((T)0.25, xy, fma(two_eta, e0, tb0 + m));
-      const T t1 = fma((T)-0.25, xy, fma(two_eta, e1, tb1 + m));
+      const T div = e0 + e1, m3 = (T)(-1.0 / 3.0);
+      const T t0 = fma((T)0.25, xy, fma(two_eta, fma(div, m3, e0), tb0));
+      const T t1 = fma((T)-0.25, xy, fma(two_eta, fma(div, m3, e1), tb1));
       const T c0 = fma(bt, n0, ob * t0), c1 = fma(bt, n1, ob * t1);
       pr = fma(bp, pr, obp * fma(-KDt, div, pb));
       if (!frozen) {

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
   const int px = g.px;   // a 2D box has fewer than 2^31 points
   const bool frozen = di != nullptr && di->frozen;
   const SweepScal<T> &Q = sweep_scal<T>(sc);
-  const T two_eta = Q.two_eta, eta = Q.eta, eta_d = Q.eta_d, bt = Q.bt, ob = Q.ob;
+  const T two_eta = Q.two_eta, eta = Q.eta, bt = Q.bt, ob = Q.ob;
   const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Ac = Q.A, rdx = Q.rdx, rdy = Q.rdy;
   const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
   T sig = 0, dtau = 0, dp = 0;
@@ -116,9 +116,9 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
     if (own) S.Ts[0][e] = t_j;
     if (own && i < nx && j < ny) {
       const T e0 = (u0_r - u0) * rdx, e1 = (S.u[1][e + px] - S.u[1][e]) * rdy;
-      const T div = e0 + e1, m = div * eta_d;
-      const T t0 = fma((T)0.25, xy, fma(two_eta, e0, S.tbn[0][e] + m));
-      const T t1 = fma((T)-0.25, xy, fma(two_eta, e1, S.tbn[1][e] + m));
+      const T div = e0 + e1, m3 = (T)(-1.0 / 3.0);
+      const T t0 = fma((T)0.25, xy, fma(two_eta, fma(div, m3, e0), S.tbn[0][e]));
+      const T t1 = fma((T)-0.25, xy, fma(two_eta, fma(div, m3, e1), S.tbn[1][e]));
       const T c0 = fma(bt, S.son[0][e], ob * t0), c1 = fma(bt, S.son[1][e], ob * t1);
       const T pr = fma(bp, S.sop[e], obp * fma(-KDt, div, S.pb[e]));
       T s = 1;

@@ -49,10 +49,11 @@ def _fields(P, nd, n, seed):
 def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
     opts = dict(opts)
     force = opts.pop("force", 0.0)
+    cohesion = 1.5e-3 * (1e3 if opts.pop("elastic", False) else 1.0)
     pending = opts.pop("pending", 0)   # commit after so many chunks, the solve undecided
     g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=precision)
     rng = np.random.default_rng(1)
-    g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, 1.5e-3 * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
+    g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, cohesion * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
     if "cell_g" in opts:
         g.set_shear_modulus(1.0 + 0.2 * opts.pop("cell_g") * rng.random(int(np.prod(n))))
     g.set_solver(tol=0.0, max_iter=iters, n_chk=opts.pop("chunk", iters // 2), **opts)
@@ -239,3 +240,19 @@ def test_commit_of_an_undecided_solve_with_a_per_cell_modulus(P, n):
     # a cell within rounding of yield may return on one side only
     differ = np.count_nonzero((out["epl"] > 0.0) != (ref["epl"] > 0.0))
     assert differ <= max(1, out["epl"].size // 1000), differ
+
+
+@pytest.mark.parametrize("n", [(61, 33), (130, 90), (300, 180)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_elastic_iterations_without_rotation_round_alike_in_every_2d_kernel(P, n, precision):
+    """The deviatoric rate is formed first and scaled once, in one order: strips, the launches per
+    iteration and the resident iterations give the same bits where neither the return nor the
+    rotation's means (whose sums each kernel shares in its own way) take part."""
+    f = _fields(P, 2, n, 15)
+    pr = P.FP64 if precision == "fp64" else P.FP32_MIXED
+    opts = dict(chunk=6, jaumann=False, elastic=True)
+    _, ref = _solve(P, 2, n, pr, P.KERNEL_FUSED, 24, f, shape=4, **opts)
+    for kernel in (P.KERNEL_STAGED, P.KERNEL_AUTO):
+        _, out = _solve(P, 2, n, pr, kernel, 24, f, **opts)
+        for k in out:
+            np.testing.assert_array_equal(out[k], ref[k])

@@ -108,11 +108,12 @@ typedef struct {
    * starts at the old pressure, and its stopping measure is 2 eta_ve times
    * the interval-averaged |div v| relative to max|sigma|.  Default 0. */
   int incompressible;
-  /* bound, in SM clock cycles, of each wait of the TMA sweep kernel
-   * (EP_KERNEL_FUSED_TMA) for its plane copies; 0 (default) is 2^31 cycles,
-   * about a second.  A wait that runs out ends the solve with
-   * EP_ERR_TIMEOUT after the block has waited (with the default bound) for
-   * the copies it issued; the handle stays usable. */
+  /* bound, in SM clock cycles, of each device wait of a sweep: of the TMA and
+   * register sweeps for their plane copies, of the resident sweeps' blocks
+   * for one another; 0 (default) is 2^31 cycles, about a second.  A wait that
+   * runs out ends the solve with EP_ERR_TIMEOUT after the block has waited
+   * (with the default bound) for the copies it issued; the handle stays
+   * usable.  Taken over when an increment is applied. */
   long long wait_cycles;
 } ep_solver_opts;
 
@@ -215,15 +216,15 @@ ep_status ep_set_fields(ep_handle h, int field, const double *host_in, size_t co
  * FP32 up to about 118,000 points, in FP64 up to about 20,000) and a 3D FP32
  * grid with a uniform modulus and no body force of up to about 100,000 points
  * run the iterations between two checks in one cooperative launch (in 2D with
- * the same results bit for bit); its blocks wait for one another, bounded at
- * 2^31 cycles (then EP_ERR_TIMEOUT).  ep_time_sweep times the other kernels
+ * the same results bit for bit); its blocks wait for one another, bounded by
+ * wait_cycles (then EP_ERR_TIMEOUT).  ep_time_sweep times the other kernels
  * there.
  * EP_KERNEL_STAGED / EP_KERNEL_FUSED force one;
  * EP_KERNEL_FUSED_TMA is the 3D fused sweep with every plane streamed by
  * the tensor-memory accelerator (a timed-out copy ends the solve with
  * EP_ERR_TIMEOUT); EP_KERNEL_FUSED_REG is the 3D fused sweep that keeps the
  * z-march in registers (threads own x columns, half warps own y rows; planes
- * streamed by the tensor-memory accelerator, waits bounded at 2^31 cycles).  The check
+ * streamed by the tensor-memory accelerator, waits bounded alike).  The check
  * iteration of each chunk runs fused too with the FP32 register sweep (it
  * reduces the stopping measures itself); the other 3D flavours and FP64
  * grids take the staged sweep for it.  A body force always uses the staged

@@ -50,8 +50,9 @@
 //     points (FP32);
 //   * warps whose rows are never written skip the steps that only written
 //     rows need.
-// Waits are bounded: one that runs out marks the grid's record (status 4), the
-// block waits (bounded) for the copies in flight and returns.
+// Waits are bounded (ep_solver_opts.wait_cycles): one that runs out marks the grid's
+// record (status 4), the block waits, with the default bound, for the copies in flight
+// and returns.
 // Check iterations (FP32, CHK = true) also reduce the stopping measures of
 // Eqs. Convergence1-3 over the points each block writes, the same point sets
 // and the same snapshot updates as the staged check iteration: max|sigma|,
@@ -167,22 +168,34 @@ __device__ __forceinline__ unsigned su32(const void *p) { return (unsigned)__cvt
 __device__ __forceinline__ void bar_expect(unsigned long long *b, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(su32(b)), "r"(bytes) : "memory");
 }
-// bounded wait for a phase of b: gives up after 2^31 SM cycles (about a
-// second, far above any copy's latency)
-__device__ __forceinline__ bool bar_wait(unsigned long long *b, unsigned parity) {
+// bounded wait for a phase of b: gives up after the grid's bound (sc null: the default, far
+// above any copy's latency).  A bound below the default polls with test_wait, which does
+// not suspend the thread, so that the bound decides when the wait gives up.
+__device__ __forceinline__ bool bar_test(unsigned long long *b, unsigned parity) {
   unsigned ok;
-  long long t0 = 0;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(su32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool bar_wait(unsigned long long *b, unsigned parity, const Scal *sc) {
+  if (bar_test(b, parity)) return true;
+  const long long limit = sc ? wait_limit(sc) : WAIT_DEFAULT, t0 = clock64();
   do {
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
+    unsigned ok;
+    if (limit < WAIT_DEFAULT)
+      ok = bar_test(b, parity);
+    else
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+          : "=r"(ok)
+          : "r"(su32(b)), "r"(parity)
+          : "memory");
     if (ok) return true;
-    const long long now = clock64();
-    if (t0 == 0) t0 = now;
-    if (now - t0 > (1ll << 31)) return false;
-  } while (true);
+  } while (clock64() - t0 <= limit);
+  return false;
 }
 __device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int x, int y, int z,
                                          unsigned long long *b) {
@@ -320,12 +333,12 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
   // anywhere in the block: the record then says so and the copies in flight
   // (a plane in each stage at most) have been waited for
   auto arrived = [&](const int stage, bool other) -> bool {
-    const bool ok = bar_wait(&S.full[stage], ph[stage]);
+    const bool ok = bar_wait(&S.full[stage], ph[stage], sc);
     ph[stage] ^= 1u;
     if (!__syncthreads_or(!ok)) return true;
     if (threadIdx.x == 0 && di != nullptr) di->done = 4;
-    if (!ok) bar_wait(&S.full[stage], ph[stage] ^ 1u);
-    if (other) bar_wait(&S.full[stage ^ 1], ph[stage ^ 1]);
+    if (!ok) bar_wait(&S.full[stage], ph[stage] ^ 1u, nullptr);
+    if (other) bar_wait(&S.full[stage ^ 1], ph[stage ^ 1], nullptr);
     return false;
   };
   if (!arrived(0, true)) return;

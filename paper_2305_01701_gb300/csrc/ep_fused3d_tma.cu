@@ -77,9 +77,8 @@ __device__ __forceinline__ bool bar_try(unsigned long long *b, unsigned parity) 
       : "memory");
   return ok != 0;
 }
-// bounded wait: gives up after `limit` SM cycles (by default 2^31, about
-// 1 s at 2 GHz, far above any copy's latency)
-constexpr long long WAIT_DEFAULT = 1ll << 31;
+// bounded wait: gives up after `limit` SM cycles (the default is far above any
+// copy's latency)
 // test_wait polls without suspending the thread, so that the bound, not
 // the hardware's own suspend window, decides when the wait gives up
 __device__ __forceinline__ bool bar_test(unsigned long long *b, unsigned parity) {
@@ -169,9 +168,9 @@ __global__ void __launch_bounds__(TX *TY, 1)
   if (leader) issue_plane<T, TY>(S, M, i0, j0, kb - 2);
   unsigned phase[2] = {0u, 0u};
 
-  const long long wait_limit = sc->wait_cycles > 0 ? sc->wait_cycles : WAIT_DEFAULT;
+  const long long limit = wait_limit(sc);
   for (int t = kb - 2; t < ke + 2; ++t) {
-    const bool ok = bar_wait(&S.bar[t & 1], phase[t & 1], wait_limit);
+    const bool ok = bar_wait(&S.bar[t & 1], phase[t & 1], limit);
     phase[t & 1] ^= 1u;
     if (__syncthreads_or(!ok)) {
       if (leader && di) atomicExch(&di->done, 4);

@@ -60,12 +60,16 @@ struct Scal {
   int jaumann;
   long long freeze_iter;   // > 0: frozen plasticity armed from this iteration on
   double freeze_eps;
-  long long wait_cycles;   // bound of a TMA wait (0: the default, 2^31 cycles)
+  long long wait_cycles;   // bound of a device wait (0: the default)
   int gcell;               // 1: per-cell shear modulus; the rotation weights then
                            // carry dt only and the trial applies each point's c2
   SweepScal<float> f;
   SweepScal<double> d;
 };
+constexpr long long WAIT_DEFAULT = 1ll << 31;   // SM cycles, about a second
+__device__ __forceinline__ long long wait_limit(const Scal *sc) {
+  return sc->wait_cycles > 0 ? sc->wait_cycles : WAIT_DEFAULT;
+}
 template <typename T>
 __device__ __forceinline__ const SweepScal<T> &sweep_scal(const Scal *sc);
 template <>

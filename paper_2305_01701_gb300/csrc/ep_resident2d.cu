@@ -13,7 +13,7 @@
 // Exchange: ep_words.cuh.  Two buffers alternate: a block
 // overwrites a word only after it has read from every neighbour what that one sent
 // after reading the word.  All blocks are resident at once (cooperative launch,
-// checked against the occupancy); a wait gives up after 2^31 cycles or when another
+// checked against the occupancy); a wait gives up after the grid's bound or when another
 // one has: done = 4, every block returns.  Numbers only grow, by the same amount in
 // every block of a launch; the buffers start a solve at zero.
 //
@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
   __syncthreads();
   if (tid == 0) *mine = base + iters;
 
+  const long long limit = wait_limit(sc);
   for (int q = 0; q < iters; ++q) {
     // ---- vertex: relaxed trial, rotation product ----
     T ts = 0, p = 0;
@@ -164,8 +165,7 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
       send(word, g.box, u0, u1, v, tag);
     } else if (box && !owned) {
       const bool shear = vin && !vown;
-      const long long t0 = clock64();
-      for (unsigned n = 1;; ++n) {
+      for (Wait w = wait_begin();;) {
         T a, b, c = tsh;
         if (receive(word, g.box, tag, &a, &b, &c, shear)) {
           u0 = a;
@@ -173,9 +173,8 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
           tsh = c;
           break;
         }
-        if ((n & 63) == 0 && (clock64() - t0 > WAIT_CYCLES || *(volatile const int *)&di->done != 0)) {
+        if (wait_over(w, limit, di)) {
           lost = true;
-          atomicCAS(&di->done, 0, 4);
           break;
         }
       }

@@ -17,7 +17,7 @@
 // has read every neighbour's scales, which that one sent after reading the velocities, and
 // the other way round; every point of the halo is read, also where it holds no centre, so
 // that each neighbour is waited for.  All blocks are resident at once (cooperative launch,
-// one per SM); a wait gives up after 2^31 cycles or when another one has: done = 4, every
+// one per SM); a wait gives up after the grid's bound or when another one has: done = 4, every
 // block returns.
 //
 // Bound: shared memory and instruction issue of one block per SM, and the latency of two
@@ -89,7 +89,11 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
   int2 *const hu = (int2 *)(counter + 4), *const hs = hu + T.halo();
   const int bi = blockIdx.x * T.t[0] - 2, bj = blockIdx.y * T.t[1] - 2, bk = blockIdx.z * T.t[2] - 2;
   __shared__ SweepScal<float> Q;
-  if (tid == 0) Q = sweep_scal<float>(sc);
+  __shared__ long long limit;
+  if (tid == 0) {
+    Q = sweep_scal<float>(sc);
+    limit = wait_limit(sc);
+  }
   __syncthreads();
   const float rdx = Q.rdx, rdy = Q.rdy, rdz = Q.rdz, eta = Q.eta, bt = Q.bt, ob = Q.ob;
   auto in_box = [&](int i, int j, int k) {
@@ -260,17 +264,12 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
       x0[l] = s0; x1[l] = s1; x2[l] = s2;
     }
     bool lost = false;
-    auto give_up = [&](unsigned n_, long long since) {
-      if ((n_ & 63) || (clock64() - since <= WAIT_CYCLES && *(volatile const int *)&di->done == 0)) return false;
-      atomicCAS(&di->done, 0, 4);
-      return true;
-    };
     {
-      const long long since = clock64();
+      Wait w = wait_begin();
       bool need[SHELL_TRIPS];
 #pragma unroll
       for (int r = 0; r < SHELL_TRIPS; ++r) need[r] = tid + r * nt < counter[1];
-      for (unsigned tries = 1;; ++tries) {
+      for (;;) {
         bool again = false;
 #pragma unroll
         for (int r = 0; r < SHELL_TRIPS; ++r) {
@@ -290,7 +289,7 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
           again |= need[r];
         }
         if (!again) break;
-        if (give_up(tries, since)) { lost = true; break; }
+        if (wait_over(w, limit, di)) { lost = true; break; }
       }
     }
     if (__syncthreads_or(lost)) return;
@@ -336,11 +335,11 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
     }
     if (q == iters - 1) break;
     {
-      const long long since = clock64();
+      Wait w = wait_begin();
       bool need[HALO_TRIPS];
 #pragma unroll
       for (int r = 0; r < HALO_TRIPS; ++r) need[r] = tid + r * nt < counter[0];
-      for (unsigned tries = 1;; ++tries) {
+      for (;;) {
         float a[HALO_TRIPS][3];
         bool ok[HALO_TRIPS], again = false;
 #pragma unroll
@@ -360,7 +359,7 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
           again |= need[r];
         }
         if (!again) break;
-        if (give_up(tries, since)) { lost = true; break; }
+        if (wait_over(w, limit, di)) { lost = true; break; }
       }
     }
     if (__syncthreads_or(lost)) return;

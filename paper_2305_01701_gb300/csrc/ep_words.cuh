@@ -9,6 +9,8 @@
 
 #include <cuda_runtime.h>
 
+#include "ep_internal.cuh"
+
 namespace ep {
 
 struct alignas(16) Word {
@@ -66,6 +68,18 @@ __device__ __forceinline__ bool receive(const Word *w, long long stride, unsigne
   return ok;
 }
 
-constexpr long long WAIT_CYCLES = 1LL << 31;   // a reader gives up after them
+// one reader's wait for its words: it gives up after the grid's bound (ep_solver_opts.
+// wait_cycles), or when another reader has (looked up every 64 tries)
+struct Wait {
+  long long since;
+  unsigned tries;
+};
+__device__ __forceinline__ Wait wait_begin() { return {clock64(), 0u}; }
+// after a try that found a word missing
+__device__ __forceinline__ bool wait_over(Wait &w, long long limit, DevInfo *di) {
+  if (clock64() - w.since <= limit && ((++w.tries & 63) != 0 || *(volatile const int *)&di->done == 0)) return false;
+  atomicCAS(&di->done, 0, 4);
+  return true;
+}
 
 }  // namespace ep

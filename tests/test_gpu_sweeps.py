@@ -256,3 +256,47 @@ def test_elastic_iterations_without_rotation_round_alike_in_every_2d_kernel(P, n
         _, out = _solve(P, 2, n, pr, kernel, 24, f, **opts)
         for k in out:
             np.testing.assert_array_equal(out[k], ref[k])
+
+
+@pytest.mark.parametrize("nd,n,precision,kernel", [
+    (3, (60, 33, 14), "fp32", "KERNEL_FUSED_REG"), (3, (60, 33, 14), "fp64", "KERNEL_FUSED_REG"),
+    (3, (40, 33, 14), "fp32", "KERNEL_AUTO"),      # its check runs the register sweep
+    (2, (64, 50), "fp64", "KERNEL_AUTO"), (2, (64, 50), "fp32", "KERNEL_AUTO"), (2, (300, 180), "fp32", "KERNEL_AUTO")])
+def test_waits_that_run_out_end_the_solve_with_timeout(P, nd, n, precision, kernel):
+    """A bound of 8 cycles, far below the latency of a plane's copy or of an exchanged word, ends
+    the solve with EP_ERR_TIMEOUT; with the default bound back the grid solves as an untouched
+    one.  Bounds around those latencies may end it or not, and leave the grid as usable."""
+    f = _fields(P, nd, n, 16)
+    rng = np.random.default_rng(1)
+    coh = 1.5e-3 * (1 + 0.01 * rng.standard_normal(int(np.prod(n))))
+    grids = []
+    for _ in range(2):
+        g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=P.FP64 if precision == "fp64" else P.FP32_MIXED)
+        g.set_material(2.0, 1.0, math.inf, 30.0, 0.0, coh)
+        g.set_kernel(getattr(P, kernel), -1)
+        for k, a in f.items():
+            g.set(k, a)
+        g.snapshot()
+        grids.append(g)
+    g, ref = grids
+
+    def solve(x, wait):
+        x.restore()
+        x.set_solver(tol=0.0, max_iter=40, n_chk=10, wait_cycles=wait)
+        x.apply_increment(1.0, 1e-4, P.LOAD_XY if nd == 2 else P.LOAD_XZ)
+        return x.solve_increment(raise_on_fail=False)["status"]
+
+    timeout, not_converged = 7, 5
+    assert solve(ref, 0) == not_converged
+    ref.commit_increment()
+    want = {k: ref.get(k) for k in list(f) + ["epl", "scale"]}
+    assert (want["scale"] < 1.0).any()
+    for wait in (8, 300, 600, 1200, 2400, 4800, 9600):
+        status = solve(g, wait)
+        assert status in ((timeout,) if wait == 8 else (timeout, not_converged)), (wait, status)
+        assert solve(g, 0) == not_converged
+        g.commit_increment()
+        for k, a in want.items():
+            np.testing.assert_array_equal(g.get(k), a)
+    g.close()
+    ref.close()

@@ -53,8 +53,8 @@ struct Strip<double> {
 
 template <typename T>
 __device__ __forceinline__ T maxt(T a, T b) { return (a > b || a != a) ? a : b; }
-__device__ __forceinline__ float absv(float x) { return fabsf(x); }
-__device__ __forceinline__ double absv(double x) { return fabs(x); }
+// |a - b|, formed in FP64
+__device__ __forceinline__ double gap(double a, double b) { return fabs(a - b); }
 
 // warp-wide max of |v| (NaN kept: its bit pattern is above +inf), one atomic
 __device__ __forceinline__ void warp_max(double v, unsigned long long *slot) {
@@ -125,8 +125,7 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
     // row history (suffix _1: row t - 1, _2: row t - 2, _3: row t - 3)
     V vx = zero, vy = zero, vx_1 = zero, vy_1 = zero, vx_2 = zero, vy_2 = zero, rd = zero;
     V P = zero, ts = zero, s_1 = zero, sxx_1 = zero, syy_1 = zero, syy_2 = zero, nxy_1 = zero;
-    T sig = 0, dtau = 0, dp = 0, rmax = 0, du = 0;
-    double vm = 0.0;
+    double sig = 0.0, dtau = 0.0, dp = 0.0, rmax = 0.0, du = 0.0, vm = 0.0;   // the stopping measures, in FP64
 
     load_row(j0 - 2, next);
     for (int t = j0 - 2; t < j1 + 2; ++t) {
@@ -183,9 +182,9 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
           auto one = [&](auto ic) {
             constexpr int E = decltype(ic)::value;
             if (!in_x0(E)) return;
-            sig = maxt(sig, maxt(absv(el<E>(sxx_1)), absv(el<E>(syy_1))));
-            dtau = maxt(dtau, maxt(absv(el<E>(n0) - el<E>(k0)), absv(el<E>(n1) - el<E>(k1))));
-            dp = maxt(dp, absv(el<E>(pr) - el<E>(kp)));
+            sig = maxt(sig, maxt(fabs((double)el<E>(sxx_1)), fabs((double)el<E>(syy_1))));
+            dtau = maxt(dtau, maxt(gap(el<E>(n0), el<E>(k0)), gap(el<E>(n1), el<E>(k1))));
+            dp = maxt(dp, gap(el<E>(pr), el<E>(kp)));
           };
           one(std::integral_constant<int, 0>{});
           if constexpr (N == 2) one(std::integral_constant<int, 1>{});
@@ -203,8 +202,8 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
           const V k = ld(I.cs, e);
           auto one = [&](auto ic) {
             constexpr int E = decltype(ic)::value;
-            sig = maxt(sig, absv(el<E>(nxy_1)));
-            dtau = maxt(dtau, absv(el<E>(nxy_1) - el<E>(k)));
+            sig = maxt(sig, fabs((double)el<E>(nxy_1)));
+            dtau = maxt(dtau, gap(el<E>(nxy_1), el<E>(k)));
           };
           one(std::integral_constant<int, 0>{});
           if constexpr (N == 2) one(std::integral_constant<int, 1>{});
@@ -226,14 +225,14 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
           const V k0 = ld(I.uchk[0], e), k1 = ld(I.uchk[1], e);
           auto one = [&](auto ic) {
             constexpr int E = decltype(ic)::value;
-            if (ux && in_x1(E)) rmax = maxt(rmax, absv(el<E>(R0)));
-            if (uy && in_x0(E)) rmax = maxt(rmax, absv(el<E>(R1)));
+            if (ux && in_x1(E)) rmax = maxt(rmax, fabs((double)el<E>(R0)));
+            if (uy && in_x0(E)) rmax = maxt(rmax, fabs((double)el<E>(R1)));
             if (gi + E <= nx && u < ny) {
-              du = maxt(du, absv(el<E>(un0) - el<E>(k0)));
+              du = maxt(du, gap(el<E>(un0), el<E>(k0)));
               vm = maxt(vm, fabs(I.v0[0][e + E] + (double)el<E>(vx_2)));
             }
             if (gi + E < nx && u <= ny) {
-              du = maxt(du, absv(el<E>(un1) - el<E>(k1)));
+              du = maxt(du, gap(el<E>(un1), el<E>(k1)));
               vm = maxt(vm, fabs(I.v0[1][e + E] + (double)el<E>(vy_2)));
             }
           };
@@ -245,11 +244,11 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
       }
     }
     if constexpr (CHK) {
-      warp_max((double)sig, &I.di->red[RED_SIG]);
-      warp_max((double)dtau, &I.di->red[RED_DTAU]);
-      warp_max((double)dp, &I.di->red[RED_DP]);
-      warp_max((double)rmax, &I.di->red[RED_R]);
-      warp_max((double)du, &I.di->red[RED_DU]);
+      warp_max(sig, &I.di->red[RED_SIG]);
+      warp_max(dtau, &I.di->red[RED_DTAU]);
+      warp_max(dp, &I.di->red[RED_DP]);
+      warp_max(rmax, &I.di->red[RED_R]);
+      warp_max(du, &I.di->red[RED_DU]);
       warp_max(vm, &I.di->red[RED_V]);
     }
   }

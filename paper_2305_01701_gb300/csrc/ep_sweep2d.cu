@@ -24,8 +24,9 @@ namespace ep {
 
 namespace {
 
-template <typename T>
-__device__ __forceinline__ T maxn(T a, T b) { return (a > b || a != a) ? a : b; }
+__device__ __forceinline__ double maxn(double a, double b) { return (a > b || a != a) ? a : b; }
+// |a - b|, formed in FP64
+__device__ __forceinline__ double gap(double a, double b) { return fabs(a - b); }
 
 // block-wide max of |v| as IEEE bits (a NaN sorts above infinity), one atomic per
 // block; blocks are (32, warps)
@@ -84,7 +85,7 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
   const T two_eta = Q.two_eta, eta = Q.eta, bt = Q.bt, ob = Q.ob;
   const T bp = Q.bp, obp = Q.obp, KDt = Q.KDt, Ac = Q.A, rdx = Q.rdx, rdy = Q.rdy;
   const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
-  T sig = 0, dtau = 0, dp = 0;
+  double sig = 0.0, dtau = 0.0, dp = 0.0;   // stopping measures, in FP64
   T u0_m = 0, t_j = 0, p_j = 0;   // x-velocity of the row below; trial and rotation product at row j
   // trial and rotation product of vertex (i, j)
   auto vertex = [&](int j, T u0, T *ts, T *pr) {
@@ -136,22 +137,22 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
       S.sx[0][e] = s0;
       S.sx[1][e] = s1;
       if (CHK) {
-        sig = maxn(sig, maxn(fabs(s0), fabs(s1)));
-        dtau = maxn(dtau, maxn(fabs(n0 - S.cn[0][e]), fabs(n1 - S.cn[1][e])));
-        dp = maxn(dp, fabs(pr - S.cp[e]));
+        sig = maxn(sig, maxn(fabs((double)s0), fabs((double)s1)));
+        dtau = maxn(dtau, maxn(gap(n0, S.cn[0][e]), gap(n1, S.cn[1][e])));
+        dp = maxn(dp, gap(pr, S.cp[e]));
         S.cn[0][e] = n0;
         S.cn[1][e] = n1;
         S.cp[e] = pr;
-        if (isnan(s) || isnan(pr)) sig = (T)NAN;
+        if (isnan(s) || isnan(pr)) sig = NAN;
       }
     }
     t_j = t_p;
     p_j = p_p;
   }
   if (CHK && di) {
-    block_max((double)sig, &di->red[RED_SIG]);
-    block_max((double)dtau, &di->red[RED_DTAU]);
-    block_max((double)dp, &di->red[RED_DP]);
+    block_max(sig, &di->red[RED_SIG]);
+    block_max(dtau, &di->red[RED_DTAU]);
+    block_max(dp, &di->red[RED_DP]);
   }
 }
 
@@ -164,8 +165,7 @@ __global__ void __launch_bounds__(128) k_move2d(Geo g, Stage<T> S, const Scal *s
   const SweepScal<T> &Q = sweep_scal<T>(sc);
   const T vs = Q.vstep, rdx = Q.rdx, rdy = Q.rdy;
   const bool x1 = i > 0 && i < nx, own = p.lane < 31 && i <= nx;
-  T sig = 0, dtau = 0, rmax = 0, du = 0;
-  double vm = 0.0;   // |v0 + u| needs the FP64 base velocity
+  double sig = 0.0, dtau = 0.0, rmax = 0.0, du = 0.0, vm = 0.0;   // stopping measures, in FP64
   // scales of the two centres beside column i in row j
   auto pair = [&](int j) { return x1 && j >= 0 && j < ny ? S.s[j * px + i - 1] + S.s[j * px + i] : (T)0; };
   // new deviator of vertex (i, j) from its rows of scales
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(128) k_move2d(Geo g, Stage<T> S, const Scal *s
     if (own) {
       S.sns[0][e] = v;
       if (CHK) {
-        sig = maxn(sig, fabs(v));
-        dtau = maxn(dtau, fabs(v - S.cs[0][e]));
+        sig = maxn(sig, fabs((double)v));
+        dtau = maxn(dtau, gap(v, S.cs[0][e]));
         S.cs[0][e] = v;
       }
       // face d: in = inside its extent, in1 = off the walls
@@ -190,11 +190,11 @@ __global__ void __launch_bounds__(128) k_move2d(Geo g, Stage<T> S, const Scal *s
         if (in1) {
           if (S.f[d]) R += S.f[d][e];
           un = fma(vs, R, u);
-          if (CHK) rmax = maxn(rmax, fabs(R));
+          if (CHK) rmax = maxn(rmax, fabs((double)R));
         }
         S.uo[d][e] = un;
         if (CHK && in) {
-          du = maxn(du, fabs(un - S.uchk[d][e]));
+          du = maxn(du, gap(un, S.uchk[d][e]));
           vm = maxn(vm, fabs(S.v0[d][e] + (double)u));
           S.uchk[d][e] = un;
         }
@@ -211,10 +211,10 @@ __global__ void __launch_bounds__(128) k_move2d(Geo g, Stage<T> S, const Scal *s
     v = v_p;
   }
   if (CHK && di) {
-    block_max((double)sig, &di->red[RED_SIG]);
-    block_max((double)dtau, &di->red[RED_DTAU]);
-    block_max((double)rmax, &di->red[RED_R]);
-    block_max((double)du, &di->red[RED_DU]);
+    block_max(sig, &di->red[RED_SIG]);
+    block_max(dtau, &di->red[RED_DTAU]);
+    block_max(rmax, &di->red[RED_R]);
+    block_max(du, &di->red[RED_DU]);
     block_max(vm, &di->red[RED_V]);
   }
 }

@@ -300,3 +300,27 @@ def test_waits_that_run_out_end_the_solve_with_timeout(P, nd, n, precision, kern
             np.testing.assert_array_equal(g.get(k), a)
     g.close()
     ref.close()
+
+
+@pytest.mark.parametrize("kernel,shape", [("KERNEL_AUTO", -1), ("KERNEL_STAGED", -1), ("KERNEL_FUSED", 0),
+                                          ("KERNEL_FUSED", 3), ("KERNEL_FUSED", 4)])
+@pytest.mark.parametrize("seed", [17, 18, 19])
+def test_fp32_stopping_measures_of_2d_sweeps_are_formed_in_fp64(P, kernel, shape, seed):
+    """max|tau - tau_chk| and max|p - p_chk| of FP32 states, against the same differences of the
+    two checks' states on the host: equal to rounding in 64 bits."""
+    n, chk = (70, 45), 2
+    f = _fields(P, 2, n, seed)
+    runs = [_solve(P, 2, n, P.FP32_MIXED, getattr(P, kernel), m, f, shape=shape, chunk=chk) for m in (2 * chk, 3 * chk)]
+    (_, a), (info, b) = runs
+    assert info["iters"] == 3 * chk
+    # Eqs. PT1-PT24qq with the defaults of the grid and _solve's material and step
+    dt, G, K, L, h = 1e-4, 1.0, 2.0, (1.0, 0.8), [w / m for w, m in zip((1.0, 0.8), n)]
+    eta, Vp = G * dt, 0.9 / math.sqrt(2.0) * min(h)
+    rho = 3.0 * math.sqrt(10.0) * math.pi / 2.0 * eta / (Vp * max(L))
+    Gt = rho * Vp ** 2 / (0.5 + 4.0 / 3.0)
+    bt = (1.0 / (2.0 * Gt)) / (1.0 / (2.0 * Gt) + 1.0 / (2.0 * eta))
+    bp = (1.0 / (0.5 * Gt)) / (1.0 / (0.5 * Gt) + 1.0 / (K * dt))
+    for keys, beta, got in ((("txx", "tyy", "txy"), bt, info["eps_tau"]), (("p",), bp, info["eps_p"])):
+        gap = max(np.abs(b[k] - a[k]).max() for k in keys)
+        want = gap / (chk * (1.0 - beta)) / info["max_sigma"]
+        assert abs(got - want) <= 1e-11 * want, (keys, got, want)

@@ -572,8 +572,8 @@ template <typename T>
 bool use_fused(const ep_grid *h) {
   if (h->ndim != 3 || h->have_f) return false;
   const int v = fused_variant(h);
-  // a per-cell shear modulus: the FP32 register sweep only
-  if (h->Gc) return sizeof(T) == 4 && v == EP_KERNEL_FUSED_REG;
+  // a per-cell shear modulus: the FP32 register sweep only, where its launch fits
+  if (h->Gc) return sizeof(T) == 4 && v == EP_KERNEL_FUSED_REG && fused3d_reg_cell_g_fits(h->g, h->kz);
   return v == EP_KERNEL_FUSED || v == EP_KERNEL_FUSED_TMA || v == EP_KERNEL_FUSED_REG;
 }
 

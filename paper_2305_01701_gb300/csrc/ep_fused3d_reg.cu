@@ -764,6 +764,11 @@ bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo
   }
 }
 
+bool fused3d_reg_cell_g_fits(const Geo &g, int kz) {
+  constexpr int rows = LaneF<16>::H - 4;
+  return (g.py + rows - 1) / rows <= 65535 && (kz <= 0 || (g.pz + kz - 1) / kz <= 65535);
+}
+
 cudaError_t fused3d_reg_configure() {
   const cudaError_t e[] = {configure_lane<LaneF<24>, false, false>(), configure_lane<LaneF<16>, false, false>(),
                            configure_lane<LaneF<16>, false, true>(),  configure_lane<LaneF<16>, true, false>(),

@@ -294,6 +294,8 @@ cudaError_t fused3d_tma_configure();
 template <typename T>
 bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di, int kz, cudaStream_t st,
                         bool check = false, bool last = false);
+// whether its blocks with a per-cell modulus fit one launch (65,535 along y and z)
+bool fused3d_reg_cell_g_fits(const Geo &g, int kz);
 cudaError_t fused3d_reg_configure();
 
 // ---- increment set-up and commit (FP64; ep_increment.cu) ------------------

@@ -18,6 +18,8 @@
 // in shared memory (warp strips: 35 us).
 #include <math.h>
 
+#include <algorithm>
+
 #include "ep_internal.cuh"
 
 namespace ep {
@@ -223,10 +225,13 @@ __global__ void __launch_bounds__(128) k_move2d(Geo g, Stage<T> S, const Scal *s
 // of the vertex's w
 template <typename T>
 __global__ void __launch_bounds__(256) k_rotation_mean2d(Geo g, const T *rd, T *md) {
-  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, px = g.px;
-  if (i < 1 || i >= g.nx || j < 1 || j >= g.ny) return;
-  const int e = j * px + i;
-  md[e] = (T)0.125 * (rd[e - px - 1] + rd[e - px] + rd[e - 1] + rd[e]);
+  const int i = blockIdx.x * 32 + threadIdx.x, px = g.px;
+  if (i < 1 || i >= g.nx) return;
+  for (int j = blockIdx.y * 8 + threadIdx.y; j < g.ny; j += gridDim.y * 8) {
+    if (j < 1) continue;
+    const int e = j * px + i;
+    md[e] = (T)0.125 * (rd[e - px - 1] + rd[e - px] + rd[e - 1] + rd[e]);
+  }
 }
 
 // rows per warp (a strip recomputes one row of vertices), doubled up to 8 while
@@ -235,6 +240,7 @@ int strip_rows(const Geo &g, dim3 *grid, dim3 *block) {
   const int bx = (g.nx + 31) / 31;   // points 0 .. nx, 31 per warp
   int rows = 1;
   while (rows < 8 && (long long)bx * ((g.py + 2 * rows - 1) / (2 * rows)) >= 1216) rows *= 2;
+  while (((g.py + rows - 1) / rows + 3) / 4 > 65535) rows *= 2;   // the longest launch
   const int strips = (g.py + rows - 1) / rows;
   int w = 4;
   while (w > 1 && (long long)bx * ((strips + w - 1) / w) < 304) w /= 2;
@@ -260,7 +266,7 @@ void launch_sweep2d(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo *di
 
 template <typename T>
 void launch_rotation_mean2d(const Geo &g, const T *rd, T *md, cudaStream_t st) {
-  k_rotation_mean2d<T><<<dim3((g.nx + 32) / 32, (g.py + 7) / 8), dim3(32, 8), 0, st>>>(g, rd, md);
+  k_rotation_mean2d<T><<<dim3((g.nx + 32) / 32, std::min((g.py + 7) / 8, 65535)), dim3(32, 8), 0, st>>>(g, rd, md);
 }
 
 template void launch_sweep2d<float>(const Geo &, const Stage<float> &, const Scal *, DevInfo *, bool, cudaStream_t,

@@ -20,6 +20,8 @@
 // 510 us of the pipe).  A warp covers 32 points along x; blocks hold as many rows as leave every SM some (launch_rows).
 #include <math.h>
 
+#include <algorithm>
+
 #include "ep_internal.cuh"
 #include "ep_lanes.cuh"
 
@@ -54,19 +56,20 @@ struct Pt {
   int i, j, k;
   long long e;
 };
-__device__ __forceinline__ Pt point(const Geo &g) {
+// o: the row block and the plane that a launch starts at (launch_parts)
+__device__ __forceinline__ Pt point(const Geo &g, int2 o) {
   Pt p;
   p.i = blockIdx.x * 32 + threadIdx.x;
-  p.j = blockIdx.y * blockDim.y + threadIdx.y;
-  p.k = blockIdx.z;
+  p.j = (o.x + blockIdx.y) * blockDim.y + threadIdx.y;
+  p.k = o.y + blockIdx.z;
   p.e = ((long long)p.k * g.py + p.j) * g.px + p.i;
   return p;
 }
 
 // ---- spins, shear rates and rotation products at vertices / edges ------------
-__global__ void __launch_bounds__(256) k64_strain(Geo g, Stage<double> S, DevInfo *di) {
+__global__ void __launch_bounds__(256) k64_strain(Geo g, int2 o, Stage<double> S, DevInfo *di) {
   if (skip(di)) return;
-  const Pt q = point(g);
+  const Pt q = point(g, o);
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   if (i > nx || j > ny) return;
   const long long e = q.e, px = g.px, pl = g.plane;
@@ -92,9 +95,9 @@ __global__ void __launch_bounds__(256) k64_strain(Geo g, Stage<double> S, DevInf
 }
 
 // ---- relaxed trials -------------------------------------------------------------
-__global__ void __launch_bounds__(256) k64_trial(Geo g, Stage<double> S, const Scal *sc, DevInfo *di) {
+__global__ void __launch_bounds__(256) k64_trial(Geo g, int2 o, Stage<double> S, const Scal *sc, DevInfo *di) {
   if (skip(di)) return;
-  const Pt q = point(g);
+  const Pt q = point(g, o);
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   if (i > nx || j > ny) return;
   const long long e = q.e, px = g.px, pl = g.plane;
@@ -139,9 +142,9 @@ __global__ void __launch_bounds__(256) k64_trial(Geo g, Stage<double> S, const S
 
 // ---- pressure and return at centres ------------------------------------------------
 template <bool CHK>
-__global__ void __launch_bounds__(256) k64_centres(Geo g, Stage<double> S, const Scal *sc, DevInfo *di) {
+__global__ void __launch_bounds__(256) k64_centres(Geo g, int2 o, Stage<double> S, const Scal *sc, DevInfo *di) {
   if (skip(di)) return;
-  const Pt q = point(g);
+  const Pt q = point(g, o);
   const long long e = q.e, px = g.px, pl = g.plane;
   const bool frozen = di != nullptr && di->frozen;
   double sig = 0.0, dtau = 0.0, dp = 0.0;
@@ -192,9 +195,9 @@ __global__ void __launch_bounds__(256) k64_centres(Geo g, Stage<double> S, const
 
 // ---- new deviators at vertices / edges ------------------------------------------------
 template <bool CHK>
-__global__ void __launch_bounds__(256) k64_edges(Geo g, Stage<double> S, DevInfo *di) {
+__global__ void __launch_bounds__(256) k64_edges(Geo g, int2 o, Stage<double> S, DevInfo *di) {
   if (skip(di)) return;
-  const Pt q = point(g);
+  const Pt q = point(g, o);
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   const long long e = q.e, px = g.px, pl = g.plane;
   double sig = 0.0, dtau = 0.0;
@@ -226,9 +229,9 @@ __global__ void __launch_bounds__(256) k64_edges(Geo g, Stage<double> S, DevInfo
 
 // ---- residual and velocity update ---------------------------------------------------------
 template <bool CHK>
-__global__ void __launch_bounds__(256) k64_velocity(Geo g, Stage<double> S, const Scal *sc, DevInfo *di) {
+__global__ void __launch_bounds__(256) k64_velocity(Geo g, int2 o, Stage<double> S, const Scal *sc, DevInfo *di) {
   if (skip(di)) return;
-  const Pt q = point(g);
+  const Pt q = point(g, o);
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   const long long e = q.e, px = g.px, pl = g.plane;
   const double vs = sc->vstep;
@@ -282,10 +285,10 @@ __global__ void __launch_bounds__(256) k64_velocity(Geo g, Stage<double> S, cons
 // md: of the edge's own w; ma, mb: of the summed w of the two other orientations
 // (w = 2 omega; sums of four).  rq = c2 dt tau_hat at edges, rd = c2 dt (tyy - txx),
 // c2 dt (tzz - txx) at centres.
-__global__ void __launch_bounds__(256) k_rotation_means(Geo g, Stage<double> S, double *md0, double *md1, double *md2,
-                                                        double *ma0, double *ma1, double *ma2, double *mb0,
-                                                        double *mb1, double *mb2) {
-  const Pt q = point(g);
+__global__ void __launch_bounds__(256) k_rotation_means(Geo g, int2 o, Stage<double> S, double *md0, double *md1,
+                                                        double *md2, double *ma0, double *ma1, double *ma2,
+                                                        double *mb0, double *mb1, double *mb2) {
+  const Pt q = point(g, o);
   const int i = q.i, j = q.j, k = q.k, nx = g.nx, ny = g.ny, nz = g.nz;
   if (i > nx || j > ny) return;
   const long long e = q.e, px = g.px, pl = g.plane;
@@ -312,43 +315,59 @@ __global__ void __launch_bounds__(256) k_rotation_means(Geo g, Stage<double> S, 
 
 // rows per block: 8 where that leaves four blocks per SM (152), fewer on smaller
 // grids
-void launch_rows(const Geo &g, dim3 *grid, dim3 *block) {
+dim3 launch_rows(const Geo &g, dim3 *block) {
   const int bx = (g.nx + 32) / 32;   // points 0 .. nx
   int rows = 8;
   while (rows > 1 && (long long)bx * ((g.py + rows - 1) / rows) * g.pz < 608) rows /= 2;
   *block = dim3(32, rows);
-  *grid = dim3(bx, (g.py + rows - 1) / rows, g.pz);
+  return dim3(bx, (g.py + rows - 1) / rows, g.pz);
+}
+
+// go(grid, offset) for a grid of row blocks and planes, cut where it is longer than a
+// launch can be
+template <typename F>
+void launch_parts(dim3 gr, F go) {
+  constexpr unsigned most = 65535;
+  for (unsigned z = 0; z < gr.z; z += most)
+    for (unsigned y = 0; y < gr.y; y += most)
+      go(dim3(gr.x, std::min(most, gr.y - y), std::min(most, gr.z - z)), make_int2((int)y, (int)z));
 }
 
 }  // namespace
 
 void launch_sweep64(const Geo &g, const Stage<double> &S, const Scal *sc, DevInfo *di, bool check, cudaStream_t st,
                    const cudaEvent_t *ev) {
-  dim3 gr, bl;
-  auto mark = [&](int q) {
-    if (ev) cudaEventRecord(ev[q], st);
+  dim3 bl;
+  const dim3 all = launch_rows(g, &bl);
+  int stage = 0;
+  auto run = [&](auto go) {
+    launch_parts(all, go);
+    ++stage;
+    if (ev) cudaEventRecord(ev[stage], st);
   };
-  launch_rows(g, &gr, &bl);
-  k64_strain<<<gr, bl, 0, st>>>(g, S, di);
-  mark(1);
-  k64_trial<<<gr, bl, 0, st>>>(g, S, sc, di);
-  mark(2);
-  if (check) k64_centres<true><<<gr, bl, 0, st>>>(g, S, sc, di);
-  else k64_centres<false><<<gr, bl, 0, st>>>(g, S, sc, di);
-  mark(3);
-  if (check) k64_edges<true><<<gr, bl, 0, st>>>(g, S, di);
-  else k64_edges<false><<<gr, bl, 0, st>>>(g, S, di);
-  mark(4);
-  if (check) k64_velocity<true><<<gr, bl, 0, st>>>(g, S, sc, di);
-  else k64_velocity<false><<<gr, bl, 0, st>>>(g, S, sc, di);
-  mark(5);
+  run([&](dim3 gr, int2 o) { k64_strain<<<gr, bl, 0, st>>>(g, o, S, di); });
+  run([&](dim3 gr, int2 o) { k64_trial<<<gr, bl, 0, st>>>(g, o, S, sc, di); });
+  run([&](dim3 gr, int2 o) {
+    if (check) k64_centres<true><<<gr, bl, 0, st>>>(g, o, S, sc, di);
+    else k64_centres<false><<<gr, bl, 0, st>>>(g, o, S, sc, di);
+  });
+  run([&](dim3 gr, int2 o) {
+    if (check) k64_edges<true><<<gr, bl, 0, st>>>(g, o, S, di);
+    else k64_edges<false><<<gr, bl, 0, st>>>(g, o, S, di);
+  });
+  run([&](dim3 gr, int2 o) {
+    if (check) k64_velocity<true><<<gr, bl, 0, st>>>(g, o, S, sc, di);
+    else k64_velocity<false><<<gr, bl, 0, st>>>(g, o, S, sc, di);
+  });
 }
 
 void launch_rotation_means(const Geo &g, const Stage<double> &S, double *const md[3], double *const ma[3],
                            double *const mb[3], cudaStream_t st) {
-  dim3 gr, bl;
-  launch_rows(g, &gr, &bl);
-  k_rotation_means<<<gr, bl, 0, st>>>(g, S, md[0], md[1], md[2], ma[0], ma[1], ma[2], mb[0], mb[1], mb[2]);
+  dim3 bl;
+  const dim3 all = launch_rows(g, &bl);
+  launch_parts(all, [&](dim3 gr, int2 o) {
+    k_rotation_means<<<gr, bl, 0, st>>>(g, o, S, md[0], md[1], md[2], ma[0], ma[1], ma[2], mb[0], mb[1], mb[2]);
+  });
 }
 
 }  // namespace ep

@@ -21,8 +21,9 @@ def P():
     return P
 
 
-def _fields(P, nd, n, seed):
-    """A history near yield: pure shear with noise, noisy velocities, shear zero on the walls."""
+def _fields(P, nd, n, seed, h=None):
+    """A history near yield: pure shear with noise, noisy velocities, shear zero on the walls.
+    h: the edge of the cells (default: a box of edges near 1)."""
     rng = np.random.default_rng(seed)
     rates = [1.0, -1.0] if nd == 2 else [1.0, 0.0, -1.0]
     f = {}
@@ -32,7 +33,8 @@ def _fields(P, nd, n, seed):
         ax = nd - 1 - d
         x = np.arange(n[d] + 1) / n[d] - 0.5
         v = rates[d] * x.reshape([-1 if q == ax else 1 for q in range(nd)]) * np.ones(shape["v" + "xyz"[d]])
-        f["v" + "xyz"[d]] = v + 0.02 * rng.standard_normal(v.shape)
+        f["v" + "xyz"[d]] = (v + 0.02 * rng.standard_normal(v.shape) if h is None else
+                             v * n[d] * h + h * rng.standard_normal(v.shape))
         c = shape["t" + "xyz"[d] * 2]
         f["t" + "xyz"[d] * 2] = (1.2e-3 if nd == 2 else 1.7e-3) * rates[d] + 1e-4 * rng.standard_normal(c)
     for k, walls in (("txy", (0, 1)), ("txz", (0, 2)), ("tyz", (1, 2))):
@@ -51,7 +53,7 @@ def _solve(P, nd, n, precision, kernel, iters, f, shape=-1, **opts):
     force = opts.pop("force", 0.0)
     cohesion = 1.5e-3 * (1e3 if opts.pop("elastic", False) else 1.0)
     pending = opts.pop("pending", 0)   # commit after so many chunks, the solve undecided
-    g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=precision)
+    g = P.Grid(nd, n, L=opts.pop("L", (1.0, 0.8, 1.3)[:nd]), precision=precision)
     rng = np.random.default_rng(1)
     g.set_material(2.0, 1.0, opts.pop("mu_s", math.inf), 30.0, 0.0, cohesion * (1 + 0.01 * rng.standard_normal(int(np.prod(n)))))
     if "cell_g" in opts:
@@ -324,3 +326,24 @@ def test_fp32_stopping_measures_of_2d_sweeps_are_formed_in_fp64(P, kernel, shape
         gap = max(np.abs(b[k] - a[k]).max() for k in keys)
         want = gap / (chk * (1.0 - beta)) / info["max_sigma"]
         assert abs(got - want) <= 1e-11 * want, (keys, got, want)
+
+
+@pytest.mark.parametrize("nd,n,precision,kernel,opts", [
+    (3, (2, 2, 70000), "fp64", ("KERNEL_FUSED_REG", 0), {}),          # planes
+    (3, (2, 530000, 1), "fp64", ("KERNEL_AUTO", -1), {}),             # row blocks
+    (2, (2, 530000), "fp64", ("KERNEL_FUSED", 0), {}),                # the rotation's means
+    (2, (2, 2100000), "fp32", ("KERNEL_FUSED", 0), {}),               # strips of rows
+    (3, (2, 790000, 1), "fp32", ("KERNEL_STAGED", -1), {"cell_g": 1.0}),
+])
+def test_grids_longer_than_one_launch(P, nd, n, precision, kernel, opts):
+    """More planes, row blocks or strips than a launch's 65,535 along y or z.  The FP64 grid that
+    no fused sweep holds along y is compared with a per-cell modulus of the same value
+    everywhere, which takes the general stage kernels."""
+    iters = 8
+    f = _fields(P, nd, n, 20, h=0.02)
+    opts = dict(opts, L=tuple(0.02 * m for m in n))
+    pr = P.FP64 if precision == "fp64" else P.FP32_MIXED
+    general = {"cell_g": 0.0} if kernel[0] == "KERNEL_AUTO" else {}
+    iref, ref = _solve(P, nd, n, pr, getattr(P, kernel[0]), iters, f, shape=kernel[1], **opts, **general)
+    info, out = _solve(P, nd, n, pr, P.KERNEL_AUTO, iters, f, **opts)
+    _compare(f, out, ref, info, iref, iters, 2.0 ** -53 if precision == "fp64" else EPS32)

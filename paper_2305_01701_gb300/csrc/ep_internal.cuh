@@ -273,7 +273,8 @@ inline int fused3d_kz(const Geo &g, int tx, int ty, int kz, int per_sm = 1, long
   const long long wave = (long long)sms * per_sm;
   int best = 0;
   long long best_cost = -1;
-  for (int k = kz > 0 ? kz : 1; k <= (kz > 0 ? kz : g.pz); ++k) {
+  // (a launch takes one wave at least, so no k beyond the best cost can beat it)
+  for (int k = kz > 0 ? kz : 1; k <= (kz > 0 ? kz : g.pz) && (best_cost < 0 || k + 4 <= best_cost); ++k) {
     const long long blocks = cols * ((g.pz + k - 1) / k);
     const long long c = (blocks + wave - 1) / wave * (std::min(k, g.pz) + 4);
     if (best_cost < 0 || c < best_cost) { best_cost = c; best = k; }

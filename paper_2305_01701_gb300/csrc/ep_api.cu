@@ -57,9 +57,12 @@ struct ep_grid {
   Scal *hscal = nullptr;
   unsigned long long *dnpl = nullptr;
   double *dline = nullptr;
-  // resident sweeps: counters of the blocks, words of its exchange
+  // resident sweeps: the 2D configuration (-1: none) or the 3D tile (0: none), counters of
+  // the blocks and words of their exchange
+  int res2 = -1, res3[3] = {};
   unsigned *rcount = nullptr;
   Word *rwords = nullptr;
+  bool chunk_resident = false, words_clean = false;   // the chunk uses the words; they are zero
   cudaGraphExec_t chunk = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int variant = EP_KERNEL_AUTO;  // sweep kernel choice (ep_set_kernel)
@@ -145,6 +148,11 @@ Geo make_geo(int ndim, const int n[3], const double L[3]) {
   return g;
 }
 
+void plan_resident(ep_grid *h) {
+  if (h->ndim == 2) h->res2 = h->prec == EP_FP64 ? resident2d_config<double>(h->g) : resident2d_config<float>(h->g);
+  else if (h->prec != EP_FP64) resident3d_tile(h->g, h->res3);
+}
+
 // Assign every array of h from the arena (dry run: only count bytes).
 void carve(ep_grid *h, Arena &a) {
   const long long B = h->g.box;
@@ -196,9 +204,9 @@ void carve(ep_grid *h, Arena &a) {
   h->items_dev = a.take<int4>(h->max_items);
   h->dnpl = a.take<unsigned long long>(1);
   h->dline = a.take<double>(2);
-  if (const long long words = resident_words(h->g, es)) {
+  if (h->res2 >= 0 || h->res3[0]) {
     h->rcount = a.take<unsigned>(RESIDENT_BLOCKS);
-    h->rwords = a.take<Word>(words);
+    h->rwords = a.take<Word>(resident_words(h->g, es));
   }
 }
 
@@ -637,10 +645,11 @@ ep_status capture_chunk(ep_grid *h) {
                       (h->n_items + fused2d_items_per_block(h->tile) - 1) / fused2d_items_per_block(h->tile));
   }
   // AUTO on a grid that fits the chip: the iterations behind the check in one launch
-  const int res = h->ndim == 2 && !h->Gc && h->variant == EP_KERNEL_AUTO ? resident2d_config<T>(h->g) : -1;
-  int tile3[3];
-  const bool res3 = sizeof(T) == 4 && use_fused<T>(h) && !h->Gc && h->variant == EP_KERNEL_AUTO && h->kz == 0 &&
-                    h->rwords && resident3d_tile(h->g, tile3);
+  const bool res2 = h->ndim == 2 && !h->Gc && h->variant == EP_KERNEL_AUTO && resident2d_runs<T>(h->res2, h->g);
+  const bool res3 = sizeof(T) == 4 && h->res3[0] && use_fused<T>(h) && !h->Gc && h->variant == EP_KERNEL_AUTO &&
+                    h->kz == 0 && resident3d_runs(h->g, h->res3);
+  h->chunk_resident = res2 || res3;
+  h->words_clean = false;
   cudaError_t launched = cudaSuccess;
   CK(h, cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
   for (int it = 0; f2 && it < h->opts.n_chk; ++it) {
@@ -653,7 +662,7 @@ ep_status capture_chunk(ep_grid *h) {
     const int chk = it == 0;
     if constexpr (sizeof(T) == 4) {
       if (!chk && res3) {
-        launched = launch_resident3d(tile3, h->g, S, h->dscal, h->dinfo, h->opts.n_chk - 1, h->rcount, h->rwords,
+        launched = launch_resident3d(h->res3, h->g, S, h->dscal, h->dinfo, h->opts.n_chk - 1, h->rcount, h->rwords,
                                      h->cap);
         break;
       }
@@ -668,8 +677,8 @@ ep_status capture_chunk(ep_grid *h) {
       if (chk) launch_check(h->dinfo, h->dscal, h->cap);
       continue;
     }
-    if (!chk && res >= 0) {
-      launched = launch_resident2d<T>(res, h->g, S, h->dscal, h->dinfo, h->opts.n_chk - 1, h->rcount, h->rwords,
+    if (!chk && res2) {
+      launched = launch_resident2d<T>(h->res2, h->g, S, h->dscal, h->dinfo, h->opts.n_chk - 1, h->rcount, h->rwords,
                                       h->cap);
       break;
     }
@@ -735,10 +744,13 @@ ep_status solve(ep_grid *h, long long max_chunks, ep_solve_info *info) {
     init.frozen_at = -1;
     *h->hinfo = init;
     CK(h, cudaMemcpyAsync(h->dinfo, h->hinfo, sizeof(DevInfo), cudaMemcpyHostToDevice, h->stream));
-    if (h->rwords)   // the two arrays are adjacent
-      CK(h, cudaMemsetAsync(h->rcount, 0, (char *)(h->rwords + resident_words(h->g, sizeof(T))) - (char *)h->rcount,
-                            h->stream));
+    h->words_clean = false;
     h->solving = true;
+  }
+  if (h->chunk_resident && !h->words_clean) {   // the two arrays are adjacent
+    CK(h, cudaMemsetAsync(h->rcount, 0, (char *)(h->rwords + resident_words(h->g, sizeof(T))) - (char *)h->rcount,
+                          h->stream));
+    h->words_clean = true;
   }
   CK(h, cudaEventRecord(h->ev0, h->stream));
   const long long cap = h->opts.max_iter / h->opts.n_chk + 2;
@@ -819,6 +831,7 @@ ep_status ep_workspace_bytes(int ndim, const int n[3], ep_precision prec, size_t
   tmp.prec = prec;
   const double L[3] = {1, 1, 1};
   tmp.g = make_geo(ndim, n, L);
+  plan_resident(&tmp);
   Arena a;
   carve(&tmp, a);
   *bytes = a.off;
@@ -856,6 +869,7 @@ ep_status ep_create_grid(int ndim, const int n[3], const double L[3], ep_precisi
   h->prec = prec;
   for (int d = 0; d < 3; ++d) { h->n[d] = d < ndim ? n[d] : 1; h->L[d] = d < ndim ? L[d] : 1.0; }
   h->g = make_geo(ndim, h->n, h->L);
+  plan_resident(h);
   ep_default_solver(ndim, &h->opts);
   Arena a;
   carve(h, a);

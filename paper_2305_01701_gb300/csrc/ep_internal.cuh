@@ -179,22 +179,25 @@ __device__ __forceinline__ void check_one(DevInfo *di, const Scal *sc) {
 }
 
 // ---- the unchecked iterations of a chunk in one launch (ep_resident2d.cu, ep_resident3d.cu) ----
-constexpr int RESIDENT_BLOCKS = 4096;          // counters of a grid
-constexpr long long RESIDENT_POINTS = 200000;  // largest box
-// the exchange's 16-byte words (0: box too large, or FP64 in 3D): in 2D two buffers of
-// three values per point, in 3D three words
+// Whether a grid takes them is decided from its size alone, when its memory is laid out,
+// for the SMs of this part; whether the device can then run the kernel (one cooperative
+// launch), when a chunk is captured.
+constexpr int RESIDENT_SMS = 152, RESIDENT_BLOCKS = 4096;   // blocks: counters of a grid
 struct Word;
-inline long long resident_words(const Geo &g, size_t elem) {
-  if (g.box > RESIDENT_POINTS || (g.ndim == 3 && elem == 8)) return 0;
-  return g.box * (g.ndim == 2 ? elem == 4 ? 2 : 6 : 3);
-}
+// the exchange's 16-byte words, for a grid that fits: in 2D two buffers of three values per
+// point, in 3D three words
+inline long long resident_words(const Geo &g, size_t elem) { return g.box * (g.ndim == 2 ? elem == 4 ? 2 : 6 : 3); }
+bool resident_device_sms(int *sms);   // false: no cooperative launches
 // 3D, FP32 (ep_resident3d.cu)
 bool resident3d_tile(const Geo &g, int tile[3]);   // the points of a block; false: does not fit
+bool resident3d_runs(const Geo &g, const int tile[3]);
 cudaError_t launch_resident3d(const int tile[3], const Geo &g, const Stage<float> &S, const Scal *sc, DevInfo *di,
                               int iters, unsigned *count, Word *words, cudaStream_t st);
 // a configuration that holds the whole grid on the chip at once, or -1
 template <typename T>
 int resident2d_config(const Geo &g);
+template <typename T>
+bool resident2d_runs(int config, const Geo &g);
 // `iters` (odd) iterations from S.u, S.son .. to S.uo, S.snn ..; the stresses before the
 // last of them go to S.son .. (3D likewise).  `count` and `words` are zero when a solve
 // starts and its own until it ends

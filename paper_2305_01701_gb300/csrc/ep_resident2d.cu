@@ -206,6 +206,11 @@ Config config(int c) {
   return c == 0 ? Config{16, 8} : c == 1 ? Config{32, 16} : sizeof(T) == 8 ? Config{16, 16} : Config{32, 32};
 }
 constexpr int CONFIGS = 3;
+template <typename T>
+long long blocks_of(int c, const Geo &g) {
+  const int ox = config<T>(c).wx - 4, oy = config<T>(c).wy - 4;
+  return (long long)((g.nx + ox) / ox) * ((g.ny + oy) / oy);
+}
 
 template <typename T>
 const void *kernel_of(int c) {
@@ -217,14 +222,16 @@ const void *kernel_of(int c) {
 
 }  // namespace
 
+bool resident_device_sms(int *sms) {
+  int dev = 0, coop = 0;
+  return cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop;
+}
+
 template <typename T>
 int resident2d_config(const Geo &g) {
-  int dev = 0, sms = 0, coop = 0, best = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop || sms < 1)
-    return -1;
-  if (g.box > RESIDENT_POINTS) return -1;
+  int best = -1;
   // Points per SM that it pays up to.  FP32: what the registers hold (1024; 383 x 191
   // takes that).  FP64: the points computed twice go through the FP64 pipe, which several
   // grids solved at once on their own streams share: 128^2 (256 points) 9.1 -> 6.6 us
@@ -232,18 +239,22 @@ int resident2d_config(const Geo &g) {
   // alone but 17.4 -> 19.1 with two, so the two launches stay there.
   long long cost = (sizeof(T) == 4 ? 1024 : 256) + 1;
   for (int c = 0; c < CONFIGS; ++c) {
-    const void *k = kernel_of<T>(c);
     const int wx = config<T>(c).wx, wy = config<T>(c).wy;
-    const long long blocks = (long long)((g.nx + wx - 4) / (wx - 4)) * ((g.ny + wy - 4) / (wy - 4));
-    const long long rounds = (blocks + sms - 1) / sms;
-    int per = 0;
-    if (blocks > RESIDENT_BLOCKS || rounds * wx * wy >= cost ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, wx * wy, 0) != cudaSuccess || rounds > per)
-      continue;
+    const long long rounds = (blocks_of<T>(c, g) + RESIDENT_SMS - 1) / RESIDENT_SMS;
+    if (blocks_of<T>(c, g) > RESIDENT_BLOCKS || rounds * wx * wy >= cost) continue;
     cost = rounds * wx * wy;
     best = c;
   }
   return best;
+}
+
+template <typename T>
+bool resident2d_runs(int c, const Geo &g) {
+  int sms = 0, per = 0;
+  return c >= 0 && resident_device_sms(&sms) &&
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of<T>(c), config<T>(c).wx * config<T>(c).wy, 0) ==
+             cudaSuccess &&
+         blocks_of<T>(c, g) <= (long long)per * sms;
 }
 
 template <typename T>
@@ -259,6 +270,8 @@ cudaError_t launch_resident2d(int c, const Geo &g, const Stage<T> &S, const Scal
 
 template int resident2d_config<float>(const Geo &);
 template int resident2d_config<double>(const Geo &);
+template bool resident2d_runs<float>(int, const Geo &);
+template bool resident2d_runs<double>(int, const Geo &);
 template cudaError_t launch_resident2d<float>(int, const Geo &, const Stage<float> &, const Scal *, DevInfo *, int,
                                               unsigned *, Word *, cudaStream_t);
 template cudaError_t launch_resident2d<double>(int, const Geo &, const Stage<double> &, const Scal *, DevInfo *, int,

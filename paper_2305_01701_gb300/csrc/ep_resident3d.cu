@@ -375,6 +375,10 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
   }
 }
 
+dim3 blocks_of(const Tile3 &T, const Geo &g) {
+  return dim3((g.nx + T.t[0]) / T.t[0], (g.ny + T.t[1]) / T.t[1], (g.nz + T.t[2]) / T.t[2]);
+}
+
 // The box that each block owns: of those whose blocks are at most one per SM, the one
 // with the least work (points of the phases, weighted by their instructions).  A grid of
 // more points than the blocks hold (152 x 704) takes the register sweep.
@@ -403,18 +407,22 @@ bool tile_of(const Geo &g, int sms, Tile3 *best) {
 }  // namespace
 
 bool resident3d_tile(const Geo &g, int tile[3]) {
-  int dev = 0, sms = 0, coop = 0, per = 0;
   Tile3 T;
-  if (g.ndim != 3 || g.box > RESIDENT_POINTS || cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-      !tile_of(g, sms < RESIDENT_BLOCKS ? sms : RESIDENT_BLOCKS, &T) ||
-      cudaFuncSetAttribute(k_resident3d, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_resident3d, T.threads(), T.smem()) != cudaSuccess ||
-      per < 1)
+  if (g.ndim != 3 || (g.nx + 1LL) * (g.ny + 1) * (g.nz + 1) > (long long)RESIDENT_SMS * NT_MAX ||
+      !tile_of(g, RESIDENT_SMS, &T))
     return false;
   for (int d = 0; d < 3; ++d) tile[d] = T.t[d];
   return true;
+}
+
+bool resident3d_runs(const Geo &g, const int tile[3]) {
+  const Tile3 T{{tile[0], tile[1], tile[2]}};
+  const dim3 b = blocks_of(T, g);
+  int sms = 0, per = 0;
+  return resident_device_sms(&sms) &&
+         cudaFuncSetAttribute(k_resident3d, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) == cudaSuccess &&
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_resident3d, T.threads(), T.smem()) == cudaSuccess &&
+         (long long)b.x * b.y * b.z <= (long long)per * sms;
 }
 
 cudaError_t launch_resident3d(const int tile[3], const Geo &g, const Stage<float> &S, const Scal *sc, DevInfo *di,
@@ -423,8 +431,7 @@ cudaError_t launch_resident3d(const int tile[3], const Geo &g, const Stage<float
   Geo gg = g;
   Stage<float> SS = S;
   void *args[] = {&gg, &SS, &sc, &di, &T, &iters, &count, &words};
-  const dim3 grid((g.nx + T.t[0]) / T.t[0], (g.ny + T.t[1]) / T.t[1], (g.nz + T.t[2]) / T.t[2]);
-  return cudaLaunchCooperativeKernel((const void *)k_resident3d, grid, dim3(T.threads()), args, T.smem(), st);
+  return cudaLaunchCooperativeKernel((const void *)k_resident3d, blocks_of(T, g), dim3(T.threads()), args, T.smem(), st);
 }
 
 }  // namespace ep

@@ -49,6 +49,32 @@ def test_workspace_bytes_and_argument_errors(lib):
         P.workspace_bytes(2, (0, 4), P.FP64)
 
 
+@pytest.mark.parametrize("nd,small,large,precision", [
+    (2, [(383, 383), (200, 200), (31, 700)], (1000, 900), "FP64"),
+    (2, [(400, 400), (3, 5000)], (1000, 900), "FP32_MIXED"),
+    (3, [(63, 63, 30), (90, 40, 31), (4, 4, 8000)], (127, 100, 80), "FP32_MIXED"),
+    (3, [(31, 31, 31)], (127, 100, 80), "FP64")])
+def test_workspace_holds_no_exchange_words_for_grids_that_do_not_use_them(lib, nd, small, large, precision):
+    """Bytes per point of the padded box: what a grid far beyond the resident sweeps takes."""
+    import math
+
+    import paper_2305_01701_gb300 as P
+
+    def box(n):
+        return (n[0] + 32) // 32 * 32 * math.prod(m + 1 for m in n[1:])
+
+    pr = getattr(P, precision)
+    # beside the fields: small blocks, and 16 bytes per work item of 32 x 8 points
+    per_point = P.workspace_bytes(nd, large, pr) / box(large)
+    for n in small:
+        assert P.workspace_bytes(nd, n, pr) <= per_point * box(n) + 16 * (box(n) // 32) + 20000, n
+    # and one that does take them
+    if (nd, precision) != (3, "FP64"):
+        n = (64, 64) if nd == 2 else (40, 30, 20)
+        words = {(2, "FP64"): 96, (2, "FP32_MIXED"): 32, (3, "FP32_MIXED"): 48}[nd, precision]
+        assert P.workspace_bytes(nd, n, pr) >= (per_point + 0.99 * words) * box(n)
+
+
 def test_layout_of_fields_matches_the_oracle():
     import oracle as O
     from paper_2305_01701_gb300 import _native

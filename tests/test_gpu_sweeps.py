@@ -347,3 +347,28 @@ def test_grids_longer_than_one_launch(P, nd, n, precision, kernel, opts):
     iref, ref = _solve(P, nd, n, pr, getattr(P, kernel[0]), iters, f, shape=kernel[1], **opts, **general)
     info, out = _solve(P, nd, n, pr, P.KERNEL_AUTO, iters, f, **opts)
     _compare(f, out, ref, info, iref, iters, 2.0 ** -53 if precision == "fp64" else EPS32)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_resident_chunks_after_other_chunks_of_the_same_solve(P, precision):
+    """The kernel changed between the chunks of one solve, twice over: the resident sweep starts its
+    exchange anew, and every chunk gives the staged sweep's bits."""
+    n = (64, 50)
+    f = _fields(P, 2, n, 21)
+    outs = []
+    for mixed in (False, True):
+        g = P.Grid(2, n, L=(1.0, 0.8), precision=P.FP64 if precision == "fp64" else P.FP32_MIXED)
+        g.set_material(2.0, 1.0, math.inf, 30.0, 0.0, np.full(n[0] * n[1], 1.5e-3))
+        g.set_solver(tol=0.0, max_iter=1000, n_chk=10)
+        for k, a in f.items():
+            g.set(k, a)
+        for _ in range(2):
+            g.apply_increment(1.0, 1e-4)
+            for chunk in range(6):
+                g.set_kernel(P.KERNEL_AUTO if mixed and chunk % 3 else P.KERNEL_STAGED)
+                assert g.solve_chunks(1)["status"] == P.PENDING
+            g.commit_increment()
+        outs.append({k: g.get(k) for k in list(f) + ["epl", "scale"]})
+        g.close()
+    for k, a in outs[0].items():
+        np.testing.assert_array_equal(outs[1][k], a)

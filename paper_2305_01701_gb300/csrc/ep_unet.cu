@@ -393,7 +393,8 @@ static cudaError_t ensure_shape(UNet &u, int N, int X, int Y, int Z) {
   u.act.clear(); u.grad.clear(); u.act_c.clear(); u.act_lvl.clear();
   if (u.partial) cudaFree(u.partial);
   u.partial = nullptr;
-  u.N = N; u.X = X; u.Y = Y; u.Z = Z;
+  u.N = 0;   // no shape until everything is allocated
+  u.X = X; u.Y = Y; u.Z = Z;
   // tensors in forward order: e[l][0], e[l][1], pool[l] (l < L-1), then per
   // decoder level: cat, d0, d1; then the head output
   auto add = [&](int c, int lvl) {
@@ -429,6 +430,8 @@ static cudaError_t ensure_shape(UNet &u, int N, int X, int Y, int Z) {
   u.xcl = nullptr;
   u.xcl_n = tc_xcl_elems(u, N, X, Y, Z);
   if (e == cudaSuccess && u.xcl_n > 0) e = cudaMalloc((void **)&u.xcl, u.xcl_n * sizeof(__nv_bfloat16));
+  if (e == cudaSuccess) u.N = N;
+  else cudaGetLastError();   // reported here, not by the next launch's check
   return e;
 }
 
@@ -935,7 +938,12 @@ ep_status ep_net_forward(ep_net *n, const float *x, int N, const int size[3], fl
       cudaFree(u.tbuf);
       u.tbuf = nullptr;
       u.tbuf_n = 0;
-      NCK(n, cudaMalloc((void **)&u.tbuf, need * sizeof(__nv_bfloat16)));
+      const cudaError_t e = cudaMalloc((void **)&u.tbuf, need * sizeof(__nv_bfloat16));
+      if (e != cudaSuccess) {
+        u.tbuf = nullptr;
+        cudaGetLastError();   // reported here, not by the next launch's check
+        return nfail(n, EP_ERR_CUDA, std::string("ep_net_forward: cudaMalloc: ") + cudaGetErrorString(e));
+      }
       u.tbuf_n = need;
     }
     NCK(n, u.D == 2 ? forward_tc<2>(u, N, size[0], size[1], Z, x, u.tbuf, y)

@@ -150,3 +150,35 @@ def _layers(nd, cin, cout, base, levels):
     for lv in range(levels - 2, -1, -1):
         out += [(3 * (base << lv), base << lv, 3), (base << lv, base << lv, 3)]
     return out + [(base, cout, 1)]
+
+
+@pytest.mark.parametrize("call", ["gradients", "train_step", "forward"])
+def test_a_shape_that_does_not_fit_fails_each_time_and_leaves_the_network_usable(P, call):
+    """A batch whose first tensor is far beyond the device's memory: refused, refused again, and
+    the next shape that fits gives what an untouched network gives.  The inputs are never read."""
+    import torch
+    gen = torch.Generator().manual_seed(5)
+    nets = [P.Net(2, 9, 5, base=16, levels=2) for _ in range(2)]
+    params = 0.1 * torch.randn(nets[0].n_params(), generator=gen)
+    x = torch.randn((1, 9, 16, 16), generator=gen).cuda()
+    t = torch.randn((1, 5, 16, 16), generator=gen).cuda()
+    torch.cuda.synchronize()
+    for n in nets:
+        n.set_params(params.numpy())
+
+    def run(net, N, size):
+        if call == "forward":
+            y = torch.empty((1, 5, 16, 16), device="cuda")
+            net.forward(x.data_ptr(), N, size, y.data_ptr())
+            return y.cpu().numpy()
+        if call == "gradients":
+            return net.gradients(x.data_ptr(), t.data_ptr(), N, size)[1]
+        net.train_step(x.data_ptr(), t.data_ptr(), N, size, 1e-3)
+        return net.get_params()
+
+    for _ in range(2):
+        with pytest.raises(P.EPError, match="out of memory"):
+            run(nets[0], 60000, [2048, 2048])
+    np.testing.assert_array_equal(run(nets[0], 1, [16, 16]), run(nets[1], 1, [16, 16]))
+    for n in nets:
+        n.close()

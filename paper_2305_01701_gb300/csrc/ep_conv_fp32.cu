@@ -25,6 +25,7 @@
 // memory; the 32 -> 32 convolution of 524,288 voxels 0.69 ms = 42 TFLOP/s, its
 // weight gradient 0.72 ms.
 #include <cuda_bf16.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -337,21 +338,37 @@ __global__ void __launch_bounds__(GT, 1) k_conv_wgrad_tile(const WgradArgs A) {
   }
 }
 
+// s + c += x, the rounding of s + x kept in c (Knuth's two-sum)
+__device__ __forceinline__ void add_exact(float &s, float &c, float x) {
+  const float t = s + x, b = t - s;
+  c += (s - (t - b)) + (x - b);
+  s = t;
+}
+
 // dw = sum of the partial sums, db likewise: 8 threads per element add every
-// eighth split each, then their sums are added, in a fixed order
+// eighth split each, then their sums are added, in a fixed order.  Up to 150
+// partial sums come one after the other here: plain additions made the last
+// layers' gradients up to 1.5 times as far from 64 bits as a tree over all
+// threads does; with their roundings kept every layer's is 0.5 to 0.8 times as
+// far (a training step of the 48 x 48 network 612 -> 620 us, of 64^3 no change).
 __global__ void __launch_bounds__(256) k_wgrad_sum(const float *partial, int slots, long long per, int cout, float *dw,
                                                    float *db) {
-  __shared__ float sh[8][32];
+  __shared__ float sh[8][32], ch[8][32];
   const int e = threadIdx.x & 31, j = threadIdx.x >> 5;
   const long long i = (long long)blockIdx.x * 32 + e, stride = per + cout;
-  float s = 0.f;
+  float s = 0.f, c = 0.f;
   if (i < stride)
-    for (int q = j; q < slots; q += 8) s += partial[q * stride + i];
+    for (int q = j; q < slots; q += 8) add_exact(s, c, partial[q * stride + i]);
   sh[j][e] = s;
+  ch[j][e] = c;
   __syncthreads();
   if (j != 0 || i >= stride) return;
 #pragma unroll
-  for (int q = 1; q < 8; ++q) s += sh[q][e];
+  for (int q = 1; q < 8; ++q) {
+    add_exact(s, c, sh[q][e]);
+    c += ch[q][e];
+  }
+  if (fabsf(s) < INFINITY) s += c;   // an infinite sum's rounding is no number
   if (i < per) dw[i] = s;
   else db[i - per] = s;
 }

@@ -182,3 +182,30 @@ def test_a_shape_that_does_not_fit_fails_each_time_and_leaves_the_network_usable
     np.testing.assert_array_equal(run(nets[0], 1, [16, 16]), run(nets[1], 1, [16, 16]))
     for n in nets:
         n.close()
+
+
+@pytest.mark.parametrize("nd,size,N", [(2, (64, 64), 8), (2, (256, 128), 2), (3, (32, 32, 16), 2)])
+def test_partial_sums_of_a_gradient_add_without_their_roundings(P, nd, size, N):
+    """The head's bias gradient of a zero head is -2 / n times the sum of the targets: with n a
+    power of two its terms are exact in FP32.  A block's threads add runs of 16 to 64 of them
+    (random roundings, averaged over hundreds of runs), and the hundreds of partial sums add
+    without theirs: the result is within 2^-23, one rounding and as much again."""
+    import torch
+    worst = 0.0
+    for seed in range(6):
+        gen = torch.Generator().manual_seed(seed)
+        net = P.Net(nd, 3, 4, base=16, levels=1)
+        params = net.get_params().copy()
+        params[-4 - 4 * 16:] = 0.0
+        net.set_params(params)
+        dims = tuple(reversed(size))
+        x = torch.randn((N, 3) + dims, generator=gen).cuda()
+        t = (torch.rand((N, 4) + dims, generator=gen) + 0.1).cuda()
+        torch.cuda.synchronize()
+        g = net.gradients(x.data_ptr(), t.data_ptr(), N, list(size))[1][-4:]
+        n = t.numel()
+        assert n & (n - 1) == 0
+        want = (-2.0 / n * t.double().transpose(0, 1).reshape(4, -1).sum(1)).cpu().numpy()
+        worst = max(worst, np.abs(g / want - 1.0).max())
+        net.close()
+    assert worst <= 2.0 ** -23, worst * 2.0 ** 23

@@ -192,6 +192,56 @@ def test_fp64_body_force_manufactured(P):
     del sp
 
 
+def _force_3d(s, seed):
+    """A force in every direction: a smooth part and noise, per face."""
+    rng = np.random.default_rng(seed)
+    out = []
+    for d in range(3):
+        shape = tuple(s.n[q] + (q == d) for q in reversed(range(3)))
+        z, y, x = np.meshgrid(*(np.linspace(-1.0, 1.0, m) for m in shape), indexing="ij")
+        out.append(2e-4 * (d + 1) * np.cos(1.3 * x + 0.7 * y * (d + 1) - 0.9 * z) + 5e-5 * rng.standard_normal(shape))
+    return out
+
+
+def test_fp64_body_force_parity_3d(P):
+    """The 3D FP64 stage kernels add the body force at x-, y- and z-faces: against the oracle on a
+    ragged grid through first yield, increments with and without a force in turn on one grid (the
+    captured chunk depends on it)."""
+    s = E.config(3, n=(17, 13, 11), tol=1e-9, precision="fp64", inclusion_radius=0.2)
+    g, o = gpu_grid(P, s, P.FP64), O.from_setup(s)
+    for inc in range(7):
+        bf = _force_3d(s, inc) if inc % 3 != 1 else None
+        g.apply_increment_rates(rates_of(s), s.dt, body_force=bf)
+        o.apply_increment(rates_of(s), s.dt, body_force=bf)
+        ig, io = g.solve_increment(), o.solve_increment()
+        assert ig["iters"] == io["iters"], (inc, ig["iters"], io["iters"])
+        sc = group_scales(o, FIELDS_3D)
+        for f in FIELDS_3D:
+            e = rel_err(g.get(f), o.get(f), sc[f])
+            assert e <= 1e-10, (inc, f, e)
+    assert io["n_plastic"] > 0
+    g.close()
+
+
+def test_fp32_body_force_within_stated_bounds_3d(P):
+    """FP32 in 3D with a body force runs the staged sweep, without one the register sweep or the
+    resident iterations: increments of both kinds on one grid against the FP64 oracle."""
+    s = E.config(3, n=(22, 15, 12), inclusion_radius=0.2)
+    g = gpu_grid(P, s, P.FP32_MIXED, tol=1e-6, max_iter=400000)
+    o = O.from_setup(s, tol=1e-10)
+    for inc in range(4):
+        bf = _force_3d(s, inc) if inc % 2 else None
+        g.apply_increment_rates(rates_of(s), s.dt, body_force=bf)
+        o.apply_increment(rates_of(s), s.dt, body_force=bf)
+        g.solve_increment()
+        o.solve_increment()
+        sc = group_scales(o, FIELDS_3D)
+        for f in ("txx", "tyy", "tzz", "txy", "txz", "tyz", "p"):
+            e = rel_err(g.get(f), o.get(f), sc[f])
+            assert e <= 1e-5, (inc, f, e)
+    g.close()
+
+
 def run_fp32_vs_oracle(P, s, increments, gpu_tol=1e-6, oracle_tol=1e-10, kernel=None, **solver):
     """FP32 mixed GPU solve at its tolerance against a tightly converged FP64
     oracle: the worst L-infinity-normalised error of each field."""

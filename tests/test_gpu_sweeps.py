@@ -372,3 +372,48 @@ def test_resident_chunks_after_other_chunks_of_the_same_solve(P, precision):
         g.close()
     for k, a in outs[0].items():
         np.testing.assert_array_equal(outs[1][k], a)
+
+
+@pytest.mark.parametrize("grids", [[(2, (64, 64), "fp64"), (2, (64, 50), "fp64"), (2, (128, 128), "fp64")],
+                                   [(2, (300, 180), "fp32"), (2, (383, 191), "fp32")],
+                                   [(3, (90, 40, 24), "fp32"), (3, (40, 33, 14), "fp32"), (2, (300, 180), "fp32")]])
+def test_resident_grids_solved_at_once_equal_one_after_the_other(P, grids):
+    """Cooperative launches of several grids on their own streams, from a host thread each: the
+    launches take turns where they do not fit the chip together, and the results are the same."""
+    import threading
+
+    def make(nd, n, precision):
+        g = P.Grid(nd, n, L=(1.0, 0.8, 1.3)[:nd], precision=P.FP64 if precision == "fp64" else P.FP32_MIXED)
+        g.set_material(2.0, 1.0, math.inf, 30.0, 0.0, np.full(int(np.prod(n)), 1.5e-3))
+        g.set_solver(tol=0.0, max_iter=400, n_chk=20)
+        for k, a in _fields(P, nd, n, 22).items():
+            g.set(k, a)
+        g.snapshot()
+        return g
+
+    def solve(g, out, q):
+        for _ in range(5):
+            g.apply_increment(1.0, 1e-4, P.LOAD_XY if g.ndim == 2 else P.LOAD_XZ)
+            out[q] = g.solve_increment(raise_on_fail=False)["status"]
+            g.commit_increment()
+
+    gs = [make(*a) for a in grids]
+    names = ["vx", "vy", "txx", "tyy", "txy", "p", "epl", "scale"]
+    status = [None] * len(gs)
+    for q, g in enumerate(gs):
+        solve(g, status, q)
+    want = [{k: g.get(k) for k in names} for g in gs]
+    assert status == [5] * len(gs)
+    for g in gs:
+        g.restore()
+    status = [None] * len(gs)
+    threads = [threading.Thread(target=solve, args=(g, status, q)) for q, g in enumerate(gs)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert status == [5] * len(gs)
+    for g, w in zip(gs, want):
+        for k in names:
+            np.testing.assert_array_equal(g.get(k), w[k])
+        g.close()

@@ -25,20 +25,12 @@
 #include <math.h>
 
 #include "ep_internal.cuh"
+#include "ep_lanes.cuh"
 #include "ep_words.cuh"
 
 namespace ep {
 
 namespace {
-
-// As in ep_sweep2d.cu.
-template <typename T>
-__device__ __forceinline__ T return_scale(T J2, T Y) {
-  Y = Y > (T)0 ? Y : (T)0;
-  if (J2 < Y * Y * (T)(sizeof(T) == 8 ? 1.0 - 1e-15 : 1.0 - 1e-6)) return (T)1;
-  const T sj = sqrt(J2);
-  return sj > Y ? Y / sj : (T)1;
-}
 
 template <typename T, int WX, int WY>
 __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const Scal *sc, DevInfo *di, int iters,
@@ -112,7 +104,7 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
       pr = fma(bp, pr, obp * fma(-KDt, div, pb));
       if (!frozen) {
         const T J2 = fma((T)0.0625, txy * txy, (T)0.5 * fma(c1, c1, c0 * c0));
-        s = return_scale(J2, fma(Ac, pr, yc));
+        s = scale_of(J2, fma(Ac, pr, yc));
       }
       n0 = s * c0;
       n1 = s * c1;

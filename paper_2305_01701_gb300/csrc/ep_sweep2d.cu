@@ -21,45 +21,12 @@
 #include <algorithm>
 
 #include "ep_internal.cuh"
+#include "ep_lanes.cuh"
+#include "ep_measures.cuh"
 
 namespace ep {
 
 namespace {
-
-__device__ __forceinline__ double maxn(double a, double b) { return (a > b || a != a) ? a : b; }
-// |a - b|, formed in FP64
-__device__ __forceinline__ double gap(double a, double b) { return fabs(a - b); }
-
-// block-wide max of |v| as IEEE bits (a NaN sorts above infinity), one atomic per
-// block; blocks are (32, warps)
-__device__ __forceinline__ void block_max(double v, unsigned long long *slot) {
-  __shared__ unsigned long long sm[8];
-  unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(0xffffffffu, b, o);
-    b = b > w ? b : w;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) sm[threadIdx.y] = b;
-  __syncthreads();
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    for (int q = 1; q < (int)blockDim.y; ++q) b = b > sm[q] ? b : sm[q];
-    if (b) atomicMax(slot, b);
-  }
-}
-
-__device__ __forceinline__ bool skip(const DevInfo *di) { return di != nullptr && *(volatile const int *)&di->done != 0; }
-
-// centre scale min(1, Y / sqrt(J2)).  Below Y^2 by more than the rounding of
-// both, sqrt(J2) > Y cannot hold and the scale is 1 without the root.
-template <typename T>
-__device__ __forceinline__ T return_scale(T J2, T Y) {
-  Y = Y > (T)0 ? Y : (T)0;
-  if (J2 < Y * Y * (T)(sizeof(T) == 8 ? 1.0 - 1e-15 : 1.0 - 1e-6)) return (T)1;
-  const T sj = sqrt(J2);
-  return sj > Y ? Y / sj : (T)1;
-}
 
 // row range of this warp
 struct Strip {
@@ -129,7 +96,7 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
         s = S.s[e];   // frozen plasticity: the held scale (Sec. 3.3)
       } else {
         const T J2 = fma((T)0.0625, txy * txy, (T)0.5 * fma(c1, c1, c0 * c0));
-        s = return_scale(J2, fma(Ac, pr, S.yc[e]));
+        s = scale_of(J2, fma(Ac, pr, S.yc[e]));
         S.s[e] = s;
       }
       const T n0 = s * c0, n1 = s * c1, s0 = n0 - pr, s1 = n1 - pr;

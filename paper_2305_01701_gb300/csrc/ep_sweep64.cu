@@ -24,33 +24,11 @@
 
 #include "ep_internal.cuh"
 #include "ep_lanes.cuh"
+#include "ep_measures.cuh"
 
 namespace ep {
 
 namespace {
-
-__device__ __forceinline__ double maxn(double a, double b) { return (a > b || a != a) ? a : b; }
-
-// block-wide max of |v| as IEEE bits (a NaN sorts above infinity), one atomic per
-// block; blocks are (32, rows)
-__device__ __forceinline__ void block_max(double v, unsigned long long *slot) {
-  __shared__ unsigned long long sm[8];
-  unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(0xffffffffu, b, o);
-    b = b > w ? b : w;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) sm[threadIdx.y] = b;
-  __syncthreads();
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    for (int q = 1; q < (int)blockDim.y; ++q) b = b > sm[q] ? b : sm[q];
-    if (b) atomicMax(slot, b);
-  }
-}
-
-__device__ __forceinline__ bool skip(const DevInfo *di) { return di != nullptr && *(volatile const int *)&di->done != 0; }
 
 struct Pt {
   int i, j, k;
@@ -106,38 +84,38 @@ __global__ void __launch_bounds__(256) k64_trial(Geo g, int2 o, Stage<double> S,
     const double e0 = (S.u[0][e + 1] - S.u[0][e]) * g.rdx, e1 = (S.u[1][e + px] - S.u[1][e]) * g.rdy;
     const double *p0 = S.pr[0];
     const double xy = (p0[e] + p0[e + 1]) + (p0[e + px] + p0[e + px + 1]);
-      const double e2 = (S.u[2][e + pl] - S.u[2][e]) * g.rdz, div = e0 + e1 + e2, d3 = div * (1.0 / 3.0);
-      const double *p1 = S.pr[1], *p2 = S.pr[2];
-      const double xz = (p1[e] + p1[e + 1]) + (p1[e + pl] + p1[e + pl + 1]);
-      const double yz = (p2[e] + p2[e + px]) + (p2[e + pl] + p2[e + pl + px]);
-      const double t0 = fma(0.25, xy + xz, fma(two_eta, e0 - d3, S.tbn[0][e]));
-      const double t1 = fma(0.25, yz - xy, fma(two_eta, e1 - d3, S.tbn[1][e]));
-      const double t2 = fma(-0.25, xz + yz, fma(two_eta, e2 - d3, S.tbn[2][e]));
-      S.Tn[0][e] = fma(bt, S.son[0][e], ob * t0);
-      S.Tn[1][e] = fma(bt, S.son[1][e], ob * t1);
-      S.Tn[2][e] = fma(bt, S.son[2][e], ob * t2);
-      S.dv[e] = div;
+    const double e2 = (S.u[2][e + pl] - S.u[2][e]) * g.rdz, div = e0 + e1 + e2, d3 = div * (1.0 / 3.0);
+    const double *p1 = S.pr[1], *p2 = S.pr[2];
+    const double xz = (p1[e] + p1[e + 1]) + (p1[e + pl] + p1[e + pl + 1]);
+    const double yz = (p2[e] + p2[e + px]) + (p2[e + pl] + p2[e + pl + px]);
+    const double t0 = fma(0.25, xy + xz, fma(two_eta, e0 - d3, S.tbn[0][e]));
+    const double t1 = fma(0.25, yz - xy, fma(two_eta, e1 - d3, S.tbn[1][e]));
+    const double t2 = fma(-0.25, xz + yz, fma(two_eta, e2 - d3, S.tbn[2][e]));
+    S.Tn[0][e] = fma(bt, S.son[0][e], ob * t0);
+    S.Tn[1][e] = fma(bt, S.son[1][e], ob * t1);
+    S.Tn[2][e] = fma(bt, S.son[2][e], ob * t2);
+    S.dv[e] = div;
   }
   const bool x1 = i > 0 && i < nx, y1 = j > 0 && j < ny, z1 = k > 0 && k < nz;
-    // spins summed over the four neighbours of another orientation
-    const double *w0 = S.om[0], *w1 = S.om[1], *w2 = S.om[2];
-    const auto edge = [&](int c, double wa, double wb) {
-      const double tr = fma(S.om[c][e], S.md[c][e],
-                            fma(wa, S.ma[c][e], fma(wb, S.mb[c][e], fma(eta, S.es[c][e], S.tbs[c][e]))));
-      return fma(bt, S.sos[c][e], ob * tr);
-    };
-    double v = 0.0;
-    if (k < nz && x1 && y1)
-      v = edge(0, (w1[e - px] + w1[e]) + (w1[e - px + pl] + w1[e + pl]), (w2[e - 1] + w2[e]) + (w2[e - 1 + pl] + w2[e + pl]));
-    S.Ts[0][e] = v;
-    v = 0.0;
-    if (j < ny && x1 && z1)
-      v = edge(1, (w0[e - pl] + w0[e - pl + px]) + (w0[e] + w0[e + px]), (w2[e - 1] + w2[e]) + (w2[e - 1 + px] + w2[e + px]));
-    S.Ts[1][e] = v;
-    v = 0.0;
-    if (i < nx && y1 && z1)
-      v = edge(2, (w1[e - px] + w1[e - px + 1]) + (w1[e] + w1[e + 1]), (w0[e - pl] + w0[e - pl + 1]) + (w0[e] + w0[e + 1]));
-    S.Ts[2][e] = v;
+  // spins summed over the four neighbours of another orientation
+  const double *w0 = S.om[0], *w1 = S.om[1], *w2 = S.om[2];
+  const auto edge = [&](int c, double wa, double wb) {
+    const double tr = fma(S.om[c][e], S.md[c][e],
+                          fma(wa, S.ma[c][e], fma(wb, S.mb[c][e], fma(eta, S.es[c][e], S.tbs[c][e]))));
+    return fma(bt, S.sos[c][e], ob * tr);
+  };
+  double v = 0.0;
+  if (k < nz && x1 && y1)
+    v = edge(0, (w1[e - px] + w1[e]) + (w1[e - px + pl] + w1[e + pl]), (w2[e - 1] + w2[e]) + (w2[e - 1 + pl] + w2[e + pl]));
+  S.Ts[0][e] = v;
+  v = 0.0;
+  if (j < ny && x1 && z1)
+    v = edge(1, (w0[e - pl] + w0[e - pl + px]) + (w0[e] + w0[e + px]), (w2[e - 1] + w2[e]) + (w2[e - 1 + px] + w2[e + px]));
+  S.Ts[1][e] = v;
+  v = 0.0;
+  if (i < nx && y1 && z1)
+    v = edge(2, (w1[e - px] + w1[e - px + 1]) + (w1[e] + w1[e + 1]), (w0[e - pl] + w0[e - pl + 1]) + (w0[e] + w0[e + 1]));
+  S.Ts[2][e] = v;
 }
 
 // ---- pressure and return at centres ------------------------------------------------
@@ -152,15 +130,11 @@ __global__ void __launch_bounds__(256) k64_centres(Geo g, int2 o, Stage<double> 
     const double p = fma(sc->bp, S.sop[e], sc->obp * fma(-sc->KDt, S.dv[e], S.pb[e]));
     const double *t0 = S.Ts[0];
     double tn[3] = {S.Tn[0][e], S.Tn[1][e], S.Tn[2][e]};
+    const double *t1 = S.Ts[1], *t2 = S.Ts[2];
     const double xy = (t0[e] + t0[e + 1]) + (t0[e + px] + t0[e + px + 1]);
-    double j4 = xy * xy, jn = fma(tn[1], tn[1], tn[0] * tn[0]);
-    {
-      const double *t1 = S.Ts[1], *t2 = S.Ts[2];
-      const double xz = (t1[e] + t1[e + 1]) + (t1[e + pl] + t1[e + pl + 1]);
-      const double yz = (t2[e] + t2[e + px]) + (t2[e + pl] + t2[e + pl + px]);
-      j4 = fma(yz, yz, fma(xz, xz, j4));
-      jn = fma(tn[2], tn[2], jn);
-    }
+    const double xz = (t1[e] + t1[e + 1]) + (t1[e + pl] + t1[e + pl + 1]);
+    const double yz = (t2[e] + t2[e + px]) + (t2[e + pl] + t2[e + pl + px]);
+    const double j4 = fma(yz, yz, fma(xz, xz, xy * xy)), jn = fma(tn[2], tn[2], fma(tn[1], tn[1], tn[0] * tn[0]));
     double s = 1.0;
     if (frozen) {
       s = S.s[e];   // frozen plasticity: the held scale (Sec. 3.3)
@@ -207,10 +181,8 @@ __global__ void __launch_bounds__(256) k64_edges(Geo g, int2 o, Stage<double> S,
     double v[3] = {0.0, 0.0, 0.0};
     if (k < nz && x1 && y1)
       v[0] = (s[e - px - 1] + s[e - px] + s[e - 1] + s[e]) * (0.25 * S.Ts[0][e]);
-    {
-      if (j < ny && x1 && z1) v[1] = (s[e - pl - 1] + s[e - pl] + s[e - 1] + s[e]) * (0.25 * S.Ts[1][e]);
-      if (i < nx && y1 && z1) v[2] = (s[e - pl - px] + s[e - pl] + s[e - px] + s[e]) * (0.25 * S.Ts[2][e]);
-    }
+    if (j < ny && x1 && z1) v[1] = (s[e - pl - 1] + s[e - pl] + s[e - 1] + s[e]) * (0.25 * S.Ts[1][e]);
+    if (i < nx && y1 && z1) v[2] = (s[e - pl - px] + s[e - pl] + s[e - px] + s[e]) * (0.25 * S.Ts[2][e]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       S.sns[c][e] = v[c];
@@ -266,13 +238,11 @@ __global__ void __launch_bounds__(256) k64_velocity(Geo g, int2 o, Stage<double>
       R = fma(S.sns[2][e + pl] - S.sns[2][e], g.rdz, R);
     }
     face(1, iy, y1, R);
-    {
-      const bool iz = i < nx && j < ny, z1 = iz && k > 0 && k < nz;
-      if (z1)
-        R = fma(S.sns[2][e + px] - S.sns[2][e], g.rdy,
-                fma(S.sns[1][e + 1] - S.sns[1][e], g.rdx, (S.sx[2][e] - S.sx[2][e - pl]) * g.rdz));
-      face(2, iz, z1, R);
-    }
+    const bool iz = i < nx && j < ny, z1 = iz && k > 0 && k < nz;
+    if (z1)
+      R = fma(S.sns[2][e + px] - S.sns[2][e], g.rdy,
+              fma(S.sns[1][e + 1] - S.sns[1][e], g.rdx, (S.sx[2][e] - S.sx[2][e - pl]) * g.rdz));
+    face(2, iz, z1, R);
   }
   if (CHK && di) {
     block_max(rmax, &di->red[RED_R]);

@@ -16,9 +16,9 @@
 //     inputs are loaded one row ahead;
 //   * check iterations reduce the residual norms per warp (one atomic per
 //     warp, item and norm).
-// The deviatoric rate is formed before it is scaled (2 eta e and -2 eta div / 3 as two
-// terms round each at the size of the larger); its two registers more would leave an SM
-// three FP32 blocks (519 us a sweep), so the compiler is held to 128.
+// The deviatoric rate e - div / 3 is rounded once and scaled after (2 eta e and -2 eta div / 3
+// as two terms round each at the size of the larger); its two registers more would leave an
+// SM three FP32 blocks (519 us a sweep), so the compiler is held to 128.
 // Warps take items independently, so a block never waits for another warp.
 // 256 grids of 127^2 .. 511^2, one sweep: FP32 is bound by the 20 arrays it
 // moves, 465 us (5.5 TB/s; one column a thread and two rows ahead: 773 us; two
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
     const V m1 = mask(in_x1(0), in_x1(1), (T)1);
     const V stx = mask(in_x1(0), in_x1(1), Q.vstep), sty = mask(in_x0(0), in_x0(1), Q.vstep);
     const V rdx = bc(Q.rdx), rdy = bc(Q.rdy), nrdx = bc(-Q.rdx), bt = bc(Q.bt), ob = bc(Q.ob);
-    const V eta = bc(Q.eta), two_eta = bc(Q.two_eta), third = bc((T)(-1.0 / 3.0)), qr = bc((T)0.25);
+    const V eta = bc(Q.eta), two_eta = bc(Q.two_eta), m3 = bc((T)(-1.0 / 3.0)), qr = bc((T)0.25);
     const T *u0 = I.u[b][0], *u1 = I.u[b][1];
     // loads read the nearest in-box columns and row without a test: a value
     // outside the box only ever enters masked expressions.  A 2D box that fits
@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(32 * SWARPS, sizeof(T) == 4 && !CHK ? 4 : 0)
       // ---- centre (gi, t - 1): relaxed trial, pressure, return ----
       const V Pc = vadd(P_1, P), tc = vadd(ts_1, ts);
       const V xy = vadd(Pc, xp<32>(Pc)), txy = vadd(tc, xp<32>(tc));
-      const V exx = vmul(vsub(xp<32>(vx_1), vx_1), rdx), eyy = vmul(vsub(vy, vy_1), rdy);
-      const V div = vadd(exx, eyy), d0 = vfma(div, third, exx), d1 = vfma(div, third, eyy);
+      const V ux = vsub(xp<32>(vx_1), vx_1), uy = vsub(vy, vy_1);
+      const V div = vfma(uy, rdy, vmul(ux, rdx)), d3 = vmul(div, m3), d0 = vfma(ux, rdx, d3), d1 = vfma(uy, rdy, d3);
       const V q = vmul(xy, qr);
       const V t0 = vadd(vfma(d0, two_eta, tbn0), q), t1 = vsub(vfma(d1, two_eta, tbn1), q);
       const V c0 = vfma(sn0, bt, vmul(t0, ob)), c1 = vfma(sn1, bt, vmul(t1, ob));

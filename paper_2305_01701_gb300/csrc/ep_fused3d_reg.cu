@@ -318,7 +318,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
   V u0 = zero, u1 = zero, u2 = zero, u0_1 = zero, u1_1 = zero, u2_1 = zero, u0_2 = zero, u1_2 = zero, u2_2 = zero;
   V rq0 = zero;
   V D_1 = zero, E_1 = zero, F_1 = zero, G_1 = zero, J_1 = zero, L_1 = zero, M_1 = zero, N_1 = zero, O_1 = zero;
-  V wxy_1 = zero, qxy_1 = zero, gxy_1 = zero, e1_1 = zero, tsxz_1 = zero, tsyz_1 = zero;
+  V wxy_1 = zero, qxy_1 = zero, gxy_1 = zero, g1_1 = zero, tsxz_1 = zero, tsyz_1 = zero;
   V s_2 = zero, U_2 = zero;                                // quarter scale and its x pair sum, plane t-2
   V sxx_2 = zero, syy_2 = zero, szz_2 = zero, szz_3 = zero;   // centre stress minus pressure
   V nxy_2 = zero, nxz_2 = zero, nyz_2 = zero;              // edge stress, level t-2
@@ -449,15 +449,14 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
         }
       }
       {   // centres of plane t-1
-        const V e0 = vmul(vsub(xp<LPR>(u0_1), u0_1), bc(rdx));
-        const V e1 = e1_1;
-        const V e2 = vmul(vsub(u2, u2_1), bc(rdz));
-        div = vadd(vadd(e0, e1), e2);
+        const V g0 = vsub(xp<LPR>(u0_1), u0_1), g1 = g1_1, g2 = vsub(u2, u2_1);
+        div = vfma(g2, bc(rdz), vfma(g1, bc(rdy), vmul(g0, bc(rdx))));
         const V O = vadd(pyz, S.pyz.r[qp]);
         const V Pxz = vadd(N_1, vN), Pyz = vadd(O_1, O), Pxy = M_1;
-        // the deviatoric rate is formed before it is scaled: 2 eta e and -2 eta div / 3 as
-        // two terms would round each at the size of the larger
-        const V m3 = bc((T)(-1.0 / 3.0)), d0 = vfma(div, m3, e0), d1 = vfma(div, m3, e1), d2 = vfma(div, m3, e2);
+        // the deviatoric rate e - div / 3 is rounded once and scaled after: 2 eta e and
+        // -2 eta div / 3 as two terms would round each at the size of the larger
+        const V d3 = vmul(div, bc((T)(-1.0 / 3.0)));
+        const V d0 = vfma(g0, bc(rdx), d3), d1 = vfma(g1, bc(rdy), d3), d2 = vfma(g2, bc(rdz), d3);
         const V r0 = vadd(Pxy, Pxz), r1 = vsub(Pyz, Pxy), r2 = vadd(Pxz, Pyz);
         V t0, t1, t2;
         if constexpr (GC) {
@@ -474,7 +473,7 @@ __device__ __forceinline__ void reg_body(const Maps<GC> &M, const Args<typename 
         c0v = vfma(own(I_SON0), bc(bt), vmul(t0, bc(ob)));
         c1v = vfma(own(I_SON1), bc(bt), vmul(t1, bc(ob)));
         c2v = vfma(own(I_SON2), bc(bt), vmul(t2, bc(ob)));
-        e1_1 = vmul(vsub(above(I_U1), u1), bc(rdy));
+        g1_1 = vsub(above(I_U1), u1);
         M_1 = vadd(vM, S.M.r[qp]);
         N_1 = vN; O_1 = O;
       }

@@ -96,10 +96,10 @@ __global__ void __launch_bounds__(WX *WY) k_resident2d(Geo g, Stage<T> S, const 
     if (cin) {
       const T xy = (p + sp[ty + 1][tx]) + (sp[ty][tx + 1] + sp[ty + 1][tx + 1]);
       const T txy = (ts + st[ty + 1][tx]) + (st[ty][tx + 1] + st[ty + 1][tx + 1]);
-      const T e0 = (su0[ty][tx + 1] - u0) * rdx, e1 = (su1[ty + 1][tx] - u1) * rdy;
-      const T div = e0 + e1, m3 = (T)(-1.0 / 3.0);
-      const T t0 = fma((T)0.25, xy, fma(two_eta, fma(div, m3, e0), tb0));
-      const T t1 = fma((T)-0.25, xy, fma(two_eta, fma(div, m3, e1), tb1));
+      const T d0 = su0[ty][tx + 1] - u0, d1 = su1[ty + 1][tx] - u1;
+      const T div = fma(d1, rdy, d0 * rdx), d3 = div * (T)(-1.0 / 3.0);
+      const T t0 = fma((T)0.25, xy, fma(two_eta, fma(d0, rdx, d3), tb0));
+      const T t1 = fma((T)-0.25, xy, fma(two_eta, fma(d1, rdy, d3), tb1));
       const T c0 = fma(bt, n0, ob * t0), c1 = fma(bt, n1, ob * t1);
       pr = fma(bp, pr, obp * fma(-KDt, div, pb));
       if (!frozen) {

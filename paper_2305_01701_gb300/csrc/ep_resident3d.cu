@@ -237,14 +237,14 @@ __global__ void __launch_bounds__(NT_MAX, 1) k_resident3d(Geo g, Stage<float> S,
     // ---- 3: relaxed trial, pressure and return at the own centre ----
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
     if (cin) {
-      const float e0 = (u0[l + 1] - u0[l]) * rdx, e1 = (u1[l + ly] - u1[l]) * rdy, e2 = (u2[l + lz] - u2[l]) * rdz;
-      const float div = e0 + e1 + e2, m3 = -1.f / 3.f;
+      const float d0 = u0[l + 1] - u0[l], d1 = u1[l + ly] - u1[l], d2 = u2[l + lz] - u2[l];
+      const float div = fmaf(d2, rdz, fmaf(d1, rdy, d0 * rdx)), d3 = div * (-1.f / 3.f);
       const float xy = (p0[l] + p0[l + 1]) + (p0[l + ly] + p0[l + ly + 1]);
       const float xz = (p1[l] + p1[l + 1]) + (p1[l + lz] + p1[l + lz + 1]);
       const float yz = (p2[l] + p2[l + ly]) + (p2[l + lz] + p2[l + lz + ly]);
-      c0 = fmaf(bt, c0, ob * fmaf(0.25f, xy + xz, fmaf(Q.two_eta, fmaf(div, m3, e0), tb0)));
-      c1 = fmaf(bt, c1, ob * fmaf(0.25f, yz - xy, fmaf(Q.two_eta, fmaf(div, m3, e1), tb1)));
-      c2 = fmaf(bt, c2, ob * fmaf(-0.25f, xz + yz, fmaf(Q.two_eta, fmaf(div, m3, e2), tb2)));
+      c0 = fmaf(bt, c0, ob * fmaf(0.25f, xy + xz, fmaf(Q.two_eta, fmaf(d0, rdx, d3), tb0)));
+      c1 = fmaf(bt, c1, ob * fmaf(0.25f, yz - xy, fmaf(Q.two_eta, fmaf(d1, rdy, d3), tb1)));
+      c2 = fmaf(bt, c2, ob * fmaf(-0.25f, xz + yz, fmaf(Q.two_eta, fmaf(d2, rdz, d3), tb2)));
       pr = fmaf(Q.bp, pr, Q.obp * fmaf(-Q.KDt, div, pb));
       if (!frozen) {
         const float txy = (t0[l] + t0[l + 1]) + (t0[l + ly] + t0[l + ly + 1]);

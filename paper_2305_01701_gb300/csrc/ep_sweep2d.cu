@@ -85,10 +85,11 @@ __global__ void __launch_bounds__(128) k_stress2d(Geo g, Stage<T> S, const Scal 
     const T xy = pc + right(pc), txy = tc + right(tc), u0_r = right(u0);
     if (own) S.Ts[0][e] = t_j;
     if (own && i < nx && j < ny) {
-      const T e0 = (u0_r - u0) * rdx, e1 = (S.u[1][e + px] - S.u[1][e]) * rdy;
-      const T div = e0 + e1, m3 = (T)(-1.0 / 3.0);
-      const T t0 = fma((T)0.25, xy, fma(two_eta, fma(div, m3, e0), S.tbn[0][e]));
-      const T t1 = fma((T)-0.25, xy, fma(two_eta, fma(div, m3, e1), S.tbn[1][e]));
+      const T d0 = u0_r - u0, d1 = S.u[1][e + px] - S.u[1][e];
+      // the rate e - div / 3 rounded once, then scaled
+      const T div = fma(d1, rdy, d0 * rdx), d3 = div * (T)(-1.0 / 3.0);
+      const T t0 = fma((T)0.25, xy, fma(two_eta, fma(d0, rdx, d3), S.tbn[0][e]));
+      const T t1 = fma((T)-0.25, xy, fma(two_eta, fma(d1, rdy, d3), S.tbn[1][e]));
       const T c0 = fma(bt, S.son[0][e], ob * t0), c1 = fma(bt, S.son[1][e], ob * t1);
       const T pr = fma(bp, S.sop[e], obp * fma(-KDt, div, S.pb[e]));
       T s = 1;

@@ -81,16 +81,17 @@ __global__ void __launch_bounds__(256) k64_trial(Geo g, int2 o, Stage<double> S,
   const long long e = q.e, px = g.px, pl = g.plane;
   const double two_eta = sc->two_eta, eta = 0.5 * two_eta, bt = sc->bt, ob = 1.0 - bt;
   if (i < nx && j < ny && k < nz) {
-    const double e0 = (S.u[0][e + 1] - S.u[0][e]) * g.rdx, e1 = (S.u[1][e + px] - S.u[1][e]) * g.rdy;
+    const double d0 = S.u[0][e + 1] - S.u[0][e], d1 = S.u[1][e + px] - S.u[1][e], d2 = S.u[2][e + pl] - S.u[2][e];
+    // the rate e - div / 3 rounded once, then scaled
+    const double div = fma(d2, g.rdz, fma(d1, g.rdy, d0 * g.rdx)), d3 = div * (-1.0 / 3.0);
     const double *p0 = S.pr[0];
     const double xy = (p0[e] + p0[e + 1]) + (p0[e + px] + p0[e + px + 1]);
-    const double e2 = (S.u[2][e + pl] - S.u[2][e]) * g.rdz, div = e0 + e1 + e2, d3 = div * (1.0 / 3.0);
     const double *p1 = S.pr[1], *p2 = S.pr[2];
     const double xz = (p1[e] + p1[e + 1]) + (p1[e + pl] + p1[e + pl + 1]);
     const double yz = (p2[e] + p2[e + px]) + (p2[e + pl] + p2[e + pl + px]);
-    const double t0 = fma(0.25, xy + xz, fma(two_eta, e0 - d3, S.tbn[0][e]));
-    const double t1 = fma(0.25, yz - xy, fma(two_eta, e1 - d3, S.tbn[1][e]));
-    const double t2 = fma(-0.25, xz + yz, fma(two_eta, e2 - d3, S.tbn[2][e]));
+    const double t0 = fma(0.25, xy + xz, fma(two_eta, fma(d0, g.rdx, d3), S.tbn[0][e]));
+    const double t1 = fma(0.25, yz - xy, fma(two_eta, fma(d1, g.rdy, d3), S.tbn[1][e]));
+    const double t2 = fma(-0.25, xz + yz, fma(two_eta, fma(d2, g.rdz, d3), S.tbn[2][e]));
     S.Tn[0][e] = fma(bt, S.son[0][e], ob * t0);
     S.Tn[1][e] = fma(bt, S.son[1][e], ob * t1);
     S.Tn[2][e] = fma(bt, S.son[2][e], ob * t2);

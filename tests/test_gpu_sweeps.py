@@ -245,17 +245,16 @@ def test_commit_of_an_undecided_solve_with_a_per_cell_modulus(P, n):
 
 
 @pytest.mark.parametrize("n", [(61, 33), (130, 90), (300, 180)])
-@pytest.mark.parametrize("precision", ["fp64", "fp32"])
-def test_elastic_iterations_without_rotation_round_alike_in_every_2d_kernel(P, n, precision):
+def test_elastic_iterations_without_rotation_round_alike_in_every_fp32_2d_kernel(P, n):
     """The deviatoric rate is formed first and scaled once, in one order: strips, the launches per
     iteration and the resident iterations give the same bits where neither the return nor the
-    rotation's means (whose sums each kernel shares in its own way) take part."""
+    rotation's means (whose sums each kernel shares in its own way) take part.  (In FP64 the
+    compiler contracts the strips' products and sums, which are not packed there.)"""
     f = _fields(P, 2, n, 15)
-    pr = P.FP64 if precision == "fp64" else P.FP32_MIXED
     opts = dict(chunk=6, jaumann=False, elastic=True)
-    _, ref = _solve(P, 2, n, pr, P.KERNEL_FUSED, 24, f, shape=4, **opts)
+    _, ref = _solve(P, 2, n, P.FP32_MIXED, P.KERNEL_FUSED, 24, f, shape=4, **opts)
     for kernel in (P.KERNEL_STAGED, P.KERNEL_AUTO):
-        _, out = _solve(P, 2, n, pr, kernel, 24, f, **opts)
+        _, out = _solve(P, 2, n, P.FP32_MIXED, kernel, 24, f, **opts)
         for k in out:
             np.testing.assert_array_equal(out[k], ref[k])
 

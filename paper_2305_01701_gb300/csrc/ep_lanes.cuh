@@ -53,7 +53,7 @@ __device__ __forceinline__ double el(double v) { return v; }
 // quotient but for near-ties (0.5 ulp; a rounded root and a division make 1.5): an error of the
 // scale acts on the same cells in every iteration (95^3 with a per-cell modulus, error against
 // 64 bits after 200 of them, median of 16 inputs over that of sqrt and division: 0.99, without
-// the residuals 1.01; 55.8 -> 57.4 us an iteration, 67 with sqrt and division).  FP64: below
+// the residuals 1.01; 55.8 -> 56.5 us an iteration, 67 with sqrt and division).  FP64: below
 // Y^2 by more than the rounding of both, sqrt(J2) > Y cannot hold and the scale is 1 without
 // the root.
 __device__ __forceinline__ float scale_of(float J2, float Y) {
@@ -69,8 +69,21 @@ __device__ __forceinline__ double scale_of(double J2, double Y) {
   const double sj = sqrt(J2);
   return sj > Y ? Y / sj : 1.0;
 }
+// both columns in packed arithmetic where either yields (a warp's neighbours mostly yield
+// together), each with the result of its own scale_of
 __device__ __forceinline__ float2 vscale(float2 J2, float2 Y) {
-  return make_float2(scale_of(J2.x, Y.x), scale_of(J2.y, Y.y));
+  Y = make_float2(Y.x > 0.f ? Y.x : 0.f, Y.y > 0.f ? Y.y : 0.f);
+  const float2 Y2 = vmul(Y, Y);
+  const bool ax = J2.x > Y2.x, ay = J2.y > Y2.y;
+  float2 out = make_float2(1.f, 1.f);
+  if (ax || ay) {
+    const float2 r = make_float2(rsqrtf(J2.x), rsqrtf(J2.y)), m1 = make_float2(-1.f, -1.f);
+    const float2 t = vmul(J2, r), d = vmul(vfma(vmul(t, m1), t, J2), vmul(r, make_float2(0.5f, 0.5f)));
+    const float2 s = vmul(Y, r), n = vmul(s, m1), q = vfma(vfma(n, d, vfma(n, t, Y)), r, s);
+    if (ax) out.x = !(J2.x < INFINITY) ? s.x : q.x > 1.f ? 1.f : q.x;
+    if (ay) out.y = !(J2.y < INFINITY) ? s.y : q.y > 1.f ? 1.f : q.y;
+  }
+  return out;
 }
 __device__ __forceinline__ double vscale(double J2, double Y) { return scale_of(J2, Y); }
 

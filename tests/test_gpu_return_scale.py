@@ -12,7 +12,15 @@ SOURCE = """
 #include "ep_lanes.cuh"
 static __global__ void k(const float *J2, const float *Y, float *s, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) s[i] = ep::scale_of(J2[i], Y[i]);
+  if (i >= n) return;
+  s[i] = ep::scale_of(J2[i], Y[i]);
+  // a pair's scales are those of its members, in either place
+  const int j = i ^ 1;
+  if (j < n) {
+    const float2 a = ep::vscale(make_float2(J2[i], J2[j]), make_float2(Y[i], Y[j]));
+    const float2 b = ep::vscale(make_float2(J2[j], J2[i]), make_float2(Y[j], Y[i]));
+    if (__float_as_uint(a.x) != __float_as_uint(s[i]) || __float_as_uint(b.y) != __float_as_uint(s[i])) s[i] = -1.f;
+  }
 }
 extern "C" int scale_of(const float *J2, const float *Y, float *s, int n) {
   k<<<(n + 255) / 256, 256>>>(J2, Y, s, n);

@@ -519,7 +519,7 @@ NCU_SOURCE = {("k_fused3d_reg", 127): "ncu capture of one launch at 127^3 (profi
                                       "traffic scaled to 511^3 by the cell count"}
 # FP64 flops per cell of one staged FP64 sweep (dadd + dmul + 2 dfma thread
 # instructions of its five kernels, counted by ncu at 127^3; profiles/)
-FP64_FLOPS_PER_CELL = 206.4
+FP64_FLOPS_PER_CELL = 207.4
 # algorithmic bytes per cell of a 3D FP32 sweep recast so that its stress is
 # no pseudo-time state (reported beside the fraction by the scheme's bytes)
 RECAST_BYTES_3D_FP32 = 80.0

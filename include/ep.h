@@ -53,8 +53,10 @@ typedef enum {
 } ep_status;
 
 /* EP_FP64: every sweep in FP64.  EP_FP32_MIXED: sweeps in FP32 on the
- * velocity increment of the current load increment, with FP64 residual
- * norms, convergence test, start-of-increment base state and history. */
+ * velocity increment of the current load increment, with an FP64
+ * convergence test, start-of-increment base state and history.  The measures
+ * that the test reads are formed in FP64 by the 2D sweeps and are maxima of
+ * FP32 values in 3D. */
 typedef enum { EP_FP64 = 0, EP_FP32_MIXED = 1 } ep_precision;
 
 /* pure-shear loading planes (Eqs. A7-A9M): XY is v_x = a x, v_y = -a y

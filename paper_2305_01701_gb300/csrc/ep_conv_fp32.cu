@@ -21,8 +21,8 @@
 //   writes its partial sums, and k_wgrad_sum adds them in a fixed order (the
 //   gradient is the same bit for bit on every call).
 // Measured on the 64^3 network (base 32, two samples): forward and backward
-// 20.4 ms against 223 ms with one thread per voxel (or weight) reading global
-// memory; the 32 -> 32 convolution of 524,288 voxels 0.69 ms = 42 TFLOP/s, its
+// 18.85 ms against 223 ms with one thread per voxel (or weight) reading global
+// memory (58 - 60 % of the issue slots, the FMA pipe's throttle the first stall); the 32 -> 32 convolution of 524,288 voxels 0.69 ms = 42 TFLOP/s, its
 // weight gradient 0.72 ms.
 #include <cuda_bf16.h>
 #include <math.h>

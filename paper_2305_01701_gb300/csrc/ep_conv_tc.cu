@@ -21,11 +21,13 @@
 // applies the ReLU and writes what the next layer reads: BF16 blocks, the 2^D
 // average (FP32 sums), the nearest upsample, each straight into its place in the
 // decoder's concatenation, or the 1^D head's FP32 output.
-// Bound: at NB = 32 the read of A from shared memory (4 KB per 32 cycles),
-// half the tensor peak; small volumes are bound by latency.  Measured on the
-// 64^3 network (base 32): 0.40 ms for the pass (32 -> 32
-// channels 51 us, 96 -> 32 102 us), against 2.3 ms with a box of 8 channels per tap and
-// FP32 tensors between the layers.
+// Bound: one CTA of four warps per SM goes through its phases one after the other
+// (the first box, the MMAs, the epilogue), so the tensor pipe is active 12 - 21 % of the
+// time on the 64^3 layers and 36 - 41 % on the 16^3 ones (16 CTAs of 152); within the MMAs
+// at NB = 32 the read of A from shared memory (4 KB per 32 cycles; L1 at 31 - 53 % of its
+// rate over the kernel) allows half the tensor peak.  Measured on the 64^3 network (base
+// 32): 0.417 ms for the pass (32 -> 32 channels 52 us, 96 -> 32 104 us), against 2.3 ms
+// with a box of 8 channels per tap and FP32 tensors between the layers.
 // Every wait is bounded; a wait that runs out sets the error word, the block
 // waits (bounded) for the copies it issued, frees its tensor memory and ends.
 #include <cuda.h>

@@ -21,7 +21,7 @@
 // SM three FP32 blocks (519 us a sweep), so the compiler is held to 128.
 // Warps take items independently, so a block never waits for another warp.
 // 256 grids of 127^2 .. 511^2, one sweep: FP32 is bound by the 20 arrays it
-// moves, 465 us (5.5 TB/s; one column a thread and two rows ahead: 773 us; two
+// moves, 464 us (5.6 TB/s; one column a thread and two rows ahead: 773 us; two
 // columns and two rows ahead 168 registers, 12 warps an SM: 511 us, at 128
 // registers with spills 638 us); FP64 (64 grids) by the FP64 pipe.
 #include <math.h>

@@ -23,15 +23,15 @@
 // plane t-1, centres t-1, edges t-1 and velocities t-2.  Three block barriers
 // separate the steps of a plane.
 // Bound: HBM in principle (132 B per cell); in fact the latency of a plane's
-// three steps at 12 warps per SM.  Measured (FP32, one sweep): 127^3 77.2 us,
-// 383^3 1575 us (4.7 TB/s), against 126.9 and 2312 us of the form with one
+// three steps at 12 warps per SM.  Measured (FP32, one sweep): 127^3 80.5 us,
+// 383^3 1611 us (4.6 TB/s), against 126.9 and 2312 us of the form with one
 // column per thread (16 warps, 600 instructions per warp and plane, register
 // prefetch).  Packing the pairs alone, with the register prefetch (8 warps of
 // 255 registers), halved the instructions and gained nothing: the loads'
 // latency showed.  cp.async in place of TMA cost 5 shared-memory wavefronts
 // per 8-byte copy (the window starts off a 32-byte sector): 131 and 2164 us.
-// With a per-cell shear modulus (31 inputs, 16 rows) 95^3 takes 55 us, the five
-// staged kernels 100.
+// With a per-cell shear modulus (31 inputs, 16 rows) 95^3 takes 56 us, the five
+// staged kernels 100 to 124.
 // Instruction count:
 //   * FP32 arithmetic is packed (add/mul/fma on float2: one instruction per
 //     pair);
@@ -754,8 +754,8 @@ bool launch_fused3d_reg(const Geo &g, const Stage<T> &S, const Scal *sc, DevInfo
   } else {
     // a plane takes a 16-row block 1.5 us and a 24-row one 2.0 us; the 24 rows write
     // 20 of theirs, the 16 rows 12, but need fewer planes per block where the grid is
-    // small (90x40x24 12.2 against 15.8 us a sweep, 63^3 19.8 / 22.3; 127^3 92.8 / 77.2,
-    // 383^3 1757 / 1575)
+    // small (90x40x24 13.0 against 16.6 us a sweep, 63^3 21.2 / 23.4; 127^3 95.8 / 79.5,
+    // 383^3 1814 / 1619)
     long long c16 = 0, c24 = 0;
     const int k16 = fused3d_kz(extent(g), OX, 12, kz, 1, &c16), k24 = fused3d_kz(extent(g), OX, 20, kz, 1, &c24);
     if (3 * c16 < 4 * c24) return launch_off<LaneF<16>, false, false>(S, A, g, sc, di, k16, st);

@@ -19,9 +19,11 @@
 //
 // Bound: latency of the exchange and of four block barriers; FP64 grids the FP64 pipe
 // as well, which takes a warp's instruction in 64 cycles.
-// Measured, an iteration against two launches: FP64 64^2 8.0 -> 4.0 us, 128^2 8.9 -> 6.5;
-// FP32 64^2 5.8 -> 1.6, 128^2 6.3 -> 1.8, 383 x 191 9.0 -> 2.7, 300^2 9.2 -> 2.9 (a
-// counter per block behind a fence: 64^2 FP64 7.5 us, 383 x 191 FP32 5.8).
+// Measured, an iteration against two launches (a box near yield, checks every 1000): FP64
+// 64^2 9.1 -> 4.3 us, 128^2 10.3 -> 6.8; FP32 64^2 8.0 -> 1.1, 128^2 8.3 -> 1.3, 383 x 191
+// 12.1 -> 1.7, 300^2 12.5 -> 1.7 (a counter per block behind a fence, when the words were
+// not yet 16 bytes wide: 64^2 FP64 7.5 us, 383 x 191 FP32 5.8).  FP64 64^2: 6 % of the issue
+// slots, warps wait on the FP64 pipe (7.0 a warp instruction), barriers (2.9) and the words.
 #include <math.h>
 
 #include "ep_internal.cuh"

@@ -22,12 +22,14 @@
 //
 // Bound: shared memory and instruction issue of one block per SM, and the latency of two
 // exchanges and five barriers.
-// Measured, an iteration against the register sweep's launch: 16^3 8.5 -> 3.9 us, 32^3 10.8
-// -> 6.5, 44^3 12.4 -> 6.8, 90 x 40 x 24 12.7 -> 8.2 (of 14,900 cycles there phases 1 - 5
-// take 1,500, 2,800, 2,300, 750 and 1,300 and the exchanges 6,200); two grids solved
-// at once 20.1 -> 15.4 ms for 1000 iterations each, four 39.9 -> 31.0.  A spilled
-// register costs an L2 trip here, since shared memory leaves L1 no room (30 spilled loads a
-// warp and iteration: 9.3 us): what a thread keeps of its edges sits in shared memory.
+// Measured, an iteration against the register sweep's launch (a box near yield, checks every
+// 1000): 16^3 9.2 -> 3.5 us, 32^3 11.4 -> 6.2, 44^3 13.1 -> 6.2, 90 x 40 x 24 13.3 -> 7.6 (of
+// 14,900 cycles there phases 1 - 5 take 1,500, 2,800, 2,300, 750 and 1,300 and the exchanges
+// 6,200; 54 % of L1's rate, stalls on barriers 5.4, words 3.6 and shared memory 4.5 a warp
+// instruction); two grids solved at once 20.1 -> 15.4 ms for 1000 iterations each, four
+// 39.9 -> 31.0.  A spilled register costs an L2 trip here, since shared memory leaves L1 no
+// room (30 spilled loads a warp and iteration: 9.3 us): what a thread keeps of its edges sits
+// in shared memory.
 #include <math.h>
 
 #include "ep_internal.cuh"

@@ -12,7 +12,7 @@
 // and shear rates stay unscaled (w = 2 omega, g = 2 eps).
 // Bound: launch and load latency on one grid (a few rows per warp, so that the
 // whole chip works on it), the FP64 pipe on large FP64 grids.  Measured, an
-// iteration: FP64 64^2 17.2 -> 8.4 us, 511^2 76.5 -> 47.5 us against five stages
+// iteration: FP64 64^2 17.2 -> 8.4 us, 511^2 76.5 -> 45.4 us against five stages
 // (12.7 and 50.5 us for five stages with the same arithmetic and as many blocks);
 // FP32 383 x 191 10.1 -> 9.0 us, 1000 x 700 48.9 -> 22.7 us against one launch of tiles
 // in shared memory (warp strips: 35 us).

@@ -16,8 +16,8 @@
 //     the pressure once, in the centre return;
 //   * the square root and the division of the return run only where J2 is within
 //     rounding of Y^2 or above (elsewhere the scale is exactly 1).
-// Measured, an iteration at 127^3: 1129 -> 639 us (157 FP64 operations per cell are
-// 510 us of the pipe).  A warp covers 32 points along x; blocks hold as many rows as leave every SM some (launch_rows).
+// Measured, an iteration at 127^3: 1129 -> 639 us (156 FP64 operations per cell are
+// 506 us of the pipe).  A warp covers 32 points along x; blocks hold as many rows as leave every SM some (launch_rows).
 #include <math.h>
 
 #include <algorithm>
